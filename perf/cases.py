@@ -288,7 +288,8 @@ def work(case):
 def tolerance(case):
     # Results are bf16, rounded once (2^-9 at most, 1.7e-3 in the 2-norm); the gradients of a layer
     # with an activation come from a derivative rounded to bf16 in the same way, and the adapters'
-    # from two such intermediates. Against products in 64 bits the results measure 1.6e-3 to 3.0e-3 (fp32 gradients without such an intermediate, 4e-7).
+    # from two such intermediates. Against products in 64 bits the results measure 1.6e-3 to 3.0e-3
+    # (fp32 gradients without such an intermediate: 4e-7).
     if case["kind"] == "cast":
         return "exact"
     return {"rel": 1e-2}
