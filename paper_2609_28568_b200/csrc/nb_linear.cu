@@ -18,6 +18,7 @@
 #include "gemm_sm100.cuh"
 #include "layer_bwd_sm100.cuh"
 #include "lora_udb_sm100.cuh"
+#include "rows_sm100.cuh"
 
 namespace {
 
@@ -352,6 +353,70 @@ using FwdStoreNarrow = GemmCfg<1, 64, 7, 2, false, false, kEpiStore>;
 using DgradStoreNarrow = GemmCfg<1, 64, 7, 2, false, true, kEpiStore>;
 using WgradF32Narrow = GemmCfg<1, 64, 7, 2, true, true, kEpiF32>;
 constexpr int kNarrowN = 64;
+
+// ----------------------------------------------------------------------------- small problems
+// Launch configuration: cluster size along x, and dependent launch where it is allowed.
+void small_launch_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attrs)[2], int ctas, int threads, int cluster,
+                         uint32_t smem_bytes, cudaStream_t stream)
+{
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(static_cast<unsigned>(ctas));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = stream;
+    unsigned n = 0;
+    if (cluster > 1) {
+        attrs[n].id = cudaLaunchAttributeClusterDimension;
+        attrs[n].val.clusterDim.x = static_cast<unsigned>(cluster);
+        attrs[n].val.clusterDim.y = 1;
+        attrs[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if (dependent_launch_allowed(stream)) {
+        attrs[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attrs[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    cfg.attrs = attrs;
+    cfg.numAttrs = n;
+}
+
+// A forward product on at most kRowsMax rows. K is shared among a cluster when it is long (48 CTAs
+// of 16 features took 7.9 us for K = 3072, and 2.7 us for K = 768), as far as two CTAs per SM go.
+template <int NT, int EPI, bool MANY>
+int launch_rows(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
+{
+    RowsParams p;
+    memset(&p, 0, sizeof(p));
+    p.inp = static_cast<const __nv_bfloat16 *>(a.A);
+    p.weight = static_cast<const __nv_bfloat16 *>(a.B);
+    p.bias = static_cast<const __nv_bfloat16 *>(a.bias);
+    p.out = static_cast<__nv_bfloat16 *>(a.D);
+    p.pre = static_cast<__nv_bfloat16 *>(const_cast<void *>(a.E));
+    p.M = a.M;
+    p.K = a.K;
+    p.N = a.N;
+    p.swiglu_h = a.swiglu_h;
+    const int span = EPI == kEpiSwiglu ? a.swiglu_h : a.N;
+    const int groups = (span + kRowsFeatures - 1) / kRowsFeatures;
+    p.ksplit = 1;
+    while (p.ksplit < kRowsMaxSplit && a.K >= 1024 * p.ksplit && groups * p.ksplit <= s.num_sms) p.ksplit *= 2;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attrs[2];
+    small_launch_config(cfg, attrs, groups * p.ksplit, kRowsThreads, p.ksplit, 0, stream);
+    NB_CUDA(cudaLaunchKernelEx(&cfg, rows_kernel<NT, EPI, MANY>, p));
+    ++g_launches;
+    return NB_OK;
+}
+
+template <int EPI>
+int launch_rows_auto(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
+{
+    const int span = EPI == kEpiSwiglu ? a.swiglu_h : a.N;
+    const bool many = span > 3 * s.num_sms * kRowsFeatures;
+    if (a.M <= 8) return many ? launch_rows<1, EPI, true>(s, a, stream) : launch_rows<1, EPI, false>(s, a, stream);
+    return launch_rows<2, EPI, false>(s, a, stream);
+}
 
 bool use_pairs(int M)
 {
@@ -763,6 +828,21 @@ int run_layer_bwd(DeviceState &s, const void *dz, const void *weight, const void
     return launch_layer_bwd<LayerBwdPlain>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, stream);
 }
 
+// A forward product with its activation: on a few rows the row kernel (9 to 16 rows only up to 8 CTAs
+// per SM: 16 rows, 768 -> 50304 takes 21 us there and 17 us in gemm_kernel).
+int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
+{
+    const bool adapter = a.A2 != nullptr;
+    if (!adapter && (a.M <= 8 || (a.M <= kRowsMax && a.N <= 8 * s.num_sms * kRowsFeatures))) {
+        if (act == NB_ACT_NONE) return launch_rows_auto<kEpiStore>(s, a, stream);
+        if (act == NB_ACT_GELU) return launch_rows_auto<kEpiGelu>(s, a, stream);
+        return launch_rows_auto<kEpiSwiglu>(s, a, stream);
+    }
+    if (act == NB_ACT_SWIGLU) return launch_gemm_auto<FwdSwiglu1, FwdSwiglu2>(s, a, stream);
+    if (act == NB_ACT_GELU) return launch_gemm_auto<FwdGelu1, FwdGelu2>(s, a, stream);
+    return launch_gemm_auto<FwdStore1, FwdStore2>(s, a, stream);
+}
+
 }  // namespace
 
 // ================================================================================ C ABI
@@ -817,15 +897,13 @@ int nb_linear_forward_ex(void *out, void *pre_act, const void *inp, const void *
     a.M = static_cast<int>(BT); a.N = static_cast<int>(OC); a.K = static_cast<int>(C);
     a.bias = bias;
     a.splits = 1;
-    if (act == NB_ACT_NONE) return launch_gemm_auto<FwdStore1, FwdStore2>(*s, a, stream);
-    if (!pre_act) {
+    if (act != NB_ACT_NONE && !pre_act) {
         // the activated result without its pre-activation: only NONE can skip the second plane
         return fail(NB_ERR_INVALID_ARG, "pre_act must be given when act != NONE");
     }
-    a.E = pre_act; a.e_rows = BT; a.e_cols = OC;
-    if (act == NB_ACT_GELU) return launch_gemm_auto<FwdGelu1, FwdGelu2>(*s, a, stream);
-    a.swiglu_h = static_cast<int>(OC / 2);
-    return launch_gemm_auto<FwdSwiglu1, FwdSwiglu2>(*s, a, stream);
+    if (act != NB_ACT_NONE) { a.E = pre_act; a.e_rows = BT; a.e_cols = OC; }
+    if (act == NB_ACT_SWIGLU) a.swiglu_h = static_cast<int>(OC / 2);
+    return run_forward(*s, a, act, stream);
 }
 
 int nb_linear_forward(void *out, const void *inp, const void *weight, const void *bias, int64_t BT,

@@ -313,6 +313,11 @@ __device__ __forceinline__ void tmem_ld_32x32_x2_wait(uint32_t taddr0, uint32_t 
 }
 
 // ------------------------------------------------------------------ shared memory access
+// two floats from the shared memory of a CTA of the cluster
+__device__ __forceinline__ void ld_cluster_f32x2(uint32_t addr, float2 &v)
+{
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+}
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c,
                                              uint32_t d)
 {
