@@ -19,6 +19,7 @@
 #include "layer_bwd_sm100.cuh"
 #include "lora_udb_sm100.cuh"
 #include "rows_sm100.cuh"
+#include "tile_sm100.cuh"
 
 namespace {
 
@@ -381,6 +382,153 @@ void small_launch_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attrs)[2
     cfg.numAttrs = n;
 }
 
+constexpr uint32_t kTileSmemTwo = 113u * 1024u;  // two CTAs on an SM
+constexpr uint32_t kTileSmemOne = 200u * 1024u;
+
+// Fills a job (and the shared memory it needs) for D[M, N] in BN-wide tiles, K split over `cluster`.
+// two: the ring leaves room for a second CTA on the SM.
+template <int BN>
+void fill_tile_job(TileJob &j, uint32_t &smem_bytes, const GemmArgs &a, int epi, bool a_mn, int cluster, bool two)
+{
+    using G = TileGeom<BN>;
+    memset(&j, 0, sizeof(j));
+    const bool swiglu = epi == kEpiSwiglu;
+    j.M = a.M;
+    j.N = a.N;
+    j.tiles_m = (a.M + kBlockM - 1) / kBlockM;
+    const int span = swiglu ? BN / 2 : BN, n = swiglu ? a.swiglu_h : a.N;
+    j.tiles_n = (n + span - 1) / span;
+    j.kblocks = (a.K + kBlockK - 1) / kBlockK;
+    j.kblocks_ext = (a.A2 && a.B2 && a.k2 > 0) ? (a.k2 + kBlockK - 1) / kBlockK : 0;
+    // a K-major A tile is one box; a single row tile of fewer than 128 rows is fetched (and kept) as
+    // just those rows
+    const uint32_t rows = !a_mn && a.M < kBlockM ? static_cast<uint32_t>((a.M + 7) / 8 * 8) : kBlockM;
+    j.a_slot = rows * 128u;
+    j.ctas = j.tiles_m * j.tiles_n * cluster;
+    j.alpha = a.alpha == 0.0f ? 1.0f : a.alpha;
+    j.bias = static_cast<const __nv_bfloat16 *>(a.bias);
+    j.D = static_cast<__nv_bfloat16 *>(a.D);
+    j.d_ld = static_cast<long long>(a.d_ld ? a.d_ld : a.d_cols);
+    j.E = static_cast<__nv_bfloat16 *>(const_cast<void *>(a.E));
+    j.e_ld = static_cast<long long>(a.e_cols);
+    j.swiglu_h = a.swiglu_h;
+    j.reduce = a.reduce;
+    const uint32_t recv = cluster > 1 ? G::RECV_BYTES : 0u;
+    const uint32_t stage = j.a_slot + G::B_BYTES;
+    const int longest = (j.kblocks + cluster - 1) / cluster + j.kblocks_ext;
+    auto fit = [&](uint32_t budget) { return static_cast<int>((budget - recv - G::TAIL_BYTES) / stage); };
+    int st = fit(two ? kTileSmemTwo : kTileSmemOne);
+    if (st < 2) st = fit(kTileSmemOne);
+    if (st > kTileMaxStages) st = kTileMaxStages;
+    if (st > longest) st = longest;
+    // the result is staged in the drained stages' memory: 4 bytes an element (fp32, or bf16 result and
+    // pre-activation) or 2, for the 32-row quarters that hold rows; SwiGLU: three planes of half a tile
+    const uint32_t quarters = a.M < kBlockM ? static_cast<uint32_t>((a.M + 31) / 32) : 4u;
+    const uint32_t elem = epi == kEpiF32 || epi == kEpiGelu ? 4u : swiglu ? 3u : 2u;
+    const uint32_t staged = (epi == kEpiF32 ? 4u : quarters) * 32u * BN * elem;
+    const int min_st = cluster > 1 ? 1 : static_cast<int>((staged + stage - 1) / stage);
+    if (st < min_st) st = min_st;
+    j.stages = st;
+    smem_bytes = static_cast<uint32_t>(st) * stage + recv + G::TAIL_BYTES;
+    // the tensor core reads 128 rows from every A slot
+    const uint32_t reach = static_cast<uint32_t>(st - 1) * j.a_slot + kBlockM * 128u;
+    if (smem_bytes < reach) smem_bytes = reach;
+}
+
+template <int BN, bool B_MN, int EPI>
+int launch_tile(DeviceState &s, const GemmArgs &a, int cluster, bool two, cudaStream_t stream)
+{
+    static bool attr_set[kMaxDevices] = {};
+    int dev = 0;
+    NB_CUDA(cudaGetDevice(&dev));
+    if (!attr_set[dev]) {
+        NB_CUDA(cudaFuncSetAttribute(tile_kernel<BN, B_MN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(kTileSmemOne)));
+        attr_set[dev] = true;
+    }
+    TileParams p;
+    memset(&p, 0, sizeof(p));
+    uint32_t smem_bytes = 0;
+    fill_tile_job<BN>(p.job[0], smem_bytes, a, EPI, false, cluster, two);
+    p.cluster = cluster;
+    p.status = s.status;
+    p.timeout_ns = kDefaultTimeoutNs;
+    const uint32_t a_box = p.job[0].a_slot / 128u;
+    const uint32_t b_box = B_MN || EPI == kEpiSwiglu ? 64u : static_cast<uint32_t>(BN);
+    CUtensorMap tA, tB, tA2, tB2;
+    int rc;
+    if ((rc = get_tmap(s, &tA, a.A, a.a_rows, a.a_cols, 0, a_box, a.a_ld)) != NB_OK) return rc;
+    if ((rc = get_tmap(s, &tB, a.B, a.b_rows, a.b_cols, 0, b_box, a.b_ld)) != NB_OK) return rc;
+    tA2 = tA;
+    tB2 = tB;
+    if (p.job[0].kblocks_ext > 0) {
+        if ((rc = get_tmap(s, &tA2, a.A2, a.a2_rows, a.a2_cols, 0, a_box, a.a2_ld)) != NB_OK) return rc;
+        if ((rc = get_tmap(s, &tB2, a.B2, a.b2_rows, a.b2_cols, 0, b_box)) != NB_OK) return rc;
+    }
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attrs[2];
+    small_launch_config(cfg, attrs, p.job[0].ctas, kTileThreads, cluster, smem_bytes, stream);
+    NB_CUDA(cudaLaunchKernelEx(&cfg, tile_kernel<BN, B_MN, EPI>, tA, tB, tA2, tB2, p));
+    ++g_launches;
+    return NB_OK;
+}
+
+// Two products in one launch (tile_pair_kernel): `d` a bf16 result with a B operand that is read
+// MN-major (null: none), `w` an fp32 one with both operands MN-major (dbias optional).
+template <int BN, bool GELU_GRAD>
+int launch_tile_pair(DeviceState &s, const GemmArgs *d, const GemmArgs &w, int accumulate, int cluster, bool two,
+                     cudaStream_t stream)
+{
+    static bool attr_set[kMaxDevices] = {};
+    int dev = 0;
+    NB_CUDA(cudaGetDevice(&dev));
+    if (!attr_set[dev]) {
+        NB_CUDA(cudaFuncSetAttribute(tile_pair_kernel<BN, GELU_GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(kTileSmemOne)));
+        attr_set[dev] = true;
+    }
+    TileParams p;
+    memset(&p, 0, sizeof(p));
+    uint32_t smem_d = 0, smem_w = 0;
+    fill_tile_job<BN>(p.job[1], smem_w, w, kEpiF32, true, 1, two);
+    p.job[1].reduce = accumulate ? 1 : 0;
+    p.job[1].dbias = w.dbias;
+    p.job[1].dbias_add = accumulate ? 1 : 0;
+    p.cluster = cluster;
+    p.status = s.status;
+    p.timeout_ns = kDefaultTimeoutNs;
+    CUtensorMap tA0, tB0, tA2, tB2, tA1, tB1, tD1;
+    int rc;
+    if ((rc = get_tmap(s, &tA1, w.A, w.a_rows, w.a_cols, 0, 64, w.a_ld)) != NB_OK) return rc;
+    if ((rc = get_tmap(s, &tB1, w.B, w.b_rows, w.b_cols, 0, 64, w.b_ld)) != NB_OK) return rc;
+    if ((rc = get_tmap(s, &tD1, w.D, w.d_rows, w.d_cols, 1, 32)) != NB_OK) return rc;
+    tA0 = tA1;  // never read without d, nor the second pair without an adapter term
+    tB0 = tB1;
+    if (d) {
+        fill_tile_job<BN>(p.job[0], smem_d, *d, GELU_GRAD ? kEpiMulGeluGrad : kEpiStore, false, cluster, two);
+        const uint32_t a_box = p.job[0].a_slot / 128u;
+        if ((rc = get_tmap(s, &tA0, d->A, d->a_rows, d->a_cols, 0, a_box, d->a_ld)) != NB_OK) return rc;
+        if ((rc = get_tmap(s, &tB0, d->B, d->b_rows, d->b_cols, 0, 64, d->b_ld)) != NB_OK) return rc;
+        tA2 = tA0;
+        tB2 = tB0;
+        if (p.job[0].kblocks_ext > 0) {
+            if ((rc = get_tmap(s, &tA2, d->A2, d->a2_rows, d->a2_cols, 0, a_box, d->a2_ld)) != NB_OK) return rc;
+            if ((rc = get_tmap(s, &tB2, d->B2, d->b2_rows, d->b2_cols, 0, 64)) != NB_OK) return rc;
+        }
+    } else {
+        tA2 = tA0;
+        tB2 = tB0;
+    }
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attrs[2];
+    int ctas = p.job[0].ctas + p.job[1].ctas;
+    ctas = (ctas + cluster - 1) / cluster * cluster;
+    small_launch_config(cfg, attrs, ctas, kTileThreads, cluster, smem_d > smem_w ? smem_d : smem_w, stream);
+    NB_CUDA(cudaLaunchKernelEx(&cfg, tile_pair_kernel<BN, GELU_GRAD>, tA0, tB0, tA2, tB2, tA1, tB1, tD1, p));
+    ++g_launches;
+    return NB_OK;
+}
+
 // A forward product on at most kRowsMax rows. K is shared among a cluster when it is long (48 CTAs
 // of 16 features took 7.9 us for K = 3072, and 2.7 us for K = 768), as far as two CTAs per SM go.
 template <int NT, int EPI, bool MANY>
@@ -417,6 +565,126 @@ int launch_rows_auto(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
     if (a.M <= 8) return many ? launch_rows<1, EPI, true>(s, a, stream) : launch_rows<1, EPI, false>(s, a, stream);
     return launch_rows<2, EPI, false>(s, a, stream);
 }
+
+// What the forms of a product take, in microseconds: a fit to chained launches on B200 (1..2048 rows,
+// 768..3072 columns), good to about 15 %. They decide between kernels of very different shape, so
+// where two are close either will do.
+//
+// A CTA of the small-problem kernel: launch, set-up and epilogue, then 64-wide k-blocks. A k-block
+// costs the MMA issuer about 300 cycles whatever BN is, and more when many SMs load at once.
+struct SmallPlan {
+    int bn = 0, cluster = 1;  // bn == 0: the persistent kernels
+    bool two = false;         // ring sized for two CTAs on an SM
+    double us = 0;
+};
+constexpr double kLaunchUs = 1.0;
+
+double small_cta_us(int bn, double kblocks, int rows, int ctas, bool two)
+{
+    const double part = (rows < kBlockM ? rows : kBlockM) / 128.0 * bn / 64.0;
+    const double stage_kb = 16.0 + bn / 8.0;
+    return 1.45 + 0.5 * part + kblocks * ((two ? (bn == 128 ? 0.30 : 0.18) : 0.152) + 1e-5 * ctas * stage_kb);
+}
+// adding up the parts of a cluster that shares K
+double small_exchange_us(int bn, int rows)
+{
+    return 1.0 + 1.4 * (rows < kBlockM ? rows : kBlockM) / 128.0 * bn / 64.0;
+}
+// gemm_kernel: waves of 128 (256) x 256 tiles, 512 tensor-core cycles per k-block
+double persistent_us(int sms, int M, int N, int kblocks)
+{
+    const int tm = M > kBlockM ? 2 * kBlockM : kBlockM;
+    const long long tiles = 1ll * ((M + tm - 1) / tm) * ((N + 255) / 256);
+    const int slots = M > kBlockM ? sms / 2 : sms;
+    return 5.3 + 0.27 * kblocks * static_cast<double>((tiles + slots - 1) / slots);
+}
+
+// Tile width and K split for one product D[M, N] over `kblocks`. The tiles have to fit the chip in one
+// wave; with more of them the persistent kernels, which overlap one tile's epilogue with the next
+// one's main loop, are as fast or faster (1024 rows, 768 -> 3072, 192 tiles: 9.2 us either way).
+// `other` is what the alternative takes; split: 0 any split of K, else that one.
+SmallPlan plan_single(int sms, int M, int N, int kblocks, bool allow32, int split, int min_bn, double other)
+{
+    SmallPlan best;
+    best.us = other;
+    for (int bn = allow32 ? 32 : 64; bn <= 128; bn *= 2) {
+        if (bn < min_bn) continue;
+        const long long tiles = 1ll * ((M + kBlockM - 1) / kBlockM) * ((N + bn - 1) / bn);
+        if (tiles > sms) continue;
+        for (int cl = split ? split : 1; cl <= (split ? split : 8); cl *= 2) {
+            // a cluster lies within one GPC: not every SM finds a place in clusters of 4 or 8
+            if (tiles * cl > sms * (cl >= 8 ? 0.86 : cl >= 4 ? 0.95 : 1.0) || bn / cl < 8 || (cl > 1 && 2 * cl > kblocks)) break;
+            const double us = kLaunchUs + small_cta_us(bn, (kblocks + cl - 1) / cl, M, static_cast<int>(tiles * cl), false) +
+                              (cl > 1 ? small_exchange_us(bn, M) : 0.0);
+            if (us < best.us) best = SmallPlan{bn, cl, false, us};
+        }
+    }
+    return best;
+}
+
+// The same for a bf16 product D[M, N] (M == 0: none) and an fp32 product [Mw, Nw] over kw k-blocks in
+// one launch; `other` is what the alternative takes, `split` as above.
+SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int Nw, int kw, bool dbias, double other, bool only64)
+{
+    SmallPlan best;
+    best.us = other;
+    for (int bn = 64; bn <= (only64 ? 64 : 128); bn *= 2) {
+        const long long nd = M > 0 ? 1ll * ((M + kBlockM - 1) / kBlockM) * ((N + bn - 1) / bn) : 0;
+        const long long nw = 1ll * ((Mw + kBlockM - 1) / kBlockM) * ((Nw + bn - 1) / bn);
+        if (nd + nw > 16ll * sms) continue;
+        for (int cl = nd && split ? split : 1; cl <= (!nd ? 1 : split ? split : 8); cl *= 2) {
+            if (bn / cl < 8 || (cl > 1 && 2 * cl > kblocks)) break;
+            for (int two = 0; two <= 1; ++two) {
+                const double slots = sms * (two ? 2.0 : 1.0);
+                const double n = static_cast<double>(nd * cl + nw);
+                if (cl > 1 && n > slots * (cl >= 8 ? 0.86 : 1.2)) continue;
+                const int crowd = static_cast<int>(n < slots ? n : slots);
+                const double td = nd ? small_cta_us(bn, (kblocks + cl - 1) / cl, M, crowd, two != 0) +
+                                           (cl > 1 ? small_exchange_us(bn, M) : 0.0) : 0.0;
+                const double tw = small_cta_us(bn, kw, Mw, crowd, two != 0) + (dbias ? kw * (bn == 128 ? 0.1 : 0.05) : 0.0);
+                double us = td > tw ? td : tw;
+                if (n > slots) {
+                    const double line = (nd * cl * td + nw * tw) / slots + 0.6 * tw;
+                    if (line > us) us = line;
+                }
+                us += kLaunchUs;
+                if (us < best.us) best = SmallPlan{bn, cl, two != 0, us};
+            }
+        }
+    }
+    return best;
+}
+
+// The split of K for dinp. It fixes the order of the sums, so it depends on the problem alone and not
+// on which other gradients are asked for in the same call; above 256 rows, where the weight gradient's
+// tiles join dinp's in the persistent kernel, there is none.
+int dinp_split(int sms, int M, int N, int kblocks)
+{
+    if (M > 2 * kBlockM) return 1;
+    const SmallPlan pl = plan_single(sms, M, N, kblocks, false, 0, 0, 1e9);
+    return pl.bn ? pl.cluster : 1;
+}
+
+template <bool B_MN, int EPI>
+int launch_tile_plan(DeviceState &s, const GemmArgs &a, const SmallPlan &pl, cudaStream_t stream)
+{
+    if constexpr (!B_MN)
+        if (pl.bn == 32) return launch_tile<32, B_MN, EPI>(s, a, pl.cluster, pl.two, stream);
+    if (pl.bn == 64) return launch_tile<64, B_MN, EPI>(s, a, pl.cluster, pl.two, stream);
+    return launch_tile<128, B_MN, EPI>(s, a, pl.cluster, pl.two, stream);
+}
+
+int launch_tile_pair_plan(DeviceState &s, const GemmArgs *d, const GemmArgs &w, bool gelu_grad, int accumulate,
+                          const SmallPlan &pl, cudaStream_t stream)
+{
+    if (gelu_grad)
+        return pl.bn == 64 ? launch_tile_pair<64, true>(s, d, w, accumulate, pl.cluster, pl.two, stream)
+                           : launch_tile_pair<128, true>(s, d, w, accumulate, pl.cluster, pl.two, stream);
+    return pl.bn == 64 ? launch_tile_pair<64, false>(s, d, w, accumulate, pl.cluster, pl.two, stream)
+                       : launch_tile_pair<128, false>(s, d, w, accumulate, pl.cluster, pl.two, stream);
+}
+
+int kblocks_of(int64_t K) { return static_cast<int>((K + kBlockK - 1) / kBlockK); }
 
 bool use_pairs(int M)
 {
@@ -829,7 +1097,8 @@ int run_layer_bwd(DeviceState &s, const void *dz, const void *weight, const void
 }
 
 // A forward product with its activation: on a few rows the row kernel (9 to 16 rows only up to 8 CTAs
-// per SM: 16 rows, 768 -> 50304 takes 21 us there and 17 us in gemm_kernel).
+// per SM: 16 rows, 768 -> 50304 takes 21 us there and 17 us in gemm_kernel), then the smaller of the
+// tile and the persistent kernel's estimates.
 int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
 {
     const bool adapter = a.A2 != nullptr;
@@ -838,9 +1107,47 @@ int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
         if (act == NB_ACT_GELU) return launch_rows_auto<kEpiGelu>(s, a, stream);
         return launch_rows_auto<kEpiSwiglu>(s, a, stream);
     }
-    if (act == NB_ACT_SWIGLU) return launch_gemm_auto<FwdSwiglu1, FwdSwiglu2>(s, a, stream);
-    if (act == NB_ACT_GELU) return launch_gemm_auto<FwdGelu1, FwdGelu2>(s, a, stream);
-    return launch_gemm_auto<FwdStore1, FwdStore2>(s, a, stream);
+    const int kb = kblocks_of(a.K) + (adapter ? 1 : 0);
+    const double other = persistent_us(s.num_sms, a.M, a.N, kb);
+    if (act == NB_ACT_SWIGLU) {
+        // 64 gate and 64 up columns per tile, so N counts both halves of the weight
+        const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, false, 1, 128, other);
+        if (pl.bn) return launch_tile<128, false, kEpiSwiglu>(s, a, 1, false, stream);
+        return launch_gemm_auto<FwdSwiglu1, FwdSwiglu2>(s, a, stream);
+    }
+    const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, true, 0, 0, other);
+    if (act == NB_ACT_GELU)
+        return pl.bn ? launch_tile_plan<false, kEpiGelu>(s, a, pl, stream) : launch_gemm_auto<FwdGelu1, FwdGelu2>(s, a, stream);
+    return pl.bn ? launch_tile_plan<false, kEpiStore>(s, a, pl, stream) : launch_gemm_auto<FwdStore1, FwdStore2>(s, a, stream);
+}
+
+// A layer's backward without the small-problem kernel: layer_bwd_kernel for both products, else a
+// launch per product. An fp32 result that starts from zero costs the clearing besides.
+double backward_us(int sms, int M, int BT, int N, int Mw, int kd, int kw, bool accumulate, bool apart)
+{
+    const int slots = sms / 2;
+    const double d_tiles = static_cast<double>((M + 255) / 256) * ((N + 255) / 256);
+    const double w_tiles = static_cast<double>((Mw + 255) / 256) * ((N + 255) / 256);
+    const double clear = accumulate ? 0.0 : 2.0;
+    if (M > 0 && BT > kBlockM && !apart) {
+        const double level = (d_tiles * (kd + 3) + w_tiles * (kw + 3)) / slots;
+        return 5.3 + clear + 0.27 * (d_tiles > 0 && kd > level ? kd : level);
+    }
+    const double waves = w_tiles / slots;
+    const double w_us = 5.0 + (waves < 1.0 ? 1.0 : waves) * (0.27 * (waves < 1.0 ? kw * waves : kw) + 0.8);
+    return w_us + clear + (M > 0 ? persistent_us(sms, M, N, kd) : 0.0);
+}
+
+// D = A . B with B read MN-major (dinp and its like), plain or times gelu'(E).
+int run_dgrad(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
+{
+    const int kb = kblocks_of(a.K) + (a.A2 ? 1 : 0);
+    const int split = dinp_split(s.num_sms, a.M, a.N, kb);
+    const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, false, split, 0, split > 1 ? 1e9 : persistent_us(s.num_sms, a.M, a.N, kb));
+    if (a.E)
+        return pl.bn ? launch_tile_plan<true, kEpiMulGeluGrad>(s, a, pl, stream)
+                     : launch_gemm_auto<DgradMulGelu1, DgradMulGelu2>(s, a, stream);
+    return pl.bn ? launch_tile_plan<true, kEpiStore>(s, a, pl, stream) : launch_gemm_auto<DgradStore1, DgradStore2>(s, a, stream);
 }
 
 }  // namespace
@@ -976,31 +1283,39 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
         dz = s->workspace;
     }
 
+    GemmArgs d, w;
+    memset(&d, 0, sizeof(d));  // dinp[BT, C] = dz[BT, OC] . W[OC, C]
+    d.A = dz; d.a_rows = BT; d.a_cols = OC;
+    d.B = weight; d.b_rows = OC; d.b_cols = C;
+    d.D = dinp; d.d_rows = BT; d.d_cols = C; d.d_dtype = 0;
+    d.M = static_cast<int>(BT); d.N = static_cast<int>(C); d.K = static_cast<int>(OC);
+    d.splits = 1;
+    if (inp_pre_act) { d.E = inp_pre_act; d.e_rows = BT; d.e_cols = C; }
+    const int kd = kblocks_of(OC), kw = kblocks_of(BT);
+    const int split = dinp ? dinp_split(s->num_sms, d.M, d.N, kd) : 1;
+    if (dweight && dweight_dtype == NB_DTYPE_F32) {
+        memset(&w, 0, sizeof(w));  // dweight[OC, C] (+)= dz^T[OC, BT] . inp[BT, C]
+        w.A = dz; w.a_rows = BT; w.a_cols = OC;
+        w.B = inp; w.b_rows = BT; w.b_cols = C;
+        w.D = dweight; w.d_rows = OC; w.d_cols = C; w.d_dtype = 1;
+        w.M = static_cast<int>(OC); w.N = static_cast<int>(C); w.K = static_cast<int>(BT);
+        w.splits = 1;
+        w.dbias = static_cast<float *>(dbias);
+        const SmallPlan pl = plan_pair(s->num_sms, dinp ? d.M : 0, d.N, kd, split, w.M, w.N, kw, dbias != nullptr,
+                                       backward_us(s->num_sms, dinp ? d.M : 0, d.M, d.N, w.M, kd, kw, accumulate != 0, split > 1), false);
+        if (pl.bn) return launch_tile_pair_plan(*s, dinp ? &d : nullptr, w, inp_pre_act != nullptr, accumulate, pl, stream);
+    }
+
     // Both products of the layer in one launch (the usual case of a training step): the weight
     // gradient's k-blocks fill the waves the input gradient's tiles leave partly empty.
-    static const bool merged = env_int("NB_MERGED_BWD", 1) != 0;
-    if (merged && dinp && dweight && dweight_dtype == NB_DTYPE_F32 && use_pairs(static_cast<int>(BT))) {
+    static const bool merge_allowed = env_int("NB_MERGED_BWD", 1) != 0;
+    if (merge_allowed && dinp && dweight && dweight_dtype == NB_DTYPE_F32 && split == 1 && use_pairs(static_cast<int>(BT))) {
         rc = run_layer_bwd(*s, dz, weight, inp, dinp, inp_pre_act, dweight, static_cast<float *>(dbias), BT, C,
                            OC, accumulate, stream);
         if (rc != NB_ERR_UNSUPPORTED) return rc;
     }
 
-    if (dinp) {  // dinp[BT, C] = dz[BT, OC] . W[OC, C]
-        GemmArgs a;
-        memset(&a, 0, sizeof(a));
-        a.A = dz; a.a_rows = BT; a.a_cols = OC;
-        a.B = weight; a.b_rows = OC; a.b_cols = C;
-        a.D = dinp; a.d_rows = BT; a.d_cols = C; a.d_dtype = 0;
-        a.M = static_cast<int>(BT); a.N = static_cast<int>(C); a.K = static_cast<int>(OC);
-        a.splits = 1;
-        if (inp_pre_act) {
-            a.E = inp_pre_act; a.e_rows = BT; a.e_cols = C;
-            rc = launch_gemm_auto<DgradMulGelu1, DgradMulGelu2>(*s, a, stream);
-        } else {
-            rc = launch_gemm_auto<DgradStore1, DgradStore2>(*s, a, stream);
-        }
-        if (rc != NB_OK) return rc;
-    }
+    if (dinp && (rc = run_dgrad(*s, d, stream)) != NB_OK) return rc;
 
     if (dweight) {  // dweight[OC, C] (+)= dz^T[OC, BT] . inp[BT, C]
         GemmArgs a;

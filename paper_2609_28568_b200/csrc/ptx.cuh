@@ -149,6 +149,13 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y)
         : "memory");
 }
+// The same tile requested into L2 only: a hint, nothing is delivered and nothing has to be waited for.
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *m, int x, int y)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
+                 ::"l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y)
+                 : "memory");
+}
 // 2D tile store shared -> global (out-of-range part of the tile is clipped).
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *m, uint32_t src, int x, int y)
 {
@@ -313,6 +320,15 @@ __device__ __forceinline__ void tmem_ld_32x32_x2_wait(uint32_t taddr0, uint32_t 
 }
 
 // ------------------------------------------------------------------ shared memory access
+// 16 bytes into the shared memory of a CTA of the cluster (a shared::cluster address), counted on an
+// mbarrier of that CTA.
+__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d,
+                                            uint32_t bar)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar)
+                 : "memory");
+}
 // two floats from the shared memory of a CTA of the cluster
 __device__ __forceinline__ void ld_cluster_f32x2(uint32_t addr, float2 &v)
 {

@@ -1,14 +1,15 @@
 """The kernels for small problems at the sizes where they change form: the row kernel (1 to 16 rows, K
-shared by a cluster or not, several CTAs of features per SM). Every element against the oracle,
-canaries around every buffer; the bounds are those of the other parity tests (one rounding to bf16,
-fp32 sums)."""
+shared by a cluster or not, several CTAs of features per SM), the tile kernel (every tile width, one
+row past a tile, K split over 2, 4 and 8 CTAs, ragged K and columns), both products of a backward in
+one launch. Every element against the oracle, canaries around every buffer; the bounds are those of
+the other parity tests (one rounding to bf16, fp32 sums)."""
 import pytest
 import torch
 
 import oracle
 from paper_2609_28568_b200 import binding as nb
 from paper_2609_28568_b200 import synth
-from parity import Guarded, check_bf16, f32
+from parity import Guarded, check_bf16, check_f32, f32
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -22,6 +23,8 @@ def gen(seed, shape, std):
 @pytest.mark.parametrize("BT,C,OC", [
     (1, 8, 16), (8, 3080, 208), (9, 1032, 80), (16, 4096, 48),   # rows: K in one CTA / shared by 2, 4 and 8
     (3, 72, 7200), (16, 40, 7200),                                # rows: several CTAs of features per SM
+    (17, 264, 144), (64, 1544, 80), (128, 3072, 96),              # tiles: fewer rows than a tile, K split
+    (129, 776, 400), (300, 2056, 272), (1000, 328, 1424),         # tiles: one row past, several row tiles
 ])
 def test_small_forward(BT, C, OC, act):
     inp, w, b = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (OC,), 0.05)
@@ -35,4 +38,35 @@ def test_small_forward(BT, C, OC, act):
     if pre:
         check_bf16(pre.t, p_ref, "pre_act")
         pre.check("pre_act")
+    nb.nb_check_status()
+
+
+@pytest.mark.parametrize("fused", [False, True])
+@pytest.mark.parametrize("BT,C,OC", [
+    (1, 8, 16), (8, 136, 3072), (64, 776, 200), (128, 264, 2056),   # dinp's K split over 2, 4, 8
+    (129, 72, 136), (256, 520, 1544), (257, 520, 1544),              # the last split, the first without
+    (384, 768, 776), (1000, 264, 328),                               # more k-blocks than stages for dweight
+])
+def test_small_backward(BT, C, OC, fused):
+    inp, w, dout = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (BT, OC), 1e-3)
+    ipre = gen(4, (BT, C), 1.0) if fused else None
+    r = oracle.linear_backward(f32(dout), f32(inp), f32(w), inp_pre=f32(ipre) if fused else None)
+    dinp = Guarded((BT, C), torch.bfloat16)
+    dw, db = Guarded((OC, C), torch.float32, fill=7.0), Guarded((OC,), torch.float32, fill=-7.0)
+    for acc in range(2):
+        nb.nb_linear_backward_ex(dinp.t, dw.t, db.t, dout, inp, w, None, ipre, BT, C, OC, nb.ACT_NONE, acc)
+    check_bf16(dinp.t, r["dinp"], "dinp")
+    check_f32(dw.t, 2 * r["dweight"], "dweight")
+    check_f32(db.t, 2 * r["dbias"], "dbias")
+    for g, n in ((dinp, "dinp"), (dw, "dweight"), (db, "dbias")):
+        g.check(n)
+    # dinp has one value, whatever else is asked for
+    alone = torch.empty_like(dinp.t)
+    nb.nb_linear_backward_ex(alone, None, None, dout, None, w, None, ipre, BT, C, OC, nb.ACT_NONE, 0)
+    assert torch.equal(alone, dinp.t)
+    # dweight alone, and without a bias gradient
+    dw2 = Guarded((OC, C), torch.float32, fill=3.0)
+    nb.nb_linear_backward_ex(None, dw2.t, None, dout, inp, None, None, None, BT, C, OC, nb.ACT_NONE, 0)
+    check_f32(dw2.t, r["dweight"], "dweight alone")
+    dw2.check("dweight alone")
     nb.nb_check_status()
