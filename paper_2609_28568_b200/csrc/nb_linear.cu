@@ -1150,6 +1150,110 @@ int run_dgrad(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
     return pl.bn ? launch_tile_plan<true, kEpiStore>(s, a, pl, stream) : launch_gemm_auto<DgradStore1, DgradStore2>(s, a, stream);
 }
 
+// The rank-r products on 128 x 64 tiles, a CTA each (gemm_kernel's narrow forms).
+double narrow_us(int sms, int tiles, int kblocks)
+{
+    return 4.3 + 0.2 * kblocks * static_cast<double>((tiles + sms - 1) / sms);
+}
+
+// t[:, r] = scale * inp . A^T
+int run_lora_down(DeviceState &s, void *t, const void *inp, const void *lora_a, float scale, int64_t BT, int64_t C,
+                  int64_t r, cudaStream_t stream)
+{
+    GemmArgs a;
+    memset(&a, 0, sizeof(a));
+    a.A = inp; a.a_rows = BT; a.a_cols = C;
+    a.B = lora_a; a.b_rows = r; a.b_cols = C;
+    a.D = t; a.d_rows = BT; a.d_cols = r; a.d_dtype = 0;
+    a.M = static_cast<int>(BT); a.N = static_cast<int>(r); a.K = static_cast<int>(C);
+    a.splits = 1;
+    a.alpha = scale;
+    const int kb = kblocks_of(C);
+    const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, r <= 32, 0, 0,
+                                     narrow_us(s.num_sms, (a.M + kBlockM - 1) / kBlockM, kb));
+    return pl.bn ? launch_tile_plan<false, kEpiStore>(s, a, pl, stream) : launch_gemm<FwdStoreNarrow>(s, a, stream);
+}
+
+struct LoraBwd {
+    void *dinp, *dlora_a, *dlora_b, *u;
+    const void *dout, *inp, *weight, *lora_a, *lora_b, *t;
+    uint64_t u_ld, t_ld;  // row strides of u and t where they are column slices of stacks, else 0
+    float scale;
+    int64_t BT, C, OC, r;
+    int accumulate;
+};
+
+// Backward of one adapted projection. Three ways, by estimate:
+//   lora_udb_kernel (u, dB and dA from one pass over dout and inp, a CTA per 128 rows) and the dinp
+//   product: the one to use when there are about as many 128-row panels as SMs;
+//   two tile_pair_kernel launches (u and dB, then dinp and dA), which spread a short batch over the
+//   chip: 519 rows are five panels, and five CTAs took 22 us;
+//   the first of those and the other two products by themselves.
+int run_lora_backward(DeviceState &s, const LoraBwd &l, cudaStream_t stream)
+{
+    const int sms = s.num_sms, BT = static_cast<int>(l.BT), C = static_cast<int>(l.C), OC = static_cast<int>(l.OC), r = static_cast<int>(l.r);
+    const int kt = kblocks_of(BT), ko = kblocks_of(OC);
+    int rc;
+    GemmArgs u, dB, dx, dA;
+    memset(&u, 0, sizeof(u));  // u = scale * dout . B   (B [OC, r] read as an MN-major operand)
+    u.A = l.dout; u.a_rows = BT; u.a_cols = OC;
+    u.B = l.lora_b; u.b_rows = OC; u.b_cols = r;
+    u.D = l.u; u.d_rows = BT; u.d_cols = r; u.d_ld = l.u_ld;
+    u.M = BT; u.N = r; u.K = OC;
+    u.splits = 1;
+    u.alpha = l.scale;
+    memset(&dB, 0, sizeof(dB));  // dB [OC, r] (+)= dout^T . t      (t already carries the scale)
+    dB.A = l.dout; dB.a_rows = BT; dB.a_cols = OC;
+    dB.B = l.t; dB.b_rows = BT; dB.b_cols = r; dB.b_ld = l.t_ld;
+    dB.D = l.dlora_b; dB.d_rows = OC; dB.d_cols = r; dB.d_dtype = 1;
+    dB.M = OC; dB.N = r; dB.K = BT;
+    memset(&dx, 0, sizeof(dx));  // dinp = dout . W + u . A: r extra rows of K
+    dx.A = l.dout; dx.a_rows = BT; dx.a_cols = OC;
+    dx.B = l.weight; dx.b_rows = OC; dx.b_cols = C;
+    dx.D = l.dinp; dx.d_rows = BT; dx.d_cols = C;
+    dx.M = BT; dx.N = C; dx.K = OC;
+    dx.splits = 1;
+    dx.A2 = l.u; dx.a2_rows = BT; dx.a2_cols = r; dx.a2_ld = l.u_ld;
+    dx.B2 = l.lora_a; dx.b2_rows = r; dx.b2_cols = C;
+    dx.k2 = r;
+    memset(&dA, 0, sizeof(dA));  // dA [r, C] (+)= u^T . inp        (u already carries the scale)
+    dA.A = l.u; dA.a_rows = BT; dA.a_cols = r; dA.a_ld = l.u_ld;
+    dA.B = l.inp; dA.b_rows = BT; dA.b_cols = C;
+    dA.D = l.dlora_a; dA.d_rows = r; dA.d_cols = C; dA.d_dtype = 1;
+    dA.M = r; dA.N = C; dA.K = BT;
+
+    const bool want_x = l.dinp != nullptr, want_a = l.dlora_a != nullptr;
+    const int panels = (BT + kBlockM - 1) / kBlockM;
+    const int split = dinp_split(sms, BT, C, ko + 1);
+    const double x_us = want_x ? plan_single(sms, BT, C, ko + 1, false, split, 0, persistent_us(sms, BT, C, ko + 1)).us : 0.0;
+    if (l.dlora_b) {
+        const double clear = l.accumulate ? 0.0 : 4.0;
+        const int udb_tiles = (OC + 127) / 128 + (want_a ? (C + 127) / 128 : 0);
+        const double udb = 6.0 + clear + 0.63 * udb_tiles * static_cast<double>((panels + sms - 1) / sms) + x_us;
+        const double far = 1e9;
+        const SmallPlan none;
+        const SmallPlan ub = plan_pair(sms, BT, r, ko, 0, OC, r, kt, false, far, true);
+        const SmallPlan xa = want_x && want_a ? plan_pair(sms, BT, C, ko + 1, split, r, C, kt, false, far, false) : none;
+        const SmallPlan a1 = want_a ? plan_pair(sms, 0, 0, 0, 1, r, C, kt, false, far, false) : none;
+        const double apart = ub.us + x_us + a1.us, paired = xa.bn ? ub.us + xa.us : far;
+        if (ub.bn && (apart < udb || paired < udb)) {
+            if ((rc = launch_tile_pair_plan(s, &u, dB, false, l.accumulate, ub, stream)) != NB_OK) return rc;
+            if (paired <= apart) return launch_tile_pair_plan(s, &dx, dA, false, l.accumulate, xa, stream);
+            if (want_x && (rc = run_dgrad(s, dx, stream)) != NB_OK) return rc;
+            return want_a ? launch_tile_pair_plan(s, nullptr, dA, false, l.accumulate, a1, stream) : NB_OK;
+        }
+        if ((rc = launch_lora_udb(s, l.dout, l.lora_b, l.t, l.t_ld, l.dlora_b, l.u, l.u_ld ? l.u_ld : static_cast<uint64_t>(r),
+                                  l.scale, BT, OC, r, l.accumulate, stream, want_a ? l.inp : nullptr, l.dlora_a, C)) != NB_OK)
+            return rc;
+        return want_x ? run_dgrad(s, dx, stream) : NB_OK;
+    }
+    const SmallPlan up = plan_single(sms, BT, r, ko, false, 0, 0, narrow_us(sms, panels, ko));
+    rc = up.bn ? launch_tile_plan<true, kEpiStore>(s, u, up, stream) : launch_gemm<DgradStoreNarrow>(s, u, stream);
+    if (rc != NB_OK) return rc;
+    if (want_x && (rc = run_dgrad(s, dx, stream)) != NB_OK) return rc;
+    return want_a ? run_wgrad_f32(s, l.u, l.inp, l.dlora_a, nullptr, BT, r, C, l.accumulate, stream) : NB_OK;
+}
+
 }  // namespace
 
 // ================================================================================ C ABI
@@ -1446,15 +1550,8 @@ int nb_lora_linear_forward(void *out, void *t, const void *inp, const void *weig
     std::lock_guard<std::mutex> lock(g_mu);
     DeviceState *s;
     if ((rc = get_state(&s)) != NB_OK) return rc;
+    if ((rc = run_lora_down(*s, t, inp, lora_a, scale, BT, C, r, stream)) != NB_OK) return rc;
     GemmArgs a;
-    memset(&a, 0, sizeof(a));  // t = scale * inp . A^T
-    a.A = inp; a.a_rows = BT; a.a_cols = C;
-    a.B = lora_a; a.b_rows = r; a.b_cols = C;
-    a.D = t; a.d_rows = BT; a.d_cols = r; a.d_dtype = 0;
-    a.M = static_cast<int>(BT); a.N = static_cast<int>(r); a.K = static_cast<int>(C);
-    a.splits = 1;
-    a.alpha = scale;
-    if ((rc = launch_gemm<FwdStoreNarrow>(*s, a, stream)) != NB_OK) return rc;
     memset(&a, 0, sizeof(a));  // out = inp . W^T (+ bias) + t . B^T: r extra columns of K
     a.A = inp; a.a_rows = BT; a.a_cols = C;
     a.B = weight; a.b_rows = OC; a.b_cols = C;
@@ -1465,7 +1562,7 @@ int nb_lora_linear_forward(void *out, void *t, const void *inp, const void *weig
     a.A2 = t; a.a2_rows = BT; a.a2_cols = r;
     a.B2 = lora_b; a.b2_rows = OC; a.b2_cols = r;
     a.k2 = static_cast<int>(r);
-    return launch_gemm_auto<FwdStore1, FwdStore2>(*s, a, stream);
+    return run_forward(*s, a, NB_ACT_NONE, stream);
 }
 
 int nb_lora_linear_backward(void *dinp, void *dlora_a, void *dlora_b, void *u, const void *dout,
@@ -1494,46 +1591,8 @@ int nb_lora_linear_backward(void *dinp, void *dlora_a, void *dlora_b, void *u, c
         }
         return NB_OK;
     }
-    GemmArgs a;
-    static const bool fused_udb = env_int("NB_LORA_FUSED", 1) != 0;
-    static const bool fused_da = env_int("NB_LORA_FUSED_DA", 1) != 0;
-    if (fused_udb && dlora_b) {  // u and dB from one pass over dout; dA from one pass over inp in the same launch
-        const bool with_da = fused_da && dlora_a != nullptr;
-        if ((rc = launch_lora_udb(*s, dout, lora_b, t, 0, dlora_b, u, static_cast<uint64_t>(r), scale, BT, OC, r,
-                                  accumulate, stream, with_da ? inp : nullptr, with_da ? dlora_a : nullptr, C)) != NB_OK)
-            return rc;
-        dlora_b = nullptr;
-        if (with_da) dlora_a = nullptr;
-    } else {
-        memset(&a, 0, sizeof(a));  // u = scale * dout . B   (B [OC, r] read as an MN-major operand)
-        a.A = dout; a.a_rows = BT; a.a_cols = OC;
-        a.B = lora_b; a.b_rows = OC; a.b_cols = r;
-        a.D = u; a.d_rows = BT; a.d_cols = r; a.d_dtype = 0;
-        a.M = static_cast<int>(BT); a.N = static_cast<int>(r); a.K = static_cast<int>(OC);
-        a.splits = 1;
-        a.alpha = scale;
-        if ((rc = launch_gemm<DgradStoreNarrow>(*s, a, stream)) != NB_OK) return rc;
-    }
-    // dB right after u: both stream dout, and what the first pass brought into L2 serves the second
-    if (dlora_b)  // dB [OC, r] (+)= dout^T . t      (t already carries the scale)
-        if ((rc = run_wgrad_f32(*s, dout, t, dlora_b, nullptr, BT, OC, r, accumulate, stream)) != NB_OK)
-            return rc;
-    if (dinp) {  // dinp = dout . W + u . A: r extra rows of K
-        memset(&a, 0, sizeof(a));
-        a.A = dout; a.a_rows = BT; a.a_cols = OC;
-        a.B = weight; a.b_rows = OC; a.b_cols = C;
-        a.D = dinp; a.d_rows = BT; a.d_cols = C; a.d_dtype = 0;
-        a.M = static_cast<int>(BT); a.N = static_cast<int>(C); a.K = static_cast<int>(OC);
-        a.splits = 1;
-        a.A2 = u; a.a2_rows = BT; a.a2_cols = r;
-        a.B2 = lora_a; a.b2_rows = r; a.b2_cols = C;
-        a.k2 = static_cast<int>(r);
-        if ((rc = launch_gemm_auto<DgradStore1, DgradStore2>(*s, a, stream)) != NB_OK) return rc;
-    }
-    if (dlora_a)  // dA [r, C] (+)= u^T . inp        (u already carries the scale)
-        if ((rc = run_wgrad_f32(*s, u, inp, dlora_a, nullptr, BT, r, C, accumulate, stream)) != NB_OK)
-            return rc;
-    return NB_OK;
+    const LoraBwd l{dinp, dlora_a, dlora_b, u, dout, inp, weight, lora_a, lora_b, t, 0, 0, scale, BT, C, OC, r, accumulate};
+    return run_lora_backward(*s, l, stream);
 }
 
 // --- adapters that share an input, stacked (q, k, v; gate, up): one rank-R product for all of them
@@ -1564,15 +1623,7 @@ int nb_lora_down_stacked(void *t_stack, const void *inp, const void *a_stack, fl
     std::lock_guard<std::mutex> lock(g_mu);
     DeviceState *s;
     if ((rc = get_state(&s)) != NB_OK) return rc;
-    GemmArgs a;
-    memset(&a, 0, sizeof(a));  // t_stack = scale * inp . a_stack^T
-    a.A = inp; a.a_rows = BT; a.a_cols = C;
-    a.B = a_stack; a.b_rows = R; a.b_cols = C;
-    a.D = t_stack; a.d_rows = BT; a.d_cols = R; a.d_dtype = 0;
-    a.M = static_cast<int>(BT); a.N = static_cast<int>(R); a.K = static_cast<int>(C);
-    a.splits = 1;
-    a.alpha = scale;
-    return launch_gemm<FwdStoreNarrow>(*s, a, stream);
+    return run_lora_down(*s, t_stack, inp, a_stack, scale, BT, C, R, stream);
 }
 
 int nb_lora_linear_forward_stacked(void *out, const void *inp, const void *weight, const void *bias,
@@ -1602,7 +1653,7 @@ int nb_lora_linear_forward_stacked(void *out, const void *inp, const void *weigh
     a.A2 = static_cast<const uint16_t *>(t_stack) + off; a.a2_rows = BT; a.a2_cols = r; a.a2_ld = R;
     a.B2 = lora_b; a.b2_rows = OC; a.b2_cols = r;
     a.k2 = static_cast<int>(r);
-    return launch_gemm_auto<FwdStore1, FwdStore2>(*s, a, stream);
+    return run_forward(*s, a, NB_ACT_NONE, stream);
 }
 
 int nb_lora_linear_backward_stacked(void *dinp, void *dlora_b, void *u_stack, const void *dout,
@@ -1628,43 +1679,10 @@ int nb_lora_linear_backward_stacked(void *dinp, void *dlora_b, void *u_stack, co
         if (!accumulate && dlora_b) NB_CUDA(cudaMemsetAsync(dlora_b, 0, static_cast<size_t>(OC * r) * 4, stream));
         return NB_OK;
     }
-    uint16_t *u_slice = static_cast<uint16_t *>(u_stack) + off;
-    GemmArgs a;
-    static const bool fused_udb = env_int("NB_LORA_FUSED", 1) != 0;
-    if (fused_udb && dlora_b) {  // u_slice and dB from one pass over dout
-        if ((rc = launch_lora_udb(*s, dout, lora_b, static_cast<const uint16_t *>(t_stack) + off, static_cast<uint64_t>(R),
-                                  dlora_b, u_slice, static_cast<uint64_t>(R), scale, BT, OC, r, accumulate,
-                                  stream)) != NB_OK)
-            return rc;
-        dlora_b = nullptr;
-    } else {
-        memset(&a, 0, sizeof(a));  // u_slice = scale * dout . B
-        a.A = dout; a.a_rows = BT; a.a_cols = OC;
-        a.B = lora_b; a.b_rows = OC; a.b_cols = r;
-        a.D = u_slice; a.d_rows = BT; a.d_cols = r; a.d_dtype = 0; a.d_ld = R;
-        a.M = static_cast<int>(BT); a.N = static_cast<int>(r); a.K = static_cast<int>(OC);
-        a.splits = 1;
-        a.alpha = scale;
-        if ((rc = launch_gemm<DgradStoreNarrow>(*s, a, stream)) != NB_OK) return rc;
-    }
-    // dB right after u: both stream dout, and what the first pass brought into L2 serves the second
-    if (dlora_b)  // dB [OC, r] (+)= dout^T . t_slice
-        if ((rc = run_wgrad_f32(*s, dout, static_cast<const uint16_t *>(t_stack) + off, dlora_b, nullptr, BT, OC, r,
-                                accumulate, stream, static_cast<uint64_t>(R))) != NB_OK)
-            return rc;
-    if (dinp) {  // dinp = dout . W + u_slice . A
-        memset(&a, 0, sizeof(a));
-        a.A = dout; a.a_rows = BT; a.a_cols = OC;
-        a.B = weight; a.b_rows = OC; a.b_cols = C;
-        a.D = dinp; a.d_rows = BT; a.d_cols = C; a.d_dtype = 0;
-        a.M = static_cast<int>(BT); a.N = static_cast<int>(C); a.K = static_cast<int>(OC);
-        a.splits = 1;
-        a.A2 = u_slice; a.a2_rows = BT; a.a2_cols = r; a.a2_ld = R;
-        a.B2 = lora_a; a.b2_rows = r; a.b2_cols = C;
-        a.k2 = static_cast<int>(r);
-        if ((rc = launch_gemm_auto<DgradStore1, DgradStore2>(*s, a, stream)) != NB_OK) return rc;
-    }
-    return NB_OK;
+    const LoraBwd l{dinp, nullptr, dlora_b, static_cast<uint16_t *>(u_stack) + off, dout, nullptr, weight, lora_a, lora_b,
+                    static_cast<const uint16_t *>(t_stack) + off, static_cast<uint64_t>(R), static_cast<uint64_t>(R),
+                    scale, BT, C, OC, r, accumulate};
+    return run_lora_backward(*s, l, stream);
 }
 
 int nb_lora_da_stacked(void *da_stack, const void *u_stack, const void *inp, int64_t BT, int64_t C, int64_t R,
@@ -1684,7 +1702,17 @@ int nb_lora_da_stacked(void *da_stack, const void *u_stack, const void *inp, int
         if (!accumulate) NB_CUDA(cudaMemsetAsync(da_stack, 0, static_cast<size_t>(R * C) * 4, stream));
         return NB_OK;
     }
-    return run_wgrad_f32(*s, u_stack, inp, da_stack, nullptr, BT, R, C, accumulate, stream);  // dA (+)= u^T . inp
+    GemmArgs w;
+    memset(&w, 0, sizeof(w));  // dA (+)= u^T . inp
+    w.A = u_stack; w.a_rows = BT; w.a_cols = R;
+    w.B = inp; w.b_rows = BT; w.b_cols = C;
+    w.D = da_stack; w.d_rows = R; w.d_cols = C; w.d_dtype = 1;
+    w.M = static_cast<int>(R); w.N = static_cast<int>(C); w.K = static_cast<int>(BT);
+    const int kw = kblocks_of(BT);
+    const SmallPlan pl = plan_pair(s->num_sms, 0, 0, 0, 1, w.M, w.N, kw, false,
+                                   backward_us(s->num_sms, 0, w.K, w.N, w.M, 0, kw, accumulate != 0, true), false);
+    if (pl.bn) return launch_tile_pair_plan(*s, nullptr, w, false, accumulate, pl, stream);
+    return run_wgrad_f32(*s, u_stack, inp, da_stack, nullptr, BT, R, C, accumulate, stream);
 }
 
 int nb_cast_f32_to_bf16(void *dst, const void *src, int64_t n, void *stream_)

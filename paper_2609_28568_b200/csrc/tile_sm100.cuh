@@ -621,7 +621,10 @@ tile_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 // Two products that read the same tensor. The CTAs of job 0 form a bf16 result (A by rows, B
 // MN-major, adapter term possible), those of job 1 an fp32 one (both operands MN-major, all of its K
 // in one CTA, so nothing has to start from zero and nothing is summed in a varying order) and, with
-// it, column sums of its A operand: a layer's dinp = dz . W beside dweight (+)= dz^T . inp and dbias.
+// it, column sums of its A operand:
+//   a layer's backward       dinp = dz . W                      dweight (+)= dz^T . inp, dbias
+//   an adapter's backward    u = scale dy . B                   dB (+)= dy^T . t
+//                            dinp = dy . W + u . A              dA (+)= u^T . inp
 template <int BN, bool GELU_GRAD>
 __global__ void __launch_bounds__(kTileThreads, BN == 128 ? 1 : 2)
 tile_pair_kernel(const __grid_constant__ CUtensorMap tmA0,  // boxes of up to 128 rows

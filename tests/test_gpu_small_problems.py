@@ -1,8 +1,11 @@
 """The kernels for small problems at the sizes where they change form: the row kernel (1 to 16 rows, K
 shared by a cluster or not, several CTAs of features per SM), the tile kernel (every tile width, one
 row past a tile, K split over 2, 4 and 8 CTAs, ragged K and columns), both products of a backward in
-one launch. Every element against the oracle, canaries around every buffer; the bounds are those of
+one launch, the adapter's two launches. Every element against the oracle, canaries around every buffer; the bounds are those of
 the other parity tests (one rounding to bf16, fp32 sums)."""
+import math
+
+import numpy as np
 import pytest
 import torch
 
@@ -69,4 +72,33 @@ def test_small_backward(BT, C, OC, fused):
     nb.nb_linear_backward_ex(None, dw2.t, None, dout, inp, None, None, None, BT, C, OC, nb.ACT_NONE, 0)
     check_f32(dw2.t, r["dweight"], "dweight alone")
     dw2.check("dweight alone")
+    nb.nb_check_status()
+
+
+@pytest.mark.parametrize("BT,C,OC,r", [
+    (1, 8, 8, 8), (100, 72, 2056, 16), (129, 1544, 136, 40), (519, 1024, 776, 8), (640, 264, 3072, 64),
+])
+def test_small_adapter_layer(BT, C, OC, r):
+    scale = 32.0 / math.sqrt(r)
+    inp, w, dout = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.02), gen(3, (BT, OC), 1e-3)
+    a, b = gen(4, (r, C), 0.02), gen(5, (OC, r), 0.02)
+    out, t, u = (Guarded((BT, n), torch.bfloat16) for n in (OC, r, r))
+    dinp = Guarded((BT, C), torch.bfloat16)
+    dA, dB = Guarded((r, C), torch.float32, fill=7.0), Guarded((OC, r), torch.float32, fill=-7.0)
+    nb.nb_lora_linear_forward(out.t, t.t, inp, w, None, a, b, scale, BT, C, OC, r)
+    for acc in range(2):
+        nb.nb_lora_linear_backward(dinp.t, dA.t, dB.t, u.t, dout, inp, w, a, b, t.t, scale, BT, C, OC, r, acc)
+    t_ref = scale * oracle.linear_forward(f32(inp), f32(a))[0]
+    u_ref = scale * oracle.linear_backward(f32(dout), None, f32(b), want=("dinp",))["dinp"]
+    di_ref, dA_ref, dB_ref = oracle.lora_backward(f32(dout), f32(inp), f32(w), f32(a), f32(b), scale)
+    check_bf16(t.t, t_ref, "t")
+    check_bf16(u.t, u_ref, "u")
+    # t and u are rounded to bf16 once (2^-9 of each element), which the other factor passes on
+    check_bf16(out.t, oracle.lora_forward(f32(inp), f32(w), None, f32(a), f32(b), scale), "out",
+               extra=2.0 ** -9 * (np.abs(t_ref) @ np.abs(f32(b).T.astype(np.float64))))
+    check_bf16(dinp.t, di_ref, "dinp", extra=2.0 ** -9 * (np.abs(u_ref) @ np.abs(f32(a).astype(np.float64))))
+    check_f32(dA.t, 2 * dA_ref, "dA")
+    check_f32(dB.t, 2 * dB_ref, "dB")
+    for g, n in ((out, "out"), (t, "t"), (u, "u"), (dinp, "dinp"), (dA, "dA"), (dB, "dB")):
+        g.check(n)
     nb.nb_check_status()
