@@ -325,7 +325,7 @@ int nb_check_status(void);
 
 /*
  * Number of kernels this library has launched from the calling process since it was
- * loaded (memsets issued through the CUDA runtime are not counted).
+ * loaded (what clears gradient buffers, a memset or a kernel, is not counted).
  */
 int64_t nb_kernel_launches(void);
 

@@ -138,6 +138,25 @@ dbias_kernel(float *__restrict__ dbias, const __nv_bfloat16 *__restrict__ dz, lo
     }
 }
 
+// Zeroes two fp32 arrays (either may be empty) ahead of a kernel that reduce-adds into them. A memset in
+// its place is a node of its own kind: the kernel before it has to drain, and so has it, before the
+// kernel after it is launched (two of them cost a layer's backward 4 to 6 us). This one is a link of the
+// dependent-launch chain, and it lets its successor start as soon as its own predecessors are done:
+// a successor that loads operands and multiplies first needs the zeros only when its first sums leave,
+// and calls griddepcontrol.wait there.
+__global__ void __launch_bounds__(256)
+clear_kernel(float *__restrict__ a, long long na, float *__restrict__ b, long long nb_)
+{
+    ptx::grid_dependency_wait();      // first: what the predecessors read must not be cleared under them,
+    ptx::grid_launch_dependents();    // and whoever starts from here on may rely on their results
+    const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
+    const long long t0 = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    // 16-byte aligned, as every array the library is given; the lengths are multiples of 8
+    for (long long i = t0; i < na / 4; i += stride) reinterpret_cast<float4 *>(a)[i] = z;
+    for (long long i = t0; i < nb_ / 4; i += stride) reinterpret_cast<float4 *>(b)[i] = z;
+}
+
 // fp32 -> bf16 (round to nearest even), 8 elements per thread per iteration: two 128-bit loads, one
 // 128-bit store. HBM-bound: 6 bytes per element.
 __global__ void __launch_bounds__(256)

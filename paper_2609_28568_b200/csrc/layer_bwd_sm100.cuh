@@ -52,6 +52,9 @@ struct LayerBwdParams {
     int w_tail_full, w_last_len;
     int w_tail_begin[kMaxPairs + 1];
     float *dbias;  // [OC] or nullptr
+    int after_clear;  // the launch before this one is clear_kernel on dweight and dbias: only what adds
+                      // to them has to wait for it (that kernel let this one start once everything
+                      // before it was done)
     int *status;
     unsigned long long timeout_ns;
 };
@@ -251,7 +254,7 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
     ptx::tc_fence_after();
     // nothing above touched global memory: it may overlap the previous kernel's tail
     ptx::grid_launch_dependents();
-    ptx::grid_dependency_wait();
+    if (!p.after_clear || warp >= 4) ptx::grid_dependency_wait();
     const uint32_t tmem_base = ptx::ld_shared_u32_volatile(tmem_slot);
     const WaitCtx wctx{abort_addr, p.status, p.timeout_ns};
     // The epilogue waits for a whole unit where the issuer waits for one stage: with twice the limit

@@ -58,6 +58,7 @@ struct UdbParams {
     float alpha;
     __nv_bfloat16 *u;  // first element of this adapter's column slice of u
     int u_ld;          // elements from one row of u to the next
+    int after_clear;   // as in LayerBwdParams: only the epilogue waits for the zeros in dB and dA
     int *status;
     unsigned long long timeout_ns;
 };
@@ -128,7 +129,7 @@ lora_udb_kernel(const __grid_constant__ CUtensorMap tmDy,  // dy [BT, OC] bf16, 
     __syncthreads();
     ptx::tc_fence_after();
     ptx::grid_launch_dependents();
-    ptx::grid_dependency_wait();
+    if (!p.after_clear || warp >= 2) ptx::grid_dependency_wait();
     const uint32_t tmem_base = ptx::ld_shared_u32_volatile(tmem_slot);
     const WaitCtx wctx{abort_addr, p.status, p.timeout_ns};
     const WaitCtx wctx_epi{abort_addr, p.status, 2 * p.timeout_ns};

@@ -355,6 +355,29 @@ using DgradStoreNarrow = GemmCfg<1, 64, 7, 2, false, true, kEpiStore>;
 using WgradF32Narrow = GemmCfg<1, 64, 7, 2, true, true, kEpiF32>;
 constexpr int kNarrowN = 64;
 
+// ----------------------------------------------------------------------------- clearing
+// Zeroes up to two fp32 arrays in stream order (clear_kernel).
+int launch_clear(const DeviceState &s, void *a, int64_t na, void *b, int64_t nb_, cudaStream_t stream)
+{
+    if (!b) nb_ = 0;
+    const long long vec = (na > nb_ ? na : nb_) / 4;
+    long long blocks = (vec + 1023) / 1024;  // four stores per thread, up to four blocks per SM
+    if (blocks > 4ll * s.num_sms) blocks = 4ll * s.num_sms;
+    if (blocks < 1) blocks = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent_launch_allowed(stream) ? 1 : 0;
+    NB_CUDA(cudaLaunchKernelEx(&cfg, clear_kernel, static_cast<float *>(a), static_cast<long long>(na),
+                               static_cast<float *>(b), static_cast<long long>(nb_)));
+    return NB_OK;  // not counted in g_launches, as the memsets it replaces were not
+}
+
 // ----------------------------------------------------------------------------- small problems
 // Launch configuration: cluster size along x, and dependent launch where it is allowed.
 void small_launch_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attrs)[2], int ctas, int threads, int cluster,
@@ -803,10 +826,11 @@ int run_wgrad_f32(DeviceState &s, const void *dz, const void *inp, void *dweight
     const int splits = choose_splits(tiles, kblocks, slots);
     a.splits = splits;
     a.reduce = (accumulate || splits > 1) ? 1 : 0;
-    if (!accumulate && splits > 1)
-        NB_CUDA(cudaMemsetAsync(dweight, 0, static_cast<size_t>(M_ * N_) * 4, stream));
+    const bool clear_w = !accumulate && splits > 1, clear_b = !accumulate && dbias != nullptr;
+    int rc;
+    if (clear_w && (rc = launch_clear(s, dweight, M_ * N_, clear_b ? dbias : nullptr, M_, stream)) != NB_OK) return rc;
+    if (clear_b && !clear_w && (rc = launch_clear(s, dbias, M_, nullptr, 0, stream)) != NB_OK) return rc;
     if (dbias) {  // the bias gradient rides along: reducer warps sum dz while it is in shared memory
-        if (!accumulate) NB_CUDA(cudaMemsetAsync(dbias, 0, static_cast<size_t>(M_) * 4, stream));
         a.dbias = dbias;
         return launch_gemm_auto<WgradF32Bias1, WgradF32Bias2>(s, a, stream);
     }
@@ -845,10 +869,7 @@ int launch_lora_udb(DeviceState &s, const void *dy, const void *lora_b, const vo
         tDa = tDb;
     }
     // every panel reduce-adds its share, so a fresh gradient starts from zero
-    if (!accumulate) {
-        NB_CUDA(cudaMemsetAsync(dlora_b, 0, static_cast<size_t>(OC * r) * 4, stream));
-        if (want_da) NB_CUDA(cudaMemsetAsync(dlora_a, 0, static_cast<size_t>(r * C) * 4, stream));
-    }
+    if (!accumulate && (rc = launch_clear(s, dlora_b, OC * r, want_da ? dlora_a : nullptr, r * C, stream)) != NB_OK) return rc;
     UdbParams p;
     memset(&p, 0, sizeof(p));
     p.BT = static_cast<int>(BT);
@@ -863,6 +884,7 @@ int launch_lora_udb(DeviceState &s, const void *dy, const void *lora_b, const vo
     p.alpha = scale;
     p.u = static_cast<__nv_bfloat16 *>(u);
     p.u_ld = static_cast<int>(u_ld);
+    p.after_clear = accumulate ? 0 : 1;
     p.status = s.status;
     p.timeout_ns = kDefaultTimeoutNs;
     cudaLaunchConfig_t cfg = {};
@@ -1058,10 +1080,8 @@ int launch_layer_bwd(DeviceState &s, const void *dz, const void *weight, const v
     tPre = tDinp;
     if (Cfg::GELU_GRAD && (rc = get_tmap(s, &tPre, inp_pre, BT, C, 0, 32)) != NB_OK) return rc;
     // partial sums of every W unit are reduce-added, so a fresh gradient starts from zero
-    if (!accumulate) {
-        NB_CUDA(cudaMemsetAsync(dweight, 0, static_cast<size_t>(OC * C) * 4, stream));
-        if (Cfg::DBIAS) NB_CUDA(cudaMemsetAsync(dbias, 0, static_cast<size_t>(OC) * 4, stream));
-    }
+    p.after_clear = accumulate ? 0 : 1;
+    if (!accumulate && (rc = launch_clear(s, dweight, OC * C, Cfg::DBIAS ? dbias : nullptr, OC, stream)) != NB_OK) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(2 * p.num_pairs));
     cfg.blockDim = dim3(kLbThreads);
@@ -1128,7 +1148,7 @@ double backward_us(int sms, int M, int BT, int N, int Mw, int kd, int kw, bool a
     const int slots = sms / 2;
     const double d_tiles = static_cast<double>((M + 255) / 256) * ((N + 255) / 256);
     const double w_tiles = static_cast<double>((Mw + 255) / 256) * ((N + 255) / 256);
-    const double clear = accumulate ? 0.0 : 2.0;
+    const double clear = accumulate ? 0.0 : 1.0;
     if (M > 0 && BT > kBlockM && !apart) {
         const double level = (d_tiles * (kd + 3) + w_tiles * (kw + 3)) / slots;
         return 5.3 + clear + 0.27 * (d_tiles > 0 && kd > level ? kd : level);
@@ -1227,9 +1247,10 @@ int run_lora_backward(DeviceState &s, const LoraBwd &l, cudaStream_t stream)
     const int split = dinp_split(sms, BT, C, ko + 1);
     const double x_us = want_x ? plan_single(sms, BT, C, ko + 1, false, split, 0, persistent_us(sms, BT, C, ko + 1)).us : 0.0;
     if (l.dlora_b) {
-        const double clear = l.accumulate ? 0.0 : 4.0;
+        const double clear = l.accumulate ? 0.0 : 1.0;
         const int udb_tiles = (OC + 127) / 128 + (want_a ? (C + 127) / 128 : 0);
-        const double udb = 6.0 + clear + 0.63 * udb_tiles * static_cast<double>((panels + sms - 1) / sms) + x_us;
+        const double udb = 6.0 + clear + x_us + udb_tiles * static_cast<double>((panels + sms - 1) / sms) *
+                           (0.37 + 0.25 * (panels < sms ? panels : sms) / sms);  // reading dout takes over towards one panel per SM
         const double far = 1e9;
         const SmallPlan none;
         const SmallPlan ub = plan_pair(sms, BT, r, ko, 0, OC, r, kt, false, far, true);
