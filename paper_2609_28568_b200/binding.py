@@ -1,4 +1,5 @@
-"""ctypes binding of the nb_linear C ABI: argument marshalling only.
+"""Binding of the nb_linear C ABI: argument marshalling only. The calls of the hot path go through the
+extension module built from csrc/native.cpp, the others through ctypes.
 
 Functions named like the C entry points take torch CUDA tensors (or raw device
 pointers as ints) and pass pointers and sizes straight through; every step of
@@ -8,11 +9,13 @@ has not been built, loading raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
 
-from .build import LIB_PATH
+from .build import LIB_PATH, NATIVE_PATH
 
 NB_OK, NB_ERR_INVALID_ARG, NB_ERR_UNSUPPORTED, NB_ERR_CUDA, NB_ERR_TIMEOUT = 0, 1, 2, 3, 4
 ACT_NONE, ACT_GELU, ACT_SWIGLU = 0, 1, 2
@@ -79,6 +82,24 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native = None
+
+
+def _load_native():
+    """The extension module. Raises if it was never built: there is no fallback."""
+    global _native
+    lib()
+    if not os.path.exists(NATIVE_PATH):
+        raise RuntimeError(f"{NATIVE_PATH} is missing: build it with `python -m paper_2609_28568_b200.build`")
+    name = __package__ + "._native"
+    loader = importlib.machinery.ExtensionFileLoader(name, NATIVE_PATH)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader(name, loader))
+    loader.exec_module(module)
+    module.set_error(NbError)
+    _native = module
+    return module
+
+
 def _ptr(t):
     if t is None:
         return None
@@ -94,7 +115,7 @@ def _check(rc: int) -> None:
 
 
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def nb_version() -> int:
@@ -120,8 +141,7 @@ def nb_linear_forward(out, inp, weight, bias, BT, C, OC, act) -> None:
 
 
 def nb_linear_forward_ex(out, pre_act, inp, weight, bias, BT, C, OC, act, stream=None) -> None:
-    _check(lib().nb_linear_forward_ex(_ptr(out), _ptr(pre_act), _ptr(inp), _ptr(weight), _ptr(bias),
-                                      BT, C, OC, act, _stream() if stream is None else stream))
+    (_native or _load_native()).nb_linear_forward_ex(out, pre_act, inp, weight, bias, BT, C, OC, act, stream)
 
 
 def nb_linear_backward(dinp, dweight, dbias, dout, inp, weight, pre_act, BT, C, OC, accumulate) -> None:
@@ -132,10 +152,8 @@ def nb_linear_backward(dinp, dweight, dbias, dout, inp, weight, pre_act, BT, C, 
 
 def nb_linear_backward_ex(dinp, dweight, dbias, dout, inp, weight, pre_act, inp_pre_act, BT, C, OC,
                           act, accumulate, dweight_dtype=DTYPE_F32, stream=None) -> None:
-    _check(lib().nb_linear_backward_ex(_ptr(dinp), _ptr(dweight), _ptr(dbias), _ptr(dout), _ptr(inp),
-                                       _ptr(weight), _ptr(pre_act), _ptr(inp_pre_act), BT, C, OC, act,
-                                       int(accumulate), dweight_dtype,
-                                       _stream() if stream is None else stream))
+    (_native or _load_native()).nb_linear_backward_ex(dinp, dweight, dbias, dout, inp, weight, pre_act, inp_pre_act,
+                                                      BT, C, OC, act, int(accumulate), dweight_dtype, stream)
 
 
 def nb_reduce_dbias(dbias, dout, BT, OC, accumulate) -> None:
@@ -162,71 +180,60 @@ NOALLOC_MAX_ELEMS = 4194304
 def nb_gelu_dbias_noalloc(dbias, dout, pre_act, BT, OC, accumulate, stream=None) -> None:
     """dbias (+)= column sums of dout * gelu'(pre_act), using only the scratch array built into
     the library: for callers that may not allocate device memory. BT*OC <= NOALLOC_MAX_ELEMS."""
-    _check(lib().nb_gelu_dbias_noalloc(_ptr(dbias), _ptr(dout), _ptr(pre_act), BT, OC,
-                                       int(accumulate), _stream() if stream is None else stream))
+    (_native or _load_native()).nb_gelu_dbias_noalloc(dbias, dout, pre_act, BT, OC, int(accumulate), stream)
 
 
 def nb_lora_linear_forward(out, t, inp, weight, bias, lora_a, lora_b, scale, BT, C, OC, r, stream=None) -> None:
     """out = inp @ W.T (+ bias) + t @ B.T with t = bf16(scale * inp @ A.T), the adapter term fused in."""
-    _check(lib().nb_lora_linear_forward(_ptr(out), _ptr(t), _ptr(inp), _ptr(weight), _ptr(bias),
-                                        _ptr(lora_a), _ptr(lora_b), scale, BT, C, OC, r,
-                                        _stream() if stream is None else stream))
+    (_native or _load_native()).nb_lora_linear_forward(out, t, inp, weight, bias, lora_a, lora_b, scale, BT, C, OC, r,
+                                                       stream)
 
 
 def nb_lora_linear_backward(dinp, dlora_a, dlora_b, u, dout, inp, weight, lora_a, lora_b, t, scale, BT, C,
                             OC, r, accumulate, stream=None) -> None:
     """Gradients of the adapter layer with the base weight frozen (dinp, dA, dB)."""
-    _check(lib().nb_lora_linear_backward(_ptr(dinp), _ptr(dlora_a), _ptr(dlora_b), _ptr(u), _ptr(dout),
-                                         _ptr(inp), _ptr(weight), _ptr(lora_a), _ptr(lora_b), _ptr(t),
-                                         scale, BT, C, OC, r, int(accumulate),
-                                         _stream() if stream is None else stream))
+    (_native or _load_native()).nb_lora_linear_backward(dinp, dlora_a, dlora_b, u, dout, inp, weight, lora_a, lora_b, t,
+                                                        scale, BT, C, OC, r, int(accumulate), stream)
 
 
 def nb_lora_down_stacked(t_stack, inp, a_stack, scale, BT, C, R, stream=None) -> None:
     """t_stack = bf16(scale * inp @ a_stack.T): the down-projections of all adapters of a group at once."""
-    _check(lib().nb_lora_down_stacked(_ptr(t_stack), _ptr(inp), _ptr(a_stack), scale, BT, C, R,
-                                      _stream() if stream is None else stream))
+    (_native or _load_native()).nb_lora_down_stacked(t_stack, inp, a_stack, scale, BT, C, R, stream)
 
 
 def nb_lora_linear_forward_stacked(out, inp, weight, bias, t_stack, lora_b, BT, C, OC, r, R, off,
                                    stream=None) -> None:
     """out = inp @ W.T (+ bias) + t_stack[:, off:off+r] @ B.T, the adapter term fused in."""
-    _check(lib().nb_lora_linear_forward_stacked(_ptr(out), _ptr(inp), _ptr(weight), _ptr(bias), _ptr(t_stack),
-                                                _ptr(lora_b), BT, C, OC, r, R, off,
-                                                _stream() if stream is None else stream))
+    (_native or _load_native()).nb_lora_linear_forward_stacked(out, inp, weight, bias, t_stack, lora_b, BT, C, OC, r, R,
+                                                               off, stream)
 
 
 def nb_lora_linear_backward_stacked(dinp, dlora_b, u_stack, dout, weight, lora_a, lora_b, t_stack, scale, BT, C,
                                     OC, r, R, off, accumulate, stream=None) -> None:
     """u slice, dinp and dB of one adapted projection of a stacked group (dA comes from nb_lora_da_stacked)."""
-    _check(lib().nb_lora_linear_backward_stacked(_ptr(dinp), _ptr(dlora_b), _ptr(u_stack), _ptr(dout),
-                                                 _ptr(weight), _ptr(lora_a), _ptr(lora_b), _ptr(t_stack), scale,
-                                                 BT, C, OC, r, R, off, int(accumulate),
-                                                 _stream() if stream is None else stream))
+    (_native or _load_native()).nb_lora_linear_backward_stacked(dinp, dlora_b, u_stack, dout, weight, lora_a, lora_b,
+                                                                t_stack, scale, BT, C, OC, r, R, off,
+                                                                int(accumulate), stream)
 
 
 def nb_lora_da_stacked(da_stack, u_stack, inp, BT, C, R, accumulate, stream=None) -> None:
     """da_stack (+)= u_stack.T @ inp: the A gradients of all adapters of a group at once."""
-    _check(lib().nb_lora_da_stacked(_ptr(da_stack), _ptr(u_stack), _ptr(inp), BT, C, R, int(accumulate),
-                                    _stream() if stream is None else stream))
+    (_native or _load_native()).nb_lora_da_stacked(da_stack, u_stack, inp, BT, C, R, int(accumulate), stream)
 
 
 def nb_lm_head_ce_forward(logits, loss, lse, inp, weight, targets, BT, C, Vp, V, stream=None) -> None:
     """Head GEMM with the softmax statistics of the first V columns fused in: logits, loss, lse."""
-    _check(lib().nb_lm_head_ce_forward(_ptr(logits), _ptr(loss), _ptr(lse), _ptr(inp), _ptr(weight),
-                                       _ptr(targets), BT, C, Vp, V,
-                                       _stream() if stream is None else stream))
+    (_native or _load_native()).nb_lm_head_ce_forward(logits, loss, lse, inp, weight, targets, BT, C, Vp, V, stream)
 
 
 def nb_ce_backward(dlogits, logits, lse, targets, gscale, BT, Vp, V, stream=None) -> None:
     """dlogits = gscale * (softmax - onehot) on the first V columns, 0 on the padding."""
-    _check(lib().nb_ce_backward(_ptr(dlogits), _ptr(logits), _ptr(lse), _ptr(targets), gscale, BT, Vp, V,
-                                _stream() if stream is None else stream))
+    (_native or _load_native()).nb_ce_backward(dlogits, logits, lse, targets, gscale, BT, Vp, V, stream)
 
 
 def nb_cast_f32_to_bf16(dst, src, n, stream=None) -> None:
     """Master-weight cast: dst (bf16) = src (fp32), round to nearest even."""
-    _check(lib().nb_cast_f32_to_bf16(_ptr(dst), _ptr(src), n, _stream() if stream is None else stream))
+    (_native or _load_native()).nb_cast_f32_to_bf16(dst, src, n, stream)
 
 
 def nb_debug_split_plan(M: int, N: int, K: int, slots: int, tile_m: int):
@@ -268,27 +275,12 @@ def nb_debug_wait_timeout(limit_us: int) -> None:
 
 def linear_forward(inp, weight, bias=None, act=ACT_NONE):
     """Allocate the outputs and call nb_linear_forward_ex. Returns (out, pre_act or None)."""
-    BT, C = inp.shape
-    OC = weight.shape[0]
-    ocols = OC // 2 if act == ACT_SWIGLU else OC
-    out = torch.empty((BT, ocols), dtype=torch.bfloat16, device=inp.device)
-    pre = torch.empty((BT, OC), dtype=torch.bfloat16, device=inp.device) if act != ACT_NONE else None
-    nb_linear_forward_ex(out, pre, inp, weight, bias, BT, C, OC, act)
-    return out, pre
+    return (_native or _load_native()).linear_forward(inp, weight, bias, act)
 
 
 def linear_backward(dout, inp, weight, pre_act=None, inp_pre_act=None, act=ACT_NONE, dweight=None,
                     dbias=None, accumulate=False, need_dinp=True, need_dweight=True,
                     need_dbias=True):
     """Allocate missing outputs and call nb_linear_backward_ex. Returns (dinp, dweight, dbias)."""
-    BT = dout.shape[0]
-    OC, C = weight.shape
-    dev = dout.device
-    dinp = torch.empty((BT, C), dtype=torch.bfloat16, device=dev) if need_dinp else None
-    if need_dweight and dweight is None:
-        dweight = torch.empty((OC, C), dtype=torch.float32, device=dev)
-    if need_dbias and dbias is None:
-        dbias = torch.empty((OC,), dtype=torch.float32, device=dev)
-    nb_linear_backward_ex(dinp, dweight if need_dweight else None, dbias if need_dbias else None,
-                          dout, inp, weight, pre_act, inp_pre_act, BT, C, OC, act, accumulate)
-    return dinp, dweight, dbias
+    return (_native or _load_native()).linear_backward(dout, inp, weight, pre_act, inp_pre_act, act, dweight, dbias,
+                                                       accumulate, need_dinp, need_dweight, need_dbias)

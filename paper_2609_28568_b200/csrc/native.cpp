@@ -1,0 +1,235 @@
+// Native half of the Python binding: argument marshalling for the C entry points, without ctypes.
+//
+// A small layer's launches take the GPU a few microseconds, and the interpreter took longer than that
+// to issue them: per call 3.2 us to look up the current stream, 0.2 us per tensor for checks and
+// pointer, 2.4 us per allocated result, about a microsecond of argument conversion (forward and
+// backward of a layer with an activation: 33 us of host time for three launches). Here a call costs
+// its launches and about a microsecond. The functions take what the Python functions of the same name
+// take, in order and by position (paper: The stack under test: bindings compose training from the C ABI).
+#include <Python.h>
+
+#include <ATen/core/Tensor.h>
+#include <ATen/ops/empty.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <type_traits>
+#include <utility>
+
+#include "nb_linear.h"
+
+namespace {
+
+PyObject *g_error = nullptr;  // NbError, given by the Python side
+
+// Raises NbError(code, text) and returns null.
+PyObject *raise(int rc)
+{
+    PyObject *e = g_error ? PyObject_CallFunction(g_error, "is", rc, nb_last_error()) : nullptr;
+    if (e) {
+        PyErr_SetObject(reinterpret_cast<PyObject *>(Py_TYPE(e)), e);
+        Py_DECREF(e);
+    } else if (!PyErr_Occurred()) {
+        PyErr_Format(PyExc_RuntimeError, "nb_linear error %d: %s", rc, nb_last_error());
+    }
+    return nullptr;
+}
+
+void *current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
+
+// A device pointer from None, an address, or a contiguous CUDA tensor.
+bool to_pointer(PyObject *o, void *&p)
+{
+    if (o == Py_None) {
+        p = nullptr;
+        return true;
+    }
+    if (THPVariable_Check(o)) {
+        const at::Tensor &t = THPVariable_Unpack(o);
+        if (!t.is_cuda() || !t.is_contiguous()) {
+            PyErr_SetString(PyExc_AssertionError, "device tensors must be contiguous CUDA tensors");
+            return false;
+        }
+        p = t.data_ptr();
+        return true;
+    }
+    if (PyLong_Check(o)) {
+        p = PyLong_AsVoidPtr(o);
+        return !(p == nullptr && PyErr_Occurred());
+    }
+    PyErr_Format(PyExc_TypeError, "a tensor, an address or None is wanted, not %.100s", Py_TYPE(o)->tp_name);
+    return false;
+}
+
+template <class T>
+bool convert(PyObject *o, T &v)
+{
+    if constexpr (std::is_pointer_v<T>) {
+        void *p = nullptr;
+        if (!to_pointer(o, p)) return false;
+        v = p;
+    } else if constexpr (std::is_floating_point_v<T>) {
+        v = static_cast<T>(PyFloat_AsDouble(o));
+        if (PyErr_Occurred()) return false;
+    } else {
+        const long long x = PyLong_AsLongLong(o);
+        if (x == -1 && PyErr_Occurred()) return false;
+        v = static_cast<T>(x);
+        if (static_cast<long long>(v) != x) {
+            PyErr_SetString(PyExc_OverflowError, "argument out of range");
+            return false;
+        }
+    }
+    return true;
+}
+
+// fn(args..., stream): the last argument may be left out or None, for the current stream.
+template <class... A, size_t... I>
+PyObject *call(int (*fn)(A...), PyObject *const *args, Py_ssize_t n, std::index_sequence<I...>)
+{
+    constexpr Py_ssize_t N = sizeof...(A);
+    if (n != N && n != N - 1) {
+        PyErr_Format(PyExc_TypeError, "%zd or %zd arguments are wanted, not %zd", N - 1, N, n);
+        return nullptr;
+    }
+    std::tuple<A...> v;
+    auto one = [&](auto &dst, size_t i) {
+        if (static_cast<Py_ssize_t>(i) == N - 1 && (n == N - 1 || args[i] == Py_None)) {
+            if constexpr (std::is_pointer_v<std::decay_t<decltype(dst)>>) dst = current_stream();
+            return true;
+        }
+        return convert(args[i], dst);
+    };
+    if (!(one(std::get<I>(v), I) && ...)) return nullptr;
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = std::apply(fn, v);
+    Py_END_ALLOW_THREADS
+    if (rc != NB_OK) return raise(rc);
+    Py_RETURN_NONE;
+}
+
+template <auto fn>
+PyObject *entry(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    return [&]<class... A>(int (*f)(A...)) {
+        return call(f, args, n, std::index_sequence_for<A...>{});
+    }(fn);
+    END_HANDLE_TH_ERRORS
+}
+
+bool to_tensor(PyObject *o, at::Tensor &t)  // None: an undefined tensor
+{
+    if (o == Py_None) return true;
+    if (!THPVariable_Check(o)) {
+        PyErr_Format(PyExc_TypeError, "a tensor is wanted, not %.100s", Py_TYPE(o)->tp_name);
+        return false;
+    }
+    t = THPVariable_Unpack(o);
+    if (!t.is_cuda() || !t.is_contiguous()) {
+        PyErr_SetString(PyExc_AssertionError, "device tensors must be contiguous CUDA tensors");
+        return false;
+    }
+    return true;
+}
+bool two_dims(const at::Tensor &t, const char *name)
+{
+    if (t.defined() && t.dim() == 2) return true;
+    PyErr_Format(PyExc_ValueError, "%s must have two dimensions", name);
+    return false;
+}
+void *ptr(const at::Tensor &t) { return t.defined() ? t.data_ptr() : nullptr; }
+PyObject *wrap(at::Tensor t)
+{
+    if (!t.defined()) Py_RETURN_NONE;
+    return THPVariable_Wrap(std::move(t));
+}
+
+// linear_forward(inp, weight, bias, act) -> (out, pre_act or None)
+PyObject *linear_forward(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    at::Tensor inp, weight, bias;
+    int act = 0;
+    if (n != 4) return PyErr_Format(PyExc_TypeError, "4 arguments are wanted");
+    if (!to_tensor(args[0], inp) || !to_tensor(args[1], weight) || !to_tensor(args[2], bias) || !convert(args[3], act))
+        return nullptr;
+    if (!two_dims(inp, "inp") || !two_dims(weight, "weight")) return nullptr;
+    const int64_t BT = inp.size(0), C = inp.size(1), OC = weight.size(0);
+    const auto opt = inp.options().dtype(at::kBFloat16);
+    at::Tensor out = at::empty({BT, act == NB_ACT_SWIGLU ? OC / 2 : OC}, opt), pre;
+    if (act != NB_ACT_NONE) pre = at::empty({BT, OC}, opt);
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = nb_linear_forward_ex(ptr(out), ptr(pre), ptr(inp), ptr(weight), ptr(bias), BT, C, OC, act, current_stream());
+    Py_END_ALLOW_THREADS
+    if (rc != NB_OK) return raise(rc);
+    return Py_BuildValue("NN", wrap(std::move(out)), wrap(std::move(pre)));
+    END_HANDLE_TH_ERRORS
+}
+
+// linear_backward(dout, inp, weight, pre_act, inp_pre_act, act, dweight, dbias, accumulate, need_dinp,
+//                 need_dweight, need_dbias) -> (dinp, dweight, dbias)
+PyObject *linear_backward(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    HANDLE_TH_ERRORS
+    at::Tensor dout, inp, weight, pre, ipre, dw, db, dinp;
+    int act = 0;
+    if (n != 12) return PyErr_Format(PyExc_TypeError, "12 arguments are wanted");
+    if (!to_tensor(args[0], dout) || !to_tensor(args[1], inp) || !to_tensor(args[2], weight) || !to_tensor(args[3], pre) ||
+        !to_tensor(args[4], ipre) || !convert(args[5], act) || !to_tensor(args[6], dw) || !to_tensor(args[7], db))
+        return nullptr;
+    int flag[4];  // accumulate, need_dinp, need_dweight, need_dbias
+    for (int i = 0; i < 4; ++i)
+        if ((flag[i] = PyObject_IsTrue(args[8 + i])) < 0) return nullptr;
+    if (!two_dims(dout, "dout") || !two_dims(weight, "weight")) return nullptr;
+    const int64_t BT = dout.size(0), OC = weight.size(0), C = weight.size(1);
+    const auto opt = dout.options();
+    if (flag[1]) dinp = at::empty({BT, C}, opt.dtype(at::kBFloat16));
+    if (flag[2] && !dw.defined()) dw = at::empty({OC, C}, opt.dtype(at::kFloat));
+    if (flag[3] && !db.defined()) db = at::empty({OC}, opt.dtype(at::kFloat));
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = nb_linear_backward_ex(ptr(dinp), flag[2] ? ptr(dw) : nullptr, flag[3] ? ptr(db) : nullptr, ptr(dout), ptr(inp),
+                               ptr(weight), ptr(pre), ptr(ipre), BT, C, OC, act, flag[0], NB_DTYPE_F32, current_stream());
+    Py_END_ALLOW_THREADS
+    if (rc != NB_OK) return raise(rc);
+    return Py_BuildValue("NNN", wrap(std::move(dinp)), wrap(std::move(dw)), wrap(std::move(db)));
+    END_HANDLE_TH_ERRORS
+}
+
+PyObject *set_error(PyObject *, PyObject *cls)
+{
+    Py_INCREF(cls);
+    Py_XSETREF(g_error, cls);
+    Py_RETURN_NONE;
+}
+
+#define NB_ENTRY(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void *>(&entry<name>)), METH_FASTCALL, nullptr}
+#define NB_FAST(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void *>(&name)), METH_FASTCALL, nullptr}
+PyMethodDef g_methods[] = {
+    NB_ENTRY(nb_linear_forward_ex),
+    NB_ENTRY(nb_linear_backward_ex),
+    NB_ENTRY(nb_gelu_dbias_noalloc),
+    NB_ENTRY(nb_lora_linear_forward),
+    NB_ENTRY(nb_lora_linear_backward),
+    NB_ENTRY(nb_lora_down_stacked),
+    NB_ENTRY(nb_lora_linear_forward_stacked),
+    NB_ENTRY(nb_lora_linear_backward_stacked),
+    NB_ENTRY(nb_lora_da_stacked),
+    NB_ENTRY(nb_lm_head_ce_forward),
+    NB_ENTRY(nb_ce_backward),
+    NB_ENTRY(nb_cast_f32_to_bf16),
+    NB_FAST(linear_forward),
+    NB_FAST(linear_backward),
+    {"set_error", set_error, METH_O, nullptr},
+    {nullptr, nullptr, 0, nullptr},
+};
+PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_native", "Argument marshalling for the nb_linear C ABI.", -1, g_methods,
+                        nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__native(void) { return PyModule_Create(&g_module); }
