@@ -1,9 +1,17 @@
 // HBM-bound helper kernels around the GEMMs: activation backward (dz), the stand-alone dbias
-// column reduction, and the bounded-wait self-test.
+// column reduction, and the bounded-wait self-test. All of them are links of the dependent-launch
+// chain: they are launched while their predecessor drains (chained_start waits for it) and let their
+// successor set itself up while they run.
 #pragma once
 #include "gemm_sm100.cuh"
 
 namespace nb {
+
+__device__ __forceinline__ void chained_start()
+{
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
+}
 
 __device__ __forceinline__ float silu_bwd(float g)
 {
@@ -16,6 +24,7 @@ __global__ void __launch_bounds__(256)
 gelu_backward_kernel(uint4 *__restrict__ dz, const uint4 *__restrict__ dout,
                      const uint4 *__restrict__ pre, long long nvec)
 {
+    chained_start();
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < nvec;
          i += stride) {
@@ -40,6 +49,7 @@ __global__ void __launch_bounds__(256)
 swiglu_backward_kernel(uint4 *__restrict__ dz, const uint4 *__restrict__ dout,
                        const uint4 *__restrict__ pre, long long BT, int hvec /* H / 8 */)
 {
+    chained_start();
     const long long total = BT * hvec;
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
@@ -80,6 +90,7 @@ dbias_kernel(float *__restrict__ dbias, const __nv_bfloat16 *__restrict__ dz, lo
 {
     // 512 bytes of shared memory only: small enough to share an SM with a resident GEMM CTA
     __shared__ float part[kDbiasCols];
+    chained_start();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cv = lane & 7;   // column vector inside a 64-column half
     const int rs = lane >> 3;  // row inside a group of four
@@ -162,6 +173,7 @@ clear_kernel(float *__restrict__ a, long long na, float *__restrict__ b, long lo
 __global__ void __launch_bounds__(256)
 cast_f32_bf16_kernel(__nv_bfloat16 *__restrict__ dst, const float *__restrict__ src, long long n)
 {
+    chained_start();
     const long long nvec = n / 8;
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     const long long t0 = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -184,6 +196,7 @@ ce_reduce_kernel(float *__restrict__ loss, float *__restrict__ lse, const float2
                  int stats_ld, const __nv_bfloat16 *__restrict__ logits, long long ld,
                  const int *__restrict__ targets, long long BT, int V)
 {
+    chained_start();
     const int lane = threadIdx.x & 31;
     const long long row = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
     if (row >= BT) return;
@@ -213,6 +226,7 @@ __global__ void __launch_bounds__(256)
 ce_backward_kernel(uint4 *dlogits, const uint4 *logits, const float *__restrict__ lse,
                    const int *__restrict__ targets, float gscale, long long BT, int vec_per_row, int V)
 {
+    chained_start();
     const long long total = BT * vec_per_row;
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;

@@ -355,6 +355,24 @@ using DgradStoreNarrow = GemmCfg<1, 64, 7, 2, false, true, kEpiStore>;
 using WgradF32Narrow = GemmCfg<1, 64, 7, 2, true, true, kEpiF32>;
 constexpr int kNarrowN = 64;
 
+// ----------------------------------------------------------------------------- elementwise kernels
+// Launches a kernel that begins with chained_start.
+template <class... P, class... A>
+int launch_chained(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent_launch_allowed(stream) ? 1 : 0;
+    NB_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+    return NB_OK;
+}
+
 // ----------------------------------------------------------------------------- clearing
 // Zeroes up to two fp32 arrays in stream order (clear_kernel).
 int launch_clear(const DeviceState &s, void *a, int64_t na, void *b, int64_t nb_, cudaStream_t stream)
@@ -364,18 +382,9 @@ int launch_clear(const DeviceState &s, void *a, int64_t na, void *b, int64_t nb_
     long long blocks = (vec + 1023) / 1024;  // four stores per thread, up to four blocks per SM
     if (blocks > 4ll * s.num_sms) blocks = 4ll * s.num_sms;
     if (blocks < 1) blocks = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(blocks));
-    cfg.blockDim = dim3(256);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = dependent_launch_allowed(stream) ? 1 : 0;
-    NB_CUDA(cudaLaunchKernelEx(&cfg, clear_kernel, static_cast<float *>(a), static_cast<long long>(na),
-                               static_cast<float *>(b), static_cast<long long>(nb_)));
-    return NB_OK;  // not counted in g_launches, as the memsets it replaces were not
+    // not counted in g_launches, as the memsets it replaces were not
+    return launch_chained(clear_kernel, dim3(static_cast<unsigned>(blocks)), 256, stream, static_cast<float *>(a),
+                          static_cast<long long>(na), static_cast<float *>(b), static_cast<long long>(nb_));
 }
 
 // ----------------------------------------------------------------------------- small problems
@@ -775,7 +784,10 @@ int ensure_workspace(DeviceState &s, size_t bytes, cudaStream_t stream = nullptr
 int launch_dbias(DeviceState &s, float *dbias, const void *dz, int64_t BT, int64_t OC, int accumulate,
                  cudaStream_t stream)
 {
-    if (!accumulate) NB_CUDA(cudaMemsetAsync(dbias, 0, static_cast<size_t>(OC) * 4, stream));
+    if (!accumulate) {
+        const int crc = launch_clear(s, dbias, OC, nullptr, 0, stream);
+        if (crc != NB_OK) return crc;
+    }
     if (BT == 0) return NB_OK;
     const int col_blocks = static_cast<int>((OC + kDbiasCols - 1) / kDbiasCols);
     // about three blocks per SM: with six (or one) the same kernel was 15-25 % slower on the stack's
@@ -787,10 +799,9 @@ int launch_dbias(DeviceState &s, float *dbias, const void *dz, int64_t BT, int64
     const long long row_blocks = (BT + rows_per_block - 1) / rows_per_block;
     if (row_blocks > 65535) return fail(NB_ERR_UNSUPPORTED, "BT too large for the dbias grid");
     dim3 grid(col_blocks, static_cast<unsigned>(row_blocks));
-    dbias_kernel<<<grid, kDbiasThreads, 0, stream>>>(dbias, static_cast<const __nv_bfloat16 *>(dz), BT,
-                                                     static_cast<int>(OC),
-                                                     static_cast<int>(rows_per_block));
-    NB_CUDA(cudaGetLastError());
+    const int rc = launch_chained(dbias_kernel, grid, kDbiasThreads, stream, dbias, static_cast<const __nv_bfloat16 *>(dz), BT,
+                                  static_cast<int>(OC), static_cast<int>(rows_per_block));
+    if (rc != NB_OK) return rc;
     ++g_launches;
     return NB_OK;
 }
@@ -1394,16 +1405,16 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
         if ((rc = ensure_workspace(*s, static_cast<size_t>(BT * OC) * 2, stream)) != NB_OK) return rc;
         if (act == NB_ACT_GELU) {
             const long long nvec = BT * OC / 8;
-            gelu_backward_kernel<<<elementwise_grid(*s, nvec), 256, 0, stream>>>(
-                static_cast<uint4 *>(s->workspace), static_cast<const uint4 *>(dout),
-                static_cast<const uint4 *>(pre_act), nvec);
+            rc = launch_chained(gelu_backward_kernel, dim3(elementwise_grid(*s, nvec)), 256, stream,
+                                static_cast<uint4 *>(s->workspace), static_cast<const uint4 *>(dout),
+                                static_cast<const uint4 *>(pre_act), nvec);
         } else {
             const int hvec = static_cast<int>(OC / 16);
-            swiglu_backward_kernel<<<elementwise_grid(*s, BT * hvec), 256, 0, stream>>>(
-                static_cast<uint4 *>(s->workspace), static_cast<const uint4 *>(dout),
-                static_cast<const uint4 *>(pre_act), BT, hvec);
+            rc = launch_chained(swiglu_backward_kernel, dim3(elementwise_grid(*s, BT * hvec)), 256, stream,
+                                static_cast<uint4 *>(s->workspace), static_cast<const uint4 *>(dout),
+                                static_cast<const uint4 *>(pre_act), BT, hvec);
         }
-        NB_CUDA(cudaGetLastError());
+        if (rc != NB_OK) return rc;
         ++g_launches;
         dz = s->workspace;
     }
@@ -1522,12 +1533,11 @@ int nb_lm_head_ce_forward(void *logits, void *loss, void *lse, const void *inp, 
     a.stats_ld = stats_ld;
     a.v_real = static_cast<int>(V);
     if ((rc = launch_gemm_auto<FwdStoreStats1, FwdStoreStats2>(*s, a, stream)) != NB_OK) return rc;
-    const unsigned blocks = static_cast<unsigned>((BT + 7) / 8);
-    ce_reduce_kernel<<<blocks, 256, 0, stream>>>(static_cast<float *>(loss), static_cast<float *>(lse),
-                                                 static_cast<const float2 *>(s->workspace), stats_ld,
-                                                 static_cast<const __nv_bfloat16 *>(logits), Vp,
-                                                 static_cast<const int *>(targets), BT, static_cast<int>(V));
-    NB_CUDA(cudaGetLastError());
+    rc = launch_chained(ce_reduce_kernel, dim3(static_cast<unsigned>((BT + 7) / 8)), 256, stream, static_cast<float *>(loss),
+                        static_cast<float *>(lse), static_cast<const float2 *>(s->workspace), stats_ld,
+                        static_cast<const __nv_bfloat16 *>(logits), Vp, static_cast<const int *>(targets), BT,
+                        static_cast<int>(V));
+    if (rc != NB_OK) return rc;
     ++g_launches;
     return NB_OK;
 }
@@ -1546,10 +1556,11 @@ int nb_ce_backward(void *dlogits, const void *logits, const void *lse, const voi
     int rc = get_state(&s);
     if (rc != NB_OK) return rc;
     const int vec_per_row = static_cast<int>(Vp / 8);
-    ce_backward_kernel<<<elementwise_grid(*s, BT * vec_per_row), 256, 0, static_cast<cudaStream_t>(stream_)>>>(
-        static_cast<uint4 *>(dlogits), static_cast<const uint4 *>(logits), static_cast<const float *>(lse),
-        static_cast<const int *>(targets), gscale, BT, vec_per_row, static_cast<int>(V));
-    NB_CUDA(cudaGetLastError());
+    rc = launch_chained(ce_backward_kernel, dim3(elementwise_grid(*s, BT * vec_per_row)), 256,
+                        static_cast<cudaStream_t>(stream_), static_cast<uint4 *>(dlogits), static_cast<const uint4 *>(logits),
+                        static_cast<const float *>(lse), static_cast<const int *>(targets), gscale, BT, vec_per_row,
+                        static_cast<int>(V));
+    if (rc != NB_OK) return rc;
     ++g_launches;
     return NB_OK;
 }
@@ -1747,9 +1758,9 @@ int nb_cast_f32_to_bf16(void *dst, const void *src, int64_t n, void *stream_)
     DeviceState *s;
     int rc = get_state(&s);
     if (rc != NB_OK) return rc;
-    cast_f32_bf16_kernel<<<elementwise_grid(*s, n / 8 + 1), 256, 0, static_cast<cudaStream_t>(stream_)>>>(
-        static_cast<__nv_bfloat16 *>(dst), static_cast<const float *>(src), n);
-    NB_CUDA(cudaGetLastError());
+    rc = launch_chained(cast_f32_bf16_kernel, dim3(elementwise_grid(*s, n / 8 + 1)), 256, static_cast<cudaStream_t>(stream_),
+                        static_cast<__nv_bfloat16 *>(dst), static_cast<const float *>(src), n);
+    if (rc != NB_OK) return rc;
     ++g_launches;
     return NB_OK;
 }
@@ -1930,10 +1941,10 @@ int nb_gelu_dbias_noalloc(void *dbias, const void *dout, const void *pre_act, in
     if (BT > 0) {
         // dz = dout * gelu'(pre_act) overwrites the first BT*OC elements of the scratch
         const long long nvec = BT * OC / 8;
-        gelu_backward_kernel<<<elementwise_grid(local, nvec), 256, 0, stream>>>(
-            static_cast<uint4 *>(dz), static_cast<const uint4 *>(dout),
-            static_cast<const uint4 *>(pre_act), nvec);
-        NB_CUDA(cudaGetLastError());
+        const int rc = launch_chained(gelu_backward_kernel, dim3(elementwise_grid(local, nvec)), 256, stream,
+                                      static_cast<uint4 *>(dz), static_cast<const uint4 *>(dout),
+                                      static_cast<const uint4 *>(pre_act), nvec);
+        if (rc != NB_OK) return rc;
         ++g_launches;
     }
     return launch_dbias(local, static_cast<float *>(dbias), dz, BT, OC, accumulate, stream);
