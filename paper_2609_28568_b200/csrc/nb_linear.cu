@@ -208,6 +208,8 @@ struct GemmArgs {
     int reduce;
     int splits;
     float *dbias;  // wgrad: bias gradient fused into the pass over dz, or null
+    bool wait_ext;      // small-problem kernel only: TileJob::wait_ext, TileParams::trigger_late
+    bool trigger_late;
     // adapter term D += A2 . B2^T over k2 columns (k2 <= 64), read after the main k range
     const void *A2; uint64_t a2_rows, a2_cols;
     const void *B2; uint64_t b2_rows, b2_cols;
@@ -445,6 +447,7 @@ void fill_tile_job(TileJob &j, uint32_t &smem_bytes, const GemmArgs &a, int epi,
     j.e_ld = static_cast<long long>(a.e_cols);
     j.swiglu_h = a.swiglu_h;
     j.reduce = a.reduce;
+    j.wait_ext = a.wait_ext && j.kblocks_ext > 0;
     const uint32_t recv = cluster > 1 ? G::RECV_BYTES : 0u;
     const uint32_t stage = j.a_slot + G::B_BYTES;
     const int longest = (j.kblocks + cluster - 1) / cluster + j.kblocks_ext;
@@ -483,6 +486,7 @@ int launch_tile(DeviceState &s, const GemmArgs &a, int cluster, bool two, cudaSt
     uint32_t smem_bytes = 0;
     fill_tile_job<BN>(p.job[0], smem_bytes, a, EPI, false, cluster, two);
     p.cluster = cluster;
+    p.trigger_late = a.trigger_late;
     p.status = s.status;
     p.timeout_ns = kDefaultTimeoutNs;
     const uint32_t a_box = p.job[0].a_slot / 128u;
@@ -527,6 +531,7 @@ int launch_tile_pair(DeviceState &s, const GemmArgs *d, const GemmArgs &w, int a
     p.job[1].dbias = w.dbias;
     p.job[1].dbias_add = accumulate ? 1 : 0;
     p.cluster = cluster;
+    p.trigger_late = w.trigger_late;
     p.status = s.status;
     p.timeout_ns = kDefaultTimeoutNs;
     CUtensorMap tA0, tB0, tA2, tB2, tA1, tB1, tD1;
@@ -1187,9 +1192,9 @@ double narrow_us(int sms, int tiles, int kblocks)
     return 4.3 + 0.2 * kblocks * static_cast<double>((tiles + sms - 1) / sms);
 }
 
-// t[:, r] = scale * inp . A^T
+// t[:, r] = scale * inp . A^T. late (or null): whether the next launch may start before this one is done.
 int run_lora_down(DeviceState &s, void *t, const void *inp, const void *lora_a, float scale, int64_t BT, int64_t C,
-                  int64_t r, cudaStream_t stream)
+                  int64_t r, cudaStream_t stream, bool *late = nullptr)
 {
     GemmArgs a;
     memset(&a, 0, sizeof(a));
@@ -1202,6 +1207,7 @@ int run_lora_down(DeviceState &s, void *t, const void *inp, const void *lora_a, 
     const int kb = kblocks_of(C);
     const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, r <= 32, 0, 0,
                                      narrow_us(s.num_sms, (a.M + kBlockM - 1) / kBlockM, kb));
+    if (late) *late = a.trigger_late = pl.bn != 0;
     return pl.bn ? launch_tile_plan<false, kEpiStore>(s, a, pl, stream) : launch_gemm<FwdStoreNarrow>(s, a, stream);
 }
 
@@ -1269,6 +1275,7 @@ int run_lora_backward(DeviceState &s, const LoraBwd &l, cudaStream_t stream)
         const SmallPlan a1 = want_a ? plan_pair(sms, 0, 0, 0, 1, r, C, kt, false, far, false) : none;
         const double apart = ub.us + x_us + a1.us, paired = xa.bn ? ub.us + xa.us : far;
         if (ub.bn && (apart < udb || paired < udb)) {
+            dB.trigger_late = dx.wait_ext = want_x;
             if ((rc = launch_tile_pair_plan(s, &u, dB, false, l.accumulate, ub, stream)) != NB_OK) return rc;
             if (paired <= apart) return launch_tile_pair_plan(s, &dx, dA, false, l.accumulate, xa, stream);
             if (want_x && (rc = run_dgrad(s, dx, stream)) != NB_OK) return rc;
@@ -1582,7 +1589,8 @@ int nb_lora_linear_forward(void *out, void *t, const void *inp, const void *weig
     std::lock_guard<std::mutex> lock(g_mu);
     DeviceState *s;
     if ((rc = get_state(&s)) != NB_OK) return rc;
-    if ((rc = run_lora_down(*s, t, inp, lora_a, scale, BT, C, r, stream)) != NB_OK) return rc;
+    bool late = false;
+    if ((rc = run_lora_down(*s, t, inp, lora_a, scale, BT, C, r, stream, &late)) != NB_OK) return rc;
     GemmArgs a;
     memset(&a, 0, sizeof(a));  // out = inp . W^T (+ bias) + t . B^T: r extra columns of K
     a.A = inp; a.a_rows = BT; a.a_cols = C;
@@ -1594,6 +1602,7 @@ int nb_lora_linear_forward(void *out, void *t, const void *inp, const void *weig
     a.A2 = t; a.a2_rows = BT; a.a2_cols = r;
     a.B2 = lora_b; a.b2_rows = OC; a.b2_cols = r;
     a.k2 = static_cast<int>(r);
+    a.wait_ext = late;
     return run_forward(*s, a, NB_ACT_NONE, stream);
 }
 

@@ -50,11 +50,14 @@ struct TileJob {
     int reduce;         // fp32 result: 1 reduce-add, 0 overwrite
     float *dbias;       // fp32 result: column sums of dz, [M], or null
     int dbias_add;      // add to what dbias holds
+    int wait_ext;       // of this job's operands the launch before this one (trigger_late) makes only A2:
+                        // only the adapter term's loads wait for it
 };
 
 struct TileParams {
     TileJob job[2];
     int cluster;        // CTAs per cluster; job 0 splits K over it, job 1 does not
+    int trigger_late;   // the next launch may start once everything before this one is done, no sooner
     int *status;
     unsigned long long timeout_ns;
 };
@@ -153,8 +156,10 @@ struct WarpBox {
 // CTA's share of K among `cluster` (1: all of K). Every thread of the CTA calls it.
 template <int BN, bool A_MN, bool B_MN, int EPI>
 __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, uint32_t smem, int tile, int rank,
-                                          int cluster, int *status, unsigned long long timeout_ns)
+                                          int cluster, const TileParams &p)
 {
+    int *const status = p.status;
+    const unsigned long long timeout_ns = p.timeout_ns;
     using G = TileGeom<BN>;
     const int warp = static_cast<int>(threadIdx.x >> 5);
     const int lane = static_cast<int>(threadIdx.x & 31);
@@ -224,8 +229,9 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
     else __syncthreads();
     ptx::tc_fence_after();
     // nothing above read or wrote global memory: it may overlap the previous kernel's tail
-    ptx::grid_launch_dependents();
-    ptx::grid_dependency_wait();
+    if (!p.trigger_late) ptx::grid_launch_dependents();
+    if (!j.wait_ext) ptx::grid_dependency_wait();
+    if (p.trigger_late) ptx::grid_launch_dependents();
     const uint32_t tmem = ptx::ld_shared_u32_volatile(bar0 + kTileTmemSlot);
     const WaitCtx wctx{abort_addr, status, timeout_ns};
     const WaitCtx wctx_epi{abort_addr, status, 2 * timeout_ns};
@@ -233,6 +239,7 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
     // the loads of one k-block into its stage
     auto issue = [&](int kb, int stage) {
         const bool ext = kb >= kb1;
+        if (ext && j.wait_ext) ptx::grid_dependency_wait();
         const CUtensorMap *mapA = ext ? t.A2 : t.A;
         const CUtensorMap *mapB = ext ? t.B2 : t.B;
         const int k0 = (ext ? kb - kb1 : kb) * kBlockK;
@@ -614,8 +621,7 @@ tile_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const TileMaps t{&tmA, &tmB, &tmA2, &tmB2, nullptr};
     const int c = static_cast<int>(blockIdx.x);
-    tile_body<BN, false, B_MN, EPI>(p.job[0], t, ptx::smem_u32(smem_raw), c / p.cluster, c % p.cluster, p.cluster,
-                                    p.status, p.timeout_ns);
+    tile_body<BN, false, B_MN, EPI>(p.job[0], t, ptx::smem_u32(smem_raw), c / p.cluster, c % p.cluster, p.cluster, p);
 }
 
 // Two products that read the same tensor. The CTAs of job 0 form a bf16 result (A by rows, B
@@ -640,10 +646,10 @@ tile_pair_kernel(const __grid_constant__ CUtensorMap tmA0,  // boxes of up to 12
     if (c < n0) {
         const TileMaps t{&tmA0, &tmB0, &tmA2, &tmB2, nullptr};
         tile_body<BN, false, true, GELU_GRAD ? kEpiMulGeluGrad : kEpiStore>(
-            p.job[0], t, ptx::smem_u32(smem_raw), c / p.cluster, c % p.cluster, p.cluster, p.status, p.timeout_ns);
+            p.job[0], t, ptx::smem_u32(smem_raw), c / p.cluster, c % p.cluster, p.cluster, p);
     } else if (c - n0 < p.job[1].ctas) {
         const TileMaps t{&tmA1, &tmB1, nullptr, nullptr, &tmD1};
-        tile_body<BN, true, true, kEpiF32>(p.job[1], t, ptx::smem_u32(smem_raw), c - n0, 0, 1, p.status, p.timeout_ns);
+        tile_body<BN, true, true, kEpiF32>(p.job[1], t, ptx::smem_u32(smem_raw), c - n0, 0, 1, p);
     }
 }
 
