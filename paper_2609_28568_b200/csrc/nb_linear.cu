@@ -417,7 +417,7 @@ void small_launch_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attrs)[2
 }
 
 constexpr uint32_t kTileSmemTwo = 113u * 1024u;  // two CTAs on an SM
-constexpr uint32_t kTileSmemOne = 200u * 1024u;
+constexpr uint32_t kTileSmemOne = 220u * 1024u;
 
 // Fills a job (and the shared memory it needs) for D[M, N] in BN-wide tiles, K split over `cluster`.
 // two: the ring leaves room for a second CTA on the SM.
@@ -620,7 +620,8 @@ double small_cta_us(int bn, double kblocks, int rows, int ctas, bool two)
 {
     const double part = (rows < kBlockM ? rows : kBlockM) / 128.0 * bn / 64.0;
     const double stage_kb = 16.0 + bn / 8.0;
-    return 1.45 + 0.5 * part + kblocks * ((two ? (bn == 128 ? 0.30 : 0.18) : 0.152) + 1e-5 * ctas * stage_kb);
+    const double mma = bn > 128 ? 0.00105 * bn : 0.152;  // 2 bn cycles per k-block take over from the issue
+    return 1.45 + 0.5 * part + kblocks * ((two ? (bn == 128 ? 0.30 : 0.18) : mma) + 1e-5 * ctas * stage_kb);
 }
 // adding up the parts of a cluster that shares K
 double small_exchange_us(int bn, int rows)
@@ -638,17 +639,18 @@ double persistent_us(int sms, int M, int N, int kblocks)
 
 // Tile width and K split for one product D[M, N] over `kblocks`. The tiles have to fit the chip in one
 // wave; with more of them the persistent kernels, which overlap one tile's epilogue with the next
-// one's main loop, are as fast or faster (1024 rows, 768 -> 3072, 192 tiles: 9.2 us either way).
+// one's main loop, are as fast or faster (1024 rows, 768 -> 3072: 192 tiles of 128 columns 11.5 us,
+// persistent 9.2 us, 128 tiles of 192 columns 8.0 us; 256 columns never beat the persistent kernel).
 // `other` is what the alternative takes; split: 0 any split of K, else that one.
 SmallPlan plan_single(int sms, int M, int N, int kblocks, bool allow32, int split, int min_bn, double other)
 {
     SmallPlan best;
     best.us = other;
-    for (int bn = allow32 ? 32 : 64; bn <= 128; bn *= 2) {
-        if (bn < min_bn) continue;
+    for (int bn : {32, 64, 128, 192}) {
+        if (bn < min_bn || (bn == 32 && !allow32) || (bn > 128 && (min_bn || split > 1))) continue;
         const long long tiles = 1ll * ((M + kBlockM - 1) / kBlockM) * ((N + bn - 1) / bn);
         if (tiles > sms) continue;
-        for (int cl = split ? split : 1; cl <= (split ? split : 8); cl *= 2) {
+        for (int cl = split ? split : 1; cl <= (split ? split : bn > 128 ? 1 : 8); cl *= 2) {
             // a cluster lies within one GPC: not every SM finds a place in clusters of 4 or 8
             if (tiles * cl > sms * (cl >= 8 ? 0.86 : cl >= 4 ? 0.95 : 1.0) || bn / cl < 8 || (cl > 1 && 2 * cl > kblocks)) break;
             const double us = kLaunchUs + small_cta_us(bn, (kblocks + cl - 1) / cl, M, static_cast<int>(tiles * cl), false) +
@@ -708,6 +710,7 @@ int launch_tile_plan(DeviceState &s, const GemmArgs &a, const SmallPlan &pl, cud
     if constexpr (!B_MN)
         if (pl.bn == 32) return launch_tile<32, B_MN, EPI>(s, a, pl.cluster, pl.two, stream);
     if (pl.bn == 64) return launch_tile<64, B_MN, EPI>(s, a, pl.cluster, pl.two, stream);
+    if (pl.bn == 192) return launch_tile<192, B_MN, EPI>(s, a, 1, false, stream);
     return launch_tile<128, B_MN, EPI>(s, a, pl.cluster, pl.two, stream);
 }
 

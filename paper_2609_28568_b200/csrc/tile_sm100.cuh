@@ -4,7 +4,7 @@
 // problem of a few hundred rows has a handful of those: most SMs idle, each busy one works through
 // all of K by itself (512 tensor-core cycles per 64 of K, whatever part of the tile is padding), and
 // the epilogue of a 256-wide tile is exposed at the end. What bounds such a problem is latency, so
-// here a CTA takes a 128 x BN tile (BN = 32 / 64 / 128), and where there are far fewer tiles than SMs
+// here a CTA takes a 128 x BN tile (BN = 32 / 64 / 128, or 192 without a split), and where there are far fewer tiles than SMs
 // the CTAs of a cluster share a tile's K range: each accumulates its part in TMEM and sends every
 // other CTA that one's slice of the columns through distributed shared memory (st.async, counted in
 // bytes on the receiver's mbarrier); the receiver adds the parts in rank order (a fixed order:
@@ -69,11 +69,12 @@ struct TileMaps {  // one job's tensor maps
 template <int BN>
 struct TileGeom {
     static constexpr uint32_t B_BYTES = BN * kBlockK * 2;
-    static constexpr uint32_t TMEM_COLS = BN;
+    static constexpr uint32_t TMEM_COLS = BN == 192 ? 256 : BN;  // a power of two
     // behind the stages: slices received from the cluster (only where K is split), then the bias /
     // partial-sum line and the barriers
     static constexpr uint32_t RECV_BYTES = (kBlockM + 1) * BN * 4;
-    static constexpr uint32_t TAIL_BYTES = 512 + 512;
+    static constexpr uint32_t LINE_BYTES = BN > 128 ? BN * 4 : 512;
+    static constexpr uint32_t TAIL_BYTES = LINE_BYTES + 512;
 };
 
 // offsets inside the barrier block
@@ -167,8 +168,8 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
     const uint32_t off_b = static_cast<uint32_t>(stages) * j.a_slot;
     const uint32_t off_recv = off_b + static_cast<uint32_t>(stages) * G::B_BYTES;
     const uint32_t off_line = off_recv + (cluster > 1 ? G::RECV_BYTES : 0u);
-    const uint32_t line = smem + off_line;          // 128 floats: bias of the tile / dbias partial sums
-    const uint32_t bar0 = line + 512u;
+    const uint32_t line = smem + off_line;          // floats: bias of the tile / dbias partial sums
+    const uint32_t bar0 = line + G::LINE_BYTES;
     auto full_bar = [&](int s) { return bar0 + 8u * static_cast<uint32_t>(s); };
     auto empty_bar = [&](int s) { return bar0 + 8u * static_cast<uint32_t>(kTileMaxStages + s); };
     const uint32_t acc_bar = bar0 + kTileBarAcc, recv_bar = bar0 + kTileBarRecv;
@@ -496,31 +497,38 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
                         Box::flush(box + 2 * Box::BYTES, j.E + r0 * j.e_ld + j.swiglu_h + col, j.e_ld, rows - q * 32,
                                    j.swiglu_h - col, lane);
                     } else {
-                        using Box = WarpBox<HC>;
+                        // boxes of 64 columns (32, 16 where the warp's share is no multiple of that)
+                        constexpr int CW = HC % 64 == 0 ? 64 : HC % 32 == 0 ? 32 : 16;
+                        using Box = WarpBox<CW>;
                         constexpr int PLANES = EPI == kEpiGelu ? 2 : 1;
-                        const uint32_t box = smem + static_cast<uint32_t>(q * 2 + hf) * PLANES * Box::BYTES;
-#pragma unroll
-                        for (int h = 0; h < HC / 16; ++h) {
-                            float v[16];
-                            tile_ld16(t_acc + static_cast<uint32_t>(hf * HC + h * 16), v);
-#pragma unroll
-                            for (int i = 0; i < 2; ++i) {
-                                const int c = h * 2 + i;
-                                uint4 o, z;
-                                tile_math8<EPI>(j, &v[i * 8], line, hf * HC + c * 8, e[EPI == kEpiMulGeluGrad ? c : 0], o, z);
-                                ptx::st_shared_v4(box + Box::pos(lane, c), o.x, o.y, o.z, o.w);
-                                if (EPI == kEpiGelu)
-                                    ptx::st_shared_v4(box + Box::BYTES + Box::pos(lane, c), z.x, z.y, z.z, z.w);
-                            }
-                        }
-                        const int col = n0 + hf * HC;
+                        const uint32_t box0 = smem + static_cast<uint32_t>((q * 2 + hf) * (HC / CW)) * PLANES * Box::BYTES;
                         const long long r0 = m0 + q * 32;
-                        if (EPI == kEpiGelu)
-                            Box::flush(box + Box::BYTES, j.E + r0 * j.e_ld + col, j.e_ld, rows - q * 32, j.N - col, lane);
-                        Box::flush(box, j.D + r0 * j.d_ld + col, j.d_ld, rows - q * 32, j.N - col, lane);
+#pragma unroll
+                        for (int b = 0; b < HC / CW; ++b) {
+                            const uint32_t box = box0 + static_cast<uint32_t>(b) * PLANES * Box::BYTES;
+#pragma unroll
+                            for (int h = 0; h < CW / 16; ++h) {
+                                float v[16];
+                                const int c0 = hf * HC + b * CW + h * 16;  // column in the tile
+                                tile_ld16(t_acc + static_cast<uint32_t>(c0), v);
+#pragma unroll
+                                for (int i = 0; i < 2; ++i) {
+                                    uint4 o, z;
+                                    tile_math8<EPI>(j, &v[i * 8], line, c0 + i * 8,
+                                                    e[EPI == kEpiMulGeluGrad ? (b * CW + h * 16) / 8 + i : 0], o, z);
+                                    const uint32_t at = box + Box::pos(lane, h * 2 + i);
+                                    ptx::st_shared_v4(at, o.x, o.y, o.z, o.w);
+                                    if (EPI == kEpiGelu) ptx::st_shared_v4(at + Box::BYTES, z.x, z.y, z.z, z.w);
+                                }
+                            }
+                            const int col = n0 + hf * HC + b * CW;
+                            if (EPI == kEpiGelu)
+                                Box::flush(box + Box::BYTES, j.E + r0 * j.e_ld + col, j.e_ld, rows - q * 32, j.N - col, lane);
+                            Box::flush(box, j.D + r0 * j.d_ld + col, j.d_ld, rows - q * 32, j.N - col, lane);
+                        }
                     }
                 }
-            } else if constexpr (EPI != kEpiSwiglu) {
+            } else if constexpr (EPI != kEpiSwiglu && BN <= 128) {
                 // K is split: slice d of BN / cluster columns goes to rank d, laid out there as
                 // [sender][group of four columns][row], so that a warp's store fills 512 bytes; a
                 // group is 129 rows long, so that neighbouring groups of a row lie in other banks
@@ -613,7 +621,7 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
 
 // One product (forward, or dinp alone).
 template <int BN, bool B_MN, int EPI>
-__global__ void __launch_bounds__(kTileThreads, BN == 128 ? 1 : 2)
+__global__ void __launch_bounds__(kTileThreads, BN >= 128 ? 1 : 2)
 tile_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
             const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
             const __grid_constant__ TileParams p)

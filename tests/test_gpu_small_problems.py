@@ -28,6 +28,7 @@ def gen(seed, shape, std):
     (3, 72, 7200), (16, 40, 7200),                                # rows: several CTAs of features per SM
     (17, 264, 144), (64, 1544, 80), (128, 3072, 96),              # tiles: fewer rows than a tile, K split
     (129, 776, 400), (300, 2056, 272), (1000, 328, 1424),         # tiles: one row past, several row tiles
+    (1030, 72, 2608),                                             # tiles of 192 columns
 ])
 def test_small_forward(BT, C, OC, act):
     inp, w, b = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (OC,), 0.05)
@@ -49,6 +50,7 @@ def test_small_forward(BT, C, OC, act):
     (1, 8, 16), (8, 136, 3072), (64, 776, 200), (128, 264, 2056),   # dinp's K split over 2, 4, 8
     (129, 72, 136), (256, 520, 1544), (257, 520, 1544),              # the last split, the first without
     (384, 768, 776), (1000, 264, 328),                               # more k-blocks than stages for dweight
+    (1030, 2608, 72),                                                # dinp alone in tiles of 192 columns
 ])
 def test_small_backward(BT, C, OC, fused):
     inp, w, dout = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (BT, OC), 1e-3)
