@@ -342,7 +342,8 @@ int nb_debug_split_plan(int64_t M, int64_t N, int64_t K, int slots, int tile_m, 
  * Host-only view of how nb_linear_backward_ex schedules a layer whose dinp and fp32 dweight are
  * both requested (BT > 128): one persistent launch whose CTA pairs each walk a list of work units,
  * 256 x 256 tiles of dinp over all of K = OC and 256 x 256 tiles of dweight over ranges of 64-row
- * k-blocks of K = BT (paper: Results/Speed, stage table, the GEMM row: this is its backward half
+ * k-blocks of K = BT (the launch itself halves the width of a few dinp tiles over a long K; the view
+ * here is that of whole tiles; paper: Results/Speed, stage table, the GEMM row: this is its backward half
  * for one layer). No device is touched. `pairs` is the number of CTA pairs (SM count / 2),
  * `gelu_grad` whether the producer's GELU derivative is applied in the dinp epilogue (it makes
  * those units dearer in the balance). out[0..7] = dinp row tiles, dinp column tiles, k-blocks of

@@ -37,7 +37,8 @@ constexpr int kLbMaxRounds = 64;
 struct LayerBwdParams {
     int BT, C, OC;
     int num_pairs;
-    // D units: tiles of dinp, K = OC
+    // D units: tiles of dinp, 256 x d_w, K = OC
+    int d_w;       // 256, or 128 where a few 256-wide tiles over a long K would be the longest chain
     int d_tiles_m, d_tiles_n, d_tiles, d_group_m, d_kblocks;
     int d_rounds;  // full rounds (num_pairs tiles each)
     int d_tail;    // tiles of the partial round: pairs [0, d_tail) take one more
@@ -275,7 +276,8 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                 bool ok = true;
                 while (ok && it.next(p, u)) {
                     const int m0 = u.m_blk * 256 + static_cast<int>(rank) * 128;
-                    const int n0 = u.n_blk * 256 + static_cast<int>(rank) * 128;
+                    const int bw = u.is_w ? 128 : p.d_w / 2;  // this CTA's columns of B
+                    const int n0 = (u.n_blk * 2 + static_cast<int>(rank)) * bw;
                     const CUtensorMap *mapB = u.is_w ? &tmInp : &tmW;
                     for (int kb = u.kb0; kb < u.kb1; ++kb) {
                         ok = wait_barrier(wctx, DBIAS ? free_bar(stage) : empty_bar(stage), phase ^ 1u,
@@ -283,7 +285,7 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                         if (!ok) break;
                         // the leader's barrier collects the bytes of both CTAs of the pair
                         const uint32_t fb = ptx::mapa(full_bar(stage), 0);
-                        if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), 2 * (Cfg::A_BYTES + Cfg::B_BYTES));
+                        if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), 2 * (Cfg::A_BYTES + static_cast<uint32_t>(bw) * 128u));
                         const uint32_t sa = smem + Cfg::OFF_A + stage * Cfg::A_BYTES;
                         const uint32_t sb = smem + Cfg::OFF_B + stage * Cfg::B_BYTES;
                         const int k0 = kb * kBlockK;
@@ -296,7 +298,7 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                         }
                         // B (W for a D unit, inp for a W unit): n along the columns, k along the rows
                         ptx::tma_load_2d_pair(sb, mapB, fb, n0, k0);
-                        ptx::tma_load_2d_pair(sb + 8192u, mapB, fb, n0 + 64, k0);
+                        if (bw == 128) ptx::tma_load_2d_pair(sb + 8192u, mapB, fb, n0 + 64, k0);
                         if (++stage == STAGES) {
                             stage = 0;
                             phase ^= 1u;
@@ -307,7 +309,7 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
         } else if (warp == 1) {
             // -------------------------------------------------------- MMA issuer (leader CTA only)
             if (rank == 0 && ptx::elect_one()) {
-                constexpr uint32_t idesc_d = make_idesc(256, 256, false, true);
+                const uint32_t idesc_d = p.d_w == 256 ? make_idesc(256, 256, false, true) : make_idesc(256, 128, false, true);
                 constexpr uint32_t idesc_w = make_idesc(256, 256, true, true);
                 LbIter it(p, pair);
                 LbUnit u;
@@ -478,14 +480,15 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
             while (it.next(p, u)) {
                 if (ptx::ld_shared_u32_volatile(epi_abort_addr) != 0) break;
                 const int m0 = u.m_blk * 256 + static_cast<int>(rank) * 128;
-                const int nw = u.n_blk * 256 + hf * 128;  // this warp's first column
+                const int tw = u.is_w ? 256 : p.d_w;
+                const int nw = u.n_blk * tw + hf * (tw / 2);  // this warp's first column
                 bool ok = true;
                 if (lane == 0) ok = wait_barrier(wctx_epi, tfull_bar(acc), acc_phase, 400 + acc);
                 ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                 if (!ok) ptx::st_shared_u32_volatile(epi_abort_addr, 1);
                 ptx::tc_fence_after();
                 const uint32_t t_acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
-                                       static_cast<uint32_t>(acc * 256 + hf * 128);
+                                       static_cast<uint32_t>(acc * 256 + hf * (tw / 2));
                 uint32_t rr[4][32];
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
@@ -524,6 +527,7 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                     // ---------------- bf16 tile of dinp: 64-column boxes
 #pragma unroll
                     for (int s4 = 0; s4 < 4; ++s4) {
+                        if (!GELU_GRAD && s4 * 64 >= tw) break;  // a 128-wide tile: 64 columns per warp
                         const int step = s4 >> 1, sub = s4 & 1;
                         const uint32_t g = d_ord * 2u + static_cast<uint32_t>(step);
                         uint32_t (&r)[32] = rr[s4];

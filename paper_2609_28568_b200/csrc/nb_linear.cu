@@ -680,10 +680,11 @@ SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int N
                 const int crowd = static_cast<int>(n < slots ? n : slots);
                 const double td = nd ? small_cta_us(bn, (kblocks + cl - 1) / cl, M, crowd, two != 0) +
                                            (cl > 1 ? small_exchange_us(bn, M) : 0.0) : 0.0;
-                const double tw = small_cta_us(bn, kw, Mw, crowd, two != 0) + (dbias ? kw * (bn == 128 ? 0.1 : 0.05) : 0.0);
+                // the bias gradient's warps own a stage each: the fewer stages, the longer they hold them
+                const double tw = small_cta_us(bn, kw, Mw, crowd, two != 0) + (dbias ? kw * (two ? 0.18 : bn == 128 ? 0.115 : 0.05) : 0.0);
                 double us = td > tw ? td : tw;
                 if (n > slots) {
-                    const double line = (nd * cl * td + nw * tw) / slots + 0.6 * tw;
+                    const double line = (nd * cl * td + nw * tw) / slots + tw;
                     if (line > us) us = line;
                 }
                 us += kLaunchUs;
@@ -928,6 +929,13 @@ int env_int(const char *name, int dflt)
     return (e && *e) ? atoi(e) : dflt;
 }
 
+constexpr double kNarrowD = 0.6;
+bool layer_bwd_narrow(int d_tiles, int d_kblocks, int w_tiles, int w_kblocks, int P)
+{
+    return d_tiles * 4 <= P && d_kblocks >= 36 && d_kblocks >= 12 + 2 * d_tiles &&
+           static_cast<double>(d_kblocks) * P > 1.0 * d_tiles * d_kblocks + 1.0 * w_tiles * w_kblocks;
+}
+
 // The schedule of layer_bwd_kernel for P CTA pairs (layer_bwd_sm100.cuh describes the unit list).
 // Costs are counted in k-blocks of tensor-core time: a D unit costs its k-blocks plus eD (the part
 // of its epilogue the next main loop does not hide: larger with gelu'), a W unit its k-blocks plus
@@ -939,8 +947,13 @@ int env_int(const char *name, int dflt)
 //  3. The last D round is partial: pairs [0, d_tail) take one more tile. The W units left over are
 //     laid out as one line of k-blocks and cut into P ranges, shorter by one D unit's cost for the
 //     pairs that took a tail tile. If the line is too short for that, one W round is taken back.
+// narrow: D tiles may be 128 columns wide. They are where the 256-wide ones are at most a quarter of the
+// pairs, K is long, and a single one takes longer than a pair's share of all the work: 1500 rows,
+// 768 -> 3072, 18 tiles of 48 k-blocks, 18.9 -> 16.4 us; 1024 rows, 1024 -> 6144, 32.5 -> 24.4 us. With
+// more tiles the operand traffic of halved ones costs more than the shorter chain gives (2021 rows,
+// 768 -> 2304, 24 tiles: 16.0 -> 19.4 us). A 128-wide k-block is counted as 0.6 of a 256-wide one.
 // Returns NB_ERR_UNSUPPORTED when the shape needs more rounds than the order mask holds.
-int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad)
+int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad, bool narrow)
 {
     memset(&p, 0, sizeof(p));
     if (P < 1 || P > kMaxPairs) return fail(NB_ERR_UNSUPPORTED, "CTA pair count %d out of range", P);
@@ -955,11 +968,18 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     p.num_pairs = P;
     p.d_tiles_m = static_cast<int>((BT + 255) / 256);
     p.d_tiles_n = static_cast<int>((C + 255) / 256);
-    p.d_tiles = p.d_tiles_m * p.d_tiles_n;
     p.d_kblocks = static_cast<int>((OC + kBlockK - 1) / kBlockK);
+    p.w_tiles_n = p.d_tiles_n;
+    p.d_w = 256;
+    if (narrow && !gelu_grad && layer_bwd_narrow(p.d_tiles_m * p.d_tiles_n, p.d_kblocks,
+                                                 static_cast<int>((OC + 255) / 256) * p.w_tiles_n,
+                                                 static_cast<int>((BT + kBlockK - 1) / kBlockK), P)) {
+        p.d_w = 128;
+        p.d_tiles_n = static_cast<int>((C + 127) / 128);
+    }
+    p.d_tiles = p.d_tiles_m * p.d_tiles_n;
     p.d_group_m = (p.d_tiles_n >= 64 ? 64 : p.d_tiles_n <= 4 ? 4 : 16) / 2;
     p.w_tiles_m = static_cast<int>((OC + 255) / 256);
-    p.w_tiles_n = p.d_tiles_n;
     p.w_tiles = p.w_tiles_m * p.w_tiles_n;
     p.w_kblocks = static_cast<int>((BT + kBlockK - 1) / kBlockK);
     int chunks = (2 * P + p.w_tiles - 1) / p.w_tiles;
@@ -974,7 +994,7 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     p.w_units = static_cast<int>(w_units);
     p.d_rounds = p.d_tiles / P;
     p.d_tail = p.d_tiles % P;
-    const double cD = p.d_kblocks + eD;
+    const double cD = p.d_kblocks * (p.d_w == 128 ? kNarrowD : 1.0) + eD;
     // the units of the last chunk may be shorter than the others: they all stay in the tail, where
     // lengths are counted exactly
     p.w_last_len = p.w_kblocks - (chunks - 1) * p.w_kbc;
@@ -1085,7 +1105,7 @@ int launch_layer_bwd(DeviceState &s, const void *dz, const void *weight, const v
         attr_set[dev] = true;
     }
     LayerBwdParams p;
-    int rc = plan_layer_bwd(p, BT, C, OC, max_pairs[dev], Cfg::GELU_GRAD);
+    int rc = plan_layer_bwd(p, BT, C, OC, max_pairs[dev], Cfg::GELU_GRAD, true);
     if (rc != NB_OK) return rc;
     p.dbias = Cfg::DBIAS ? dbias : nullptr;
     p.status = s.status;
@@ -1162,15 +1182,17 @@ int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
 
 // A layer's backward without the small-problem kernel: layer_bwd_kernel for both products, else a
 // launch per product. An fp32 result that starts from zero costs the clearing besides.
-double backward_us(int sms, int M, int BT, int N, int Mw, int kd, int kw, bool accumulate, bool apart)
+double backward_us(int sms, int M, int BT, int N, int Mw, int kd, int kw, bool accumulate, bool apart, bool gelu)
 {
     const int slots = sms / 2;
     const double d_tiles = static_cast<double>((M + 255) / 256) * ((N + 255) / 256);
     const double w_tiles = static_cast<double>((Mw + 255) / 256) * ((N + 255) / 256);
-    const double clear = accumulate ? 0.0 : 1.0;
+    const double clear = accumulate ? 0.0 : 2.8;
     if (M > 0 && BT > kBlockM && !apart) {
-        const double level = (d_tiles * (kd + 3) + w_tiles * (kw + 3)) / slots;
-        return 5.3 + clear + 0.27 * (d_tiles > 0 && kd > level ? kd : level);
+        const bool narrow = !gelu && layer_bwd_narrow(static_cast<int>(d_tiles), kd, static_cast<int>(w_tiles), kw, slots);
+        const double chain = narrow ? kNarrowD * kd : kd;
+        const double level = ((narrow ? 2.0 : 1.0) * d_tiles * (chain + 3) + w_tiles * (kw + 3)) / slots;
+        return 5.3 + clear + 0.27 * (chain > level ? chain : level);
     }
     const double waves = w_tiles / slots;
     const double w_us = 5.0 + (waves < 1.0 ? 1.0 : waves) * (0.27 * (waves < 1.0 ? kw * waves : kw) + 0.8);
@@ -1267,7 +1289,7 @@ int run_lora_backward(DeviceState &s, const LoraBwd &l, cudaStream_t stream)
     const int split = dinp_split(sms, BT, C, ko + 1);
     const double x_us = want_x ? plan_single(sms, BT, C, ko + 1, false, split, 0, persistent_us(sms, BT, C, ko + 1)).us : 0.0;
     if (l.dlora_b) {
-        const double clear = l.accumulate ? 0.0 : 1.0;
+        const double clear = l.accumulate ? 0.0 : 2.8;
         const int udb_tiles = (OC + 127) / 128 + (want_a ? (C + 127) / 128 : 0);
         const double udb = 6.0 + clear + x_us + udb_tiles * static_cast<double>((panels + sms - 1) / sms) *
                            (0.37 + 0.25 * (panels < sms ? panels : sms) / sms);  // reading dout takes over towards one panel per SM
@@ -1448,7 +1470,7 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
         w.splits = 1;
         w.dbias = static_cast<float *>(dbias);
         const SmallPlan pl = plan_pair(s->num_sms, dinp ? d.M : 0, d.N, kd, split, w.M, w.N, kw, dbias != nullptr,
-                                       backward_us(s->num_sms, dinp ? d.M : 0, d.M, d.N, w.M, kd, kw, accumulate != 0, split > 1), false);
+                                       backward_us(s->num_sms, dinp ? d.M : 0, d.M, d.N, w.M, kd, kw, accumulate != 0, split > 1, inp_pre_act != nullptr), false);
         if (pl.bn) return launch_tile_pair_plan(*s, dinp ? &d : nullptr, w, inp_pre_act != nullptr, accumulate, pl, stream);
     }
 
@@ -1754,7 +1776,7 @@ int nb_lora_da_stacked(void *da_stack, const void *u_stack, const void *inp, int
     w.M = static_cast<int>(R); w.N = static_cast<int>(C); w.K = static_cast<int>(BT);
     const int kw = kblocks_of(BT);
     const SmallPlan pl = plan_pair(s->num_sms, 0, 0, 0, 1, w.M, w.N, kw, false,
-                                   backward_us(s->num_sms, 0, w.K, w.N, w.M, 0, kw, accumulate != 0, true), false);
+                                   backward_us(s->num_sms, 0, w.K, w.N, w.M, 0, kw, accumulate != 0, true, false), false);
     if (pl.bn) return launch_tile_pair_plan(*s, nullptr, w, false, accumulate, pl, stream);
     return run_wgrad_f32(*s, u_stack, inp, da_stack, nullptr, BT, R, C, accumulate, stream);
 }
@@ -1844,7 +1866,7 @@ int nb_debug_layer_bwd_plan(int64_t BT, int64_t C, int64_t OC, int pairs, int ge
 {
     if (!out || cap < 8 || BT <= 0 || C <= 0 || OC <= 0) return -fail(NB_ERR_INVALID_ARG, "bad argument");
     LayerBwdParams p;
-    const int rc = plan_layer_bwd(p, BT, C, OC, pairs, gelu_grad != 0);
+    const int rc = plan_layer_bwd(p, BT, C, OC, pairs, gelu_grad != 0, false);
     if (rc != NB_OK) return -rc;
     out[0] = p.d_tiles_m; out[1] = p.d_tiles_n; out[2] = p.d_kblocks;
     out[3] = p.w_tiles_m; out[4] = p.w_tiles_n; out[5] = p.w_kblocks;

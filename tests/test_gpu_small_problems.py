@@ -51,6 +51,7 @@ def test_small_forward(BT, C, OC, act):
     (129, 72, 136), (256, 520, 1544), (257, 520, 1544),              # the last split, the first without
     (384, 768, 776), (1000, 264, 328),                               # more k-blocks than stages for dweight
     (1030, 2608, 72),                                                # dinp alone in tiles of 192 columns
+    (1500, 776, 3080), (1030, 1000, 6152),                           # the persistent launch, dinp in halved tiles
 ])
 def test_small_backward(BT, C, OC, fused):
     inp, w, dout = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (BT, OC), 1e-3)
