@@ -684,9 +684,10 @@ SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int N
                 const double tw = small_cta_us(bn, kw, Mw, crowd, two != 0) + (dbias ? kw * (two ? 0.18 : bn == 128 ? 0.115 : 0.05) : 0.0);
                 double us = td > tw ? td : tw;
                 if (n > slots) {
-                    const double line = (nd * cl * td + nw * tw) / slots + tw;
+                    const double line = (nd * cl * td + nw * tw) / slots + 0.6 * tw;
                     if (line > us) us = line;
                 }
+                if (two && bn == 128) us *= 1.2;  // three stages each: short rings that wait for each other
                 us += kLaunchUs;
                 if (us < best.us) best = SmallPlan{bn, cl, two != 0, us};
             }
@@ -1190,7 +1191,7 @@ double backward_us(int sms, int M, int BT, int N, int Mw, int kd, int kw, bool a
     const double clear = accumulate ? 0.0 : 2.8;
     if (M > 0 && BT > kBlockM && !apart) {
         const bool narrow = !gelu && layer_bwd_narrow(static_cast<int>(d_tiles), kd, static_cast<int>(w_tiles), kw, slots);
-        const double chain = narrow ? kNarrowD * kd : kd;
+        const double chain = narrow ? 0.7 * kd : kd;
         const double level = ((narrow ? 2.0 : 1.0) * d_tiles * (chain + 3) + w_tiles * (kw + 3)) / slots;
         return 5.3 + clear + 0.27 * (chain > level ? chain : level);
     }
