@@ -12,8 +12,8 @@
 // before the kernel waits for the one before it. Where K is long and there are few features, the
 // CTAs of a cluster share K and read each other's sums.
 //
-// Chained launches, 8 rows, weights from DRAM, against gemm_kernel: 768 -> 768 2.2 us (6.7),
-// 768 -> 3072 3.0 us (7.8), 3072 -> 768 3.7 us (19.9), 768 -> 50304 14.3 us (17.2; 77 MB of weights
+// Chained launches, 8 rows, weights from DRAM, against gemm_kernel: 768 -> 768 2.1 us (6.7),
+// 768 -> 3072 2.7 us (7.8), 3072 -> 768 3.3 us (19.9), 768 -> 50304 14.4 us (17.2; 77 MB of weights
 // take 12 us).
 #pragma once
 #include "gemm_sm100.cuh"
@@ -51,14 +51,14 @@ __device__ __forceinline__ uint4 ld_stream(const __nv_bfloat16 *p)
 }
 
 // NT: groups of eight rows. MANY: there are several CTAs of work per SM (the head's 50304 features):
-// fewer pieces of K in flight per thread and more CTAs on an SM (8 rows, 768 -> 50304: 14.3 us
-// against 24.2 us; for 768 -> 768 the other form takes 2.2 us against 2.7).
+// fewer pieces of K in flight per thread and four CTAs on an SM (8 rows, 768 -> 50304: 14.4 us
+// against 22.7 us with two; five or six have too few registers, 15.7 and 17.1 us).
 template <int NT, int EPI, bool MANY>
-__global__ void __launch_bounds__(kRowsThreads, MANY ? 6 : 1)
+__global__ void __launch_bounds__(kRowsThreads, MANY ? 4 : 1)
 rows_kernel(const RowsParams p)
 {
     constexpr int SETS = EPI == kEpiSwiglu ? 2 : 1;  // gate and up rows
-    constexpr int U = MANY ? 2 : SETS == 2 ? 3 : 6;  // pieces of K in flight
+    constexpr int U = MANY ? 3 : SETS == 2 ? 3 : 6;  // pieces of K in flight
     constexpr int LD = 18;  // floats from one row's sixteen partial sums to the next
     __shared__ float part[SETS][kRowsWarps][NT * 8][LD];
     const int warp = static_cast<int>(threadIdx.x >> 5), lane = static_cast<int>(threadIdx.x & 31);
@@ -88,6 +88,23 @@ rows_kernel(const RowsParams p)
     }
     ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
+
+    // two neighbouring features of one row per thread at the end; their bias is fetched with the operands
+    // (fetched when it is needed it adds an L2 latency to the chain)
+    constexpr int ITEMS = NT * 8 * (kRowsFeatures / 2);
+    static_assert(ITEMS <= kRowsThreads, "one item per thread");
+    const int m = static_cast<int>(threadIdx.x) / (kRowsFeatures / 2), f = (static_cast<int>(threadIdx.x) % (kRowsFeatures / 2)) * 2;
+    const bool mine = static_cast<int>(threadIdx.x) < ITEMS && (p.ksplit == 1 || m % p.ksplit == rank) && m < p.M &&
+                      f0 + f < span;
+    float bias[SETS][2];
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+        bias[s][0] = bias[s][1] = 0.0f;
+        if (!MANY && mine && p.bias != nullptr) {  // only 2-byte aligned: element by element
+            bias[s][0] = __bfloat162float(p.bias[s * p.swiglu_h + f0 + f]);
+            bias[s][1] = __bfloat162float(p.bias[s * p.swiglu_h + f0 + f + 1]);
+        }
+    }
 
     float acc[SETS][NT][4];
 #pragma unroll
@@ -133,16 +150,12 @@ rows_kernel(const RowsParams p)
             part[s][warp][n * 8 + 2 * t + 1][g + 8] = acc[s][n][3];
         }
     __syncthreads();
-    // two neighbouring features of one row per thread
-    constexpr int ITEMS = NT * 8 * (kRowsFeatures / 2);
-    static_assert(ITEMS <= kRowsThreads, "one item per thread");
-    const int m = static_cast<int>(threadIdx.x) / (kRowsFeatures / 2), f = (static_cast<int>(threadIdx.x) % (kRowsFeatures / 2)) * 2;
-    const bool mine = static_cast<int>(threadIdx.x) < ITEMS;
     float z[SETS][2];
+    const bool split = p.ksplit > 1;
 #pragma unroll
     for (int s = 0; s < SETS; ++s) {
         z[s][0] = z[s][1] = 0.0f;
-        if (mine)
+        if (static_cast<int>(threadIdx.x) < ITEMS)
 #pragma unroll
             for (int w = 0; w < kRowsWarps; ++w) {
                 const float2 v = *reinterpret_cast<const float2 *>(&part[s][w][m][f]);
@@ -150,15 +163,14 @@ rows_kernel(const RowsParams p)
                 z[s][1] += v.y;
             }
     }
-    const bool split = p.ksplit > 1;
     if (split) {
         // the CTA's sums stand where warp 0's were (each thread overwrites what it alone has read);
         // rank r finishes the rows m with m % ksplit == r
 #pragma unroll
         for (int s = 0; s < SETS; ++s)
-            if (mine) *reinterpret_cast<float2 *>(&part[s][0][m][f]) = make_float2(z[s][0], z[s][1]);
+            if (static_cast<int>(threadIdx.x) < ITEMS) *reinterpret_cast<float2 *>(&part[s][0][m][f]) = make_float2(z[s][0], z[s][1]);
         ptx::cluster_sync();
-        if (mine && m % p.ksplit == rank)
+        if (mine)
 #pragma unroll
             for (int s = 0; s < SETS; ++s) {
                 z[s][0] = z[s][1] = 0.0f;
@@ -172,14 +184,19 @@ rows_kernel(const RowsParams p)
             }
         ptx::cluster_sync();  // nobody leaves while a peer may still read its sums
     }
+    if (!mine) return;
     const int col = f0 + f;
-    if (!mine || (split && m % p.ksplit != rank) || m >= p.M || col >= span) return;
-    if (p.bias != nullptr)
+    if (MANY && p.bias != nullptr)  // other CTAs of the SM cover the latency, and registers are scarce
 #pragma unroll
         for (int s = 0; s < SETS; ++s) {
-            z[s][0] += __bfloat162float(p.bias[s * p.swiglu_h + col]);
-            z[s][1] += __bfloat162float(p.bias[s * p.swiglu_h + col + 1]);
+            bias[s][0] = __bfloat162float(p.bias[s * p.swiglu_h + col]);
+            bias[s][1] = __bfloat162float(p.bias[s * p.swiglu_h + col + 1]);
         }
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+        z[s][0] += bias[s][0];
+        z[s][1] += bias[s][1];
+    }
     const long long row = m;
     uint32_t o;
     if (EPI == kEpiStore) {
