@@ -303,25 +303,29 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     const uint32_t epi_abort_addr = bar0 + 248;
     static_assert(8 * (3 * STAGES + 8) <= 240, "barrier region");
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            ptx::mbar_init(full_bar(s), 1);
-            ptx::mbar_init(empty_bar(s), 1);  // MMAs that read the stage are done
-            ptx::mbar_init(free_bar(s), 4);   // DBIAS: the four reducer warps have read it too
+    if (warp == 0) {  // a lane per barrier: one after the other they delay the first load
+        if (lane < STAGES) {
+            ptx::mbar_init(full_bar(lane), 1);
+            ptx::mbar_init(empty_bar(lane), 1);  // MMAs that read the stage are done
+            ptx::mbar_init(free_bar(lane), 4);   // DBIAS: the four reducer warps have read it too
+        } else if (lane < STAGES + 2) {
+            ptx::mbar_init(tfull_bar(lane - STAGES), 1);
+            ptx::mbar_init(tempty_bar(lane - STAGES), kEpiWarps * CG);  // one arrive per epilogue warp of the tile
         }
-        for (int b = 0; b < 2; ++b) {
-            ptx::mbar_init(tfull_bar(b), 1);
-            ptx::mbar_init(tempty_bar(b), kEpiWarps * CG);  // one arrive per epilogue warp of the tile
+        if (Cfg::WARP_EPI && EPI == kEpiMulGeluGrad && lane < 2 * kEpiWarps)  // two per epilogue warp, above the common slots
+            ptx::mbar_init(bar0 + 256u + 8u * lane, 1);
+        if (lane == 31) {
+            ptx::st_shared_u32_volatile(abort_addr, 0);
+            ptx::st_shared_u32_volatile(epi_abort_addr, 0);
         }
-        if (Cfg::WARP_EPI && EPI == kEpiMulGeluGrad)  // two per epilogue warp, above the common slots
-            for (int b = 0; b < 2 * kEpiWarps; ++b) ptx::mbar_init(bar0 + 256u + 8u * b, 1);
-        ptx::st_shared_u32_volatile(abort_addr, 0);
-        ptx::st_shared_u32_volatile(epi_abort_addr, 0);
         ptx::fence_barrier_init();
-        ptx::prefetch_tmap(&tmA);
-        ptx::prefetch_tmap(&tmB);
-        ptx::prefetch_tmap(&tmD);
-        if (EPI == kEpiGelu || EPI == kEpiSwiglu || EPI == kEpiMulGeluGrad) ptx::prefetch_tmap(&tmE);
+        if (lane == 30) {
+            ptx::prefetch_tmap(&tmA);
+            ptx::prefetch_tmap(&tmB);
+            ptx::prefetch_tmap(&tmD);
+            if (EPI == kEpiGelu || EPI == kEpiSwiglu || EPI == kEpiMulGeluGrad) ptx::prefetch_tmap(&tmE);
+        }
+        __syncwarp();
     }
     if (warp == 1) {
         ptx::tmem_alloc<CG>(tmem_slot, Cfg::TMEM_COLS);

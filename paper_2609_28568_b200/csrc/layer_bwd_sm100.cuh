@@ -225,26 +225,30 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
     const uint32_t abort_addr = bar0 + 484;
     const uint32_t epi_abort_addr = bar0 + 488;
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            ptx::mbar_init(full_bar(s), 1);
-            ptx::mbar_init(empty_bar(s), 1);
-            ptx::mbar_init(free_bar(s), 1);
+    if (warp == 0) {  // a lane per barrier: one after the other they delay the first load
+        if (lane < STAGES) {
+            ptx::mbar_init(full_bar(lane), 1);
+            ptx::mbar_init(empty_bar(lane), 1);
+            ptx::mbar_init(free_bar(lane), 1);
+        } else if (lane < STAGES + 2) {
+            ptx::mbar_init(tfull_bar(lane - STAGES), 1);
+            ptx::mbar_init(tempty_bar(lane - STAGES), kEpiWarps * 2);
         }
-        for (int b = 0; b < 2; ++b) {
-            ptx::mbar_init(tfull_bar(b), 1);
-            ptx::mbar_init(tempty_bar(b), kEpiWarps * 2);
+        if (lane < 16) ptx::mbar_init(aux_bar(static_cast<uint32_t>(lane)), 1);
+        if (lane == 31) {
+            ptx::st_shared_u32_volatile(abort_addr, 0);
+            ptx::st_shared_u32_volatile(epi_abort_addr, 0);
         }
-        for (uint32_t b = 0; b < 16; ++b) ptx::mbar_init(aux_bar(b), 1);
-        ptx::st_shared_u32_volatile(abort_addr, 0);
-        ptx::st_shared_u32_volatile(epi_abort_addr, 0);
         ptx::fence_barrier_init();
-        ptx::prefetch_tmap(&tmDz);
-        ptx::prefetch_tmap(&tmW);
-        ptx::prefetch_tmap(&tmInp);
-        ptx::prefetch_tmap(&tmDinp);
-        ptx::prefetch_tmap(&tmDw);
-        if (GELU_GRAD) ptx::prefetch_tmap(&tmPre);
+        if (lane == 30) {
+            ptx::prefetch_tmap(&tmDz);
+            ptx::prefetch_tmap(&tmW);
+            ptx::prefetch_tmap(&tmInp);
+            ptx::prefetch_tmap(&tmDinp);
+            ptx::prefetch_tmap(&tmDw);
+            if (GELU_GRAD) ptx::prefetch_tmap(&tmPre);
+        }
+        __syncwarp();
     }
     if (warp == 2) {
         ptx::tmem_alloc<2>(tmem_slot, Cfg::TMEM_COLS);

@@ -10,10 +10,11 @@
 // bytes on the receiver's mbarrier); the receiver adds the parts in rank order (a fixed order:
 // results do not vary) and runs the epilogue on its slice.
 //
-//   warp 0      TMA producer; before it waits for the previous kernel of the stream it asks for the
-//               weight tiles of the CTA to be brought into L2 (a hint: nothing is read into the SM)
+//   warp 0      TMA producer
 //   warp 1      MMA issuer, TMEM allocation
-//   warps 2..9  epilogue: TMEM -> registers -> bias / activation -> the warp's box in the drained
+//   warps 2..9  before they wait for the previous kernel of the stream they ask for the first weight
+//               tiles of the CTA to be brought into L2 (a hint: nothing is read into the SM); then
+//               epilogue: TMEM -> registers -> bias / activation -> the warp's box in the drained
 //               pipeline stages -> whole rows of the box to global memory (no TMA store to wait for:
 //               a shorter chain), or, for fp32 weight gradients, TMA stores / reduce-adds
 //
@@ -31,6 +32,7 @@ namespace nb {
 
 constexpr int kTileMaxStages = 16;
 constexpr int kTileThreads = 320;
+constexpr int kTilePrefetch = 1;  // weight k-blocks each epilogue warp asks for ahead of time
 
 struct TileJob {
     int M, N;
@@ -188,21 +190,27 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
     if (!smem_ok && threadIdx.x == 0 && atomicCAS(status, 0, kStatusBadSmem) == 0)
         status[2] = static_cast<int>(blockIdx.x);
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < stages; ++s) {
-            ptx::mbar_init(full_bar(s), 1);
+    if (warp == 0) {
+        // one lane per stage: a lane after the other would spend longer here than a k-block takes
+        if (lane < stages) {
+            ptx::mbar_init(full_bar(lane), 1);
             // the tensor core has read the stage; with the bias gradient one epilogue warp has too
-            ptx::mbar_init(empty_bar(s), sum_dz ? 2 : 1);
+            ptx::mbar_init(empty_bar(lane), sum_dz ? 2 : 1);
         }
-        ptx::mbar_init(acc_bar, 1);
-        ptx::mbar_init(recv_bar, 1);
-        // every rank sends this CTA its part of rows x (BN / cluster) columns
-        if (cluster > 1) ptx::mbar_expect_tx(recv_bar, static_cast<uint32_t>(rows) * BN * 4u);
-        ptx::st_shared_u32_volatile(abort_addr, 0);
+        if (lane == 31) {
+            ptx::mbar_init(acc_bar, 1);
+            ptx::mbar_init(recv_bar, 1);
+            // every rank sends this CTA its part of rows x (BN / cluster) columns
+            if (cluster > 1) ptx::mbar_expect_tx(recv_bar, static_cast<uint32_t>(rows) * BN * 4u);
+            ptx::st_shared_u32_volatile(abort_addr, 0);
+        }
         ptx::fence_barrier_init();
-        ptx::prefetch_tmap(t.A);
-        ptx::prefetch_tmap(t.B);
-        if (EPI == kEpiF32) ptx::prefetch_tmap(t.D);
+        if (lane == 30) {
+            ptx::prefetch_tmap(t.A);
+            ptx::prefetch_tmap(t.B);
+            if (EPI == kEpiF32) ptx::prefetch_tmap(t.D);
+        }
+        __syncwarp();
     }
     if (warp == 1) {
         ptx::tmem_alloc<1>(bar0 + kTileTmemSlot, G::TMEM_COLS);
@@ -213,15 +221,20 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
     constexpr int B_BOXES = EPI == kEpiSwiglu ? 2 : B_MN ? BN / 64 : 1;
     constexpr uint32_t B_BOX_BYTES = G::B_BYTES / B_BOXES;
     auto b_row = [&](int i) { return EPI == kEpiSwiglu ? i * j.swiglu_h + n0 : n0; };
-    if (warp == 0 && EPI != kEpiF32) {
-        // B is the weight: its tiles may be brought into L2 while the previous kernel still runs
+    if (warp >= 2 && EPI != kEpiF32) {
+        // B is the weight: its tiles may be brought into L2 while the previous kernel still runs (issued
+        // by one thread this took longer than the rest of the set-up)
         if (ptx::elect_one()) {
-            for (int kb = kb0; kb < kb1; ++kb)
+#pragma unroll
+            for (int r = 0; r < kTilePrefetch; ++r) {
+                const int kb = kb0 + warp - 2 + r * kEpiWarps;
+                if (kb >= kb1) break;
 #pragma unroll
                 for (int i = 0; i < B_BOXES; ++i) {
                     if (B_MN) ptx::tma_prefetch_2d(t.B, n0 + i * 64, kb * kBlockK);
                     else ptx::tma_prefetch_2d(t.B, kb * kBlockK, b_row(i));
                 }
+            }
         }
         __syncwarp();
     }
