@@ -200,16 +200,30 @@ ce_reduce_kernel(float *__restrict__ loss, float *__restrict__ lse, const float2
     const int lane = threadIdx.x & 31;
     const long long row = static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5);
     if (row >= BT) return;
+    // one pass, eight partials of the row in flight per lane (two passes, one load at a time, took
+    // 19 us for 16384 rows of 394 partials, 52 MB)
     const float2 *st = stats + row * stats_ld;
-    float m = -INFINITY;
-    for (int k = lane; k < stats_ld; k += 32) m = fmaxf(m, st[k].x);
+    float m = -INFINITY, s = 0.0f;
+    for (int k0 = lane; k0 < stats_ld; k0 += 32 * 8) {
+        float2 v[8];
+        float mx = m;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    float s = 0.0f;
-    for (int k = lane; k < stats_ld; k += 32) {
-        const float2 v = st[k];
-        if (v.x > -INFINITY) s += v.y * __expf(v.x - m);
+        for (int i = 0; i < 8; ++i) {
+            v[i] = k0 + 32 * i < stats_ld ? __ldg(st + k0 + 32 * i) : make_float2(-INFINITY, 0.0f);
+            mx = fmaxf(mx, v[i].x);
+        }
+        if (mx > -INFINITY) {
+            s *= __expf(m - mx);  // 0 while m = -inf
+            m = mx;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) s += v[i].y * __expf(v[i].x - m);
+        }
     }
+    float mw = m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mw = fmaxf(mw, __shfl_xor_sync(0xffffffffu, mw, o));
+    if (m > -INFINITY) s *= __expf(m - mw);
+    m = mw;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {

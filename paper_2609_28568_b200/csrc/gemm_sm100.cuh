@@ -728,7 +728,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         }
                     }
                 }
-                float sv[EPI == kEpiStoreStats ? 32 : 1];
+                uint32_t sw2[EPI == kEpiStoreStats ? 16 : 1];  // kEpiStoreStats: the 32 stored (rounded) values
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const uint32_t pos = chunk_pos(sub * 4 + j);
@@ -762,11 +762,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         const uint32_t w0 = pack_f2_bf16x2(z[0]), w1 = pack_f2_bf16x2(z[1]),
                                        w2 = pack_f2_bf16x2(z[2]), w3 = pack_f2_bf16x2(z[3]);
                         ptx::st_shared_v4(stg + pos, w0, w1, w2, w3);
-                        if (EPI == kEpiStoreStats) {  // keep the eight stored (rounded) values
-                            sv[j * 8 + 0] = ptx::bf16_lo(w0); sv[j * 8 + 1] = ptx::bf16_hi(w0);
-                            sv[j * 8 + 2] = ptx::bf16_lo(w1); sv[j * 8 + 3] = ptx::bf16_hi(w1);
-                            sv[j * 8 + 4] = ptx::bf16_lo(w2); sv[j * 8 + 5] = ptx::bf16_hi(w2);
-                            sv[j * 8 + 6] = ptx::bf16_lo(w3); sv[j * 8 + 7] = ptx::bf16_hi(w3);
+                        if (EPI == kEpiStoreStats) {
+                            sw2[j * 4] = w0;
+                            sw2[j * 4 + 1] = w1;
+                            sw2[j * 4 + 2] = w2;
+                            sw2[j * 4 + 3] = w3;
                         }
                     }
                 }
@@ -774,25 +774,37 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     // online softmax statistics of this thread's 32 stored values: running
                     // maximum st_m and sum of exp(value - st_m), columns >= v_real left out
                     const int g0 = nw + s4 * 32;
-                    float mx = -INFINITY;
                     if (g0 + 32 > p.v_real) {  // only the tile that straddles v_real masks
 #pragma unroll
-                        for (int k = 0; k < 32; ++k)
-                            if (g0 + k >= p.v_real) sv[k] = -INFINITY;
+                        for (int k = 0; k < 16; ++k) {
+                            if (g0 + 2 * k >= p.v_real) sw2[k] = 0xff80ff80u;  // minus infinity, twice
+                            else if (g0 + 2 * k + 1 >= p.v_real) sw2[k] = (sw2[k] & 0xffffu) | 0xff800000u;
+                        }
                     }
+                    // maximum of pairs, and pairs through the multiply-add and the sum: half the
+                    // instructions of one value at a time
+                    uint32_t mx2 = sw2[0];
 #pragma unroll
-                    for (int k = 0; k < 32; ++k) mx = fmaxf(mx, sv[k]);
+                    for (int k = 1; k < 16; ++k) mx2 = ptx::max_bf16x2(mx2, sw2[k]);
+                    const float mx = fmaxf(ptx::bf16_lo(mx2), ptx::bf16_hi(mx2));
                     if (mx > st_m) {
                         st_s *= exp2f((st_m - mx) * 1.4426950408889634f);  // 0 while st_m = -inf
                         st_m = mx;
                     }
                     if (st_m > -INFINITY) {
                         const float ms = st_m * 1.4426950408889634f;
-                        float acc_s = 0.0f;
+                        const ptx::f2 l2e = ptx::make_f2(1.4426950408889634f, 1.4426950408889634f);
+                        const ptx::f2 nms = ptx::make_f2(-ms, -ms);
+                        ptx::f2 acc_s[2] = {ptx::make_f2(0.0f, 0.0f), ptx::make_f2(0.0f, 0.0f)};
 #pragma unroll
-                        for (int k = 0; k < 32; ++k)
-                            acc_s += ptx::ex2_approx(fmaf(sv[k], 1.4426950408889634f, -ms));
-                        st_s += acc_s;
+                        for (int k = 0; k < 16; ++k) {
+                            float a0, a1;
+                            ptx::split_f2(ptx::fma2(ptx::make_f2_bits(sw2[k] << 16, sw2[k] & 0xffff0000u), l2e, nms), a0, a1);
+                            acc_s[k & 1] = ptx::add2(acc_s[k & 1], ptx::make_f2(ptx::ex2_approx(a0), ptx::ex2_approx(a1)));
+                        }
+                        float s0, s1;
+                        ptx::split_f2(ptx::add2(acc_s[0], acc_s[1]), s0, s1);
+                        st_s += s0 + s1;
                     }
                 }
                 if (sub == 1) {
