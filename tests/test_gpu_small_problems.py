@@ -105,3 +105,22 @@ def test_small_adapter_layer(BT, C, OC, r):
     for g, n in ((out, "out"), (t, "t"), (u, "u"), (dinp, "dinp"), (dA, "dA"), (dB, "dB")):
         g.check(n)
     nb.nb_check_status()
+
+
+@pytest.mark.parametrize("BT,Vp,V", [
+    (1, 8, 1), (700001, 8, 5),           # a vector per row; more vectors than one pass of the grid takes
+    (40000, 136, 129), (7, 50304, 50257),
+    (3, 2 * 148 * 2048 * 8 + 24, 2 * 148 * 2048 * 8 + 1),  # rows longer than a pass
+])
+def test_dlogits_row_and_column_carried_along(BT, Vp, V):
+    logits = gen(1, (BT, Vp), 2.0)
+    targets = ((torch.arange(BT, device="cuda", dtype=torch.int64) * 7919 + V - 1) % V).to(torch.int32)
+    lse = torch.logsumexp(logits[:, :V].double(), 1).float()
+    _, _, ref = oracle.cross_entropy(f32(logits), targets.cpu().numpy(), V, 0.5)
+    out = Guarded((BT, Vp), torch.bfloat16)
+    nb.nb_ce_backward(out.t, logits, lse, targets, 0.5, BT, Vp, V)
+    check_bf16(out.t, ref, "dlogits")
+    out.check("dlogits")
+    assert torch.all(out.t[:, V:] == 0)
+    nb.nb_ce_backward(logits, logits, lse, targets, 0.5, BT, Vp, V)
+    assert torch.equal(logits, out.t)
