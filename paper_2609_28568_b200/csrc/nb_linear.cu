@@ -623,10 +623,12 @@ double small_cta_us(int bn, double kblocks, int rows, int ctas, bool two)
     const double mma = bn > 128 ? 0.00105 * bn : 0.152;  // 2 bn cycles per k-block take over from the issue
     return 1.45 + 0.5 * part + kblocks * ((two ? (bn == 128 ? 0.30 : 0.18) : mma) + 1e-5 * ctas * stage_kb);
 }
-// adding up the parts of a cluster that shares K
-double small_exchange_us(int bn, int rows)
+// Adding up the parts of a cluster that shares K; the network between the SMs slows down where more
+// than half of them use it (768 columns from 3072, 128-wide tiles over two: 72 CTAs 10.5 us, 96 11.7).
+double small_exchange_us(int bn, int rows, int ctas)
 {
-    return 1.0 + 1.4 * (rows < kBlockM ? rows : kBlockM) / 128.0 * bn / 64.0;
+    const double part = (rows < kBlockM ? rows : kBlockM) / 128.0 * bn / 64.0;
+    return 0.6 + part * (1.2 + (ctas > 74 ? 0.015 * (ctas - 74) : 0.0));
 }
 // gemm_kernel: waves of 128 (256) x 256 tiles, 512 tensor-core cycles per k-block
 double persistent_us(int sms, int M, int N, int kblocks)
@@ -654,7 +656,7 @@ SmallPlan plan_single(int sms, int M, int N, int kblocks, bool allow32, int spli
             // a cluster lies within one GPC: not every SM finds a place in clusters of 4 or 8
             if (tiles * cl > sms * (cl >= 8 ? 0.86 : cl >= 4 ? 0.95 : 1.0) || bn / cl < 8 || (cl > 1 && 2 * cl > kblocks)) break;
             const double us = kLaunchUs + small_cta_us(bn, (kblocks + cl - 1) / cl, M, static_cast<int>(tiles * cl), false) +
-                              (cl > 1 ? small_exchange_us(bn, M) : 0.0);
+                              (cl > 1 ? small_exchange_us(bn, M, static_cast<int>(tiles * cl)) : 0.0);
             if (us < best.us) best = SmallPlan{bn, cl, false, us};
         }
     }
@@ -679,7 +681,7 @@ SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int N
                 if (cl > 1 && n > slots * (cl >= 8 ? 0.86 : 1.2)) continue;
                 const int crowd = static_cast<int>(n < slots ? n : slots);
                 const double td = nd ? small_cta_us(bn, (kblocks + cl - 1) / cl, M, crowd, two != 0) +
-                                           (cl > 1 ? small_exchange_us(bn, M) : 0.0) : 0.0;
+                                           (cl > 1 ? small_exchange_us(bn, M, static_cast<int>(nd * cl)) : 0.0) : 0.0;
                 // the bias gradient's warps own a stage each: the fewer stages, the longer they hold them
                 const double tw = small_cta_us(bn, kw, Mw, crowd, two != 0) + (dbias ? kw * (two ? 0.18 : bn == 128 ? 0.115 : 0.05) : 0.0);
                 double us = td > tw ? td : tw;
