@@ -600,6 +600,8 @@ int launch_rows_auto(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
     const int span = EPI == kEpiSwiglu ? a.swiglu_h : a.N;
     const bool many = span > 3 * s.num_sms * kRowsFeatures;
     if (a.M <= 8) return many ? launch_rows<1, EPI, true>(s, a, stream) : launch_rows<1, EPI, false>(s, a, stream);
+    if constexpr (EPI != kEpiSwiglu)  // gate and up rows: too few registers (1024 -> 16384 12.6 us, with two CTAs 8.6)
+        if (many) return launch_rows<2, EPI, true>(s, a, stream);
     return launch_rows<2, EPI, false>(s, a, stream);
 }
 
@@ -1159,7 +1161,7 @@ int run_layer_bwd(DeviceState &s, const void *dz, const void *weight, const void
 }
 
 // A forward product with its activation: on a few rows the row kernel (9 to 16 rows only up to 8 CTAs
-// per SM: 16 rows, 768 -> 50304 takes 21 us there and 17 us in gemm_kernel), then the smaller of the
+// per SM: 16 rows, 768 -> 50304 takes 19.5 us there and 17.3 us in gemm_kernel), then the smaller of the
 // tile and the persistent kernel's estimates.
 int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
 {

@@ -50,15 +50,19 @@ __device__ __forceinline__ uint4 ld_stream(const __nv_bfloat16 *p)
     return v;
 }
 
-// NT: groups of eight rows. MANY: there are several CTAs of work per SM (the head's 50304 features):
-// fewer pieces of K in flight per thread and four CTAs on an SM (8 rows, 768 -> 50304: 14.4 us
-// against 22.7 us with two; five or six have too few registers, 15.7 and 17.1 us).
+// NT: groups of eight rows. At least two CTAs have to fit an SM (128 registers a thread), or the next
+// launch of the chain cannot start while this one runs: 16 rows, or gate and up rows, with one CTA (138
+// and 168 registers, more pieces of K in flight) took 6.0 us against 3.6 (16 rows, 3072 -> 768), 4.2
+// against 2.9 (768 -> 3072), 10.3 against 4.2 (8 rows, SwiGLU, 4096 -> 1024). MANY: there are several
+// CTAs of work per SM: fewer pieces of K in flight per thread and four CTAs on an SM (8 rows,
+// 768 -> 50304: 14.4 us against 22.7 us with two, five or six have too few registers, 15.7 and 17.1 us;
+// 16 rows, 1024 -> 8192: 4.7 us against 5.8 us with two and 6.1 us with three).
 template <int NT, int EPI, bool MANY>
-__global__ void __launch_bounds__(kRowsThreads, MANY ? 4 : 1)
+__global__ void __launch_bounds__(kRowsThreads, MANY ? 4 : 2)
 rows_kernel(const RowsParams p)
 {
     constexpr int SETS = EPI == kEpiSwiglu ? 2 : 1;  // gate and up rows
-    constexpr int U = MANY ? 3 : SETS == 2 ? 3 : 6;  // pieces of K in flight
+    constexpr int U = MANY ? (NT == 2 ? 2 : 3) : (SETS == 2 || NT == 2) ? 3 : 6;  // pieces of K in flight
     constexpr int LD = 18;  // floats from one row's sixteen partial sums to the next
     __shared__ float part[SETS][kRowsWarps][NT * 8][LD];
     const int warp = static_cast<int>(threadIdx.x >> 5), lane = static_cast<int>(threadIdx.x & 31);
