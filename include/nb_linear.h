@@ -206,10 +206,11 @@ int nb_ce_backward(void *dlogits, const void *logits, const void *lse, const voi
  *     dlora_a (+)= u^T . inp                                    [r, C]    fp32
  * dinp, dlora_a, dlora_b may be NULL (skipped); accumulate as in nb_linear_backward. t and u are
  * rounded to bf16 once each (they are tensor-core operands); everything else follows the
- * conventions at the top of this file. When dlora_b is asked for, u and dlora_b come out of one
- * kernel that reads dout once (both products are bound by that read); when dlora_a is asked for
- * as well, the same launch also reads inp once and forms dlora_a. Both gradients are summed by
- * reduce-adds of per-row-panel partial sums, in no fixed order.
+ * conventions at the top of this file. On large batches, when dlora_b is asked for, u and dlora_b
+ * come out of one kernel that reads dout once (both products are bound by that read); when dlora_a
+ * is asked for as well, the same launch also reads inp once and forms dlora_a; both gradients are
+ * then summed by reduce-adds of per-row-panel partial sums, in no fixed order. On short batches u
+ * and dlora_b are one launch and dinp and dlora_a another, summed in a fixed order.
  *
  * Projections that share an input and are laid out as one layer (a qkv or a gate_up projection:
  * weights stacked by rows) can use these two calls as they are, with r = the sum of the members'
@@ -325,7 +326,7 @@ int nb_check_status(void);
 
 /*
  * Number of kernels this library has launched from the calling process since it was
- * loaded (what clears gradient buffers, a memset or a kernel, is not counted).
+ * loaded (what clears gradient buffers is not counted).
  */
 int64_t nb_kernel_launches(void);
 
