@@ -74,6 +74,15 @@ __device__ __forceinline__ void cluster_sync()
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
                  ::: "memory");
 }
+// the two halves of cluster_sync (every thread of the cluster arrives once, then waits)
+__device__ __forceinline__ void cluster_arrive()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 // arrive on an mbarrier that may live in another CTA of the cluster (shared::cluster address)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 {
@@ -320,14 +329,10 @@ __device__ __forceinline__ void tmem_ld_32x32_x2_wait(uint32_t taddr0, uint32_t 
 }
 
 // ------------------------------------------------------------------ shared memory access
-// 16 bytes into the shared memory of a CTA of the cluster (a shared::cluster address), counted on an
-// mbarrier of that CTA.
-__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d,
-                                            uint32_t bar)
+// 16 bytes into the shared memory of a CTA of the cluster (a shared::cluster address)
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-                 ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar)
-                 : "memory");
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 // two floats from the shared memory of a CTA of the cluster
 __device__ __forceinline__ void ld_cluster_f32x2(uint32_t addr, float2 &v)

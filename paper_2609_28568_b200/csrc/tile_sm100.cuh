@@ -6,9 +6,9 @@
 // the epilogue of a 256-wide tile is exposed at the end. What bounds such a problem is latency, so
 // here a CTA takes a 128 x BN tile (BN = 32 / 64 / 128, or 192 without a split), and where there are far fewer tiles than SMs
 // the CTAs of a cluster share a tile's K range: each accumulates its part in TMEM and sends every
-// other CTA that one's slice of the columns through distributed shared memory (st.async, counted in
-// bytes on the receiver's mbarrier); the receiver adds the parts in rank order (a fixed order:
-// results do not vary) and runs the epilogue on its slice.
+// other CTA that one's slice of the columns through distributed shared memory, and after a barrier
+// of the cluster adds the parts it got in rank order (a fixed order: results do not vary) and runs the
+// epilogue on its slice.
 //
 //   warp 0      TMA producer
 //   warp 1      MMA issuer, TMEM allocation
@@ -81,9 +81,9 @@ struct TileGeom {
 
 // offsets inside the barrier block
 //   8 s          full[s]          8 (16 + s)  empty[s]
-//   8 * 32       accumulator complete          8 * 33  slices received
+//   8 * 32       accumulator complete
 //   8 * 34       TMEM base address (4 bytes), abort flag (4 bytes)
-constexpr uint32_t kTileBarAcc = 8 * 32, kTileBarRecv = 8 * 33, kTileTmemSlot = 8 * 34, kTileAbort = 8 * 34 + 4;
+constexpr uint32_t kTileBarAcc = 8 * 32, kTileTmemSlot = 8 * 34, kTileAbort = 8 * 34 + 4;
 
 // Sixteen columns of this thread's row.
 __device__ __forceinline__ void tile_ld16(uint32_t taddr, float (&v)[16])
@@ -174,7 +174,7 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
     const uint32_t bar0 = line + G::LINE_BYTES;
     auto full_bar = [&](int s) { return bar0 + 8u * static_cast<uint32_t>(s); };
     auto empty_bar = [&](int s) { return bar0 + 8u * static_cast<uint32_t>(kTileMaxStages + s); };
-    const uint32_t acc_bar = bar0 + kTileBarAcc, recv_bar = bar0 + kTileBarRecv;
+    const uint32_t acc_bar = bar0 + kTileBarAcc;
     const uint32_t abort_addr = bar0 + kTileAbort;
 
     const int m_blk = tile % j.tiles_m, n_blk = tile / j.tiles_m;
@@ -199,9 +199,6 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
         }
         if (lane == 31) {
             ptx::mbar_init(acc_bar, 1);
-            ptx::mbar_init(recv_bar, 1);
-            // every other rank sends this CTA its part of rows x (BN / cluster) columns
-            if (cluster > 1) ptx::mbar_expect_tx(recv_bar, static_cast<uint32_t>(rows) * (BN - BN / cluster) * 4u);
             ptx::st_shared_u32_volatile(abort_addr, 0);
         }
         ptx::fence_barrier_init();
@@ -547,8 +544,10 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
                 // group is 129 rows long, so that neighbouring groups of a row lie in other banks. The
                 // network between the SMs is the slow part, so the CTA's own slice stays off it: 128
                 // columns over two CTAs 8.4 -> 6.9 us (128 rows, 768 -> 768), 13.5 -> 11.7 us (1024
-                // rows, 3072 -> 768), 32 columns over two 5.2 -> 4.5 us. (Bulk copies from shared
-                // memory to shared memory in place of st.async: 0.6 us slower.)
+                // rows, 3072 -> 768), 32 columns over two 5.2 -> 4.5 us. Plain stores and one barrier of the
+                // cluster; st.async with the bytes counted on the receiver's mbarrier took 0.1 to 0.5 us
+                // longer (64 rows, 768 -> 768: 3.80 -> 3.65 us; 519 rows, 3072 -> 1024: 12.0 -> 11.4), bulk
+                // copies from shared memory to shared memory another 0.6 us.
                 const int sl = BN / cluster;
                 auto slice_pos = [&](int sender, int r, int c) {
                     return static_cast<uint32_t>(((sender * (sl / 4) + c / 4) * (kBlockM + 1) + r) * 16);
@@ -571,10 +570,12 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
                                 const uint32_t x0 = __float_as_uint(v[i * 4]), x1 = __float_as_uint(v[i * 4 + 1]),
                                                x2 = __float_as_uint(v[i * 4 + 2]), x3 = __float_as_uint(v[i * 4 + 3]);
                                 if (d == rank) ptx::st_shared_v4(at, x0, x1, x2, x3);
-                                else ptx::st_async_v4(ptx::mapa(at, d), x0, x1, x2, x3, ptx::mapa(recv_bar, d));
+                                else ptx::st_cluster_v4(ptx::mapa(at, d), x0, x1, x2, x3);
                             }
                     }
                 }
+                __syncwarp();
+                ptx::cluster_arrive();
                 // eight columns of one row per item, neighbouring items along the row
                 const int pieces = sl / 8;
                 const int items = rows * pieces;
@@ -585,11 +586,8 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
                     if (col < j.N)
                         e0 = __ldg(reinterpret_cast<const uint4 *>(j.E + static_cast<long long>(m0 + et / pieces) * j.e_ld + col));
                 }
-                bool got = true;
-                if (lane == 0) got = wait_barrier(wctx_epi, recv_bar, 0, 450);
-                got = __shfl_sync(0xffffffffu, got ? 1 : 0, 0) != 0;
-                ptx::named_bar_sync(1, kEpiThreads);  // and this CTA's own part
-                for (int it = et; got && it < items; it += kEpiThreads) {
+                ptx::cluster_wait();  // every part has arrived
+                for (int it = et; ok && it < items; it += kEpiThreads) {
                     const int rw = it / pieces, piece = it % pieces;
                     const int cl = cbase + piece * 8;
                     const int col = n0 + cl;
@@ -620,16 +618,16 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
 
     // ---------------------------------------------------------------- common exit
     __syncwarp();
+    constexpr bool SPLIT = EPI != kEpiF32 && EPI != kEpiSwiglu && BN <= 128;
+    if (SPLIT && cluster > 1 && (warp < 2 || !smem_ok)) ptx::cluster_sync();  // the epilogue's warps have passed it
     ptx::tc_fence_before();
     __syncthreads();
     if (ptx::ld_shared_u32_volatile(abort_addr) != 0) {
-        // A wait expired somewhere: give copies and MMAs still in flight time to land. In a cluster
-        // a peer may still send to this CTA's memory, so it stays until every peer has left or
-        // stands here too (a CTA that leaves normally has received all its parts: nobody sends to it).
+        // A wait expired somewhere: give copies and MMAs still in flight time to land. (A peer sends nothing
+        // after the cluster's barrier.)
         const uint64_t t0 = ptx::globaltimer_ns();
         while (ptx::globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
         __syncwarp();
-        if (cluster > 1) ptx::cluster_sync();
     }
     if (warp == 1) {
         ptx::tc_fence_after();
