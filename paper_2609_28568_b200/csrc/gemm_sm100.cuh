@@ -90,6 +90,10 @@ struct GemmCfg {
     static constexpr uint32_t A_BYTES = kBlockM * kBlockK * 2;
     static constexpr int B_ROWS = BLOCK_N / CG_;  // rows of B's N extent held by one CTA
     static constexpr uint32_t B_BYTES = B_ROWS * kBlockK * 2;
+    // rows per box of a K-major operand; 96 rows of B are one box, and A's 128 then are too (issuing three
+    // boxes would take the producer longer than the 384 cycles of a 192-wide k-block)
+    static constexpr int A_BOX_ROWS = B_ROWS % 64 ? kBlockM : 64;
+    static constexpr int B_BOX_ROWS = B_ROWS % 64 ? B_ROWS : 64;
     static constexpr uint32_t OFF_A = 0;
     static constexpr uint32_t OFF_B = STAGES * A_BYTES;
     static constexpr uint32_t OFF_STG = STAGES * (A_BYTES + B_BYTES);
@@ -101,7 +105,7 @@ struct GemmCfg {
     // Warp-private epilogue (bf16 results of full-width tiles): every epilogue warp stages and
     // stores its own 32-row boxes, no barrier joins the warps. The bias then lives in two buffers
     // (by tile parity) and each warp has its own pair of pre-activation barriers.
-    static constexpr bool WARP_EPI = BLOCK_N_ == 256 &&
+    static constexpr bool WARP_EPI = BLOCK_N_ >= 192 &&
                                      (EPI_ == kEpiStore || EPI_ == kEpiStoreStats || EPI_ == kEpiGelu ||
                                       EPI_ == kEpiMulGeluGrad || EPI_ == kEpiF32);
     // boxes of staging per epilogue warp: one per stored plane; fp32 results alternate between two
@@ -121,7 +125,8 @@ struct GemmCfg {
     static constexpr int STEPS = (EPI == kEpiF32) ? BLOCK_N / 32
                                  : (EPI == kEpiSwiglu) ? BLOCK_N / 128 : BLOCK_N / 64;
     static_assert(CG_ == 1 || CG_ == 2, "CTAs per tile");
-    static_assert(BLOCK_N % (64 * CG_) == 0 && BLOCK_N >= 64 && BLOCK_N <= 256, "BLOCK_N");
+    static_assert((BLOCK_N % (64 * CG_) == 0 && BLOCK_N >= 64 && BLOCK_N <= 256) ||
+                      (BLOCK_N == 192 && CG_ == 2 && !A_MN_ && !B_MN_ && (EPI_ == kEpiStore || EPI_ == kEpiGelu)), "BLOCK_N");
     static_assert(2 * BLOCK_N <= 512, "two accumulators must fit in TMEM");
     static_assert(NSTG % BUFS_PER_STEP == 0 && SLOTS >= 1, "staging ring");
     static_assert(EPI != kEpiMulGeluGrad || SLOTS >= 2, "staging ring");
@@ -397,8 +402,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                             load(sa + j * 8192u, mapA, fb, m0 + j * 64, k0);
                     } else {          // tensor [M rows, K cols]: boxes of 64(k) x 64(m)
 #pragma unroll
-                        for (int j = 0; j < kBlockM / 64; ++j)
-                            load(sa + j * 8192u, mapA, fb, k0, m0 + j * 64);
+                        for (int j = 0; j < kBlockM / Cfg::A_BOX_ROWS; ++j)
+                            load(sa + j * 8192u, mapA, fb, k0, m0 + j * Cfg::A_BOX_ROWS);
                     }
                     // this CTA's share of B's N extent: all of it, or its half of the pair's tile
                     if (Cfg::B_MN) {
@@ -419,8 +424,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     } else {                          // boxes of 64(k) x 64(n)
                         const int n0 = n_blk * BLOCK_N + static_cast<int>(rank) * Cfg::B_ROWS;
 #pragma unroll
-                        for (int j = 0; j < Cfg::B_ROWS / 64; ++j)
-                            load(sb + j * 8192u, mapB, fb, k0, n0 + j * 64);
+                        for (int j = 0; j < Cfg::B_ROWS / Cfg::B_BOX_ROWS; ++j)
+                            load(sb + j * 8192u, mapB, fb, k0, n0 + j * Cfg::B_BOX_ROWS);
                     }
                     if (++stage == STAGES) {
                         stage = 0;
@@ -613,6 +618,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             decode_unit(p, u, m_blk, n_blk, split);
             const int m0 = m_blk * Cfg::TILE_M + static_cast<int>(rank) * kBlockM;
             const int nw = n_blk * BLOCK_N + hf * 128;  // this warp's first column
+            // 32-column pieces of this warp: a 192-wide tile's second half has two
+            const int s4_end = BLOCK_N == 256 || hf == 0 ? 4 : (BLOCK_N - 128) / 32;
             // this lane's four of the warp's 128 bias values, fetched while the tile is still in the
             // tensor core
             uint32_t bv[4] = {0u, 0u, 0u, 0u};
@@ -636,7 +643,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const uint32_t bias_t = smem + Cfg::OFF_BIAS + (tile_i & 1u) * (BLOCK_N * 4u) +
                                     static_cast<uint32_t>(hf) * 512u;
             if (has_bias) {
-                ptx::st_shared_v4(bias_t + static_cast<uint32_t>(lane) * 16u, bv[0], bv[1], bv[2], bv[3]);
+                if (lane < s4_end * 8) ptx::st_shared_v4(bias_t + static_cast<uint32_t>(lane) * 16u, bv[0], bv[1], bv[2], bv[3]);
                 __syncwarp();
             }
             const uint32_t t_acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
@@ -652,6 +659,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             float st_m = -INFINITY, st_s = 0.0f;  // kEpiStoreStats: this thread's row statistics
 #pragma unroll
             for (int s4 = 0; s4 < 4; ++s4) {  // 32 columns at a time; two make a stored box
+                if (s4 >= s4_end) break;
                 const int step = s4 >> 1, sub = s4 & 1;
                 const uint32_t g = tile_i * 2u + static_cast<uint32_t>(step);
                 // the bias of 16 columns at a time, ahead of the arithmetic that uses it (the loads
@@ -745,7 +753,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     } else {
                         if (j == 2) {
                             load_bias16(1);
-                            if (s4 == 3) release_acc(acc);  // kBiasEpi: the tile's last bias loads are out
+                            if (s4 == s4_end - 1) release_acc(acc);  // kBiasEpi: the tile's last bias loads are out
                         }
                         const float4 b0 = bb[2 * (j & 1)], b1 = bb[2 * (j & 1) + 1];
                         ptx::f2 z[4];  // eight columns as four packed pairs

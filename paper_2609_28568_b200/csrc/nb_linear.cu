@@ -255,9 +255,9 @@ int launch_gemm(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
     }
     CUtensorMap tA, tB, tD, tE;
     int rc;
-    // operands are fetched as 64 x 64 boxes; results (and the aux tile) move as 128-row chunks
-    if ((rc = get_tmap(s, &tA, a.A, a.a_rows, a.a_cols, 0, 64, a.a_ld)) != NB_OK) return rc;
-    if ((rc = get_tmap(s, &tB, a.B, a.b_rows, a.b_cols, 0, 64, a.b_ld)) != NB_OK) return rc;
+    // operands are fetched as 64 x 64 boxes (192-wide tiles: 128 and 96 rows of 64); results (and the aux tile) move as 128-row chunks
+    if ((rc = get_tmap(s, &tA, a.A, a.a_rows, a.a_cols, 0, Cfg::A_BOX_ROWS, a.a_ld)) != NB_OK) return rc;
+    if ((rc = get_tmap(s, &tB, a.B, a.b_rows, a.b_cols, 0, Cfg::B_BOX_ROWS, a.b_ld)) != NB_OK) return rc;
     if ((rc = get_tmap(s, &tD, a.D, a.d_rows, a.d_cols, a.d_dtype, Cfg::OUT_BOX_ROWS, a.d_ld)) != NB_OK) return rc;
     if (a.E) {
         if ((rc = get_tmap(s, &tE, a.E, a.e_rows, a.e_cols, 0, Cfg::OUT_BOX_ROWS)) != NB_OK) return rc;
@@ -266,8 +266,8 @@ int launch_gemm(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
     }
     CUtensorMap tA2 = tA, tB2 = tB;
     if (a.A2 && a.B2 && a.k2 > 0) {
-        if ((rc = get_tmap(s, &tA2, a.A2, a.a2_rows, a.a2_cols, 0, 64, a.a2_ld)) != NB_OK) return rc;
-        if ((rc = get_tmap(s, &tB2, a.B2, a.b2_rows, a.b2_cols, 0, 64)) != NB_OK) return rc;
+        if ((rc = get_tmap(s, &tA2, a.A2, a.a2_rows, a.a2_cols, 0, Cfg::A_BOX_ROWS, a.a2_ld)) != NB_OK) return rc;
+        if ((rc = get_tmap(s, &tB2, a.B2, a.b2_rows, a.b2_cols, 0, Cfg::B_BOX_ROWS)) != NB_OK) return rc;
     }
     GemmParams p;
     memset(&p, 0, sizeof(p));
@@ -342,6 +342,9 @@ using FwdStore2 = GemmCfg<2, 256, 6, 2, false, false, kEpiStore>;
 using FwdStoreStats1 = GemmCfg<1, 256, 4, 2, false, false, kEpiStoreStats>;
 using FwdStoreStats2 = GemmCfg<2, 256, 6, 2, false, false, kEpiStoreStats>;
 using FwdGelu2 = GemmCfg<2, 256, 5, 4, false, false, kEpiGelu>;
+// 192-wide pair tiles, where these make fewer or shorter waves (narrower_tiles)
+using FwdStore2N = GemmCfg<2, 192, 6, 2, false, false, kEpiStore>;
+using FwdGelu2N = GemmCfg<2, 192, 5, 4, false, false, kEpiGelu>;
 using FwdSwiglu2 = GemmCfg<2, 256, 5, 3, false, false, kEpiSwiglu>;
 using DgradStore2 = GemmCfg<2, 256, 6, 2, false, true, kEpiStore>;
 using DgradMulGelu2 = GemmCfg<2, 256, 4, 2, false, true, kEpiMulGeluGrad>;
@@ -1160,6 +1163,22 @@ int run_layer_bwd(DeviceState &s, const void *dz, const void *weight, const void
     return launch_layer_bwd<LayerBwdPlain>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, stream);
 }
 
+// Whether a forward product in CTA pairs runs in 192-column tiles: where it takes several waves of the pairs
+// and as many with these as with 256-column ones, each wave is shorter (2021 rows, 768 -> 3072 with GELU,
+// two waves: 17.4 -> 15.0 us; 8192 rows, 3072 -> 768: 35.3 -> 32.0 us; 4600 rows, 768 -> 2304, three
+// waves: 18.0 -> 16.1 us). One more wave costs more than that (4096 rows, 768 -> 2304: 14.9 -> 15.7 us),
+// and in a single wave the SMs' ports to L2 take back what the tensor cores save (4096 rows, 3072 -> 768:
+// 18.6 us either way; 73 operand bytes per clock and SM against 64).
+bool narrower_tiles(int sms, int M, int N)
+{
+    if (!use_pairs(M)) return false;
+    auto waves = [&](int bn) {
+        const long long tiles = 1ll * ((M + 2 * kBlockM - 1) / (2 * kBlockM)) * ((N + bn - 1) / bn);
+        return (tiles + sms / 2 - 1) / (sms / 2);
+    };
+    return waves(256) > 1 && waves(192) == waves(256);
+}
+
 // A forward product with its activation: on a few rows the row kernel (9 to 16 rows only up to 8 CTAs
 // per SM: 16 rows, 768 -> 50304 takes 19.5 us there and 17.3 us in gemm_kernel), then the smaller of the
 // tile and the persistent kernel's estimates.
@@ -1180,6 +1199,8 @@ int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
         return launch_gemm_auto<FwdSwiglu1, FwdSwiglu2>(s, a, stream);
     }
     const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, true, 0, 0, other);
+    if (!pl.bn && narrower_tiles(s.num_sms, a.M, a.N))
+        return act == NB_ACT_GELU ? launch_gemm<FwdGelu2N>(s, a, stream) : launch_gemm<FwdStore2N>(s, a, stream);
     if (act == NB_ACT_GELU)
         return pl.bn ? launch_tile_plan<false, kEpiGelu>(s, a, pl, stream) : launch_gemm_auto<FwdGelu1, FwdGelu2>(s, a, stream);
     return pl.bn ? launch_tile_plan<false, kEpiStore>(s, a, pl, stream) : launch_gemm_auto<FwdStore1, FwdStore2>(s, a, stream);

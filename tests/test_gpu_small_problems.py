@@ -124,3 +124,28 @@ def test_dlogits_row_and_column_carried_along(BT, Vp, V):
     assert torch.all(out.t[:, V:] == 0)
     nb.nb_ce_backward(logits, logits, lse, targets, 0.5, BT, Vp, V)
     assert torch.equal(logits, out.t)
+
+
+@pytest.mark.parametrize("act", [nb.ACT_NONE, nb.ACT_GELU])
+@pytest.mark.parametrize("BT,C,OC,r", [(1990, 136, 3080, 8), (1800, 72, 3264, 64), (4500, 200, 2120, 16)])
+def test_forward_in_192_column_pair_tiles(act, BT, C, OC, r):
+    """Several waves of the CTA pairs, as many as with 256 columns: one column past a tile, a full last
+    tile, a ragged one; with an adapter term, whose k-blocks go through the same boxes."""
+    inp, w, bias = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (OC,), 0.1)
+    ref, pre_ref = oracle.linear_forward(f32(inp), f32(w), f32(bias), act=act)
+    out, pre = Guarded((BT, OC), torch.bfloat16), Guarded((BT, OC), torch.bfloat16)
+    nb.nb_linear_forward_ex(out.t, pre.t if act else None, inp, w, bias, BT, C, OC, act)
+    check_bf16(out.t, ref, "out")
+    out.check("out")
+    if act:
+        check_bf16(pre.t, pre_ref, "pre")
+        pre.check("pre")
+        return
+    a, b, scale = gen(4, (r, C), 0.02), gen(5, (OC, r), 0.02), 4.0
+    t = Guarded((BT, r), torch.bfloat16)
+    nb.nb_lora_linear_forward(out.t, t.t, inp, w, bias, a, b, scale, BT, C, OC, r)
+    t_ref = scale * oracle.linear_forward(f32(inp), f32(a))[0]
+    check_bf16(out.t, oracle.lora_forward(f32(inp), f32(w), f32(bias), f32(a), f32(b), scale), "out with adapter",
+               extra=2.0 ** -9 * (np.abs(t_ref) @ np.abs(f32(b).T.astype(np.float64))))
+    out.check("out with adapter")
+    nb.nb_check_status()
