@@ -683,7 +683,8 @@ SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int N
             for (int two = 0; two <= 1; ++two) {
                 const double slots = sms * (two ? 2.0 : 1.0);
                 const double n = static_cast<double>(nd * cl + nw);
-                if (cl > 1 && n > slots * (cl >= 8 ? 0.86 : 1.2)) continue;
+                // job 0's clusters come first and have to find their places; job 1's tiles fill up behind them
+                if (cl >= 8 ? n > 0.86 * slots : cl > 1 && nd * cl > 0.95 * slots) continue;
                 const int crowd = static_cast<int>(n < slots ? n : slots);
                 const double td = nd ? small_cta_us(bn, (kblocks + cl - 1) / cl, M, crowd, two != 0) +
                                            (cl > 1 ? small_exchange_us(bn, M, static_cast<int>(nd * cl)) : 0.0) : 0.0;
@@ -691,10 +692,13 @@ SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int N
                 const double tw = small_cta_us(bn, kw, Mw, crowd, two != 0) + (dbias ? kw * (two ? 0.18 : bn == 128 ? 0.115 : 0.05) : 0.0);
                 double us = td > tw ? td : tw;
                 if (n > slots) {
-                    const double line = (nd * cl * td + nw * tw) / slots + 0.6 * tw;
+                    const double line = (nd * cl * td + nw * tw) / slots + tw;
                     if (line > us) us = line;
                 }
-                if (two && bn == 128) us *= 1.2;  // three stages each: short rings that wait for each other
+                // three stages each: from eight k-blocks of dweight on, short rings that wait for each other (1003
+                // rows, 776 -> 1416: 18 us against 12.6); up to four, one CTA's stores run under the other's
+                // loads (130 rows, 4096 -> 1024: 9.5 us against 12.8; 256 rows, 4096 x 4096: 36.8 against 42.8)
+                if (two && bn == 128 && kw > 4) us *= 1.0 + 0.1 * (kw < 8 ? kw - 4 : 4);
                 us += kLaunchUs;
                 if (us < best.us) best = SmallPlan{bn, cl, two != 0, us};
             }
@@ -705,12 +709,20 @@ SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int N
 
 // The split of K for dinp. It fixes the order of the sums, so it depends on the problem alone and not
 // on which other gradients are asked for in the same call; above 256 rows, where the weight gradient's
-// tiles join dinp's in the persistent kernel, there is none.
+// tiles join dinp's in the persistent kernel, there is none. At most four CTAs share K: eight find no place
+// in a GPC among the weight gradient's tiles (128 rows, 768 -> 3072, both products: 9.3 us with eight, 7.4
+// with four; 64 rows, 768 -> 2304: 7.7 and 5.9; dinp alone 6.3 and 6.6). Where those tiles fill the chip
+// twice over, the clusters take no more than 32 places (256 rows, 4096 x 4096: 53 us with two CTAs
+// sharing K, 37 without; 200 rows, 1024 -> 6144: 20.9 with four, 18.7 with two, 21.4 without).
 int dinp_split(int sms, int M, int N, int kblocks)
 {
     if (M > 2 * kBlockM) return 1;
     const SmallPlan pl = plan_single(sms, M, N, kblocks, false, 0, 0, 1e9);
-    return pl.bn ? pl.cluster : 1;
+    int split = pl.bn ? (pl.cluster < 4 ? pl.cluster : 4) : 1;
+    const int cols = (N + kBlockM - 1) / kBlockM;
+    if ((kblocks + 1) / 2 * cols > 2 * sms)
+        while (split > 1 && (M + kBlockM - 1) / kBlockM * cols * split > 32) split /= 2;
+    return split;
 }
 
 template <bool B_MN, int EPI>
@@ -1213,12 +1225,13 @@ double backward_us(int sms, int M, int BT, int N, int Mw, int kd, int kw, bool a
     const int slots = sms / 2;
     const double d_tiles = static_cast<double>((M + 255) / 256) * ((N + 255) / 256);
     const double w_tiles = static_cast<double>((Mw + 255) / 256) * ((N + 255) / 256);
-    const double clear = accumulate ? 0.0 : 2.8;
+    // the fp32 result is cleared (unless it is added to) and reduce-added into
+    const double clear = (accumulate ? 0.0 : 2.8) + 1e-6 * Mw * N;
     if (M > 0 && BT > kBlockM && !apart) {
         const bool narrow = !gelu && layer_bwd_narrow(static_cast<int>(d_tiles), kd, static_cast<int>(w_tiles), kw, slots);
         const double chain = narrow ? 0.7 * kd : kd;
         const double level = ((narrow ? 2.0 : 1.0) * d_tiles * (chain + 3) + w_tiles * (kw + 3)) / slots;
-        return 5.3 + clear + 0.27 * (chain > level ? chain : level);
+        return 6.0 + clear + 0.27 * (chain > level ? chain : level);
     }
     const double waves = w_tiles / slots;
     const double w_us = 5.0 + (waves < 1.0 ? 1.0 : waves) * (0.27 * (waves < 1.0 ? kw * waves : kw) + 0.8);
