@@ -47,7 +47,7 @@ def test_small_forward(BT, C, OC, act):
 
 @pytest.mark.parametrize("fused", [False, True])
 @pytest.mark.parametrize("BT,C,OC", [
-    (1, 8, 16), (8, 136, 3072), (64, 776, 200), (128, 264, 2056),   # dinp's K split over 2, 4, 8
+    (1, 8, 16), (8, 136, 3072), (64, 776, 200), (128, 264, 2056),   # dinp's K split over 2 and 4
     (129, 72, 136), (256, 520, 1544), (257, 520, 1544),              # the last split, the first without
     (384, 768, 776), (1000, 264, 328),                               # more k-blocks than stages for dweight
     (1030, 2608, 72),                                                # dinp alone in tiles of 192 columns
