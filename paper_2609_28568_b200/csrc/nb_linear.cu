@@ -214,7 +214,7 @@ struct GemmArgs {
     const void *A2; uint64_t a2_rows, a2_cols;
     const void *B2; uint64_t b2_rows, b2_cols;
     int k2;
-    float alpha;   // D = alpha * acc (+ bias); 0 is read as 1
+    float alpha = 1.0f;   // D = alpha * acc (+ bias)
     uint64_t a_ld, b_ld, d_ld, a2_ld;  // row strides in elements of A, B, D, A2 when they are column slices (0: dense)
     float2 *stats; // forward with softmax statistics: [M, stats_ld]
     int stats_ld;
@@ -287,7 +287,7 @@ int launch_gemm(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
     // column tile. Many column tiles (the head): a tall group keeps the weight tiles' reuse in L2;
     // few column tiles: a short group keeps the row tiles' (measured on B200, 1-2 % either way)
     p.kblocks_ext = (a.A2 && a.B2 && a.k2 > 0 && p.splits == 1) ? (a.k2 + kBlockK - 1) / kBlockK : 0;
-    p.alpha = a.alpha == 0.0f ? 1.0f : a.alpha;
+    p.alpha = a.alpha;
     p.group_m = (p.tiles_n >= 64 ? 64 : p.tiles_n <= 4 ? 4 : 16) / Cfg::CG;
     p.swiglu_h = a.swiglu_h;
     p.reduce = a.reduce;
@@ -442,7 +442,7 @@ void fill_tile_job(TileJob &j, uint32_t &smem_bytes, const GemmArgs &a, int epi,
     const uint32_t rows = !a_mn && a.M < kBlockM ? static_cast<uint32_t>((a.M + 7) / 8 * 8) : kBlockM;
     j.a_slot = rows * 128u;
     j.ctas = j.tiles_m * j.tiles_n * cluster;
-    j.alpha = a.alpha == 0.0f ? 1.0f : a.alpha;
+    j.alpha = a.alpha;
     j.bias = static_cast<const __nv_bfloat16 *>(a.bias);
     j.D = static_cast<__nv_bfloat16 *>(a.D);
     j.d_ld = static_cast<long long>(a.d_ld ? a.d_ld : a.d_cols);
@@ -850,8 +850,7 @@ int run_wgrad_f32(DeviceState &s, const void *dz, const void *inp, void *dweight
                   int64_t BT, int64_t M_, int64_t N_, int accumulate, cudaStream_t stream,
                   uint64_t inp_ld = 0)
 {
-    GemmArgs a;
-    memset(&a, 0, sizeof(a));
+    GemmArgs a{};
     a.A = dz; a.a_rows = BT; a.a_cols = M_;
     a.B = inp; a.b_rows = BT; a.b_cols = N_; a.b_ld = inp_ld;
     a.D = dweight; a.d_rows = M_; a.d_cols = N_; a.d_dtype = 1;
@@ -1260,8 +1259,7 @@ double narrow_us(int sms, int tiles, int kblocks)
 int run_lora_down(DeviceState &s, void *t, const void *inp, const void *lora_a, float scale, int64_t BT, int64_t C,
                   int64_t r, cudaStream_t stream, bool *late = nullptr)
 {
-    GemmArgs a;
-    memset(&a, 0, sizeof(a));
+    GemmArgs a{};
     a.A = inp; a.a_rows = BT; a.a_cols = C;
     a.B = lora_a; a.b_rows = r; a.b_cols = C;
     a.D = t; a.d_rows = BT; a.d_cols = r; a.d_dtype = 0;
@@ -1295,20 +1293,19 @@ int run_lora_backward(DeviceState &s, const LoraBwd &l, cudaStream_t stream)
     const int sms = s.num_sms, BT = static_cast<int>(l.BT), C = static_cast<int>(l.C), OC = static_cast<int>(l.OC), r = static_cast<int>(l.r);
     const int kt = kblocks_of(BT), ko = kblocks_of(OC);
     int rc;
-    GemmArgs u, dB, dx, dA;
-    memset(&u, 0, sizeof(u));  // u = scale * dout . B   (B [OC, r] read as an MN-major operand)
+    GemmArgs u{};  // u = scale * dout . B   (B [OC, r] read as an MN-major operand)
     u.A = l.dout; u.a_rows = BT; u.a_cols = OC;
     u.B = l.lora_b; u.b_rows = OC; u.b_cols = r;
     u.D = l.u; u.d_rows = BT; u.d_cols = r; u.d_ld = l.u_ld;
     u.M = BT; u.N = r; u.K = OC;
     u.splits = 1;
     u.alpha = l.scale;
-    memset(&dB, 0, sizeof(dB));  // dB [OC, r] (+)= dout^T . t      (t already carries the scale)
+    GemmArgs dB{};  // dB [OC, r] (+)= dout^T . t      (t already carries the scale)
     dB.A = l.dout; dB.a_rows = BT; dB.a_cols = OC;
     dB.B = l.t; dB.b_rows = BT; dB.b_cols = r; dB.b_ld = l.t_ld;
     dB.D = l.dlora_b; dB.d_rows = OC; dB.d_cols = r; dB.d_dtype = 1;
     dB.M = OC; dB.N = r; dB.K = BT;
-    memset(&dx, 0, sizeof(dx));  // dinp = dout . W + u . A: r extra rows of K
+    GemmArgs dx{};  // dinp = dout . W + u . A: r extra rows of K
     dx.A = l.dout; dx.a_rows = BT; dx.a_cols = OC;
     dx.B = l.weight; dx.b_rows = OC; dx.b_cols = C;
     dx.D = l.dinp; dx.d_rows = BT; dx.d_cols = C;
@@ -1317,7 +1314,7 @@ int run_lora_backward(DeviceState &s, const LoraBwd &l, cudaStream_t stream)
     dx.A2 = l.u; dx.a2_rows = BT; dx.a2_cols = r; dx.a2_ld = l.u_ld;
     dx.B2 = l.lora_a; dx.b2_rows = r; dx.b2_cols = C;
     dx.k2 = r;
-    memset(&dA, 0, sizeof(dA));  // dA [r, C] (+)= u^T . inp        (u already carries the scale)
+    GemmArgs dA{};  // dA [r, C] (+)= u^T . inp        (u already carries the scale)
     dA.A = l.u; dA.a_rows = BT; dA.a_cols = r; dA.a_ld = l.u_ld;
     dA.B = l.inp; dA.b_rows = BT; dA.b_cols = C;
     dA.D = l.dlora_a; dA.d_rows = r; dA.d_cols = C; dA.d_dtype = 1;
@@ -1403,8 +1400,7 @@ int nb_linear_forward_ex(void *out, void *pre_act, const void *inp, const void *
     DeviceState *s;
     if ((rc = get_state(&s)) != NB_OK) return rc;
 
-    GemmArgs a;
-    memset(&a, 0, sizeof(a));
+    GemmArgs a{};
     a.A = inp; a.a_rows = BT; a.a_cols = C;
     a.B = weight; a.b_rows = OC; a.b_cols = C;
     a.D = out; a.d_rows = BT; a.d_cols = (act == NB_ACT_SWIGLU) ? OC / 2 : OC; a.d_dtype = 0;
@@ -1490,8 +1486,8 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
         dz = s->workspace;
     }
 
-    GemmArgs d, w;
-    memset(&d, 0, sizeof(d));  // dinp[BT, C] = dz[BT, OC] . W[OC, C]
+    GemmArgs d{}, w{};
+    // dinp[BT, C] = dz[BT, OC] . W[OC, C]
     d.A = dz; d.a_rows = BT; d.a_cols = OC;
     d.B = weight; d.b_rows = OC; d.b_cols = C;
     d.D = dinp; d.d_rows = BT; d.d_cols = C; d.d_dtype = 0;
@@ -1501,7 +1497,7 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
     const int kd = kblocks_of(OC), kw = kblocks_of(BT);
     const int split = dinp ? dinp_split(s->num_sms, d.M, d.N, kd) : 1;
     if (dweight && dweight_dtype == NB_DTYPE_F32) {
-        memset(&w, 0, sizeof(w));  // dweight[OC, C] (+)= dz^T[OC, BT] . inp[BT, C]
+        // dweight[OC, C] (+)= dz^T[OC, BT] . inp[BT, C]
         w.A = dz; w.a_rows = BT; w.a_cols = OC;
         w.B = inp; w.b_rows = BT; w.b_cols = C;
         w.D = dweight; w.d_rows = OC; w.d_cols = C; w.d_dtype = 1;
@@ -1525,8 +1521,7 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
     if (dinp && (rc = run_dgrad(*s, d, stream)) != NB_OK) return rc;
 
     if (dweight) {  // dweight[OC, C] (+)= dz^T[OC, BT] . inp[BT, C]
-        GemmArgs a;
-        memset(&a, 0, sizeof(a));
+        GemmArgs a{};
         a.A = dz; a.a_rows = BT; a.a_cols = OC;
         a.B = inp; a.b_rows = BT; a.b_cols = C;
         a.D = dweight; a.d_rows = OC; a.d_cols = C;
@@ -1593,8 +1588,7 @@ int nb_lm_head_ce_forward(void *logits, void *loss, void *lse, const void *inp, 
     if ((rc = get_state(&s)) != NB_OK) return rc;
     const int stats_ld = 2 * static_cast<int>((Vp + 255) / 256);
     if ((rc = ensure_workspace(*s, static_cast<size_t>(BT) * stats_ld * sizeof(float2), stream)) != NB_OK) return rc;
-    GemmArgs a;
-    memset(&a, 0, sizeof(a));
+    GemmArgs a{};
     a.A = inp; a.a_rows = BT; a.a_cols = C;
     a.B = weight; a.b_rows = Vp; a.b_cols = C;
     a.D = logits; a.d_rows = BT; a.d_cols = Vp; a.d_dtype = 0;
@@ -1655,8 +1649,7 @@ int nb_lora_linear_forward(void *out, void *t, const void *inp, const void *weig
     if ((rc = get_state(&s)) != NB_OK) return rc;
     bool late = false;
     if ((rc = run_lora_down(*s, t, inp, lora_a, scale, BT, C, r, stream, &late)) != NB_OK) return rc;
-    GemmArgs a;
-    memset(&a, 0, sizeof(a));  // out = inp . W^T (+ bias) + t . B^T: r extra columns of K
+    GemmArgs a{};  // out = inp . W^T (+ bias) + t . B^T: r extra columns of K
     a.A = inp; a.a_rows = BT; a.a_cols = C;
     a.B = weight; a.b_rows = OC; a.b_cols = C;
     a.D = out; a.d_rows = BT; a.d_cols = OC; a.d_dtype = 0;
@@ -1747,8 +1740,7 @@ int nb_lora_linear_forward_stacked(void *out, const void *inp, const void *weigh
     std::lock_guard<std::mutex> lock(g_mu);
     DeviceState *s;
     if ((rc = get_state(&s)) != NB_OK) return rc;
-    GemmArgs a;
-    memset(&a, 0, sizeof(a));  // out = inp . W^T (+ bias) + t_slice . B^T: r extra columns of K
+    GemmArgs a{};  // out = inp . W^T (+ bias) + t_slice . B^T: r extra columns of K
     a.A = inp; a.a_rows = BT; a.a_cols = C;
     a.B = weight; a.b_rows = OC; a.b_cols = C;
     a.D = out; a.d_rows = BT; a.d_cols = OC; a.d_dtype = 0;
@@ -1807,8 +1799,7 @@ int nb_lora_da_stacked(void *da_stack, const void *u_stack, const void *inp, int
         if (!accumulate) NB_CUDA(cudaMemsetAsync(da_stack, 0, static_cast<size_t>(R * C) * 4, stream));
         return NB_OK;
     }
-    GemmArgs w;
-    memset(&w, 0, sizeof(w));  // dA (+)= u^T . inp
+    GemmArgs w{};  // dA (+)= u^T . inp
     w.A = u_stack; w.a_rows = BT; w.a_cols = R;
     w.B = inp; w.b_rows = BT; w.b_cols = C;
     w.D = da_stack; w.d_rows = R; w.d_cols = C; w.d_dtype = 1;
@@ -1937,8 +1928,7 @@ int nb_debug_gemm_timeout(void *out, const void *inp, const void *weight, int64_
     int rc = get_state(&s);
     if (rc != NB_OK) return rc;
     const int64_t BT = 128, C = 256, OC = 256;  // one tile, one CTA, four k-blocks
-    GemmArgs a;
-    memset(&a, 0, sizeof(a));
+    GemmArgs a{};
     a.A = inp; a.a_rows = BT; a.a_cols = C;
     a.B = weight; a.b_rows = OC; a.b_cols = C;
     a.D = out; a.d_rows = BT; a.d_cols = OC; a.d_dtype = 0;

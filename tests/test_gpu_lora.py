@@ -270,6 +270,32 @@ def test_adapter_stack_driver_two_micro_steps(stacked):
                       (3072, 1024)))
 
 
+@pytest.mark.parametrize("with_b", [True, False])
+@pytest.mark.parametrize("BT,C,OC,r", [
+    (8, 72, 136, 8), (100, 264, 1032, 16), (519, 1024, 776, 40),   # products spread over the chip
+    (19000, 64, 72, 16),                                            # a CTA per 128 rows
+])
+def test_adapter_with_scale_zero_is_the_base_layer(BT, C, OC, r, with_b):
+    """scale = 0 is a scale like any other: t and u are zeros, the adapter's gradients too, and out and dinp
+    are what the base layer alone gives. (t and u exactly: 0 times a finite sum.)"""
+    inp, w, _, a, bb, dout = _tensors(BT, C, OC, r, False, seed=950)
+    out, t, u = (torch.full((BT, n), 3.0, dtype=torch.bfloat16, device=DEV) for n in (OC, r, r))
+    dinp = torch.full((BT, C), 3.0, dtype=torch.bfloat16, device=DEV)
+    dA = torch.full((r, C), 3.0, device=DEV)
+    dB = torch.full((OC, r), 3.0, device=DEV) if with_b else None
+    nb.nb_lora_linear_forward(out, t, inp, w, None, a, bb, 0.0, BT, C, OC, r)
+    nb.nb_lora_linear_backward(dinp, dA, dB, u, dout, inp, w, a, bb, t, 0.0, BT, C, OC, r, 0)
+    assert not t.any() and not u.any() and not dA.any()
+    assert dB is None or not dB.any()
+    check_bf16(out, oracle.linear_forward(f32(inp), f32(w))[0], "out")
+    check_bf16(dinp, oracle.linear_backward(f32(dout), None, f32(w), want=("dinp",))["dinp"], "dinp")
+    ts = torch.full((BT, r), 3.0, dtype=torch.bfloat16, device=DEV)
+    nb.nb_lora_down_stacked(ts, inp, a, 0.0, BT, C, r)
+    us = torch.full((BT, r), 3.0, dtype=torch.bfloat16, device=DEV)
+    nb.nb_lora_linear_backward_stacked(None, dB, us, dout, None, a, bb, ts, 0.0, BT, C, OC, r, r, 0, 0)
+    assert not ts.any() and not us.any()
+
+
 def test_adapter_stack_driver_fused_groups():
     """The projections of a group as one linear layer (weights stacked by rows, B block-diagonal): every
     member's output columns, adapter gradients and the group's summed input gradient against the oracle
