@@ -1,7 +1,8 @@
 // HBM-bound helper kernels around the GEMMs: activation backward (dz), the stand-alone dbias
 // column reduction, and the bounded-wait self-test. All of them are links of the dependent-launch
 // chain: they are launched while their predecessor drains (chained_start waits for it) and let their
-// successor set itself up while they run.
+// successor set itself up while they run. Their inputs may be written while they are resident: no __restrict__ and no
+// read-only loads (ptx::ld_global_*).
 #pragma once
 #include "gemm_sm100.cuh"
 
@@ -21,15 +22,14 @@ __device__ __forceinline__ float silu_bwd(float g)
 
 // dz = dout * gelu'(pre), 8 bf16 per thread per iteration (128-bit loads and stores).
 __global__ void __launch_bounds__(256)
-gelu_backward_kernel(uint4 *__restrict__ dz, const uint4 *__restrict__ dout,
-                     const uint4 *__restrict__ pre, long long nvec)
+gelu_backward_kernel(uint4 *dz, const uint4 *dout, const uint4 *pre, long long nvec)
 {
     chained_start();
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < nvec;
          i += stride) {
-        const uint4 d = __ldg(dout + i);
-        const uint4 x = __ldg(pre + i);
+        const uint4 d = ptx::ld_global_v4(dout + i);
+        const uint4 x = ptx::ld_global_v4(pre + i);
         const uint32_t dv[4] = {d.x, d.y, d.z, d.w};
         const uint32_t xv[4] = {x.x, x.y, x.z, x.w};
         uint32_t o[4];
@@ -46,8 +46,7 @@ gelu_backward_kernel(uint4 *__restrict__ dz, const uint4 *__restrict__ dout,
 // SwiGLU backward: dout [BT, H], pre [BT, 2H] = [gate | up]  ->  dz [BT, 2H].
 //   dz[:, j] = dout * up * silu'(gate) ; dz[:, H + j] = dout * silu(gate)
 __global__ void __launch_bounds__(256)
-swiglu_backward_kernel(uint4 *__restrict__ dz, const uint4 *__restrict__ dout,
-                       const uint4 *__restrict__ pre, long long BT, int hvec /* H / 8 */)
+swiglu_backward_kernel(uint4 *dz, const uint4 *dout, const uint4 *pre, long long BT, int hvec /* H / 8 */)
 {
     chained_start();
     const long long total = BT * hvec;
@@ -56,9 +55,9 @@ swiglu_backward_kernel(uint4 *__restrict__ dz, const uint4 *__restrict__ dout,
          i += stride) {
         const long long m = i / hvec;
         const int j = static_cast<int>(i - m * hvec);
-        const uint4 d = __ldg(dout + i);
-        const uint4 g = __ldg(pre + m * 2 * hvec + j);
-        const uint4 u = __ldg(pre + m * 2 * hvec + hvec + j);
+        const uint4 d = ptx::ld_global_v4(dout + i);
+        const uint4 g = ptx::ld_global_v4(pre + m * 2 * hvec + j);
+        const uint4 u = ptx::ld_global_v4(pre + m * 2 * hvec + hvec + j);
         const uint32_t dv[4] = {d.x, d.y, d.z, d.w};
         const uint32_t gv[4] = {g.x, g.y, g.z, g.w};
         const uint32_t uv[4] = {u.x, u.y, u.z, u.w};
@@ -85,8 +84,7 @@ constexpr int kDbiasCols = 128;
 constexpr int kDbiasThreads = 256;
 
 __global__ void __launch_bounds__(kDbiasThreads)
-dbias_kernel(float *__restrict__ dbias, const __nv_bfloat16 *__restrict__ dz, long long BT, int OC,
-             int rows_per_block)
+dbias_kernel(float *dbias, const __nv_bfloat16 *dz, long long BT, int OC, int rows_per_block)
 {
     // 512 bytes of shared memory only: small enough to share an SM with a resident GEMM CTA
     __shared__ float part[kDbiasCols];
@@ -115,8 +113,8 @@ dbias_kernel(float *__restrict__ dbias, const __nv_bfloat16 *__restrict__ dz, lo
             v1[i] = make_uint4(0, 0, 0, 0);
             if (r < r_end) {
                 const __nv_bfloat16 *rowp = dz + r * OC + col0 + cv * 8;
-                if (in0) v0[i] = __ldg(reinterpret_cast<const uint4 *>(rowp));
-                if (in1) v1[i] = __ldg(reinterpret_cast<const uint4 *>(rowp + 64));
+                if (in0) v0[i] = ptx::ld_global_v4(rowp);
+                if (in1) v1[i] = ptx::ld_global_v4(rowp + 64);
             }
         }
 #pragma unroll
@@ -156,7 +154,7 @@ dbias_kernel(float *__restrict__ dbias, const __nv_bfloat16 *__restrict__ dz, lo
 // a successor that loads operands and multiplies first needs the zeros only when its first sums leave,
 // and calls griddepcontrol.wait there.
 __global__ void __launch_bounds__(256)
-clear_kernel(float *__restrict__ a, long long na, float *__restrict__ b, long long nb_)
+clear_kernel(float *a, long long na, float *b, long long nb_)
 {
     ptx::grid_dependency_wait();      // first: what the predecessors read must not be cleared under them,
     ptx::grid_launch_dependents();    // and whoever starts from here on may rely on their results
@@ -171,7 +169,7 @@ clear_kernel(float *__restrict__ a, long long na, float *__restrict__ b, long lo
 // fp32 -> bf16 (round to nearest even), 8 elements per thread per iteration: two 128-bit loads, one
 // 128-bit store. HBM-bound: 6 bytes per element.
 __global__ void __launch_bounds__(256)
-cast_f32_bf16_kernel(__nv_bfloat16 *__restrict__ dst, const float *__restrict__ src, long long n)
+cast_f32_bf16_kernel(__nv_bfloat16 *dst, const float *src, long long n)
 {
     chained_start();
     const long long nvec = n / 8;
@@ -180,8 +178,8 @@ cast_f32_bf16_kernel(__nv_bfloat16 *__restrict__ dst, const float *__restrict__ 
     const float4 *s4 = reinterpret_cast<const float4 *>(src);
     uint4 *d4 = reinterpret_cast<uint4 *>(dst);
     for (long long i = t0; i < nvec; i += stride) {
-        const float4 a = __ldg(s4 + 2 * i);
-        const float4 b = __ldg(s4 + 2 * i + 1);
+        const float4 a = ptx::ld_global_f32x4(s4 + 2 * i);
+        const float4 b = ptx::ld_global_f32x4(s4 + 2 * i + 1);
         d4[i] = make_uint4(ptx::pack_bf16x2(a.x, a.y), ptx::pack_bf16x2(a.z, a.w),
                            ptx::pack_bf16x2(b.x, b.y), ptx::pack_bf16x2(b.z, b.w));
     }
@@ -192,9 +190,8 @@ cast_f32_bf16_kernel(__nv_bfloat16 *__restrict__ dst, const float *__restrict__ 
 // the forward GEMM wrote: one warp per row combines the partial (max, sum exp) pairs into
 // lse = log sum_j exp(logit_j) and loss = lse - logit[target]. A target outside [0, V) gives NaN.
 __global__ void __launch_bounds__(256)
-ce_reduce_kernel(float *__restrict__ loss, float *__restrict__ lse, const float2 *__restrict__ stats,
-                 int stats_ld, const __nv_bfloat16 *__restrict__ logits, long long ld,
-                 const int *__restrict__ targets, long long BT, int V)
+ce_reduce_kernel(float *loss, float *lse, const float2 *stats, int stats_ld, const __nv_bfloat16 *logits, long long ld,
+                 const int *targets, long long BT, int V)
 {
     chained_start();
     const int lane = threadIdx.x & 31;
@@ -209,7 +206,7 @@ ce_reduce_kernel(float *__restrict__ loss, float *__restrict__ lse, const float2
         float mx = m;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            v[i] = k0 + 32 * i < stats_ld ? __ldg(st + k0 + 32 * i) : make_float2(-INFINITY, 0.0f);
+            v[i] = k0 + 32 * i < stats_ld ? ptx::ld_global_f32x2(st + k0 + 32 * i) : make_float2(-INFINITY, 0.0f);
             mx = fmaxf(mx, v[i].x);
         }
         if (mx > -INFINITY) {
@@ -242,8 +239,8 @@ ce_reduce_kernel(float *__restrict__ loss, float *__restrict__ lse, const float2
 // single columns: 550 -> 518 us at 16384 x 50304 (in place 563 -> 521, 3.3 GB), 37.3 -> 34.5 at
 // 1024 x 50304, 20.8 -> 14.1 in place at 8000 x 4096.
 __global__ void __launch_bounds__(256)
-ce_backward_kernel(uint4 *dlogits, const uint4 *logits, const float *__restrict__ lse,
-                   const int *__restrict__ targets, float gscale, long long BT, int vec_per_row, int V)
+ce_backward_kernel(uint4 *dlogits, const uint4 *logits, const float *lse, const int *targets, float gscale, long long BT,
+                   int vec_per_row, int V)
 {
     chained_start();
     const long long total = BT * vec_per_row;

@@ -629,7 +629,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     // element loads: the bias pointer is only required to be 2-byte aligned
                     const unsigned short *bp = reinterpret_cast<const unsigned short *>(p.bias) + col;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) bv[k] = static_cast<uint32_t>(__ldg(bp + k)) << 16;
+                    for (int k = 0; k < 4; ++k) bv[k] = ptx::ld_global_u16(bp + k) << 16;
                 }
             }
             bool ok = true;

@@ -328,6 +328,36 @@ __device__ __forceinline__ void tmem_ld_32x32_x2_wait(uint32_t taddr0, uint32_t 
         : "memory");
 }
 
+// ------------------------------------------------------------------ global memory access
+// Plain loads of what an earlier launch writes. A link of the dependent-launch chain is resident while its
+// producer still runs, so its inputs are not read-only for its whole life: the read-only path (__ldg, or a
+// const __restrict__ pointer) is not defined for them, and a load on it may be moved above
+// griddepcontrol.wait. Volatile keeps these behind it.
+__device__ __forceinline__ uint4 ld_global_v4(const void *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_global_f32x4(const void *p)
+{
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_global_f32x2(const void *p)
+{
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_global_u16(const void *p)
+{
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+
 // ------------------------------------------------------------------ shared memory access
 // 16 bytes into the shared memory of a CTA of the cluster (a shared::cluster address)
 __device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)

@@ -131,7 +131,7 @@ rows_kernel(const RowsParams p)
                 for (int h = 0; h < 2; ++h) a[u][s][h] = in ? ld_stream(wrow[s][h] + k) : zero;
 #pragma unroll
             for (int n = 0; n < NT; ++n)
-                b[u][n] = in ? __ldg(reinterpret_cast<const uint4 *>(xrow[n] + k)) : zero;
+                b[u][n] = in ? ptx::ld_global_v4(xrow[n] + k) : zero;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u)

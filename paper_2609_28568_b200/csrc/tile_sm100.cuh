@@ -458,7 +458,7 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
                         const int col = n0 + hf * HC + i * 8;
                         e[i] = make_uint4(0, 0, 0, 0);
                         if (row_ok && col < j.N)
-                            e[i] = __ldg(reinterpret_cast<const uint4 *>(j.E + grow * j.e_ld + col));
+                            e[i] = ptx::ld_global_v4(j.E + grow * j.e_ld + col);
                     }
                 }
                 bool ok = true;
@@ -584,7 +584,7 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
                 if (EPI == kEpiMulGeluGrad && et < items) {
                     const int col = n0 + cbase + (et % pieces) * 8;
                     if (col < j.N)
-                        e0 = __ldg(reinterpret_cast<const uint4 *>(j.E + static_cast<long long>(m0 + et / pieces) * j.e_ld + col));
+                        e0 = ptx::ld_global_v4(j.E + static_cast<long long>(m0 + et / pieces) * j.e_ld + col);
                 }
                 ptx::cluster_wait();  // every part has arrived
                 for (int it = et; ok && it < items; it += kEpiThreads) {
@@ -604,7 +604,7 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
                     if (col < j.N) {
                         uint4 e = e0;
                         if (EPI == kEpiMulGeluGrad && it != et)
-                            e = __ldg(reinterpret_cast<const uint4 *>(j.E + static_cast<long long>(m0 + rw) * j.e_ld + col));
+                            e = ptx::ld_global_v4(j.E + static_cast<long long>(m0 + rw) * j.e_ld + col);
                         uint4 o, z;
                         tile_math8<EPI>(j, v, line, cl, e, o, z);
                         const long long r = static_cast<long long>(m0) + rw;

@@ -149,3 +149,76 @@ def test_forward_in_192_column_pair_tiles(act, BT, C, OC, r):
                extra=2.0 ** -9 * (np.abs(t_ref) @ np.abs(f32(b).T.astype(np.float64))))
     out.check("out with adapter")
     nb.nb_check_status()
+
+
+def _layers_loop(BT, C, H, fused, sync):
+    """Two layers, forward and backward, over and over on two alternating sets of buffers: every tensor a
+    launch reads was written by one of the launches just before it, over what it held two passes earlier.
+    The weights shrink what goes through them, so the values settle where the biases put them."""
+    w1, w2 = gen(11, (H, C), 0.4 * C ** -0.5), gen(12, (C, H), 0.4 * H ** -0.5)
+    b1, b2 = gen(13, (H,), 0.1), gen(14, (C,), 0.1)
+    bf = dict(dtype=torch.bfloat16, device=DEV)
+    x = [gen(15, (BT, C), 1.0), torch.empty((BT, C), **bf)]
+    h, pre, dh = ([torch.empty((BT, H), **bf) for _ in range(2)] for _ in range(3))
+    y = [torch.empty((BT, C), **bf) for _ in range(2)]
+    dw = [torch.empty((C, H), device=DEV) for _ in range(2)]
+    wc = [torch.empty((C, H), **bf) for _ in range(2)]
+    for i in range(24):
+        k = i & 1
+        calls = (
+            lambda: nb.nb_linear_forward_ex(h[k], pre[k], x[k], w1, b1, BT, C, H, nb.ACT_GELU),
+            lambda: nb.nb_linear_forward_ex(y[k], None, h[k], w2, b2, BT, H, C, nb.ACT_NONE),
+            lambda: nb.nb_linear_backward_ex(dh[k], dw[k], None, y[k], h[k], w2, None, pre[k] if fused else None, BT, H, C,
+                                             nb.ACT_NONE, 0),
+            lambda: nb.nb_cast_f32_to_bf16(wc[k], dw[k], C * H),
+            lambda: nb.nb_linear_backward_ex(x[1 - k], None, None, dh[k], None, w1, None if fused else pre[k], None, BT, C, H,
+                                             nb.ACT_NONE if fused else nb.ACT_GELU, 0),
+        )
+        for call in calls:
+            call()
+            if sync:
+                torch.cuda.synchronize()
+    torch.cuda.synchronize()
+    for a, b in zip(wc, dw):
+        assert torch.equal(a, b.to(torch.bfloat16))
+    return x + h + pre + y + dh
+
+
+@pytest.mark.parametrize("fused", [False, True])
+@pytest.mark.parametrize("BT,C,H", [(8, 768, 3072), (3, 1032, 520), (72, 768, 776), (300, 520, 1544), (2100, 776, 1032)])
+def test_chained_launches_over_two_alternating_buffers(BT, C, H, fused):
+    """A launch may start while its producer runs; what it then reads has to be what that one wrote, not what
+    the buffer held before: the same bits as with the device idle between launches."""
+    for a, b in zip(_layers_loop(BT, C, H, fused, False), _layers_loop(BT, C, H, fused, True)):
+        assert torch.isfinite(a).all() and a.any()
+        assert torch.equal(a, b)
+    nb.nb_check_status()
+
+
+@pytest.mark.parametrize("BT", [5, 300])
+def test_chained_head_over_two_alternating_buffers(BT):
+    C, Vp, V = 264, 1016, 1009
+    w = gen(21, (Vp, C), C ** -0.5)
+    targets = (torch.arange(BT, device=DEV) * 31 % V).to(torch.int32)
+    got = []
+    for sync in (False, True):
+        x = [gen(22, (BT, C), 1.0), torch.empty((BT, C), dtype=torch.bfloat16, device=DEV)]
+        logits = [torch.empty((BT, Vp), dtype=torch.bfloat16, device=DEV) for _ in range(2)]
+        loss, lse = ([torch.empty(BT, device=DEV) for _ in range(2)] for _ in range(2))
+        for i in range(24):
+            k = i & 1
+            for call in (
+                lambda: nb.nb_lm_head_ce_forward(logits[k], loss[k], lse[k], x[k], w, targets, BT, C, Vp, V),
+                lambda: nb.nb_ce_backward(logits[k], logits[k], lse[k], targets, 2.0, BT, Vp, V),
+                lambda: nb.nb_linear_backward_ex(x[1 - k], None, None, logits[k], None, w, None, None, BT, C, Vp,
+                                                 nb.ACT_NONE, 0),
+            ):
+                call()
+                if sync:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        got.append(x + logits + loss + lse)
+    for a, b in zip(*got):
+        assert torch.isfinite(a).all() and a.any()
+        assert torch.equal(a, b)
+    nb.nb_check_status()
