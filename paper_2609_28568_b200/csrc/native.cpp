@@ -161,9 +161,12 @@ PyObject *linear_forward(PyObject *, PyObject *const *args, Py_ssize_t n)
     const auto opt = inp.options().dtype(at::kBFloat16);
     at::Tensor out = at::empty({BT, act == NB_ACT_SWIGLU ? OC / 2 : OC}, opt), pre;
     if (act != NB_ACT_NONE) pre = at::empty({BT, OC}, opt);
+    // whatever of torch can throw comes before the interpreter's lock is given up
+    void *const po = ptr(out), *const pp = ptr(pre), *const pi = ptr(inp), *const pw = ptr(weight), *const pb = ptr(bias);
+    void *const stream = current_stream();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = nb_linear_forward_ex(ptr(out), ptr(pre), ptr(inp), ptr(weight), ptr(bias), BT, C, OC, act, current_stream());
+    rc = nb_linear_forward_ex(po, pp, pi, pw, pb, BT, C, OC, act, stream);
     Py_END_ALLOW_THREADS
     if (rc != NB_OK) return raise(rc);
     return Py_BuildValue("NN", wrap(std::move(out)), wrap(std::move(pre)));
@@ -190,10 +193,13 @@ PyObject *linear_backward(PyObject *, PyObject *const *args, Py_ssize_t n)
     if (flag[1]) dinp = at::empty({BT, C}, opt.dtype(at::kBFloat16));
     if (flag[2] && !dw.defined()) dw = at::empty({OC, C}, opt.dtype(at::kFloat));
     if (flag[3] && !db.defined()) db = at::empty({OC}, opt.dtype(at::kFloat));
+    // whatever of torch can throw comes before the interpreter's lock is given up
+    void *const px = ptr(dinp), *const pdw = flag[2] ? ptr(dw) : nullptr, *const pdb = flag[3] ? ptr(db) : nullptr;
+    void *const pd = ptr(dout), *const pi = ptr(inp), *const pw = ptr(weight), *const pp = ptr(pre), *const pe = ptr(ipre);
+    void *const stream = current_stream();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = nb_linear_backward_ex(ptr(dinp), flag[2] ? ptr(dw) : nullptr, flag[3] ? ptr(db) : nullptr, ptr(dout), ptr(inp),
-                               ptr(weight), ptr(pre), ptr(ipre), BT, C, OC, act, flag[0], NB_DTYPE_F32, current_stream());
+    rc = nb_linear_backward_ex(px, pdw, pdb, pd, pi, pw, pp, pe, BT, C, OC, act, flag[0], NB_DTYPE_F32, stream);
     Py_END_ALLOW_THREADS
     if (rc != NB_OK) return raise(rc);
     return Py_BuildValue("NNN", wrap(std::move(dinp)), wrap(std::move(dw)), wrap(std::move(db)));
