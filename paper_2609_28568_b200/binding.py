@@ -95,7 +95,7 @@ def _load_native():
     loader = importlib.machinery.ExtensionFileLoader(name, NATIVE_PATH)
     module = importlib.util.module_from_spec(importlib.util.spec_from_loader(name, loader))
     loader.exec_module(module)
-    module.set_error(NbError)
+    module.set_python(NbError, _ptr, _stream_address)
     _native = module
     return module
 
@@ -107,6 +107,15 @@ def _ptr(t):
         return t
     assert t.is_cuda and t.is_contiguous(), "device tensors must be contiguous CUDA tensors"
     return t.data_ptr()
+
+
+def _stream_address(s):
+    """The address in a stream object: a c_void_p, or what carries one as _as_parameter_ (torch.cuda.Stream)."""
+    while not (s is None or isinstance(s, (int, ctypes.c_void_p))):
+        if not hasattr(s, "_as_parameter_"):
+            raise TypeError(f"a stream or its address is wanted, not {type(s).__name__}")
+        s = s._as_parameter_
+    return s.value if isinstance(s, ctypes.c_void_p) else s
 
 
 def _check(rc: int) -> None:

@@ -14,6 +14,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <tuple>
 #include <type_traits>
 #include <utility>
 
@@ -21,7 +22,8 @@
 
 namespace {
 
-PyObject *g_error = nullptr;  // NbError, given by the Python side
+// given by the Python side: NbError, and what turns the rarer kinds of arguments into addresses
+PyObject *g_error = nullptr, *g_pointer_of = nullptr, *g_stream_of = nullptr;
 
 // Raises NbError(code, text) and returns null.
 PyObject *raise(int rc)
@@ -38,13 +40,24 @@ PyObject *raise(int rc)
 
 void *current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// A device pointer from None, an address, or a contiguous CUDA tensor.
+bool to_address(PyObject *o, void *&p)  // None or an int
+{
+    p = o == Py_None ? nullptr : PyLong_AsVoidPtr(o);
+    return !(p == nullptr && PyErr_Occurred());
+}
+bool by_python(PyObject *convert, PyObject *o, void *&p)
+{
+    if (!convert) return PyErr_Format(PyExc_TypeError, "a tensor, an address or None is wanted, not %.100s", Py_TYPE(o)->tp_name), false;
+    PyObject *a = PyObject_CallOneArg(convert, o);
+    if (!a) return false;
+    const bool ok = to_address(a, p);
+    Py_DECREF(a);
+    return ok;
+}
+
+// A device pointer from None, an address, a contiguous CUDA tensor, or (by Python) what behaves like one.
 bool to_pointer(PyObject *o, void *&p)
 {
-    if (o == Py_None) {
-        p = nullptr;
-        return true;
-    }
     if (THPVariable_Check(o)) {
         const at::Tensor &t = THPVariable_Unpack(o);
         if (!t.is_cuda() || !t.is_contiguous()) {
@@ -54,13 +67,11 @@ bool to_pointer(PyObject *o, void *&p)
         p = t.data_ptr();
         return true;
     }
-    if (PyLong_Check(o)) {
-        p = PyLong_AsVoidPtr(o);
-        return !(p == nullptr && PyErr_Occurred());
-    }
-    PyErr_Format(PyExc_TypeError, "a tensor, an address or None is wanted, not %.100s", Py_TYPE(o)->tp_name);
-    return false;
+    if (o == Py_None || PyLong_Check(o)) return to_address(o, p);
+    return by_python(g_pointer_of, o, p);
 }
+// A stream from an address or (by Python) a stream object.
+bool to_stream(PyObject *o, void *&p) { return PyLong_Check(o) ? to_address(o, p) : by_python(g_stream_of, o, p); }
 
 template <class T>
 bool convert(PyObject *o, T &v)
@@ -89,16 +100,18 @@ template <class... A, size_t... I>
 PyObject *call(int (*fn)(A...), PyObject *const *args, Py_ssize_t n, std::index_sequence<I...>)
 {
     constexpr Py_ssize_t N = sizeof...(A);
+    static_assert(std::is_same_v<std::tuple_element_t<N - 1, std::tuple<A...>>, void *>, "the last argument is the stream");
     if (n != N && n != N - 1) {
         PyErr_Format(PyExc_TypeError, "%zd or %zd arguments are wanted, not %zd", N - 1, N, n);
         return nullptr;
     }
     std::tuple<A...> v;
     auto one = [&](auto &dst, size_t i) {
-        if (static_cast<Py_ssize_t>(i) == N - 1 && (n == N - 1 || args[i] == Py_None)) {
-            if constexpr (std::is_pointer_v<std::decay_t<decltype(dst)>>) dst = current_stream();
-            return true;
-        }
+        if constexpr (std::is_same_v<std::decay_t<decltype(dst)>, void *>)
+            if (static_cast<Py_ssize_t>(i) == N - 1) {
+                if (n < N || args[i] == Py_None) return dst = current_stream(), true;
+                return to_stream(args[i], dst);
+            }
         return convert(args[i], dst);
     };
     if (!(one(std::get<I>(v), I) && ...)) return nullptr;
@@ -120,9 +133,8 @@ PyObject *entry(PyObject *, PyObject *const *args, Py_ssize_t n)
     END_HANDLE_TH_ERRORS
 }
 
-bool to_tensor(PyObject *o, at::Tensor &t)  // None: an undefined tensor
+bool to_tensor(PyObject *o, at::Tensor &t)
 {
-    if (o == Py_None) return true;
     if (!THPVariable_Check(o)) {
         PyErr_Format(PyExc_TypeError, "a tensor is wanted, not %.100s", Py_TYPE(o)->tp_name);
         return false;
@@ -134,11 +146,10 @@ bool to_tensor(PyObject *o, at::Tensor &t)  // None: an undefined tensor
     }
     return true;
 }
-bool two_dims(const at::Tensor &t, const char *name)
+bool dims(const at::Tensor &t, bool ok, const char *name)
 {
-    if (t.defined() && t.dim() == 2) return true;
-    PyErr_Format(PyExc_ValueError, "%s must have two dimensions", name);
-    return false;
+    if (!ok) PyErr_Format(PyExc_ValueError, "%s has %lld dimensions", name, static_cast<long long>(t.dim()));
+    return ok;
 }
 void *ptr(const at::Tensor &t) { return t.defined() ? t.data_ptr() : nullptr; }
 PyObject *wrap(at::Tensor t)
@@ -151,18 +162,20 @@ PyObject *wrap(at::Tensor t)
 PyObject *linear_forward(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     HANDLE_TH_ERRORS
-    at::Tensor inp, weight, bias;
+    at::Tensor inp, weight;
+    void *pb = nullptr;
     int act = 0;
     if (n != 4) return PyErr_Format(PyExc_TypeError, "4 arguments are wanted");
-    if (!to_tensor(args[0], inp) || !to_tensor(args[1], weight) || !to_tensor(args[2], bias) || !convert(args[3], act))
+    if (!to_tensor(args[0], inp) || !to_tensor(args[1], weight) || !to_pointer(args[2], pb) || !convert(args[3], act))
         return nullptr;
-    if (!two_dims(inp, "inp") || !two_dims(weight, "weight")) return nullptr;
+    // of the weight only the number of rows is taken: it may have its columns in more than one dimension
+    if (!dims(inp, inp.dim() == 2, "inp") || !dims(weight, weight.dim() >= 1, "weight")) return nullptr;
     const int64_t BT = inp.size(0), C = inp.size(1), OC = weight.size(0);
     const auto opt = inp.options().dtype(at::kBFloat16);
     at::Tensor out = at::empty({BT, act == NB_ACT_SWIGLU ? OC / 2 : OC}, opt), pre;
     if (act != NB_ACT_NONE) pre = at::empty({BT, OC}, opt);
     // whatever of torch can throw comes before the interpreter's lock is given up
-    void *const po = ptr(out), *const pp = ptr(pre), *const pi = ptr(inp), *const pw = ptr(weight), *const pb = ptr(bias);
+    void *const po = ptr(out), *const pp = ptr(pre), *const pi = ptr(inp), *const pw = ptr(weight);
     void *const stream = current_stream();
     int rc;
     Py_BEGIN_ALLOW_THREADS
@@ -178,38 +191,44 @@ PyObject *linear_forward(PyObject *, PyObject *const *args, Py_ssize_t n)
 PyObject *linear_backward(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     HANDLE_TH_ERRORS
-    at::Tensor dout, inp, weight, pre, ipre, dw, db, dinp;
+    at::Tensor dout, weight, dinp, new_dw, new_db;
+    void *pi = nullptr, *pp = nullptr, *pe = nullptr, *pdw = nullptr, *pdb = nullptr;
     int act = 0;
     if (n != 12) return PyErr_Format(PyExc_TypeError, "12 arguments are wanted");
-    if (!to_tensor(args[0], dout) || !to_tensor(args[1], inp) || !to_tensor(args[2], weight) || !to_tensor(args[3], pre) ||
-        !to_tensor(args[4], ipre) || !convert(args[5], act) || !to_tensor(args[6], dw) || !to_tensor(args[7], db))
-        return nullptr;
     int flag[4];  // accumulate, need_dinp, need_dweight, need_dbias
     for (int i = 0; i < 4; ++i)
         if ((flag[i] = PyObject_IsTrue(args[8 + i])) < 0) return nullptr;
-    if (!two_dims(dout, "dout") || !two_dims(weight, "weight")) return nullptr;
+    // a gradient that is not asked for goes back as it came, whatever it is
+    if (!to_tensor(args[0], dout) || !to_pointer(args[1], pi) || !to_tensor(args[2], weight) || !to_pointer(args[3], pp) ||
+        !to_pointer(args[4], pe) || !convert(args[5], act) || (flag[2] && !to_pointer(args[6], pdw)) ||
+        (flag[3] && !to_pointer(args[7], pdb)))
+        return nullptr;
+    // of dout only the number of rows is taken
+    if (!dims(dout, dout.dim() >= 1, "dout") || !dims(weight, weight.dim() == 2, "weight")) return nullptr;
     const int64_t BT = dout.size(0), OC = weight.size(0), C = weight.size(1);
     const auto opt = dout.options();
     if (flag[1]) dinp = at::empty({BT, C}, opt.dtype(at::kBFloat16));
-    if (flag[2] && !dw.defined()) dw = at::empty({OC, C}, opt.dtype(at::kFloat));
-    if (flag[3] && !db.defined()) db = at::empty({OC}, opt.dtype(at::kFloat));
+    if (flag[2] && args[6] == Py_None) pdw = ptr(new_dw = at::empty({OC, C}, opt.dtype(at::kFloat)));
+    if (flag[3] && args[7] == Py_None) pdb = ptr(new_db = at::empty({OC}, opt.dtype(at::kFloat)));
     // whatever of torch can throw comes before the interpreter's lock is given up
-    void *const px = ptr(dinp), *const pdw = flag[2] ? ptr(dw) : nullptr, *const pdb = flag[3] ? ptr(db) : nullptr;
-    void *const pd = ptr(dout), *const pi = ptr(inp), *const pw = ptr(weight), *const pp = ptr(pre), *const pe = ptr(ipre);
-    void *const stream = current_stream();
+    void *const px = ptr(dinp), *const pd = ptr(dout), *const pw = ptr(weight), *const stream = current_stream();
     int rc;
     Py_BEGIN_ALLOW_THREADS
     rc = nb_linear_backward_ex(px, pdw, pdb, pd, pi, pw, pp, pe, BT, C, OC, act, flag[0], NB_DTYPE_F32, stream);
     Py_END_ALLOW_THREADS
     if (rc != NB_OK) return raise(rc);
-    return Py_BuildValue("NNN", wrap(std::move(dinp)), wrap(std::move(dw)), wrap(std::move(db)));
+    auto given = [](PyObject *o, at::Tensor &t) { return t.defined() ? wrap(std::move(t)) : Py_NewRef(o); };
+    return Py_BuildValue("NNN", wrap(std::move(dinp)), given(args[6], new_dw), given(args[7], new_db));
     END_HANDLE_TH_ERRORS
 }
 
-PyObject *set_error(PyObject *, PyObject *cls)
+// set_python(NbError, pointer_of, stream_of)
+PyObject *set_python(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
-    Py_INCREF(cls);
-    Py_XSETREF(g_error, cls);
+    if (n != 3) return PyErr_Format(PyExc_TypeError, "3 arguments are wanted");
+    Py_XSETREF(g_error, Py_NewRef(args[0]));
+    Py_XSETREF(g_pointer_of, Py_NewRef(args[1]));
+    Py_XSETREF(g_stream_of, Py_NewRef(args[2]));
     Py_RETURN_NONE;
 }
 
@@ -230,7 +249,7 @@ PyMethodDef g_methods[] = {
     NB_ENTRY(nb_cast_f32_to_bf16),
     NB_FAST(linear_forward),
     NB_FAST(linear_backward),
-    {"set_error", set_error, METH_O, nullptr},
+    NB_FAST(set_python),
     {nullptr, nullptr, 0, nullptr},
 };
 PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_native", "Argument marshalling for the nb_linear C ABI.", -1, g_methods,
