@@ -948,7 +948,7 @@ int env_int(const char *name, int dflt)
     return (e && *e) ? atoi(e) : dflt;
 }
 
-constexpr double kNarrowD = 0.6;
+constexpr double kNarrowD = 0.6;  // in the level share of the work; backward_us takes 0.7 for the chain of one such tile
 bool layer_bwd_narrow(int d_tiles, int d_kblocks, int w_tiles, int w_kblocks, int P)
 {
     return d_tiles * 4 <= P && d_kblocks >= 36 && d_kblocks >= 12 + 2 * d_tiles &&
@@ -966,8 +966,8 @@ bool layer_bwd_narrow(int d_tiles, int d_kblocks, int w_tiles, int w_kblocks, in
 //  3. The last D round is partial: pairs [0, d_tail) take one more tile. The W units left over are
 //     laid out as one line of k-blocks and cut into P ranges, shorter by one D unit's cost for the
 //     pairs that took a tail tile. If the line is too short for that, one W round is taken back.
-// narrow: D tiles may be 128 columns wide. They are where the 256-wide ones are at most a quarter of the
-// pairs, K is long, and a single one takes longer than a pair's share of all the work: 1500 rows,
+// narrow (as it is launched): D tiles are 128 columns wide (layer_bwd_narrow; not with gelu') where the 256-wide ones are
+// at most a quarter of the pairs, K is long, and a single one takes longer than a pair's share of all the work: 1500 rows,
 // 768 -> 3072, 18 tiles of 48 k-blocks, 18.9 -> 16.4 us; 1024 rows, 1024 -> 6144, 32.5 -> 24.4 us. With
 // more tiles the operand traffic of halved ones costs more than the shorter chain gives (2021 rows,
 // 768 -> 2304, 24 tiles: 16.0 -> 19.4 us). A 128-wide k-block is counted as 0.6 of a 256-wide one.
@@ -1218,7 +1218,8 @@ int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
 }
 
 // A layer's backward without the small-problem kernel: layer_bwd_kernel for both products, else a
-// launch per product. An fp32 result that starts from zero costs the clearing besides.
+// launch per product. An fp32 result that starts from zero costs the clearing besides. (sms / 2: the CTA pairs that
+// the launch's occupancy query finds on B200.)
 double backward_us(int sms, int M, int BT, int N, int Mw, int kd, int kw, bool accumulate, bool apart, bool gelu)
 {
     const int slots = sms / 2;
@@ -1891,12 +1892,12 @@ int nb_debug_split_plan(int64_t M, int64_t N, int64_t K, int slots, int tile_m, 
     return NB_OK;
 }
 
-int nb_debug_layer_bwd_plan(int64_t BT, int64_t C, int64_t OC, int pairs, int gelu_grad, int *out,
+int nb_debug_layer_bwd_plan(int64_t BT, int64_t C, int64_t OC, int pairs, int flags, int *out,
                             int64_t cap)
 {
     if (!out || cap < 8 || BT <= 0 || C <= 0 || OC <= 0) return -fail(NB_ERR_INVALID_ARG, "bad argument");
     LayerBwdParams p;
-    const int rc = plan_layer_bwd(p, BT, C, OC, pairs, gelu_grad != 0, false);
+    const int rc = plan_layer_bwd(p, BT, C, OC, pairs, (flags & NB_PLAN_GELU_GRAD) != 0, (flags & NB_PLAN_LAUNCHED) != 0);
     if (rc != NB_OK) return -rc;
     out[0] = p.d_tiles_m; out[1] = p.d_tiles_n; out[2] = p.d_kblocks;
     out[3] = p.w_tiles_m; out[4] = p.w_tiles_n; out[5] = p.w_kblocks;

@@ -182,3 +182,36 @@ def test_layer_backward_plan_on_drawn_shapes(L):
         assert (d_seen == 1).all(), tag
         assert (w_cov == 1).all(), tag
     assert declined < 100   # the drawn set mostly exercises the planner, not its refusal
+
+
+def test_layer_backward_plan_with_halved_dinp_tiles(L):
+    """A few dinp tiles over a long K are 128 columns wide in the launch's own plan: they
+    partition the work like whole ones. At most a quarter of the pairs as whole tiles, at least 36 and 12 + two a tile of
+    k-blocks, and one tile longer than a pair's share; never with the GELU derivative."""
+    import numpy as np
+    rng = np.random.default_rng(7)
+    cases = [(1500, 760, 3080, 74), (1030, 760, 6152, 74), (1500, 768, 3072, 74), (1024, 1024, 6144, 74), (512, 768, 50304, 74),
+             (300, 8, 2304, 66), (257, 136, 4104, 33)]
+    while len(cases) < 60:
+        cases.append((int(rng.integers(129, 1600)), 8 * int(rng.integers(1, 160)), 8 * int(rng.integers(288, 1500)),
+                      int(rng.choice((74, 66, 33)))))
+    halved = 0
+    for BT, C, OC, pairs in cases:
+        tiles, dkb, wkb = -(-BT // 256) * -(-C // 256), -(-OC // 64), -(-BT // 64)
+        wt = -(-OC // 256) * -(-C // 256)
+        narrow = tiles * 4 <= pairs and dkb >= 36 and dkb >= 12 + 2 * tiles and dkb * pairs > tiles * dkb + wt * wkb
+        for gelu in (False, True):
+            hdr, recs = binding.nb_debug_layer_bwd_plan(BT, C, OC, pairs, gelu, launched=True)
+            width = 128 if narrow and not gelu else 256
+            tag = (BT, C, OC, pairs, gelu)
+            assert hdr[:6] == (-(-BT // 256), -(-C // width), dkb, -(-OC // 256), -(-C // 256), wkb), tag
+            d = sorted((m, n, kb0, kb1) for _, is_w, m, n, kb0, kb1 in recs if not is_w)
+            assert d == [(m, n, 0, dkb) for m in range(hdr[0]) for n in range(hdr[1])], tag
+            cov = np.zeros((hdr[3], hdr[4], wkb), dtype=np.int64)
+            for _, is_w, m, n, kb0, kb1 in recs:
+                if is_w:
+                    cov[m, n, kb0:kb1] += 1
+            assert (cov == 1).all(), tag
+        halved += narrow
+    assert halved >= 20
+    assert all(t in cases for t in ((1500, 760, 3080, 74), (1030, 760, 6152, 74)))  # also on the GPU: test_gpu_small_problems
