@@ -360,6 +360,36 @@ int nb_debug_layer_bwd_plan(int64_t BT, int64_t C, int64_t OC, int pairs, int fl
                             int64_t cap);
 
 /*
+ * Host-only view of the kernels that a call takes on a device of `sms` SMs, as the call itself decides
+ * it from its sizes (no device is touched; one product of the paper's path may run in several forms).
+ *   call   NB_CALL_FORWARD (act as in nb_linear_forward_ex), NB_CALL_BACKWARD, NB_CALL_LORA_FORWARD,
+ *          NB_CALL_LORA_BACKWARD (r: the rank; else ignored)
+ *   flags  what a backward call is asked for: NB_CALL_DINP, NB_CALL_DWEIGHT (fp32; adapters: dlora_a),
+ *          NB_CALL_DBIAS (adapters: dlora_b), NB_CALL_GELU_GRAD (inp_pre_act given), NB_CALL_ACCUMULATE
+ *   out    up to 12 ints, four per launch: kernel (NB_ROUTE_*), width of its tiles in columns (weight rows
+ *          for NB_ROUTE_ROWS), CTAs of a cluster that share K, CTAs per SM that it is sized for
+ * Clearing and elementwise launches are left out. Returns the number of launches, or minus an NB_ERR_* code.
+ */
+#define NB_CALL_FORWARD 0
+#define NB_CALL_BACKWARD 1
+#define NB_CALL_LORA_FORWARD 2
+#define NB_CALL_LORA_BACKWARD 3
+#define NB_CALL_DINP 1
+#define NB_CALL_DWEIGHT 2
+#define NB_CALL_DBIAS 4
+#define NB_CALL_GELU_GRAD 8
+#define NB_CALL_ACCUMULATE 16
+#define NB_ROUTE_ROWS 1      /* rows_kernel */
+#define NB_ROUTE_TILE 2      /* tile_kernel */
+#define NB_ROUTE_TILE_PAIR 3 /* tile_pair_kernel */
+#define NB_ROUTE_GEMM 4      /* gemm_kernel */
+#define NB_ROUTE_GEMM_192 5  /* gemm_kernel in 192-column pair tiles */
+#define NB_ROUTE_LAYER_BWD 6 /* layer_bwd_kernel */
+#define NB_ROUTE_LORA_UDB 7  /* lora_udb_kernel */
+int nb_debug_route(int call, int64_t BT, int64_t C, int64_t OC, int64_t r, int act, int flags, int sms,
+                   int *out);
+
+/*
  * Self-test of the bounded-wait mechanism: launches a one-block kernel that waits, for
  * at most `limit_us` microseconds, on a barrier nothing ever signals, then returns
  * normally after recording the expiry. nb_check_status() afterwards reports

@@ -29,8 +29,11 @@ EXPORTS = (
     "nb_debug_split_plan", "nb_cast_f32_to_bf16", "nb_lm_head_ce_forward", "nb_ce_backward",
     "nb_lora_linear_forward", "nb_lora_linear_backward", "nb_debug_layer_bwd_plan", "nb_debug_gemm_timeout",
     "nb_lora_down_stacked", "nb_lora_linear_forward_stacked", "nb_lora_linear_backward_stacked",
-    "nb_lora_da_stacked",
+    "nb_lora_da_stacked", "nb_debug_route",
 )
+
+CALL_FORWARD, CALL_BACKWARD, CALL_LORA_FORWARD, CALL_LORA_BACKWARD = range(4)
+ROUTES = {1: "rows", 2: "tile", 3: "tile_pair", 4: "gemm", 5: "gemm", 6: "layer_bwd", 7: "lora_udb"}
 
 _lib = None
 _vp, _i64, _int = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int
@@ -78,6 +81,7 @@ def lib() -> ctypes.CDLL:
         L.nb_debug_split_plan.argtypes = [_i64, _i64, _i64, _int, _int, ctypes.POINTER(_int)]
         L.nb_debug_gemm_timeout.argtypes = [_vp, _vp, _vp, _i64]
         L.nb_debug_layer_bwd_plan.argtypes = [_i64, _i64, _i64, _int, _int, ctypes.POINTER(_int), _i64]
+        L.nb_debug_route.argtypes = [_int] + [_i64] * 4 + [_int] * 3 + [ctypes.POINTER(_int)]
         _lib = L
     return _lib
 
@@ -264,6 +268,19 @@ def nb_debug_layer_bwd_plan(BT: int, C: int, OC: int, pairs: int, gelu_grad: boo
         raise NbError(-n, lib().nb_last_error().decode())
     recs = [tuple(out[8 + 6 * i: 14 + 6 * i]) for i in range(n)]
     return tuple(out[:8]), recs
+
+
+def nb_debug_route(call: int, BT: int, C: int, OC: int, *, r: int = 0, act: int = ACT_NONE, dinp: bool = True,
+                   dweight: bool = True, dbias: bool = True, gelu_grad: bool = False, accumulate: bool = False,
+                   sms: int = 148):
+    """The launches of a call as (kernel, tile width, CTAs sharing K, CTAs per SM), by name; adapters: dweight
+    stands for dlora_a and dbias for dlora_b."""
+    out = (_int * 12)()
+    flags = sum(bool(f) << i for i, f in enumerate((dinp, dweight, dbias, gelu_grad, accumulate)))
+    n = lib().nb_debug_route(call, BT, C, OC, r, act, flags, sms, out)
+    if n < 0:
+        raise NbError(-n, lib().nb_last_error().decode())
+    return [(ROUTES[out[4 * i]], *out[4 * i + 1:4 * i + 4]) for i in range(n)]
 
 
 def nb_kernel_launches() -> int:

@@ -571,6 +571,18 @@ int launch_tile_pair(DeviceState &s, const GemmArgs *d, const GemmArgs &w, int a
 
 // A forward product on at most kRowsMax rows. K is shared among a cluster when it is long (48 CTAs
 // of 16 features took 7.9 us for K = 3072, and 2.7 us for K = 768), as far as two CTAs per SM go.
+int rows_split(int sms, int groups, int K)
+{
+    int split = 1;
+    while (split < kRowsMaxSplit && K >= 1024 * split && groups * split <= sms) split *= 2;
+    return split;
+}
+// Several CTAs of features per SM: the form with four of them on an SM. Not for the gate and up rows of 9 to 16
+// rows: too few registers (1024 -> 16384 12.6 us, with two CTAs 8.6).
+bool rows_many(int sms, int M, int span, bool swiglu)
+{
+    return span > 3 * sms * kRowsFeatures && !(swiglu && M > 8);
+}
 template <int NT, int EPI, bool MANY>
 int launch_rows(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
 {
@@ -585,10 +597,8 @@ int launch_rows(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
     p.K = a.K;
     p.N = a.N;
     p.swiglu_h = a.swiglu_h;
-    const int span = EPI == kEpiSwiglu ? a.swiglu_h : a.N;
-    const int groups = (span + kRowsFeatures - 1) / kRowsFeatures;
-    p.ksplit = 1;
-    while (p.ksplit < kRowsMaxSplit && a.K >= 1024 * p.ksplit && groups * p.ksplit <= s.num_sms) p.ksplit *= 2;
+    const int groups = ((EPI == kEpiSwiglu ? a.swiglu_h : a.N) + kRowsFeatures - 1) / kRowsFeatures;
+    p.ksplit = rows_split(s.num_sms, groups, a.K);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attrs[2];
     small_launch_config(cfg, attrs, groups * p.ksplit, kRowsThreads, p.ksplit, 0, stream);
@@ -600,10 +610,9 @@ int launch_rows(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
 template <int EPI>
 int launch_rows_auto(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
 {
-    const int span = EPI == kEpiSwiglu ? a.swiglu_h : a.N;
-    const bool many = span > 3 * s.num_sms * kRowsFeatures;
+    const bool many = rows_many(s.num_sms, a.M, EPI == kEpiSwiglu ? a.swiglu_h : a.N, EPI == kEpiSwiglu);
     if (a.M <= 8) return many ? launch_rows<1, EPI, true>(s, a, stream) : launch_rows<1, EPI, false>(s, a, stream);
-    if constexpr (EPI != kEpiSwiglu)  // gate and up rows: too few registers (1024 -> 16384 12.6 us, with two CTAs 8.6)
+    if constexpr (EPI != kEpiSwiglu)
         if (many) return launch_rows<2, EPI, true>(s, a, stream);
     return launch_rows<2, EPI, false>(s, a, stream);
 }
@@ -1190,31 +1199,45 @@ bool narrower_tiles(int sms, int M, int N)
     return waves(256) > 1 && waves(192) == waves(256);
 }
 
+// Which kernel forms a product, and in which form.
+struct Route {
+    int kernel = NB_ROUTE_GEMM;
+    SmallPlan pl;  // the tile kernels
+};
+
 // A forward product with its activation: on a few rows the row kernel (9 to 16 rows only up to 8 CTAs
 // per SM: 16 rows, 768 -> 50304 takes 19.5 us there and 17.3 us in gemm_kernel), then the smaller of the
 // tile and the persistent kernel's estimates.
+Route route_forward(int sms, int M, int N, int K, int act, bool adapter)
+{
+    if (!adapter && (M <= 8 || (M <= kRowsMax && N <= 8 * sms * kRowsFeatures))) return {NB_ROUTE_ROWS, {}};
+    const int kb = kblocks_of(K) + (adapter ? 1 : 0);
+    const double other = persistent_us(sms, M, N, kb);
+    // SwiGLU: 64 gate and 64 up columns per tile, so N counts both halves of the weight
+    const SmallPlan pl = act == NB_ACT_SWIGLU ? plan_single(sms, M, N, kb, false, 1, 128, other)
+                                              : plan_single(sms, M, N, kb, true, 0, 0, other);
+    if (pl.bn) return {NB_ROUTE_TILE, pl};
+    return {act != NB_ACT_SWIGLU && narrower_tiles(sms, M, N) ? NB_ROUTE_GEMM_192 : NB_ROUTE_GEMM, pl};
+}
+
 int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
 {
-    const bool adapter = a.A2 != nullptr;
-    if (!adapter && (a.M <= 8 || (a.M <= kRowsMax && a.N <= 8 * s.num_sms * kRowsFeatures))) {
+    const Route r = route_forward(s.num_sms, a.M, a.N, a.K, act, a.A2 != nullptr);
+    if (r.kernel == NB_ROUTE_ROWS) {
         if (act == NB_ACT_NONE) return launch_rows_auto<kEpiStore>(s, a, stream);
         if (act == NB_ACT_GELU) return launch_rows_auto<kEpiGelu>(s, a, stream);
         return launch_rows_auto<kEpiSwiglu>(s, a, stream);
     }
-    const int kb = kblocks_of(a.K) + (adapter ? 1 : 0);
-    const double other = persistent_us(s.num_sms, a.M, a.N, kb);
-    if (act == NB_ACT_SWIGLU) {
-        // 64 gate and 64 up columns per tile, so N counts both halves of the weight
-        const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, false, 1, 128, other);
-        if (pl.bn) return launch_tile<128, false, kEpiSwiglu>(s, a, 1, false, stream);
-        return launch_gemm_auto<FwdSwiglu1, FwdSwiglu2>(s, a, stream);
+    if (r.kernel == NB_ROUTE_TILE) {
+        if (act == NB_ACT_SWIGLU) return launch_tile<128, false, kEpiSwiglu>(s, a, 1, false, stream);
+        return act == NB_ACT_GELU ? launch_tile_plan<false, kEpiGelu>(s, a, r.pl, stream)
+                                  : launch_tile_plan<false, kEpiStore>(s, a, r.pl, stream);
     }
-    const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, true, 0, 0, other);
-    if (!pl.bn && narrower_tiles(s.num_sms, a.M, a.N))
+    if (r.kernel == NB_ROUTE_GEMM_192)
         return act == NB_ACT_GELU ? launch_gemm<FwdGelu2N>(s, a, stream) : launch_gemm<FwdStore2N>(s, a, stream);
-    if (act == NB_ACT_GELU)
-        return pl.bn ? launch_tile_plan<false, kEpiGelu>(s, a, pl, stream) : launch_gemm_auto<FwdGelu1, FwdGelu2>(s, a, stream);
-    return pl.bn ? launch_tile_plan<false, kEpiStore>(s, a, pl, stream) : launch_gemm_auto<FwdStore1, FwdStore2>(s, a, stream);
+    if (act == NB_ACT_NONE) return launch_gemm_auto<FwdStore1, FwdStore2>(s, a, stream);
+    if (act == NB_ACT_GELU) return launch_gemm_auto<FwdGelu1, FwdGelu2>(s, a, stream);
+    return launch_gemm_auto<FwdSwiglu1, FwdSwiglu2>(s, a, stream);
 }
 
 // A layer's backward without the small-problem kernel: layer_bwd_kernel for both products, else a
@@ -1239,21 +1262,50 @@ double backward_us(int sms, int M, int BT, int N, int Mw, int kd, int kw, bool a
 }
 
 // D = A . B with B read MN-major (dinp and its like), plain or times gelu'(E).
+Route route_dgrad(int sms, int M, int N, int kb)
+{
+    const int split = dinp_split(sms, M, N, kb);
+    const SmallPlan pl = plan_single(sms, M, N, kb, false, split, 0, split > 1 ? 1e9 : persistent_us(sms, M, N, kb));
+    return {pl.bn ? NB_ROUTE_TILE : NB_ROUTE_GEMM, pl};
+}
+
 int run_dgrad(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
 {
-    const int kb = kblocks_of(a.K) + (a.A2 ? 1 : 0);
-    const int split = dinp_split(s.num_sms, a.M, a.N, kb);
-    const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, false, split, 0, split > 1 ? 1e9 : persistent_us(s.num_sms, a.M, a.N, kb));
+    const Route r = route_dgrad(s.num_sms, a.M, a.N, kblocks_of(a.K) + (a.A2 ? 1 : 0));
     if (a.E)
-        return pl.bn ? launch_tile_plan<true, kEpiMulGeluGrad>(s, a, pl, stream)
-                     : launch_gemm_auto<DgradMulGelu1, DgradMulGelu2>(s, a, stream);
-    return pl.bn ? launch_tile_plan<true, kEpiStore>(s, a, pl, stream) : launch_gemm_auto<DgradStore1, DgradStore2>(s, a, stream);
+        return r.pl.bn ? launch_tile_plan<true, kEpiMulGeluGrad>(s, a, r.pl, stream)
+                       : launch_gemm_auto<DgradMulGelu1, DgradMulGelu2>(s, a, stream);
+    return r.pl.bn ? launch_tile_plan<true, kEpiStore>(s, a, r.pl, stream) : launch_gemm_auto<DgradStore1, DgradStore2>(s, a, stream);
+}
+
+// A layer's backward with an fp32 dweight: both products (dinp: with dinp) in tiles of one launch, both in the
+// persistent launch, or each by itself (NB_ROUTE_GEMM; dinp then by route_dgrad).
+Route route_backward(int sms, bool dinp, bool dbias, bool gelu, bool accumulate, int BT, int C, int OC)
+{
+    static const bool merge_allowed = env_int("NB_MERGED_BWD", 1) != 0;
+    const int kd = kblocks_of(OC), kw = kblocks_of(BT);
+    const int split = dinp ? dinp_split(sms, BT, C, kd) : 1;
+    const SmallPlan pl = plan_pair(sms, dinp ? BT : 0, C, kd, split, OC, C, kw, dbias,
+                                   backward_us(sms, dinp ? BT : 0, BT, C, OC, kd, kw, accumulate, split > 1, gelu), false);
+    if (pl.bn) return {NB_ROUTE_TILE_PAIR, pl};
+    return {merge_allowed && dinp && split == 1 && use_pairs(BT) ? NB_ROUTE_LAYER_BWD : NB_ROUTE_GEMM, pl};
 }
 
 // The rank-r products on 128 x 64 tiles, a CTA each (gemm_kernel's narrow forms).
 double narrow_us(int sms, int tiles, int kblocks)
 {
     return 4.3 + 0.2 * kblocks * static_cast<double>((tiles + sms - 1) / sms);
+}
+
+SmallPlan plan_lora_down(int sms, int M, int r, int kb)
+{
+    return plan_single(sms, M, r, kb, r <= 32, 0, 0, narrow_us(sms, (M + kBlockM - 1) / kBlockM, kb));
+}
+
+// u[:, r] by itself
+SmallPlan plan_lora_u(int sms, int M, int r, int kb)
+{
+    return plan_single(sms, M, r, kb, false, 0, 0, narrow_us(sms, (M + kBlockM - 1) / kBlockM, kb));
 }
 
 // t[:, r] = scale * inp . A^T. late (or null): whether the next launch may start before this one is done.
@@ -1267,9 +1319,7 @@ int run_lora_down(DeviceState &s, void *t, const void *inp, const void *lora_a, 
     a.M = static_cast<int>(BT); a.N = static_cast<int>(r); a.K = static_cast<int>(C);
     a.splits = 1;
     a.alpha = scale;
-    const int kb = kblocks_of(C);
-    const SmallPlan pl = plan_single(s.num_sms, a.M, a.N, kb, r <= 32, 0, 0,
-                                     narrow_us(s.num_sms, (a.M + kBlockM - 1) / kBlockM, kb));
+    const SmallPlan pl = plan_lora_down(s.num_sms, a.M, a.N, kblocks_of(C));
     if (late) *late = a.trigger_late = pl.bn != 0;
     return pl.bn ? launch_tile_plan<false, kEpiStore>(s, a, pl, stream) : launch_gemm<FwdStoreNarrow>(s, a, stream);
 }
@@ -1289,10 +1339,33 @@ struct LoraBwd {
 //   two tile_pair_kernel launches (u and dB, then dinp and dA), which spread a short batch over the
 //   chip: 519 rows are five panels, and five CTAs took 22 us;
 //   the first of those and the other two products by themselves.
+struct LoraRoute {
+    SmallPlan ub, xa, a1;  // u with dB (bn == 0: lora_udb_kernel); dinp with dA, or (xa.bn == 0) dA alone
+};
+LoraRoute route_lora_backward(int sms, int BT, int C, int OC, int r, bool want_x, bool want_a, bool accumulate)
+{
+    const int kt = kblocks_of(BT), ko = kblocks_of(OC);
+    const int panels = (BT + kBlockM - 1) / kBlockM;
+    const int split = dinp_split(sms, BT, C, ko + 1);
+    const double x_us = want_x ? plan_single(sms, BT, C, ko + 1, false, split, 0, persistent_us(sms, BT, C, ko + 1)).us : 0.0;
+    const double clear = accumulate ? 0.0 : 2.8;
+    const int udb_tiles = (OC + 127) / 128 + (want_a ? (C + 127) / 128 : 0);
+    const double udb = 6.0 + clear + x_us + udb_tiles * static_cast<double>((panels + sms - 1) / sms) *
+                       (0.37 + 0.25 * (panels < sms ? panels : sms) / sms);  // reading dout takes over towards one panel per SM
+    const double far = 1e9;
+    LoraRoute l;
+    l.ub = plan_pair(sms, BT, r, ko, 0, OC, r, kt, false, far, true);
+    if (want_x && want_a) l.xa = plan_pair(sms, BT, C, ko + 1, split, r, C, kt, false, far, false);
+    if (want_a) l.a1 = plan_pair(sms, 0, 0, 0, 1, r, C, kt, false, far, false);
+    const double apart = l.ub.us + x_us + l.a1.us, paired = l.xa.bn ? l.ub.us + l.xa.us : far;
+    if (!l.ub.bn || (apart >= udb && paired >= udb)) return {};
+    if (paired > apart) l.xa = {};
+    return l;
+}
+
 int run_lora_backward(DeviceState &s, const LoraBwd &l, cudaStream_t stream)
 {
     const int sms = s.num_sms, BT = static_cast<int>(l.BT), C = static_cast<int>(l.C), OC = static_cast<int>(l.OC), r = static_cast<int>(l.r);
-    const int kt = kblocks_of(BT), ko = kblocks_of(OC);
     int rc;
     GemmArgs u{};  // u = scale * dout . B   (B [OC, r] read as an MN-major operand)
     u.A = l.dout; u.a_rows = BT; u.a_cols = OC;
@@ -1322,33 +1395,21 @@ int run_lora_backward(DeviceState &s, const LoraBwd &l, cudaStream_t stream)
     dA.M = r; dA.N = C; dA.K = BT;
 
     const bool want_x = l.dinp != nullptr, want_a = l.dlora_a != nullptr;
-    const int panels = (BT + kBlockM - 1) / kBlockM;
-    const int split = dinp_split(sms, BT, C, ko + 1);
-    const double x_us = want_x ? plan_single(sms, BT, C, ko + 1, false, split, 0, persistent_us(sms, BT, C, ko + 1)).us : 0.0;
     if (l.dlora_b) {
-        const double clear = l.accumulate ? 0.0 : 2.8;
-        const int udb_tiles = (OC + 127) / 128 + (want_a ? (C + 127) / 128 : 0);
-        const double udb = 6.0 + clear + x_us + udb_tiles * static_cast<double>((panels + sms - 1) / sms) *
-                           (0.37 + 0.25 * (panels < sms ? panels : sms) / sms);  // reading dout takes over towards one panel per SM
-        const double far = 1e9;
-        const SmallPlan none;
-        const SmallPlan ub = plan_pair(sms, BT, r, ko, 0, OC, r, kt, false, far, true);
-        const SmallPlan xa = want_x && want_a ? plan_pair(sms, BT, C, ko + 1, split, r, C, kt, false, far, false) : none;
-        const SmallPlan a1 = want_a ? plan_pair(sms, 0, 0, 0, 1, r, C, kt, false, far, false) : none;
-        const double apart = ub.us + x_us + a1.us, paired = xa.bn ? ub.us + xa.us : far;
-        if (ub.bn && (apart < udb || paired < udb)) {
+        const LoraRoute w = route_lora_backward(sms, BT, C, OC, r, want_x, want_a, l.accumulate != 0);
+        if (w.ub.bn) {
             dB.trigger_late = dx.wait_ext = want_x;
-            if ((rc = launch_tile_pair_plan(s, &u, dB, false, l.accumulate, ub, stream)) != NB_OK) return rc;
-            if (paired <= apart) return launch_tile_pair_plan(s, &dx, dA, false, l.accumulate, xa, stream);
+            if ((rc = launch_tile_pair_plan(s, &u, dB, false, l.accumulate, w.ub, stream)) != NB_OK) return rc;
+            if (w.xa.bn) return launch_tile_pair_plan(s, &dx, dA, false, l.accumulate, w.xa, stream);
             if (want_x && (rc = run_dgrad(s, dx, stream)) != NB_OK) return rc;
-            return want_a ? launch_tile_pair_plan(s, nullptr, dA, false, l.accumulate, a1, stream) : NB_OK;
+            return want_a ? launch_tile_pair_plan(s, nullptr, dA, false, l.accumulate, w.a1, stream) : NB_OK;
         }
         if ((rc = launch_lora_udb(s, l.dout, l.lora_b, l.t, l.t_ld, l.dlora_b, l.u, l.u_ld ? l.u_ld : static_cast<uint64_t>(r),
                                   l.scale, BT, OC, r, l.accumulate, stream, want_a ? l.inp : nullptr, l.dlora_a, C)) != NB_OK)
             return rc;
         return want_x ? run_dgrad(s, dx, stream) : NB_OK;
     }
-    const SmallPlan up = plan_single(sms, BT, r, ko, false, 0, 0, narrow_us(sms, panels, ko));
+    const SmallPlan up = plan_lora_u(sms, BT, r, kblocks_of(OC));
     rc = up.bn ? launch_tile_plan<true, kEpiStore>(s, u, up, stream) : launch_gemm<DgradStoreNarrow>(s, u, stream);
     if (rc != NB_OK) return rc;
     if (want_x && (rc = run_dgrad(s, dx, stream)) != NB_OK) return rc;
@@ -1495,8 +1556,6 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
     d.M = static_cast<int>(BT); d.N = static_cast<int>(C); d.K = static_cast<int>(OC);
     d.splits = 1;
     if (inp_pre_act) { d.E = inp_pre_act; d.e_rows = BT; d.e_cols = C; }
-    const int kd = kblocks_of(OC), kw = kblocks_of(BT);
-    const int split = dinp ? dinp_split(s->num_sms, d.M, d.N, kd) : 1;
     if (dweight && dweight_dtype == NB_DTYPE_F32) {
         // dweight[OC, C] (+)= dz^T[OC, BT] . inp[BT, C]
         w.A = dz; w.a_rows = BT; w.a_cols = OC;
@@ -1505,18 +1564,17 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
         w.M = static_cast<int>(OC); w.N = static_cast<int>(C); w.K = static_cast<int>(BT);
         w.splits = 1;
         w.dbias = static_cast<float *>(dbias);
-        const SmallPlan pl = plan_pair(s->num_sms, dinp ? d.M : 0, d.N, kd, split, w.M, w.N, kw, dbias != nullptr,
-                                       backward_us(s->num_sms, dinp ? d.M : 0, d.M, d.N, w.M, kd, kw, accumulate != 0, split > 1, inp_pre_act != nullptr), false);
-        if (pl.bn) return launch_tile_pair_plan(*s, dinp ? &d : nullptr, w, inp_pre_act != nullptr, accumulate, pl, stream);
-    }
-
-    // Both products of the layer in one launch (the usual case of a training step): the weight
-    // gradient's k-blocks fill the waves the input gradient's tiles leave partly empty.
-    static const bool merge_allowed = env_int("NB_MERGED_BWD", 1) != 0;
-    if (merge_allowed && dinp && dweight && dweight_dtype == NB_DTYPE_F32 && split == 1 && use_pairs(static_cast<int>(BT))) {
-        rc = run_layer_bwd(*s, dz, weight, inp, dinp, inp_pre_act, dweight, static_cast<float *>(dbias), BT, C,
-                           OC, accumulate, stream);
-        if (rc != NB_ERR_UNSUPPORTED) return rc;
+        const Route r = route_backward(s->num_sms, dinp != nullptr, dbias != nullptr, inp_pre_act != nullptr, accumulate != 0,
+                                       d.M, d.N, w.M);
+        if (r.kernel == NB_ROUTE_TILE_PAIR)
+            return launch_tile_pair_plan(*s, dinp ? &d : nullptr, w, inp_pre_act != nullptr, accumulate, r.pl, stream);
+        // Both products of the layer in one launch (the usual case of a training step): the weight
+        // gradient's k-blocks fill the waves the input gradient's tiles leave partly empty.
+        if (r.kernel == NB_ROUTE_LAYER_BWD) {
+            rc = run_layer_bwd(*s, dz, weight, inp, dinp, inp_pre_act, dweight, static_cast<float *>(dbias), BT, C,
+                               OC, accumulate, stream);
+            if (rc != NB_ERR_UNSUPPORTED) return rc;
+        }
     }
 
     if (dinp && (rc = run_dgrad(*s, d, stream)) != NB_OK) return rc;
@@ -1915,6 +1973,68 @@ int nb_debug_layer_bwd_plan(int64_t BT, int64_t C, int64_t OC, int pairs, int fl
         }
     }
     return records;
+}
+
+int nb_debug_route(int call, int64_t BT, int64_t C, int64_t OC, int64_t r, int act, int flags, int sms, int *out)
+{
+    if (!out || BT <= 0 || C <= 0 || OC <= 0 || sms < 2 || BT >= (1ll << 31) || C >= (1ll << 31) || OC >= (1ll << 31))
+        return -fail(NB_ERR_INVALID_ARG, "bad argument");
+    const int M = static_cast<int>(BT), K = static_cast<int>(C), N = static_cast<int>(OC), R = static_cast<int>(r);
+    const bool adapter = call == NB_CALL_LORA_FORWARD || call == NB_CALL_LORA_BACKWARD;
+    if (adapter && (r < 8 || r > 64 || r % 8 != 0)) return -fail(NB_ERR_UNSUPPORTED, "rank must be 8..64, a multiple of 8");
+    const bool dinp = flags & NB_CALL_DINP, dweight = flags & NB_CALL_DWEIGHT, dbias = flags & NB_CALL_DBIAS;
+    const bool gelu = flags & NB_CALL_GELU_GRAD, accumulate = flags & NB_CALL_ACCUMULATE;
+    int n = 0;
+    auto put = [&](int kernel, int width, int shared, int per_sm) {
+        out[4 * n] = kernel; out[4 * n + 1] = width; out[4 * n + 2] = shared; out[4 * n + 3] = per_sm;
+        ++n;
+    };
+    auto tiles = [&](int kernel, const SmallPlan &pl) { put(kernel, pl.bn, pl.cluster, pl.two ? 2 : 1); };
+    auto product = [&](const Route &t) {
+        if (t.kernel == NB_ROUTE_TILE) tiles(t.kernel, t.pl);
+        else put(t.kernel, t.kernel == NB_ROUTE_GEMM_192 ? 192 : 256, 1, 1);
+    };
+    auto narrow = [&](const SmallPlan &pl) {
+        if (pl.bn) tiles(NB_ROUTE_TILE, pl);
+        else put(NB_ROUTE_GEMM, kNarrowN, 1, 1);
+    };
+    if (call == NB_CALL_FORWARD || call == NB_CALL_LORA_FORWARD) {
+        if (adapter) narrow(plan_lora_down(sms, M, R, kblocks_of(K)));
+        const Route t = route_forward(sms, M, N, K, adapter ? NB_ACT_NONE : act, adapter);
+        const int span = act == NB_ACT_SWIGLU ? N / 2 : N;
+        if (t.kernel == NB_ROUTE_ROWS)
+            put(t.kernel, kRowsFeatures, rows_split(sms, (span + kRowsFeatures - 1) / kRowsFeatures, K),
+                rows_many(sms, M, span, act == NB_ACT_SWIGLU) ? 4 : 2);
+        else product(t);
+    } else if (call == NB_CALL_BACKWARD) {
+        const Route t = dweight ? route_backward(sms, dinp, dbias, gelu, accumulate, M, K, N) : Route{};
+        if (t.kernel == NB_ROUTE_TILE_PAIR) {
+            tiles(t.kernel, t.pl);
+        } else if (t.kernel == NB_ROUTE_LAYER_BWD) {
+            LayerBwdParams p;
+            const int rc = plan_layer_bwd(p, BT, C, OC, sms / 2 < kMaxPairs ? sms / 2 : kMaxPairs, gelu, true);
+            if (rc != NB_OK) return -rc;
+            put(t.kernel, p.d_w, 1, 1);
+        } else {
+            if (dinp) product(route_dgrad(sms, M, K, kblocks_of(N)));
+            if (dweight) put(NB_ROUTE_GEMM, 256, 1, 1);
+        }
+    } else if (call == NB_CALL_LORA_BACKWARD) {
+        const LoraRoute t = dbias ? route_lora_backward(sms, M, K, N, R, dinp, dweight, accumulate) : LoraRoute{};
+        if (t.ub.bn) tiles(NB_ROUTE_TILE_PAIR, t.ub);
+        else if (dbias) put(NB_ROUTE_LORA_UDB, kNarrowN, 1, 1);
+        else narrow(plan_lora_u(sms, M, R, kblocks_of(N)));
+        if (t.xa.bn) {
+            tiles(NB_ROUTE_TILE_PAIR, t.xa);
+        } else {
+            if (dinp) product(route_dgrad(sms, M, K, kblocks_of(N) + 1));
+            if (dweight && t.ub.bn) tiles(NB_ROUTE_TILE_PAIR, t.a1);
+            else if (dweight && !dbias) put(NB_ROUTE_GEMM, 256, 1, 1);
+        }
+    } else {
+        return -fail(NB_ERR_INVALID_ARG, "unknown call %d", call);
+    }
+    return n;
 }
 
 int nb_debug_gemm_timeout(void *out, const void *inp, const void *weight, int64_t limit_us)

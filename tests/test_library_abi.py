@@ -215,3 +215,33 @@ def test_layer_backward_plan_with_halved_dinp_tiles(L):
         halved += narrow
     assert halved >= 20
     assert all(t in cases for t in ((1500, 760, 3080, 74), (1030, 760, 6152, 74)))  # also on the GPU: test_gpu_small_problems
+
+
+def test_route_view(L):
+    """The view of the kernels that calls take: what it refuses, and the promise on dinp: the number of CTAs that
+    share its K, which fixes the order of its sums, does not depend on what else the call is asked for."""
+    import numpy as np
+    assert L.nb_debug_route(9, 8, 8, 8, 0, 0, 7, 148, (binding.ctypes.c_int * 12)()) == -binding.NB_ERR_INVALID_ARG
+    assert L.nb_debug_route(0, 0, 8, 8, 0, 0, 7, 148, (binding.ctypes.c_int * 12)()) == -binding.NB_ERR_INVALID_ARG
+    with pytest.raises(binding.NbError):
+        binding.nb_debug_route(binding.CALL_LORA_FORWARD, 8, 8, 8, r=12)
+    assert binding.nb_debug_route(binding.CALL_FORWARD, 8, 768, 3072) == [("rows", 16, 1, 2)]
+    assert binding.nb_debug_route(binding.CALL_FORWARD, 16384, 768, 3072) == [("gemm", 256, 1, 1)]
+    assert binding.nb_debug_route(binding.CALL_BACKWARD, 16384, 768, 3072) == [("layer_bwd", 256, 1, 1)]
+    assert [k[0] for k in binding.nb_debug_route(binding.CALL_LORA_BACKWARD, 16384, 1024, 2048, r=16)] == ["lora_udb", "gemm"]
+    rng = np.random.default_rng(3)
+    shared = 0
+    for _ in range(1500):
+        BT = int(2 ** rng.uniform(0, 11.2))
+        C, OC = (8 * int(2 ** rng.uniform(0, 9)) for _ in range(2))
+        (alone,) = binding.nb_debug_route(binding.CALL_BACKWARD, BT, C, OC, dweight=False, dbias=False)
+        shared += alone[2] > 1
+        assert alone[0] in ("tile", "gemm") and alone[2] in (1, 2, 4)
+        for gelu in (False, True):
+            for dbias in (False, True):
+                for accumulate in (False, True):
+                    route = binding.nb_debug_route(binding.CALL_BACKWARD, BT, C, OC, dbias=dbias, gelu_grad=gelu,
+                                                   accumulate=accumulate)
+                    assert route[0][0] in ("tile_pair", "layer_bwd", "tile", "gemm")
+                    assert route[0][2] == alone[2], (BT, C, OC, route, alone)
+    assert shared > 200
