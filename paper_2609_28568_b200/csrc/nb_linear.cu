@@ -422,12 +422,48 @@ void small_launch_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attrs)[2
 constexpr uint32_t kTileSmemTwo = 113u * 1024u;  // two CTAs on an SM
 constexpr uint32_t kTileSmemOne = 220u * 1024u;
 
+// The ring of a job in BN-wide tiles: bytes of an A tile, stages, the CTA's shared memory. `longest`: the most
+// k-blocks a CTA works through. two: sized for two CTAs on an SM, where that leaves two stages
+// (pair_fits_twice asks whether it does).
+struct TileRing {
+    uint32_t a_slot;
+    int stages;
+    uint32_t bytes;
+};
+template <int BN>
+TileRing tile_ring(int M, int epi, bool a_mn, int cluster, int longest, bool two)
+{
+    using G = TileGeom<BN>;
+    TileRing r;
+    // a K-major A tile is one box; a single row tile of fewer than 128 rows is fetched (and kept) as
+    // just those rows
+    r.a_slot = (!a_mn && M < kBlockM ? static_cast<uint32_t>((M + 7) / 8 * 8) : kBlockM) * 128u;
+    const uint32_t recv = cluster > 1 ? G::RECV_BYTES : 0u;
+    const uint32_t stage = r.a_slot + G::B_BYTES;
+    auto fit = [&](uint32_t budget) { return static_cast<int>((budget - recv - G::TAIL_BYTES) / stage); };
+    int st = fit(two ? kTileSmemTwo : kTileSmemOne);
+    if (st < 2) st = fit(kTileSmemOne);
+    if (st > kTileMaxStages) st = kTileMaxStages;
+    if (st > longest) st = longest;
+    // the result is staged in the drained stages' memory: 4 bytes an element (fp32, or bf16 result and
+    // pre-activation) or 2, for the 32-row quarters that hold rows; SwiGLU: three planes of half a tile
+    const uint32_t quarters = M < kBlockM ? static_cast<uint32_t>((M + 31) / 32) : 4u;
+    const uint32_t elem = epi == kEpiF32 || epi == kEpiGelu ? 4u : epi == kEpiSwiglu ? 3u : 2u;
+    const uint32_t staged = (epi == kEpiF32 ? 4u : quarters) * 32u * BN * elem;
+    const int min_st = cluster > 1 ? 1 : static_cast<int>((staged + stage - 1) / stage);
+    if (st < min_st) st = min_st;
+    r.stages = st;
+    r.bytes = static_cast<uint32_t>(st) * stage + recv + G::TAIL_BYTES;
+    // the tensor core reads 128 rows from every A slot
+    const uint32_t reach = static_cast<uint32_t>(st - 1) * r.a_slot + kBlockM * 128u;
+    if (r.bytes < reach) r.bytes = reach;
+    return r;
+}
+
 // Fills a job (and the shared memory it needs) for D[M, N] in BN-wide tiles, K split over `cluster`.
-// two: the ring leaves room for a second CTA on the SM.
 template <int BN>
 void fill_tile_job(TileJob &j, uint32_t &smem_bytes, const GemmArgs &a, int epi, bool a_mn, int cluster, bool two)
 {
-    using G = TileGeom<BN>;
     memset(&j, 0, sizeof(j));
     const bool swiglu = epi == kEpiSwiglu;
     j.M = a.M;
@@ -437,10 +473,6 @@ void fill_tile_job(TileJob &j, uint32_t &smem_bytes, const GemmArgs &a, int epi,
     j.tiles_n = (n + span - 1) / span;
     j.kblocks = (a.K + kBlockK - 1) / kBlockK;
     j.kblocks_ext = (a.A2 && a.B2 && a.k2 > 0) ? (a.k2 + kBlockK - 1) / kBlockK : 0;
-    // a K-major A tile is one box; a single row tile of fewer than 128 rows is fetched (and kept) as
-    // just those rows
-    const uint32_t rows = !a_mn && a.M < kBlockM ? static_cast<uint32_t>((a.M + 7) / 8 * 8) : kBlockM;
-    j.a_slot = rows * 128u;
     j.ctas = j.tiles_m * j.tiles_n * cluster;
     j.alpha = a.alpha;
     j.bias = static_cast<const __nv_bfloat16 *>(a.bias);
@@ -451,30 +483,14 @@ void fill_tile_job(TileJob &j, uint32_t &smem_bytes, const GemmArgs &a, int epi,
     j.swiglu_h = a.swiglu_h;
     j.reduce = a.reduce;
     j.wait_ext = a.wait_ext && j.kblocks_ext > 0;
-    const uint32_t recv = cluster > 1 ? G::RECV_BYTES : 0u;
-    const uint32_t stage = j.a_slot + G::B_BYTES;
-    const int longest = (j.kblocks + cluster - 1) / cluster + j.kblocks_ext;
-    auto fit = [&](uint32_t budget) { return static_cast<int>((budget - recv - G::TAIL_BYTES) / stage); };
-    int st = fit(two ? kTileSmemTwo : kTileSmemOne);
-    if (st < 2) st = fit(kTileSmemOne);
-    if (st > kTileMaxStages) st = kTileMaxStages;
-    if (st > longest) st = longest;
-    // the result is staged in the drained stages' memory: 4 bytes an element (fp32, or bf16 result and
-    // pre-activation) or 2, for the 32-row quarters that hold rows; SwiGLU: three planes of half a tile
-    const uint32_t quarters = a.M < kBlockM ? static_cast<uint32_t>((a.M + 31) / 32) : 4u;
-    const uint32_t elem = epi == kEpiF32 || epi == kEpiGelu ? 4u : swiglu ? 3u : 2u;
-    const uint32_t staged = (epi == kEpiF32 ? 4u : quarters) * 32u * BN * elem;
-    const int min_st = cluster > 1 ? 1 : static_cast<int>((staged + stage - 1) / stage);
-    if (st < min_st) st = min_st;
-    j.stages = st;
-    smem_bytes = static_cast<uint32_t>(st) * stage + recv + G::TAIL_BYTES;
-    // the tensor core reads 128 rows from every A slot
-    const uint32_t reach = static_cast<uint32_t>(st - 1) * j.a_slot + kBlockM * 128u;
-    if (smem_bytes < reach) smem_bytes = reach;
+    const TileRing r = tile_ring<BN>(a.M, epi, a_mn, cluster, (j.kblocks + cluster - 1) / cluster + j.kblocks_ext, two);
+    j.a_slot = r.a_slot;
+    j.stages = r.stages;
+    smem_bytes = r.bytes;
 }
 
 template <int BN, bool B_MN, int EPI>
-int launch_tile(DeviceState &s, const GemmArgs &a, int cluster, bool two, cudaStream_t stream)
+int launch_tile(DeviceState &s, const GemmArgs &a, int cluster, cudaStream_t stream)
 {
     static bool attr_set[kMaxDevices] = {};
     int dev = 0;
@@ -487,7 +503,7 @@ int launch_tile(DeviceState &s, const GemmArgs &a, int cluster, bool two, cudaSt
     TileParams p;
     memset(&p, 0, sizeof(p));
     uint32_t smem_bytes = 0;
-    fill_tile_job<BN>(p.job[0], smem_bytes, a, EPI, false, cluster, two);
+    fill_tile_job<BN>(p.job[0], smem_bytes, a, EPI, false, cluster, false);
     p.cluster = cluster;
     p.trigger_late = a.trigger_late;
     p.status = s.status;
@@ -625,7 +641,7 @@ int launch_rows_auto(DeviceState &s, const GemmArgs &a, cudaStream_t stream)
 // costs the MMA issuer about 300 cycles whatever BN is, and more when many SMs load at once.
 struct SmallPlan {
     int bn = 0, cluster = 1;  // bn == 0: the persistent kernels
-    bool two = false;         // ring sized for two CTAs on an SM
+    bool two = false;         // tile_pair_kernel: ring sized for two CTAs on an SM
     double us = 0;
 };
 constexpr double kLaunchUs = 1.0;
@@ -677,9 +693,20 @@ SmallPlan plan_single(int sms, int M, int N, int kblocks, bool allow32, int spli
     return best;
 }
 
+// Whether two CTAs of tile_pair_kernel fit an SM: by the shared memory of both jobs' rings (with K split,
+// 128-wide tiles of more than 56 rows do not: the slices received take 66 KB), and by registers (gelu' in 128-wide
+// tiles takes 156 a thread; 102 are what two CTAs leave).
+template <int BN>
+bool pair_fits_twice(int M, int longest, int cluster, int Mw, int kw, bool gelu)
+{
+    if (BN == 128 && gelu) return false;
+    return tile_ring<BN>(Mw, kEpiF32, true, 1, kw, true).bytes <= kTileSmemTwo &&
+           (M == 0 || tile_ring<BN>(M, gelu ? kEpiMulGeluGrad : kEpiStore, false, cluster, longest, true).bytes <= kTileSmemTwo);
+}
+
 // The same for a bf16 product D[M, N] (M == 0: none) and an fp32 product [Mw, Nw] over kw k-blocks in
-// one launch; `other` is what the alternative takes, `split` as above.
-SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int Nw, int kw, bool dbias, double other, bool only64)
+// one launch; `other` is what the alternative takes, `split` as above; gelu: the bf16 product times gelu'.
+SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int Nw, int kw, bool dbias, bool gelu, double other, bool only64)
 {
     SmallPlan best;
     best.us = other;
@@ -690,12 +717,14 @@ SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int N
         for (int cl = nd && split ? split : 1; cl <= (!nd ? 1 : split ? split : 8); cl *= 2) {
             if (bn / cl < 8 || (cl > 1 && 2 * cl > kblocks)) break;
             for (int two = 0; two <= 1; ++two) {
+                const int longest = (kblocks + cl - 1) / cl;
+                if (two && !(bn == 64 ? pair_fits_twice<64>(M, longest, cl, Mw, kw, gelu) : pair_fits_twice<128>(M, longest, cl, Mw, kw, gelu))) continue;
                 const double slots = sms * (two ? 2.0 : 1.0);
                 const double n = static_cast<double>(nd * cl + nw);
                 // job 0's clusters come first and have to find their places; job 1's tiles fill up behind them
                 if (cl >= 8 ? n > 0.86 * slots : cl > 1 && nd * cl > 0.95 * slots) continue;
                 const int crowd = static_cast<int>(n < slots ? n : slots);
-                const double td = nd ? small_cta_us(bn, (kblocks + cl - 1) / cl, M, crowd, two != 0) +
+                const double td = nd ? small_cta_us(bn, longest, M, crowd, two != 0) +
                                            (cl > 1 ? small_exchange_us(bn, M, static_cast<int>(nd * cl)) : 0.0) : 0.0;
                 // the bias gradient's warps own a stage each: the fewer stages, the longer they hold them
                 const double tw = small_cta_us(bn, kw, Mw, crowd, two != 0) + (dbias ? kw * (two ? 0.18 : bn == 128 ? 0.115 : 0.05) : 0.0);
@@ -738,10 +767,10 @@ template <bool B_MN, int EPI>
 int launch_tile_plan(DeviceState &s, const GemmArgs &a, const SmallPlan &pl, cudaStream_t stream)
 {
     if constexpr (!B_MN)
-        if (pl.bn == 32) return launch_tile<32, B_MN, EPI>(s, a, pl.cluster, pl.two, stream);
-    if (pl.bn == 64) return launch_tile<64, B_MN, EPI>(s, a, pl.cluster, pl.two, stream);
-    if (pl.bn == 192) return launch_tile<192, B_MN, EPI>(s, a, 1, false, stream);
-    return launch_tile<128, B_MN, EPI>(s, a, pl.cluster, pl.two, stream);
+        if (pl.bn == 32) return launch_tile<32, B_MN, EPI>(s, a, pl.cluster, stream);
+    if (pl.bn == 64) return launch_tile<64, B_MN, EPI>(s, a, pl.cluster, stream);
+    if (pl.bn == 192) return launch_tile<192, B_MN, EPI>(s, a, 1, stream);
+    return launch_tile<128, B_MN, EPI>(s, a, pl.cluster, stream);
 }
 
 int launch_tile_pair_plan(DeviceState &s, const GemmArgs *d, const GemmArgs &w, bool gelu_grad, int accumulate,
@@ -1229,7 +1258,7 @@ int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
         return launch_rows_auto<kEpiSwiglu>(s, a, stream);
     }
     if (r.kernel == NB_ROUTE_TILE) {
-        if (act == NB_ACT_SWIGLU) return launch_tile<128, false, kEpiSwiglu>(s, a, 1, false, stream);
+        if (act == NB_ACT_SWIGLU) return launch_tile<128, false, kEpiSwiglu>(s, a, 1, stream);
         return act == NB_ACT_GELU ? launch_tile_plan<false, kEpiGelu>(s, a, r.pl, stream)
                                   : launch_tile_plan<false, kEpiStore>(s, a, r.pl, stream);
     }
@@ -1285,7 +1314,7 @@ Route route_backward(int sms, bool dinp, bool dbias, bool gelu, bool accumulate,
     static const bool merge_allowed = env_int("NB_MERGED_BWD", 1) != 0;
     const int kd = kblocks_of(OC), kw = kblocks_of(BT);
     const int split = dinp ? dinp_split(sms, BT, C, kd) : 1;
-    const SmallPlan pl = plan_pair(sms, dinp ? BT : 0, C, kd, split, OC, C, kw, dbias,
+    const SmallPlan pl = plan_pair(sms, dinp ? BT : 0, C, kd, split, OC, C, kw, dbias, gelu,
                                    backward_us(sms, dinp ? BT : 0, BT, C, OC, kd, kw, accumulate, split > 1, gelu), false);
     if (pl.bn) return {NB_ROUTE_TILE_PAIR, pl};
     return {merge_allowed && dinp && split == 1 && use_pairs(BT) ? NB_ROUTE_LAYER_BWD : NB_ROUTE_GEMM, pl};
@@ -1354,9 +1383,9 @@ LoraRoute route_lora_backward(int sms, int BT, int C, int OC, int r, bool want_x
                        (0.37 + 0.25 * (panels < sms ? panels : sms) / sms);  // reading dout takes over towards one panel per SM
     const double far = 1e9;
     LoraRoute l;
-    l.ub = plan_pair(sms, BT, r, ko, 0, OC, r, kt, false, far, true);
-    if (want_x && want_a) l.xa = plan_pair(sms, BT, C, ko + 1, split, r, C, kt, false, far, false);
-    if (want_a) l.a1 = plan_pair(sms, 0, 0, 0, 1, r, C, kt, false, far, false);
+    l.ub = plan_pair(sms, BT, r, ko, 0, OC, r, kt, false, false, far, true);
+    if (want_x && want_a) l.xa = plan_pair(sms, BT, C, ko + 1, split, r, C, kt, false, false, far, false);
+    if (want_a) l.a1 = plan_pair(sms, 0, 0, 0, 1, r, C, kt, false, false, far, false);
     const double apart = l.ub.us + x_us + l.a1.us, paired = l.xa.bn ? l.ub.us + l.xa.us : far;
     if (!l.ub.bn || (apart >= udb && paired >= udb)) return {};
     if (paired > apart) l.xa = {};
@@ -1864,7 +1893,7 @@ int nb_lora_da_stacked(void *da_stack, const void *u_stack, const void *inp, int
     w.D = da_stack; w.d_rows = R; w.d_cols = C; w.d_dtype = 1;
     w.M = static_cast<int>(R); w.N = static_cast<int>(C); w.K = static_cast<int>(BT);
     const int kw = kblocks_of(BT);
-    const SmallPlan pl = plan_pair(s->num_sms, 0, 0, 0, 1, w.M, w.N, kw, false,
+    const SmallPlan pl = plan_pair(s->num_sms, 0, 0, 0, 1, w.M, w.N, kw, false, false,
                                    backward_us(s->num_sms, 0, w.K, w.N, w.M, 0, kw, accumulate != 0, true, false), false);
     if (pl.bn) return launch_tile_pair_plan(*s, nullptr, w, false, accumulate, pl, stream);
     return run_wgrad_f32(*s, u_stack, inp, da_stack, nullptr, BT, R, C, accumulate, stream);

@@ -656,7 +656,7 @@ tile_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 //   an adapter's backward    u = scale dy . B                   dB (+)= dy^T . t
 //                            dinp = dy . W + u . A              dA (+)= u^T . inp
 template <int BN, bool GELU_GRAD>
-__global__ void __launch_bounds__(kTileThreads, BN == 128 ? 1 : 2)
+__global__ void __launch_bounds__(kTileThreads, BN == 128 && GELU_GRAD ? 1 : 2)  // two where the planner may count on two
 tile_pair_kernel(const __grid_constant__ CUtensorMap tmA0,  // boxes of up to 128 rows
                  const __grid_constant__ CUtensorMap tmB0,  // 64 x 64 boxes, as all that follow
                  const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,

@@ -245,3 +245,35 @@ def test_route_view(L):
                     assert route[0][0] in ("tile_pair", "layer_bwd", "tile", "gemm")
                     assert route[0][2] == alone[2], (BT, C, OC, route, alone)
     assert shared > 200
+
+
+def test_backward_forms_that_count_on_two_ctas_fit_them(L):
+    """Where the tile kernel of a backward is planned with two CTAs on an SM, two have to fit: 228 KB of shared
+    memory of which each CTA reserves one, counted here from the tiles alone (A of 128 rows of 64 bf16, or only the rows
+    there are; B of 64 x width; at least two stages where a CTA has more than one k-block; with K shared, one row more than a tile of fp32
+    slices received; results staged in the stages), and registers: the form with gelu' in 128-wide tiles has too many."""
+    import numpy as np
+    rng = np.random.default_rng(4)
+
+    def kb(rows, mn_major, width, kblocks, shared, staged):
+        a = 128 if mn_major or rows >= 128 else -(-rows // 8) * 8
+        stages = max(min(2, kblocks), 1 if shared > 1 else -(-staged // (128 * (a + width))))
+        return (stages * 128 * (a + width) + (129 * width * 4 if shared > 1 else 0)) / 1024
+
+    two = 0
+    for _ in range(6000):
+        BT = int(2 ** rng.uniform(0, 10.5))
+        C, OC = (8 * int(2 ** rng.uniform(3, 10)) for _ in range(2))
+        gelu = bool(rng.integers(0, 2))
+        for kernel, width, shared, per_sm in binding.nb_debug_route(binding.CALL_BACKWARD, BT, C, OC, gelu_grad=gelu):
+            if kernel != "tile_pair" or per_sm != 2:
+                continue
+            two += 1
+            tag = (BT, C, OC, gelu, width, shared)
+            assert not (width == 128 and gelu), tag
+            longest = -(-(-(-OC // 64)) // shared)
+            quarters = -(-min(BT, 128) // 32)
+            dinp = kb(BT, False, width, longest, shared, quarters * 32 * width * 2)
+            dweight = kb(OC, True, width, -(-BT // 64), 1, 128 * width * 4)
+            assert max(dinp, dweight) + 1 <= 114, tag
+    assert two > 500
