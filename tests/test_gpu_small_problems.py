@@ -1,7 +1,8 @@
 """The kernels for small problems at the sizes where they change form: the row kernel (1 to 16 rows, K
 shared by a cluster or not, several CTAs of features per SM), the tile kernel (every tile width, one
 row past a tile, K split over 2, 4 and 8 CTAs, ragged K and columns), both products of a backward in
-one launch, the adapter's two launches. Every element against the oracle, canaries around every buffer; the bounds are those of
+one launch, the adapter's two launches. The tests whose name ends in `forms` state the form that each case is
+there for and check it by the host's view of the route. Every element against the oracle, canaries around every buffer; the bounds are those of
 the other parity tests (one rounding to bf16, fp32 sums)."""
 import math
 
@@ -25,7 +26,7 @@ def gen(seed, shape, std):
 @pytest.mark.parametrize("act", [nb.ACT_NONE, nb.ACT_GELU, nb.ACT_SWIGLU])
 @pytest.mark.parametrize("BT,C,OC", [
     (1, 8, 16), (8, 3080, 208), (9, 1032, 80), (16, 4096, 48),   # rows: K in one CTA / shared by 2, 4 and 8
-    (3, 72, 7200), (16, 40, 7200),                                # rows: several CTAs of features per SM
+    (3, 72, 7200), (16, 40, 7200),                                # rows: several CTAs of features per SM (not SwiGLU)
     (17, 264, 144), (64, 1544, 80), (128, 3072, 96),              # tiles: fewer rows than a tile, K split
     (129, 776, 400), (300, 2056, 272), (1000, 328, 1424),         # tiles: one row past, several row tiles
     (1030, 72, 2608),                                             # tiles of 192 columns
@@ -47,11 +48,11 @@ def test_small_forward(BT, C, OC, act):
 
 @pytest.mark.parametrize("fused", [False, True])
 @pytest.mark.parametrize("BT,C,OC", [
-    (1, 8, 16), (8, 136, 3072), (64, 776, 200), (128, 264, 2056),   # dinp's K split over 2 and 4
+    (1, 8, 16), (8, 136, 3072), (64, 776, 200), (128, 264, 2056),   # dinp's K split over 4, or not
     (129, 72, 136), (256, 520, 1544), (257, 520, 1544),              # the last split, the first without
     (384, 768, 776), (1000, 264, 328),                               # more k-blocks than stages for dweight
     (1030, 2608, 72),                                                # dinp alone in tiles of 192 columns
-    (1500, 776, 3080), (1030, 1000, 6152),                           # the persistent launch, dinp in halved tiles
+    (1500, 776, 3080), (1030, 1000, 6152),                           # the persistent launch, or (second, from zero) tiles
 ])
 def test_small_backward(BT, C, OC, fused):
     inp, w, dout = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (BT, OC), 1e-3)
@@ -222,3 +223,93 @@ def test_chained_head_over_two_alternating_buffers(BT):
         assert torch.isfinite(a).all() and a.any()
         assert torch.equal(a, b)
     nb.nb_check_status()
+
+
+def _seen(route, form):
+    assert route == [form], (route, form)
+
+
+@pytest.mark.parametrize("act", [nb.ACT_NONE, nb.ACT_GELU])
+@pytest.mark.parametrize("BT,C,OC,form", [
+    (2, 1048, 24, ("rows", 16, 2, 2)), (7, 2248, 40, ("rows", 16, 4, 2)), (13, 4152, 24, ("rows", 16, 8, 2)),
+    (9, 136, 7208, ("rows", 16, 1, 4)),
+    (60, 840, 1616, ("tile", 32, 2, 1)), (139, 1208, 560, ("tile", 32, 2, 1)), (129, 672, 48, ("tile", 32, 4, 1)),
+    (144, 40, 2448, ("tile", 64, 1, 1)), (35, 856, 2512, ("tile", 64, 2, 1)), (130, 1440, 560, ("tile", 64, 4, 1)),
+    (134, 2896, 48, ("tile", 64, 8, 1)), (139, 40, 5520, ("tile", 128, 1, 1)), (26, 1112, 5008, ("tile", 128, 2, 1)),
+    (135, 3272, 1200, ("tile", 128, 4, 1)), (25, 1296, 1136, ("tile", 128, 8, 1)), (296, 40, 6320, ("tile", 192, 1, 1)),
+    (552, 40, 6384, ("gemm", 192, 1, 1)), (419, 40, 7200, ("gemm", 256, 1, 1)),
+])
+def test_forward_forms(BT, C, OC, form, act):
+    _seen(nb.nb_debug_route(nb.CALL_FORWARD, BT, C, OC, act=act), form)
+    test_small_forward(BT, C, OC, act)
+
+
+@pytest.mark.parametrize("BT,C,OC,form", [
+    (5, 136, 14256, ("rows", 16, 1, 4)), (11, 136, 14256, ("rows", 16, 1, 2)), (3, 1048, 48, ("rows", 16, 2, 2)),
+    (16, 4152, 32, ("rows", 16, 8, 2)), (17, 264, 144, ("tile", 128, 1, 1)), (300, 40, 6480, ("gemm", 256, 1, 1)),
+])
+def test_forward_swiglu_forms(BT, C, OC, form):
+    _seen(nb.nb_debug_route(nb.CALL_FORWARD, BT, C, OC, act=nb.ACT_SWIGLU), form)
+    test_small_forward(BT, C, OC, nb.ACT_SWIGLU)
+
+
+@pytest.mark.parametrize("BT,C,OC,fused,form", [
+    (139, 3312, 96, False, ("tile_pair", 64, 1, 2)), (139, 3312, 96, True, ("tile_pair", 64, 1, 2)),
+    (9, 2024, 2448, False, ("tile_pair", 64, 2, 2)), (142, 1272, 1712, True, ("tile_pair", 64, 2, 2)),
+    (205, 536, 8080, False, ("tile_pair", 64, 2, 1)), (205, 536, 8080, True, ("tile_pair", 64, 2, 1)),
+    (135, 40, 1008, True, ("tile_pair", 64, 4, 1)),
+    (131, 552, 1040, False, ("tile_pair", 64, 4, 2)), (131, 552, 1040, True, ("tile_pair", 64, 4, 2)),
+    (130, 3184, 48, False, ("tile_pair", 128, 1, 1)), (130, 3184, 48, True, ("tile_pair", 128, 1, 1)),
+    (133, 3808, 288, False, ("tile_pair", 128, 1, 2)),
+    (134, 800, 5552, False, ("tile_pair", 128, 2, 1)), (134, 800, 5552, True, ("tile_pair", 128, 2, 1)),
+    (36, 2616, 880, False, ("tile_pair", 128, 2, 2)),
+    (9, 72, 4640, False, ("tile_pair", 128, 4, 1)), (9, 72, 4640, True, ("tile_pair", 128, 4, 1)),
+    (9, 2104, 560, False, ("tile_pair", 128, 4, 2)),
+    # the persistent launch: ragged edges, and dinp in halved tiles
+    (1990, 8, 16, False, ("layer_bwd", 256, 1, 1)), (1990, 8, 16, True, ("layer_bwd", 256, 1, 1)),
+    (1424, 808, 48, False, ("layer_bwd", 256, 1, 1)), (1424, 808, 48, True, ("layer_bwd", 256, 1, 1)),
+    (2300, 72, 136, False, ("layer_bwd", 256, 1, 1)), (2300, 72, 136, True, ("layer_bwd", 256, 1, 1)),
+    (1375, 648, 3088, False, ("layer_bwd", 128, 1, 1)),
+])
+def test_backward_forms(BT, C, OC, fused, form):
+    """With a bias gradient, from zero and accumulating: both take the form."""
+    for accumulate in (False, True):
+        _seen(nb.nb_debug_route(nb.CALL_BACKWARD, BT, C, OC, gelu_grad=fused, accumulate=accumulate), form)
+    test_small_backward(BT, C, OC, fused)
+
+
+@pytest.mark.parametrize("accumulate", [0, 1])
+@pytest.mark.parametrize("BT,C,OC,bias", [(1500, 760, 3080, False), (1500, 760, 3080, True), (1030, 760, 6152, True)])
+def test_backward_with_halved_dinp_tiles_forms(BT, C, OC, bias, accumulate):
+    """Ragged columns in the last halved tile, ragged rows, ragged K, every element."""
+    _seen(nb.nb_debug_route(nb.CALL_BACKWARD, BT, C, OC, dbias=bias, accumulate=bool(accumulate)), ("layer_bwd", 128, 1, 1))
+    inp, w, dout = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (BT, OC), 1e-3)
+    r = oracle.linear_backward(f32(dout), f32(inp), f32(w))
+    dinp = Guarded((BT, C), torch.bfloat16)
+    dw = Guarded((OC, C), torch.float32, fill=0.5)
+    db = Guarded((OC,), torch.float32, fill=-0.25) if bias else None
+    nb.nb_linear_backward_ex(dinp.t, dw.t, db.t if bias else None, dout, inp, w, None, None, BT, C, OC, nb.ACT_NONE, accumulate)
+    check_bf16(dinp.t, r["dinp"], "dinp")
+    check_f32(dw.t - 0.5 * accumulate, r["dweight"], "dweight")
+    if bias:
+        check_f32(db.t + 0.25 * accumulate, r["dbias"], "dbias")
+    for g, n in ((dinp, "dinp"), (dw, "dweight"), (db, "dbias")):
+        if g is not None:
+            g.check(n)
+    nb.nb_check_status()
+
+
+@pytest.mark.parametrize("BT,C,OC,r,down,up,back", [
+    (83, 784, 1168, 24, ("tile", 32, 4, 1), ("tile", 32, 2, 1), ["tile_pair", "tile_pair"]),
+    (134, 968, 736, 64, ("tile", 64, 8, 1), ("tile", 32, 1, 1), ["tile_pair", "tile_pair"]),
+    (26, 992, 4544, 16, ("tile", 64, 8, 1), ("tile", 64, 2, 1), ["tile_pair", "tile_pair"]),
+    (532, 8, 6352, 16, ("tile", 32, 1, 1), ("gemm", 192, 1, 1), ["tile_pair", "tile_pair"]),
+    (852, 2496, 32, 8, ("tile", 32, 4, 1), ("tile", 32, 4, 1), ["tile_pair", "tile", "tile_pair"]),
+    (1550, 8, 16, 48, ("tile", 64, 1, 1), ("tile", 32, 1, 1), ["lora_udb", "tile"]),
+])
+def test_adapter_forms(BT, C, OC, r, down, up, back):
+    assert nb.nb_debug_route(nb.CALL_LORA_FORWARD, BT, C, OC, r=r) == [down, up]
+    for accumulate in (False, True):
+        got = nb.nb_debug_route(nb.CALL_LORA_BACKWARD, BT, C, OC, r=r, accumulate=accumulate)
+        assert [k[0] for k in got] == back, got
+    test_small_adapter_layer(BT, C, OC, r)
