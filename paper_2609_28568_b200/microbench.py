@@ -1,20 +1,24 @@
 """Time one kind of library call on one shape (also the small case used for ncu captures).
 
-    python -m paper_2609_28568_b200.microbench KIND BT C OC [REPS] [energy]
+    python -m paper_2609_28568_b200.microbench KIND BT C OC [REPS] [energy | chain]
 
 KIND: fwd, fwd_nobias, fwd_gelu, fwd_swiglu, dgrad, dgrad_fused (dgrad with the producer's GELU
 backward in the epilogue), wgrad (accumulating), wgrad_bias (wgrad with the fused bias gradient),
 dbias (stand-alone column reduction), bwd (dinp + dweight + dbias in one call), bwd_nobias (dinp +
-dweight), bwd_fused (bwd with the producer's GELU backward in the dinp epilogue), cast (fp32 -> bf16
+dweight), bwd_fused (bwd with the producer's GELU backward in the dinp epilogue), bwd_zero and
+bwd_fused_zero (the same from zero instead of accumulating), cast (fp32 -> bf16
 master-weight cast of OC*C elements; reports GB/s), head_ce (head forward with the fused softmax
 statistics, vocabulary OC with the last 47 columns as padding), ce_bwd (dlogits from logits, GB/s),
+ce_bwd_inplace (over the logits),
 lora_fwd / lora_bwd (rank-16 adapter beside a frozen weight; TFLOP/s counts base + adapter flops).
 Prints microseconds per call and TFLOP/s from CUDA events around REPS back-to-back calls.
 
 With the word `energy` after REPS (GEMM kinds only) the call is instead replayed from a CUDA graph for
 about 2.5 seconds over rotating sets of buffers (inputs come from DRAM, as inside a training step, and the
 part settles at its power cap), and the GPU's energy counter (NVML, read-only) is read around the loop:
-microseconds, TFLOP/s, millijoules per call, picojoules per flop and average watts.
+microseconds, TFLOP/s, millijoules per call, picojoules per flop and average watts. With the word `chain`
+(the same kinds) it is the median of REPS replays of a captured graph of 24 calls one after the other over the
+rotating buffers, which is how launches follow each other in a step: microseconds per call.
 """
 from __future__ import annotations
 
@@ -26,13 +30,10 @@ from . import binding as nb
 from . import synth
 
 
-def sustained_energy(kind: str, BT: int, C: int, OC: int) -> int:
-    """Energy per call under sustained load: see the module docstring."""
+def replayed(kind: str, BT: int, C: int, OC: int, chain: int = 0) -> int:
+    """Calls replayed from a graph: energy per call under sustained load, or (chain > 0: replays) the time of a
+    call in a chain of them. See the module docstring."""
     import time
-
-    import pynvml
-    pynvml.nvmlInit()
-    h = pynvml.nvmlDeviceGetHandleByIndex(torch.cuda.current_device())
     dev, bf, f32 = "cuda", torch.bfloat16, torch.float32
     nbuf = 2 if BT * OC > (1 << 28) else 6
     inp = [synth.normal(1 + i, (BT, C), 1.0, dev) for i in range(nbuf)]
@@ -58,6 +59,9 @@ def sustained_energy(kind: str, BT: int, C: int, OC: int) -> int:
                                                          OC, 0, 1),
         "bwd_fused": lambda i: nb.nb_linear_backward_ex(dinp[i], dw, db, dout[i], inp[i], w, None, ipre[i], BT, C,
                                                         OC, 0, 1),
+        "bwd_zero": lambda i: nb.nb_linear_backward_ex(dinp[i], dw, db, dout[i], inp[i], w, None, None, BT, C, OC, 0, 0),
+        "bwd_fused_zero": lambda i: nb.nb_linear_backward_ex(dinp[i], dw, db, dout[i], inp[i], w, None, ipre[i], BT, C,
+                                                             OC, 0, 0),
     }
     if kind not in calls:
         print(__doc__)
@@ -74,7 +78,7 @@ def sustained_energy(kind: str, BT: int, C: int, OC: int) -> int:
     e1.record()
     torch.cuda.synchronize()
     per_graph = nbuf * 4
-    reps = max(2, int(2500.0 / (e0.elapsed_time(e1) / 20)) // per_graph)
+    reps = chain or max(2, int(2500.0 / (e0.elapsed_time(e1) / 20)) // per_graph)
     g, cap = torch.cuda.CUDAGraph(), torch.cuda.Stream()
     cap.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(cap):
@@ -84,6 +88,20 @@ def sustained_energy(kind: str, BT: int, C: int, OC: int) -> int:
     torch.cuda.current_stream().wait_stream(cap)
     g.replay()
     torch.cuda.synchronize()
+    if chain:
+        times = []
+        for _ in range(reps):
+            e0.record()
+            g.replay()
+            e1.record()
+            torch.cuda.synchronize()
+            times.append(e0.elapsed_time(e1) * 1e3 / per_graph)
+        nb.nb_check_status()
+        print(f"{kind} BT={BT} C={C} OC={OC} in a chain of {per_graph}: {sorted(times)[reps // 2]:.2f} us/call")
+        return 0
+    import pynvml
+    pynvml.nvmlInit()
+    h = pynvml.nvmlDeviceGetHandleByIndex(torch.cuda.current_device())
     j0, t0 = pynvml.nvmlDeviceGetTotalEnergyConsumption(h), time.time()
     e0.record()
     for _ in range(reps):
@@ -106,7 +124,9 @@ def main(argv) -> int:
     kind, BT, C, OC = argv[1], int(argv[2]), int(argv[3]), int(argv[4])
     reps = int(argv[5]) if len(argv) > 5 else 20
     if len(argv) > 6 and argv[6] == "energy":
-        return sustained_energy(kind, BT, C, OC)
+        return replayed(kind, BT, C, OC)
+    if len(argv) > 6 and argv[6] == "chain":
+        return replayed(kind, BT, C, OC, reps)
     dev = "cuda"
     bf, f32 = torch.bfloat16, torch.float32
     inp = synth.normal(1, (BT, C), 1.0, dev)
@@ -140,7 +160,7 @@ def main(argv) -> int:
         src = torch.randn(n, dtype=f32, device=dev)
         dst = torch.empty(n, dtype=bf, device=dev)
         calls["cast"] = lambda: nb.nb_cast_f32_to_bf16(dst, src, n)
-    if kind in ("head_ce", "ce_bwd"):
+    if kind in ("head_ce", "ce_bwd", "ce_bwd_inplace"):
         V = OC - 47 if OC > 47 else OC
         tg = torch.randint(0, V, (BT,), dtype=torch.int32, device=dev)
         loss = torch.empty(BT, dtype=f32, device=dev)
@@ -149,6 +169,9 @@ def main(argv) -> int:
         if kind == "ce_bwd":
             calls["head_ce"]()
             calls["ce_bwd"] = lambda: nb.nb_ce_backward(pre, out, lse, tg, 1.0 / BT, BT, OC, V)
+        if kind == "ce_bwd_inplace":
+            calls["head_ce"]()
+            calls["ce_bwd_inplace"] = lambda: nb.nb_ce_backward(out, out, lse, tg, 1.0 / BT, BT, OC, V)
     if kind in ("lora_fwd", "lora_bwd"):
         r, scale = 16, 8.0
         la = synth.normal(6, (r, C), 0.02, dev)
@@ -179,8 +202,8 @@ def main(argv) -> int:
     if kind == "cast":
         print(f"cast n={OC * C}: {ms * 1e3:.1f} us/call  {OC * C * 6 / ms / 1e6:.1f} GB/s")
         return 0
-    if kind == "ce_bwd":
-        print(f"ce_bwd BT={BT} Vp={OC}: {ms * 1e3:.1f} us/call  {BT * OC * 4 / ms / 1e6:.1f} GB/s")
+    if kind.startswith("ce_bwd"):
+        print(f"{kind} BT={BT} Vp={OC}: {ms * 1e3:.1f} us/call  {BT * OC * 4 / ms / 1e6:.1f} GB/s")
         return 0
     flops = 2 * BT * C * OC * (2 if kind.startswith("bwd") else 1)
     if kind == "lora_fwd":
