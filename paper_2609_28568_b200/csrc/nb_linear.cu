@@ -718,13 +718,6 @@ SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int N
             if (bn / cl < 8 || (cl > 1 && 2 * cl > kblocks)) break;
             for (int two = 0; two <= 1; ++two) {
                 const int longest = (kblocks + cl - 1) / cl;
-                // Where two do not fit, the form runs one per SM with the whole ring, and this is a second estimate of
-                // that: where its tiles take more than a wave it lies nearer than the first one, which adds a
-                // whole last tile. 700 drawn problems, the chosen form against the fastest: 2.6 % with it on average, 2.5 %
-                // without, but without it eleven small ones lose 3 to 11 % (100 rows, 1536 -> 1536 with gelu': 64-wide
-                // tiles 9.4 us, 128-wide ones 8.4; 519 rows, 3072 -> 768: layer_bwd_kernel 15.8, 128-wide tiles 13.2).
-                const bool fits = two && (bn == 64 ? pair_fits_twice<64>(M, longest, cl, Mw, kw, gelu)
-                                                   : pair_fits_twice<128>(M, longest, cl, Mw, kw, gelu));
                 const double slots = sms * (two ? 2.0 : 1.0);
                 const double n = static_cast<double>(nd * cl + nw);
                 // job 0's clusters come first and have to find their places; job 1's tiles fill up behind them
@@ -744,9 +737,19 @@ SmallPlan plan_pair(int sms, int M, int N, int kblocks, int split, int Mw, int N
                 // loads (130 rows, 4096 -> 1024: 9.5 us against 12.8; 256 rows, 4096 x 4096: 36.8 against 42.8)
                 if (two && bn == 128 && kw > 4) us *= 1.0 + 0.1 * (kw < 8 ? kw - 4 : 4);
                 us += kLaunchUs;
-                if (us < best.us) best = SmallPlan{bn, cl, fits, us};
+                if (us < best.us) best = SmallPlan{bn, cl, two != 0, us};
             }
         }
+    }
+    // Where two do not fit, the form runs one per SM with the whole ring, and the estimate of two is a second one of
+    // that: where its tiles take more than a wave it lies nearer than the first one, which adds a whole last tile. 700
+    // drawn problems, the chosen form against the fastest: 2.6 % with it on average, 2.5 % without, but without it eleven
+    // small ones lose 3 to 11 % (100 rows, 1536 -> 1536 with gelu': 64-wide tiles 9.4 us, 128-wide ones 8.4; 519 rows,
+    // 3072 -> 768: layer_bwd_kernel 15.8, 128-wide tiles 13.2).
+    if (best.two) {
+        const int longest = (kblocks + best.cluster - 1) / best.cluster;
+        best.two = best.bn == 64 ? pair_fits_twice<64>(M, longest, best.cluster, Mw, kw, gelu)
+                                 : pair_fits_twice<128>(M, longest, best.cluster, Mw, kw, gelu);
     }
     return best;
 }
@@ -1221,7 +1224,7 @@ int run_layer_bwd(DeviceState &s, const void *dz, const void *weight, const void
 // Whether a forward product in CTA pairs runs in 192-column tiles: where it takes several waves of the pairs
 // and as many with these as with 256-column ones, each wave is shorter (2021 rows, 768 -> 3072 with GELU,
 // two waves: 17.4 -> 15.0 us; 8192 rows, 3072 -> 768: 35.3 -> 32.0 us; 4600 rows, 768 -> 2304, three
-// waves: 18.0 -> 16.1 us). One more wave costs more than that (4096 rows, 768 -> 2304: 14.9 -> 15.7 us),
+// waves: 18.0 -> 16.1 us; no upper limit on the waves). One more wave costs more than that (4096 rows, 768 -> 2304: 14.9 -> 15.7 us),
 // and in a single wave the SMs' ports to L2 take back what the tensor cores save (4096 rows, 3072 -> 768:
 // 18.6 us either way; 73 operand bytes per clock and SM against 64).
 bool narrower_tiles(int sms, int M, int N)
