@@ -210,7 +210,8 @@ int nb_ce_backward(void *dlogits, const void *logits, const void *lse, const voi
  * come out of one kernel that reads dout once (both products are bound by that read); when dlora_a
  * is asked for as well, the same launch also reads inp once and forms dlora_a; both gradients are
  * then summed by reduce-adds of per-row-panel partial sums, in no fixed order. On short batches u
- * and dlora_b are one launch and dinp and dlora_a another, summed in a fixed order.
+ * and dlora_b are one launch and dinp and dlora_a another, summed in a fixed order. Which of the two
+ * it is depends on the sizes, on what is asked for and on accumulate, so the last bit of u may too.
  *
  * Projections that share an input and are laid out as one layer (a qkv or a gate_up projection:
  * weights stacked by rows) can use these two calls as they are, with r = the sum of the members'
@@ -251,8 +252,9 @@ int nb_lora_linear_backward(void *dinp, void *dlora_a, void *dlora_b, void *u, c
  *
  * r and off are multiples of 8, off + r <= R <= 64, R a multiple of 8. Column slices of t_stack and
  * u_stack are addressed in place (row stride R); columns outside a slice are neither read into a
- * product nor written. Every result equals what the unstacked calls give for that adapter; rounding
- * points and all other conventions are those of nb_lora_linear_forward / _backward.
+ * product nor written. Every result is what the unstacked calls give for that adapter, up to the order
+ * of the fp32 sums (r and R may split K differently); rounding points and all other conventions are those
+ * of nb_lora_linear_forward / _backward.
  */
 int nb_lora_down_stacked(void *t_stack, const void *inp, const void *a_stack, float scale, int64_t BT,
                          int64_t C, int64_t R, void *stream);
@@ -326,7 +328,8 @@ int nb_check_status(void);
 
 /*
  * Number of kernels this library has launched from the calling process since it was
- * loaded (what clears gradient buffers is not counted).
+ * loaded (what clears gradient buffers is not counted: a memset, or a small kernel ahead of the one
+ * that adds into them).
  */
 int64_t nb_kernel_launches(void);
 

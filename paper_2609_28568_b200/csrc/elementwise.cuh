@@ -236,8 +236,8 @@ ce_reduce_kernel(float *loss, float *lse, const float2 *stats, int stats_ld, con
 // Bound by its two passes over the logits where these exceed L2, and by instructions where they do not
 // or where the power cap holds the SMs down after the head's GEMM. So row and column are carried along
 // instead of divided out of a 64-bit index, and only the vectors that hold the target or cross V look at
-// single columns: 550 -> 518 us at 16384 x 50304 (in place 563 -> 521, 3.3 GB), 37.3 -> 34.5 at
-// 1024 x 50304, 20.8 -> 14.1 in place at 8000 x 4096.
+// single columns: 550 -> 518 us at 16384 x 50304 (in place 563 -> 521, 3.3 GB), 37.3 -> 34.3 at
+// 1024 x 50304, 20.9 -> 14.7 in place at 8000 x 4096.
 __global__ void __launch_bounds__(256)
 ce_backward_kernel(uint4 *dlogits, const uint4 *logits, const float *lse, const int *targets, float gscale, long long BT,
                    int vec_per_row, int V)

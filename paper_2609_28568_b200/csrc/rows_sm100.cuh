@@ -12,9 +12,8 @@
 // before the kernel waits for the one before it. Where K is long and there are few features, the
 // CTAs of a cluster share K and read each other's sums.
 //
-// Chained launches, 8 rows, weights from DRAM, against gemm_kernel: 768 -> 768 2.1 us (6.7),
-// 768 -> 3072 2.7 us (7.8), 3072 -> 768 3.3 us (19.9), 768 -> 50304 14.4 us (17.2; 77 MB of weights
-// take 12 us).
+// Chained launches, 8 rows, against gemm_kernel: 768 -> 768 1.8 us (6.7), 768 -> 3072 2.5 us (7.8),
+// 3072 -> 768 3.2 us (19.9), 768 -> 50304 14.5 us (17.2; 77 MB of weights take 12 us).
 #pragma once
 #include "gemm_sm100.cuh"
 
@@ -55,8 +54,8 @@ __device__ __forceinline__ uint4 ld_stream(const __nv_bfloat16 *p)
 // and 168 registers, more pieces of K in flight) took 6.0 us against 3.6 (16 rows, 3072 -> 768), 4.2
 // against 2.9 (768 -> 3072), 10.3 against 4.2 (8 rows, SwiGLU, 4096 -> 1024). MANY: there are several
 // CTAs of work per SM: fewer pieces of K in flight per thread and four CTAs on an SM (8 rows,
-// 768 -> 50304: 14.4 us against 22.7 us with two, five or six have too few registers, 15.7 and 17.1 us;
-// 16 rows, 1024 -> 8192: 4.7 us against 5.8 us with two and 6.1 us with three).
+// 768 -> 50304: 14.5 us against 22.7 us with two, five or six have too few registers, 15.7 and 17.1 us;
+// 16 rows, 1024 -> 8192: 4.6 us against 5.8 us with two and 6.1 us with three).
 template <int NT, int EPI, bool MANY>
 __global__ void __launch_bounds__(kRowsThreads, MANY ? 4 : 2)
 rows_kernel(const RowsParams p)

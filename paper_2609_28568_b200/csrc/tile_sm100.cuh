@@ -7,8 +7,8 @@
 // here a CTA takes a 128 x BN tile (BN = 32 / 64 / 128, or 192 without a split), and where there are far fewer tiles than SMs
 // the CTAs of a cluster share a tile's K range: each accumulates its part in TMEM and sends every
 // other CTA that one's slice of the columns through distributed shared memory, and after a barrier
-// of the cluster adds the parts it got in rank order (a fixed order: results do not vary) and runs the
-// epilogue on its slice.
+// of the cluster adds the parts it got in rank order (a fixed order: products do not vary; the bias
+// gradient's partial sums meet in shared memory in any order) and runs the epilogue on its slice.
 //
 //   warp 0      TMA producer
 //   warp 1      MMA issuer, TMEM allocation
@@ -22,9 +22,9 @@
 // tensor core then multiplies whatever follows in shared memory for the other rows, which touches
 // no valid row of the result.
 //
-// Chained launches against the persistent kernels: forward 1024 rows 768 -> 2304 6.7 us (8.7),
-// 1024 rows 3072 -> 768 11.1 us (18.5), 128 rows 768 -> 768 4.7 us (7.3); dinp 2048 rows 3072 -> 768
-// 13.9 us (18.5); backward 512 rows 768 x 768 5.4 us (14.1 with the clearing of dweight, 8.3 without).
+// Chained launches against the persistent kernels: forward 1024 rows 768 -> 2304 6.2 us (8.7),
+// 1024 rows 3072 -> 768 11.4 us (18.5), 128 rows 768 -> 768 4.4 us (7.3); dinp 2048 rows 3072 -> 768
+// 13.1 us (18.5); backward 512 rows 768 x 768 5.5 us (14.1 with the clearing of dweight, 8.3 without).
 #pragma once
 #include "gemm_sm100.cuh"
 
@@ -544,7 +544,7 @@ __device__ __forceinline__ void tile_body(const TileJob &j, const TileMaps &t, u
                 // group is 129 rows long, so that neighbouring groups of a row lie in other banks. The
                 // network between the SMs is the slow part, so the CTA's own slice stays off it: 128
                 // columns over two CTAs 8.4 -> 6.9 us (128 rows, 768 -> 768), 13.5 -> 11.7 us (1024
-                // rows, 3072 -> 768), 32 columns over two 5.2 -> 4.5 us. Plain stores and one barrier of the
+                // rows, 3072 -> 768, a form it no longer takes), 32 columns over two 5.2 -> 4.5 us. Plain stores and one barrier of the
                 // cluster; st.async with the bytes counted on the receiver's mbarrier took 0.1 to 0.5 us
                 // longer (64 rows, 768 -> 768: 3.80 -> 3.65 us; 519 rows, 3072 -> 1024: 12.0 -> 11.4), bulk
                 // copies from shared memory to shared memory another 0.6 us.
