@@ -78,6 +78,25 @@ struct TmapKeyHash {
     }
 };
 
+struct PlanKey {
+    int64_t BT, C, OC;
+    int pairs;
+    bool gelu_grad;
+    bool operator==(const PlanKey &o) const
+    {
+        return BT == o.BT && C == o.C && OC == o.OC && pairs == o.pairs && gelu_grad == o.gelu_grad;
+    }
+};
+struct PlanKeyHash {
+    size_t operator()(const PlanKey &k) const
+    {
+        const uint64_t h = (static_cast<uint64_t>(k.BT) * 0x9E3779B97F4A7C15ull) ^ (static_cast<uint64_t>(k.C) * 0xBF58476D1CE4E5B9ull) ^
+                           (static_cast<uint64_t>(k.OC) * 0x94D049BB133111EBull) ^ (static_cast<uint64_t>(k.pairs) << 1) ^
+                           static_cast<uint64_t>(k.gelu_grad);
+        return static_cast<size_t>(h ^ (h >> 31));
+    }
+};
+
 struct DeviceState {
     bool init = false;
     int num_sms = 0;
@@ -85,6 +104,7 @@ struct DeviceState {
     void *workspace = nullptr;
     size_t workspace_bytes = 0;
     std::unordered_map<TmapKey, CUtensorMap, TmapKeyHash> tmaps;
+    std::unordered_map<PlanKey, LayerBwdParams, PlanKeyHash> plans;
 };
 
 std::mutex g_mu;
@@ -1002,17 +1022,84 @@ bool layer_bwd_narrow(int d_tiles, int d_kblocks, int w_tiles, int w_kblocks, in
            static_cast<double>(d_kblocks) * P > 1.0 * d_tiles * d_kblocks + 1.0 * w_tiles * w_kblocks;
 }
 
-// The schedule of layer_bwd_kernel for P CTA pairs (layer_bwd_sm100.cuh describes the unit list).
-// Costs are counted in k-blocks of tensor-core time: a D unit costs its k-blocks plus eD (the part
-// of its epilogue the next main loop does not hide: larger with gelu'), a W unit its k-blocks plus
-// eW. Every pair should end up with the same cost.
-//  1. K = BT of the weight gradient is cut into chunks so that there are about two W units per
-//     pair, none shorter than 32 k-blocks (every unit reduce-adds a whole fp32 tile: fewer, longer
-//     units mean less traffic; in-step timings did not tell 16 to 128 k-blocks apart).
+// What a unit costs beside its k-blocks, in k-blocks of 0.33 us, from the times at which the pairs of twelve launches ended
+// (2021 and 4096 rows): a W unit's fp32 boxes, 128 KB an SM, take up to 2.3 us of the main loop they leave under, a D unit's
+// bf16 boxes 0.4, and gelu' some arithmetic on top. (5 to 7 for a W unit measure alike; 3, as before, leaves the pairs with
+// several of them 3 to 5 us behind the others.)
+constexpr int kCostD = 1, kCostDGelu = 2, kCostW = 5;
+constexpr int kMaxChunk = 64;  // k-blocks
+constexpr int kMinPiece = 2;  // k-blocks of a W unit that are worth a cut
+
+// The W units that are left after the whole rounds, as one line of k-blocks: `full` of them in units of kbc, the rest in
+// units of last.
+struct LbLine {
+    long long total, full;
+    int kbc, last;
+    long long unit_left(long long x) const  // k-blocks from x to the end of its unit
+    {
+        return x < full ? kbc - x % kbc : last - (x - full) % last;
+    }
+};
+// Cuts the line into a range per pair such that no pair's cost (fixed_tail for the first d_tail of them, a range, kCostW
+// for each unit that it touches) exceeds `limit`; ranges end at their unit's end or at least kMinPiece k-blocks from either
+// end of it, and the last pair takes what is left. begin (or null): P + 1 range borders. pieces: set to their number; where it is given (not 0), as the number that such a cut
+// makes, a pair takes no more than the mean of what is left and `slack`, so that what the limit leaves over is spread and not
+// all the last pair's.
+struct LbCut {
+    double most, least, mean;  // of the pairs' costs
+};
+LbCut cut_line(const LbLine &l, int P, int d_tail, double fixed_tail, double limit, int *begin, int &pieces, double slack = 0.0)
+{
+    long long x = 0;
+    int n = 0;
+    double carry = 0.0;  // of a k-block that the pair before this one had room for
+    LbCut c{0.0, 1e30, 0.0};
+    for (int q = 0; q < P; ++q) {
+        if (begin) begin[q] = static_cast<int>(x);
+        double target = limit;
+        if (pieces > 0) {
+            const double mean = (static_cast<double>(l.total - x) + kCostW * (pieces > n ? pieces - n : 0) +
+                                 fixed_tail * (q < d_tail ? d_tail - q : 0)) / (P - q) + slack;
+            if (mean < target) target = mean;
+        }
+        target += carry;
+        carry = 0.0;
+        double cost = q < d_tail ? fixed_tail : 0.0;
+        while (x < l.total) {
+            const long long left = l.unit_left(x);
+            const long long room = q == P - 1 ? left : static_cast<long long>(target - cost - kCostW);
+            long long take = room < left ? room : left;
+            if (take < left && take > left - kMinPiece) take = left - kMinPiece;
+            if (take < left && take < kMinPiece) break;
+            x += take;
+            ++n;
+            cost += kCostW + static_cast<double>(take);
+            if (take < left) {
+                carry = target - cost < 1.0 ? target - cost : 1.0;
+                break;
+            }
+        }
+        if (cost > c.most) c.most = cost;
+        if (cost < c.least) c.least = cost;
+        c.mean += cost / P;
+    }
+    if (begin) begin[P] = static_cast<int>(l.total);
+    if (pieces == 0) pieces = n;
+    return c;
+}
+
+// The schedule of layer_bwd_kernel for P CTA pairs (layer_bwd_sm100.cuh describes the unit list). Costs are counted in
+// k-blocks of tensor-core time (kCostD, kCostW above); every pair should end up with the same cost.
+//  1. K = BT of the weight gradient is cut into chunks. Every number of them from one to the one that gives two W units per
+//     pair is tried, of 16 to kMaxChunk k-blocks where that leaves a choice, and the one whose dearest pair is cheapest is taken.
 //  2. Whole rounds (one unit per pair) are dealt first; W rounds are spread evenly among D rounds.
-//  3. The last D round is partial: pairs [0, d_tail) take one more tile. The W units left over are
-//     laid out as one line of k-blocks and cut into P ranges, shorter by one D unit's cost for the
-//     pairs that took a tail tile. If the line is too short for that, one W round is taken back.
+//  3. The last D round is partial: pairs [0, d_tail) take one more tile. The W units left over are laid out as one line of
+//     k-blocks and cut into P ranges at the lowest limit at which cut_line finds a place for all of it. If the line is so
+//     short that the tail D tiles alone exceed the level, a W round is taken back into it.
+// Against ranges levelled one after the other with 3 k-blocks a unit, over about two chunks a pair of 32 k-blocks or more
+// (chained launches, accumulating, us): 4096 rows, 768 -> 768 16.3 -> 14.1, 768 -> 2304 27.0 -> 25.5, 1024 -> 6144 77.8 -> 73.6,
+// 3072 -> 1024 42.8 -> 40.0; 8192 rows, 768 -> 768 23.5 -> 20.4; 16384 rows, 768 -> 768 38.5 -> 34.9, 768 -> 2304
+// 90.9 -> 88.2. Chunks of up to 256 k-blocks cost 16384 rows, 768 -> 3072 4 % (the pairs drift apart).
 // narrow (as it is launched): D tiles are 128 columns wide (layer_bwd_narrow; not with gelu') where the 256-wide ones are
 // at most a quarter of the pairs, K is long, and a single one takes longer than a pair's share of all the work: 1500 rows,
 // 768 -> 3072, 18 tiles of 48 k-blocks, 18.9 -> 16.4 us; 1024 rows, 1024 -> 6144, 32.5 -> 24.4 us. With
@@ -1023,11 +1110,6 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
 {
     memset(&p, 0, sizeof(p));
     if (P < 1 || P > kMaxPairs) return fail(NB_ERR_UNSUPPORTED, "CTA pair count %d out of range", P);
-    static const int eD_plain = env_int("NB_LB_ED", 3);
-    static const int eD_gelu = env_int("NB_LB_ED_GELU", 8);
-    static const int eW = env_int("NB_LB_EW", 3);
-    static const int kbc_forced = env_int("NB_LB_KBC", 0);
-    const int eD = gelu_grad ? eD_gelu : eD_plain;
     p.BT = static_cast<int>(BT);
     p.C = static_cast<int>(C);
     p.OC = static_cast<int>(OC);
@@ -1037,101 +1119,118 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     p.d_kblocks = static_cast<int>((OC + kBlockK - 1) / kBlockK);
     p.w_tiles_n = p.d_tiles_n;
     p.d_w = 256;
-    if (narrow && !gelu_grad && layer_bwd_narrow(p.d_tiles_m * p.d_tiles_n, p.d_kblocks,
-                                                 static_cast<int>((OC + 255) / 256) * p.w_tiles_n,
-                                                 static_cast<int>((BT + kBlockK - 1) / kBlockK), P)) {
-        p.d_w = 128;
-        p.d_tiles_n = static_cast<int>((C + 127) / 128);
-    }
-    p.d_tiles = p.d_tiles_m * p.d_tiles_n;
-    p.d_group_m = (p.d_tiles_n >= 64 ? 64 : p.d_tiles_n <= 4 ? 4 : 16) / 2;
     p.w_tiles_m = static_cast<int>((OC + 255) / 256);
     p.w_tiles = p.w_tiles_m * p.w_tiles_n;
     p.w_kblocks = static_cast<int>((BT + kBlockK - 1) / kBlockK);
-    int chunks = (2 * P + p.w_tiles - 1) / p.w_tiles;
-    const int max_chunks = p.w_kblocks / 32 > 1 ? p.w_kblocks / 32 : 1;
-    if (chunks > max_chunks) chunks = max_chunks;
-    if (chunks < 1) chunks = 1;
-    p.w_kbc = (p.w_kblocks + chunks - 1) / chunks;
-    if (kbc_forced > 0) p.w_kbc = kbc_forced < p.w_kblocks ? kbc_forced : p.w_kblocks;
-    chunks = (p.w_kblocks + p.w_kbc - 1) / p.w_kbc;
-    const long long w_units = 1ll * chunks * p.w_tiles;
-    if (w_units >= (1ll << 24) || p.d_tiles >= (1 << 24)) return fail(NB_ERR_UNSUPPORTED, "too many work units");
-    p.w_units = static_cast<int>(w_units);
+    if (narrow && !gelu_grad && layer_bwd_narrow(p.d_tiles_m * p.d_tiles_n, p.d_kblocks, p.w_tiles, p.w_kblocks, P)) {
+        p.d_w = 128;
+        p.d_tiles_n = static_cast<int>((C + 127) / 128);
+    }
+    if (1ll * p.d_tiles_m * p.d_tiles_n >= (1 << 24)) return fail(NB_ERR_UNSUPPORTED, "too many work units");
+    p.d_tiles = p.d_tiles_m * p.d_tiles_n;
+    p.d_group_m = (p.d_tiles_n >= 64 ? 64 : p.d_tiles_n <= 4 ? 4 : 16) / 2;
     p.d_rounds = p.d_tiles / P;
     p.d_tail = p.d_tiles % P;
-    const double cD = p.d_kblocks * (p.d_w == 128 ? kNarrowD : 1.0) + eD;
-    // the units of the last chunk may be shorter than the others: they all stay in the tail, where
-    // lengths are counted exactly
-    p.w_last_len = p.w_kblocks - (chunks - 1) * p.w_kbc;
-    const int even_units = p.w_last_len == p.w_kbc ? p.w_units : p.w_units - p.w_tiles;
-    int aW = even_units / P;
-    double b_hi = 0.0, b_lo = 0.0;  // tail k-blocks of a pair without / with a tail D tile
-    long long Rk = 0;
-    for (;; --aW) {
-        const long long tail_full = 1ll * (even_units - aW * P) * p.w_kbc;
-        Rk = tail_full + 1ll * (p.w_units - even_units) * p.w_last_len;
-        p.w_tail_full = static_cast<int>(tail_full < (1ll << 30) ? tail_full : (1ll << 30));
-        b_hi = static_cast<double>(Rk) / P + cD * p.d_tail / P;
-        b_lo = b_hi - cD;
-        const bool fits = p.d_tail == 0 ? (Rk == 0 || Rk >= 8ll * P) : b_lo >= 8.0;
-        if (fits || aW == 0) break;
-    }
-    if (Rk >= (1ll << 30)) return fail(NB_ERR_UNSUPPORTED, "weight-gradient tail too long");
-    p.w_rounds = aW;
-    const int rounds = p.d_rounds + p.w_rounds;
-    if (rounds > kLbMaxRounds) return fail(NB_ERR_UNSUPPORTED, "more than %d rounds", kLbMaxRounds);
-    p.round_is_w = 0;
-    for (int r = 0; r < rounds; ++r)
-        if (1ll * (r + 1) * aW / rounds > 1ll * r * aW / rounds) p.round_is_w |= 1ull << r;
-    // Tail ranges. Pair q's share is what levels the cost of the pairs still to be served: the
-    // k-blocks and per-piece allowances left on the line plus their fixed costs (tail D tile),
-    // divided among them, minus its own fixed cost. A range ends on a multiple of four k-blocks of
-    // its unit or at the unit's end.
-    (void)b_hi;
-    (void)b_lo;
-    const int tail_units = p.w_units - aW * P;
-    const long long full_units = p.w_tail_full / p.w_kbc;
-    auto unit_at = [&](long long x, long long &u_idx, long long &u_left) {
-        if (x < p.w_tail_full) {
-            u_idx = x / p.w_kbc;
-            u_left = p.w_kbc - x % p.w_kbc;
-        } else {
-            const long long xr = x - p.w_tail_full;
-            u_idx = full_units + xr / p.w_last_len;
-            u_left = p.w_last_len - xr % p.w_last_len;
-        }
-    };
-    long long x = 0;
-    p.w_tail_begin[0] = 0;
-    for (int q = 0; q < P; ++q) {
-        if (q == P - 1) {
-            x = Rk;
-        } else if (x < Rk) {
-            long long u_idx, u_left;
-            unit_at(x, u_idx, u_left);
-            const int pairs_left = P - q;
-            const int tail_d_left = p.d_tail > q ? p.d_tail - q : 0;
-            const double line_cost = static_cast<double>(Rk - x) + 1.0 * eW * (tail_units - u_idx) +
-                                     1.0 * eW * (pairs_left - 1);
-            double rem = (line_cost + cD * tail_d_left) / pairs_left - (q < p.d_tail ? cD : 0.0);
-            while (x < Rk && rem >= eW + 4) {
-                unit_at(x, u_idx, u_left);
-                long long take = static_cast<long long>(rem - eW);
-                if (take >= u_left) {
-                    take = u_left;
-                } else {
-                    take = take / 4 * 4;
-                    if (take <= 0) break;
-                }
-                x += take;
-                rem -= eW + take;
-                if (take < u_left) break;
+    const double cD = p.d_kblocks * (p.d_w == 128 ? kNarrowD : 1.0) + (gelu_grad ? kCostDGelu : kCostD);
+
+    int max_chunks = (2 * P + p.w_tiles - 1) / p.w_tiles;
+    if (max_chunks > p.w_kblocks / 16) max_chunks = p.w_kblocks / 16;
+    if (max_chunks < 1) max_chunks = 1;
+    double best = -1.0;
+    long long best_total = 0;
+    for (int want = 1; want <= max_chunks; ++want) {
+        const int kbc = (p.w_kblocks + want - 1) / want;
+        const int chunks = (p.w_kblocks + kbc - 1) / kbc;
+        if (chunks != want || (want < max_chunks && kbc > kMaxChunk)) continue;  // the same length again
+        const long long w_units = 1ll * chunks * p.w_tiles;
+        if (w_units >= (1ll << 24)) break;
+        // the units of the last chunk may be shorter than the others: they all stay in the tail, where lengths are
+        // counted exactly
+        const int last = p.w_kblocks - (chunks - 1) * kbc;
+        const long long even = last == kbc ? w_units : w_units - p.w_tiles;
+        const int aW_max = static_cast<int>(even / P);
+        // as many W rounds as leave the pairs with a tail D tile below the level, give or take one
+        const double mean = (1.0 * p.w_kblocks * p.w_tiles + 1.0 * kCostW * (w_units + P) + cD * p.d_tail) / P;
+        int aW_hi = p.d_tail ? static_cast<int>((mean - cD) / (kbc + kCostW)) + 1 : aW_max;
+        aW_hi = aW_hi < 0 ? 0 : aW_hi < aW_max ? aW_hi : aW_max;
+        for (int aW = aW_hi; aW >= 0 && aW >= aW_hi - 2; --aW) {
+            const long long full = (even - 1ll * aW * P) * kbc;
+            const LbLine line{full + (w_units - even) * last, full, kbc, last};
+            if (line.total >= (1ll << 30) || p.d_rounds + aW > kLbMaxRounds) continue;
+            const double rounds = 1.0 * aW * (kbc + kCostW);  // beside the D rounds, which are the same for all plans
+            // no cut costs less than this: every pair with a range pays for a piece at least, and every unit
+            const long long units = w_units - 1ll * aW * P;
+            const double floor_ = (1.0 * line.total + kCostW * static_cast<double>(units > P - p.d_tail ? units : P - p.d_tail) + cD * p.d_tail) / P;
+            if (best >= 0.0 && (rounds + floor_) * 1.5 >= best) continue;
+            double lo = floor_ - 1.0, hi = floor_ + kCostW;
+            auto fits = [&](double limit) {
+                int n = 0;
+                return cut_line(line, P, p.d_tail, cD, limit, nullptr, n).most <= (cD > limit && p.d_tail ? cD : limit) + 1.0;
+            };
+            while (!fits(hi)) hi = 1.25 * hi + kCostW;
+            while (hi - lo > 0.25) {
+                const double mid = 0.5 * (lo + hi);
+                if (fits(mid)) hi = mid;
+                else lo = mid;
             }
+            // That cut, or one that spreads its room over the pairs. The dearest pair counts and, where the chip is at its
+            // power limit, what all of them do (each piece adds to it); a very cheap one is a share that could be others'.
+            // Where the tail D tiles are the longest chain whatever the others do, higher limits leave more units whole.
+            const bool chain = p.d_tail && cD > hi;
+            auto price = [&](const LbCut &c) { return c.most + 0.5 * c.mean + (chain ? 0.0 : (c.most - c.least) / 8); };
+            int pieces = 0;
+            double slack = 1e9, limit = hi, cost = price(cut_line(line, P, p.d_tail, cD, hi, nullptr, pieces));
+            if (chain) {
+                for (double at = 1.05 * hi; at < 0.9 * cD; at *= 1.05) {
+                    int n = 0;
+                    const double c = price(cut_line(line, P, p.d_tail, cD, at, nullptr, n));
+                    if (c >= cost) continue;
+                    cost = c;
+                    limit = at;
+                }
+                pieces = 0;
+            } else {
+                for (int i = 0; i < 24; ++i) {
+                    const double c = price(cut_line(line, P, p.d_tail, cD, 1e9, nullptr, pieces, 0.125 * i));
+                    if (c >= cost) continue;
+                    cost = c;
+                    slack = 0.125 * i;
+                    limit = 1e9;
+                }
+            }
+            cost += rounds * 1.5;
+            if (best >= 0.0 && cost >= best) continue;
+            best = cost;
+            best_total = line.total;
+            p.w_kbc = kbc;
+            p.w_units = static_cast<int>(w_units);
+            p.w_rounds = aW;
+            p.w_last_len = last;
+            p.w_tail_full = static_cast<int>(full);
+            (void)cut_line(line, P, p.d_tail, cD, limit, p.w_tail_begin, pieces, slack);
         }
-        p.w_tail_begin[q + 1] = static_cast<int>(x);
     }
-    for (int q = P + 1; q <= kMaxPairs; ++q) p.w_tail_begin[q] = static_cast<int>(Rk);
+    if (best < 0.0) return fail(NB_ERR_UNSUPPORTED, "more than %d rounds", kLbMaxRounds);
+    const int rounds = p.d_rounds + p.w_rounds;
+    for (int r = 0; r < rounds; ++r)
+        if (1ll * (r + 1) * p.w_rounds / rounds > 1ll * r * p.w_rounds / rounds) p.round_is_w |= 1ull << r;
+    for (int q = P + 1; q <= kMaxPairs; ++q) p.w_tail_begin[q] = static_cast<int>(best_total);
+    return NB_OK;
+}
+
+// The plan of a launch. Finding one takes 60 to 300 us, so the plans of the last sizes are kept (they hold sizes only).
+int cached_layer_bwd_plan(DeviceState &s, LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad)
+{
+    const PlanKey key{BT, C, OC, P, gelu_grad};
+    const auto it = s.plans.find(key);
+    if (it != s.plans.end()) {
+        p = it->second;
+        return NB_OK;
+    }
+    const int rc = plan_layer_bwd(p, BT, C, OC, P, gelu_grad, true);
+    if (rc != NB_OK) return rc;
+    if (s.plans.size() >= 512) s.plans.clear();
+    s.plans.emplace(key, p);
     return NB_OK;
 }
 
@@ -1171,7 +1270,7 @@ int launch_layer_bwd(DeviceState &s, const void *dz, const void *weight, const v
         attr_set[dev] = true;
     }
     LayerBwdParams p;
-    int rc = plan_layer_bwd(p, BT, C, OC, max_pairs[dev], Cfg::GELU_GRAD, true);
+    int rc = cached_layer_bwd_plan(s, p, BT, C, OC, max_pairs[dev], Cfg::GELU_GRAD);
     if (rc != NB_OK) return rc;
     p.dbias = Cfg::DBIAS ? dbias : nullptr;
     p.status = s.status;
