@@ -20,11 +20,24 @@ __device__ __forceinline__ float silu_bwd(float g)
     return s * (1.0f + g * (1.0f - s));
 }
 
-// dz = dout * gelu'(pre), 8 bf16 per thread per iteration (128-bit loads and stores).
+// Zeroes an fp32 array (null: none; 16-byte aligned, its length a multiple of 4) with all threads of the grid.
+__device__ __forceinline__ void clear_f32(float *a, long long n)
+{
+    if (a == nullptr) return;
+    const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
+    for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n / 4; i += stride)
+        reinterpret_cast<float4 *>(a)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+}
+
+// dz = dout * gelu'(pre), 8 bf16 per thread per iteration (128-bit loads and stores). cw, cb (or null): gradients that the
+// layer's products, which follow, add to, cleared on the way (a launch of its own for that is 2.5 us on the chain).
 __global__ void __launch_bounds__(256)
-gelu_backward_kernel(uint4 *dz, const uint4 *dout, const uint4 *pre, long long nvec)
+gelu_backward_kernel(uint4 *dz, const uint4 *dout, const uint4 *pre, long long nvec, float *cw, long long nw, float *cb,
+                     long long nb_)
 {
     chained_start();
+    clear_f32(cw, nw);
+    clear_f32(cb, nb_);
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < nvec;
          i += stride) {
@@ -46,9 +59,12 @@ gelu_backward_kernel(uint4 *dz, const uint4 *dout, const uint4 *pre, long long n
 // SwiGLU backward: dout [BT, H], pre [BT, 2H] = [gate | up]  ->  dz [BT, 2H].
 //   dz[:, j] = dout * up * silu'(gate) ; dz[:, H + j] = dout * silu(gate)
 __global__ void __launch_bounds__(256)
-swiglu_backward_kernel(uint4 *dz, const uint4 *dout, const uint4 *pre, long long BT, int hvec /* H / 8 */)
+swiglu_backward_kernel(uint4 *dz, const uint4 *dout, const uint4 *pre, long long BT, int hvec /* H / 8 */, float *cw,
+                       long long nw, float *cb, long long nb_)
 {
     chained_start();
+    clear_f32(cw, nw);
+    clear_f32(cb, nb_);
     const long long total = BT * hvec;
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;

@@ -53,6 +53,8 @@ struct LayerBwdParams {
     int w_tail_full, w_last_len;
     int w_tail_begin[kMaxPairs + 1];
     float *dbias;  // [OC] or nullptr
+    int w_whole;      // every W unit is a tile's whole K
+    int store_w;      // dweight and dbias start from nothing and every W unit is whole: stored, not added
     int after_clear;  // the launch before this one is clear_kernel on dweight and dbias: only what adds
                       // to them has to wait for it (that kernel let this one start once everything
                       // before it was done)
@@ -428,7 +430,11 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                 for (int k = 0; k < 8; ++k) atomicAdd_shared_f32(part_s + 4u * (cc * 8 + k), sum[k]);
                 ptx::named_bar_sync(2, 128);
                 const int m = u.m_blk * 256 + static_cast<int>(rank) * 128 + rt;
-                if (ok && m < p.OC) atomicAdd(p.dbias + m, ptx::ld_shared_f32(part_s + 4u * rt));
+                if (ok && m < p.OC) {
+                    const float v = ptx::ld_shared_f32(part_s + 4u * rt);
+                    if (p.store_w) p.dbias[m] = v;
+                    else atomicAdd(p.dbias + m, v);
+                }
                 ptx::st_shared_f32(part_s + 4u * rt, 0.0f);
                 ptx::named_bar_sync(2, 128);
             }
@@ -507,7 +513,7 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                 release_acc(acc);  // the accumulator is in registers
 
                 if (u.is_w) {
-                    // ---------------- fp32 tile of dweight: 32-column boxes, reduce-added
+                    // ---------------- fp32 tile of dweight: 32-column boxes, reduce-added (whole ones of a fresh one stored)
 #pragma unroll
                     for (int s4 = 0; s4 < 4; ++s4) {
                         uint32_t (&r)[32] = rr[s4];
@@ -522,7 +528,10 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                         if (ptx::elect_one()) {
                             const int x = nw + s4 * 32;
                             const int y = m0 + q * 32;
-                            if (ok && x < p.C && y < p.OC) ptx::tma_reduce_add_2d(&tmDw, fb, x, y);
+                            if (ok && x < p.C && y < p.OC) {
+                                if (p.store_w) ptx::tma_store_2d(&tmDw, fb, x, y);
+                                else ptx::tma_reduce_add_2d(&tmDw, fb, x, y);
+                            }
                             ptx::bulk_commit_group();
                         }
                         __syncwarp();

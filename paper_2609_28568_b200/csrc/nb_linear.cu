@@ -81,18 +81,18 @@ struct TmapKeyHash {
 struct PlanKey {
     int64_t BT, C, OC;
     int pairs;
-    bool gelu_grad;
+    bool gelu_grad, fresh;
     bool operator==(const PlanKey &o) const
     {
-        return BT == o.BT && C == o.C && OC == o.OC && pairs == o.pairs && gelu_grad == o.gelu_grad;
+        return BT == o.BT && C == o.C && OC == o.OC && pairs == o.pairs && gelu_grad == o.gelu_grad && fresh == o.fresh;
     }
 };
 struct PlanKeyHash {
     size_t operator()(const PlanKey &k) const
     {
         const uint64_t h = (static_cast<uint64_t>(k.BT) * 0x9E3779B97F4A7C15ull) ^ (static_cast<uint64_t>(k.C) * 0xBF58476D1CE4E5B9ull) ^
-                           (static_cast<uint64_t>(k.OC) * 0x94D049BB133111EBull) ^ (static_cast<uint64_t>(k.pairs) << 1) ^
-                           static_cast<uint64_t>(k.gelu_grad);
+                           (static_cast<uint64_t>(k.OC) * 0x94D049BB133111EBull) ^ (static_cast<uint64_t>(k.pairs) << 2) ^
+                           (static_cast<uint64_t>(k.gelu_grad) << 1) ^ static_cast<uint64_t>(k.fresh);
         return static_cast<size_t>(h ^ (h >> 31));
     }
 };
@@ -1028,6 +1028,7 @@ bool layer_bwd_narrow(int d_tiles, int d_kblocks, int w_tiles, int w_kblocks, in
 // several of them 3 to 5 us behind the others.)
 constexpr int kCostD = 1, kCostDGelu = 2, kCostW = 5;
 constexpr int kMaxChunk = 64;  // k-blocks
+constexpr int kCostClear = 8;  // the launch that clears a fresh dweight, 2.5 to 3 us on the chain
 constexpr int kMinPiece = 2;  // k-blocks of a W unit that are worth a cut
 
 // The W units that are left after the whole rounds, as one line of k-blocks: `full` of them in units of kbc, the rest in
@@ -1100,13 +1101,15 @@ LbCut cut_line(const LbLine &l, int P, int d_tail, double fixed_tail, double lim
 // (chained launches, accumulating, us): 4096 rows, 768 -> 768 16.3 -> 14.1, 768 -> 2304 27.0 -> 25.5, 1024 -> 6144 77.8 -> 73.6,
 // 3072 -> 1024 42.8 -> 40.0; 8192 rows, 768 -> 768 23.5 -> 20.4; 16384 rows, 768 -> 768 38.5 -> 34.9, 768 -> 2304
 // 90.9 -> 88.2. Chunks of up to 256 k-blocks cost 16384 rows, 768 -> 3072 4 % (the pairs drift apart).
+// fresh: dweight starts from nothing. Where every W unit is a tile's whole K it is stored and the clearing launch saved
+// (2021 rows, 768 -> 3072 22.7 -> 20.7 us, 768 -> 50304 298 -> 265; 1100 rows, 1024 -> 4096 34.3 -> 29.4), which is worth kCostClear.
 // narrow (as it is launched): D tiles are 128 columns wide (layer_bwd_narrow; not with gelu') where the 256-wide ones are
 // at most a quarter of the pairs, K is long, and a single one takes longer than a pair's share of all the work: 1500 rows,
 // 768 -> 3072, 18 tiles of 48 k-blocks, 18.9 -> 16.4 us; 1024 rows, 1024 -> 6144, 32.5 -> 24.4 us. With
 // more tiles the operand traffic of halved ones costs more than the shorter chain gives (2021 rows,
 // 768 -> 2304, 24 tiles: 16.0 -> 19.4 us). A 128-wide k-block is counted as 0.6 of a 256-wide one.
 // Returns NB_ERR_UNSUPPORTED when the shape needs more rounds than the order mask holds.
-int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad, bool narrow)
+int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad, bool narrow, bool fresh)
 {
     memset(&p, 0, sizeof(p));
     if (P < 1 || P > kMaxPairs) return fail(NB_ERR_UNSUPPORTED, "CTA pair count %d out of range", P);
@@ -1180,14 +1183,19 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
             auto price = [&](const LbCut &c) { return c.most + 0.5 * c.mean + (chain ? 0.0 : (c.most - c.least) / 8); };
             int pieces = 0;
             double slack = 1e9, limit = hi, cost = price(cut_line(line, P, p.d_tail, cD, hi, nullptr, pieces));
-            if (chain) {
-                for (double at = 1.05 * hi; at < 0.9 * cD; at *= 1.05) {
+            const bool may_store = fresh && chunks == 1;
+            if (chain || may_store) {
+                const double end = may_store ? (chain ? cD : hi) + 2.0 * kCostClear : 0.9 * cD;
+                for (double at = hi; at < end; at *= 1.05) {
                     int n = 0;
-                    const double c = price(cut_line(line, P, p.d_tail, cD, at, nullptr, n));
+                    double c = price(cut_line(line, P, p.d_tail, cD, at, nullptr, n));
+                    if (may_store && n == units) c -= kCostClear;
                     if (c >= cost) continue;
                     cost = c;
                     limit = at;
                 }
+            }
+            if (chain) {
                 pieces = 0;
             } else {
                 for (int i = 0; i < 24; ++i) {
@@ -1197,6 +1205,7 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
                     slack = 0.125 * i;
                     limit = 1e9;
                 }
+                if (slack == 1e9) pieces = 0;
             }
             cost += rounds * 1.5;
             if (best >= 0.0 && cost >= best) continue;
@@ -1215,23 +1224,34 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     for (int r = 0; r < rounds; ++r)
         if (1ll * (r + 1) * p.w_rounds / rounds > 1ll * r * p.w_rounds / rounds) p.round_is_w |= 1ull << r;
     for (int q = P + 1; q <= kMaxPairs; ++q) p.w_tail_begin[q] = static_cast<int>(best_total);
+    p.w_whole = p.w_kbc == p.w_kblocks;
+    for (int q = 0; q < P; ++q) p.w_whole &= p.w_tail_begin[q] % p.w_kbc == 0;
     return NB_OK;
 }
 
 // The plan of a launch. Finding one takes 60 to 300 us, so the plans of the last sizes are kept (they hold sizes only).
-int cached_layer_bwd_plan(DeviceState &s, LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad)
+int cached_layer_bwd_plan(DeviceState &s, LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad, bool fresh)
 {
-    const PlanKey key{BT, C, OC, P, gelu_grad};
+    const PlanKey key{BT, C, OC, P, gelu_grad, fresh};
     const auto it = s.plans.find(key);
     if (it != s.plans.end()) {
         p = it->second;
         return NB_OK;
     }
-    const int rc = plan_layer_bwd(p, BT, C, OC, P, gelu_grad, true);
+    const int rc = plan_layer_bwd(p, BT, C, OC, P, gelu_grad, true, fresh);
     if (rc != NB_OK) return rc;
     if (s.plans.size() >= 512) s.plans.clear();
     s.plans.emplace(key, p);
     return NB_OK;
+}
+
+// Whether the launch will store a fresh dweight. (It decides for the pairs that it finds room for; where those are not
+// half the SMs this may be wrong, and the gradient is cleared once too often or by a launch of its own.)
+bool layer_bwd_stores(DeviceState &s, int64_t BT, int64_t C, int64_t OC, bool gelu_grad)
+{
+    LayerBwdParams p;
+    const int P = s.num_sms / 2 < kMaxPairs ? s.num_sms / 2 : kMaxPairs;
+    return cached_layer_bwd_plan(s, p, BT, C, OC, P, gelu_grad, true) == NB_OK && p.w_whole;
 }
 
 using LayerBwdPlain = LbCfg<false, false>;
@@ -1242,7 +1262,7 @@ using LayerBwdGeluBias = LbCfg<true, true>;
 template <class Cfg>
 int launch_layer_bwd(DeviceState &s, const void *dz, const void *weight, const void *inp, void *dinp,
                      const void *inp_pre, void *dweight, float *dbias, int64_t BT, int64_t C, int64_t OC,
-                     int accumulate, cudaStream_t stream)
+                     int accumulate, bool cleared, cudaStream_t stream)
 {
     static bool attr_set[kMaxDevices] = {};
     static int max_pairs[kMaxDevices] = {};
@@ -1270,7 +1290,7 @@ int launch_layer_bwd(DeviceState &s, const void *dz, const void *weight, const v
         attr_set[dev] = true;
     }
     LayerBwdParams p;
-    int rc = cached_layer_bwd_plan(s, p, BT, C, OC, max_pairs[dev], Cfg::GELU_GRAD);
+    int rc = cached_layer_bwd_plan(s, p, BT, C, OC, max_pairs[dev], Cfg::GELU_GRAD, !accumulate);
     if (rc != NB_OK) return rc;
     p.dbias = Cfg::DBIAS ? dbias : nullptr;
     p.status = s.status;
@@ -1283,9 +1303,10 @@ int launch_layer_bwd(DeviceState &s, const void *dz, const void *weight, const v
     if ((rc = get_tmap(s, &tDw, dweight, OC, C, 1, 32)) != NB_OK) return rc;
     tPre = tDinp;
     if (Cfg::GELU_GRAD && (rc = get_tmap(s, &tPre, inp_pre, BT, C, 0, 32)) != NB_OK) return rc;
-    // partial sums of every W unit are reduce-added, so a fresh gradient starts from zero
-    p.after_clear = accumulate ? 0 : 1;
-    if (!accumulate && (rc = launch_clear(s, dweight, OC * C, Cfg::DBIAS ? dbias : nullptr, OC, stream)) != NB_OK) return rc;
+    // partial sums of W units are reduce-added, so a fresh gradient starts from zero unless all of them are whole
+    p.store_w = !accumulate && p.w_whole;
+    p.after_clear = !accumulate && !p.store_w && !cleared;
+    if (p.after_clear && (rc = launch_clear(s, dweight, OC * C, Cfg::DBIAS ? dbias : nullptr, OC, stream)) != NB_OK) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(2 * p.num_pairs));
     cfg.blockDim = dim3(kLbThreads);
@@ -1310,14 +1331,14 @@ int launch_layer_bwd(DeviceState &s, const void *dz, const void *weight, const v
 // then issues the products one by one.
 int run_layer_bwd(DeviceState &s, const void *dz, const void *weight, const void *inp, void *dinp,
                   const void *inp_pre, void *dweight, float *dbias, int64_t BT, int64_t C, int64_t OC,
-                  int accumulate, cudaStream_t stream)
+                  int accumulate, bool cleared, cudaStream_t stream)
 {
     if (inp_pre) {
-        if (dbias) return launch_layer_bwd<LayerBwdGeluBias>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, stream);
-        return launch_layer_bwd<LayerBwdGelu>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, stream);
+        if (dbias) return launch_layer_bwd<LayerBwdGeluBias>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, cleared, stream);
+        return launch_layer_bwd<LayerBwdGelu>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, cleared, stream);
     }
-    if (dbias) return launch_layer_bwd<LayerBwdBias>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, stream);
-    return launch_layer_bwd<LayerBwdPlain>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, stream);
+    if (dbias) return launch_layer_bwd<LayerBwdBias>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, cleared, stream);
+    return launch_layer_bwd<LayerBwdPlain>(s, dz, weight, inp, dinp, inp_pre, dweight, dbias, BT, C, OC, accumulate, cleared, stream);
 }
 
 // Whether a forward product in CTA pairs runs in 192-column tiles: where it takes several waves of the pairs
@@ -1667,18 +1688,30 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
 
     // dz: either dout itself, or dout times this layer's activation derivative (workspace)
     const void *dz = dout;
+    // The pass that forms dz also clears a dweight that layer_bwd_kernel adds to, which saves that launch (4096 rows,
+    // 1024 -> 6144 SwiGLU: 106 -> 96 us with the new schedule).
+    Route r;
+    if (dweight && dweight_dtype == NB_DTYPE_F32)
+        r = route_backward(s->num_sms, dinp != nullptr, dbias != nullptr, inp_pre_act != nullptr, accumulate != 0,
+                           static_cast<int>(BT), static_cast<int>(C), static_cast<int>(OC));
+    float *clear_w = nullptr;
     if (act != NB_ACT_NONE) {
+        if (dweight && dweight_dtype == NB_DTYPE_F32 && !accumulate && r.kernel == NB_ROUTE_LAYER_BWD &&
+            !layer_bwd_stores(*s, BT, C, OC, inp_pre_act != nullptr))
+            clear_w = static_cast<float *>(dweight);
+        float *const clear_b = clear_w ? static_cast<float *>(dbias) : nullptr;
+        const long long nw = clear_w ? static_cast<long long>(OC * C) : 0, nb_ = clear_b ? static_cast<long long>(OC) : 0;
         if ((rc = ensure_workspace(*s, static_cast<size_t>(BT * OC) * 2, stream)) != NB_OK) return rc;
         if (act == NB_ACT_GELU) {
             const long long nvec = BT * OC / 8;
             rc = launch_chained(gelu_backward_kernel, dim3(elementwise_grid(*s, nvec)), 256, stream,
                                 static_cast<uint4 *>(s->workspace), static_cast<const uint4 *>(dout),
-                                static_cast<const uint4 *>(pre_act), nvec);
+                                static_cast<const uint4 *>(pre_act), nvec, clear_w, nw, clear_b, nb_);
         } else {
             const int hvec = static_cast<int>(OC / 16);
             rc = launch_chained(swiglu_backward_kernel, dim3(elementwise_grid(*s, BT * hvec)), 256, stream,
                                 static_cast<uint4 *>(s->workspace), static_cast<const uint4 *>(dout),
-                                static_cast<const uint4 *>(pre_act), BT, hvec);
+                                static_cast<const uint4 *>(pre_act), BT, hvec, clear_w, nw, clear_b, nb_);
         }
         if (rc != NB_OK) return rc;
         ++g_launches;
@@ -1701,15 +1734,13 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
         w.M = static_cast<int>(OC); w.N = static_cast<int>(C); w.K = static_cast<int>(BT);
         w.splits = 1;
         w.dbias = static_cast<float *>(dbias);
-        const Route r = route_backward(s->num_sms, dinp != nullptr, dbias != nullptr, inp_pre_act != nullptr, accumulate != 0,
-                                       d.M, d.N, w.M);
         if (r.kernel == NB_ROUTE_TILE_PAIR)
             return launch_tile_pair_plan(*s, dinp ? &d : nullptr, w, inp_pre_act != nullptr, accumulate, r.pl, stream);
         // Both products of the layer in one launch (the usual case of a training step): the weight
         // gradient's k-blocks fill the waves the input gradient's tiles leave partly empty.
         if (r.kernel == NB_ROUTE_LAYER_BWD) {
             rc = run_layer_bwd(*s, dz, weight, inp, dinp, inp_pre_act, dweight, static_cast<float *>(dbias), BT, C,
-                               OC, accumulate, stream);
+                               OC, accumulate, clear_w != nullptr, stream);
             if (rc != NB_ERR_UNSUPPORTED) return rc;
         }
     }
@@ -2092,7 +2123,8 @@ int nb_debug_layer_bwd_plan(int64_t BT, int64_t C, int64_t OC, int pairs, int fl
 {
     if (!out || cap < 8 || BT <= 0 || C <= 0 || OC <= 0) return -fail(NB_ERR_INVALID_ARG, "bad argument");
     LayerBwdParams p;
-    const int rc = plan_layer_bwd(p, BT, C, OC, pairs, (flags & NB_PLAN_GELU_GRAD) != 0, (flags & NB_PLAN_LAUNCHED) != 0);
+    const int rc = plan_layer_bwd(p, BT, C, OC, pairs, (flags & NB_PLAN_GELU_GRAD) != 0, (flags & NB_PLAN_LAUNCHED) != 0,
+                                  (flags & NB_PLAN_FRESH) != 0);
     if (rc != NB_OK) return -rc;
     out[0] = p.d_tiles_m; out[1] = p.d_tiles_n; out[2] = p.d_kblocks;
     out[3] = p.w_tiles_m; out[4] = p.w_tiles_n; out[5] = p.w_kblocks;
@@ -2149,7 +2181,7 @@ int nb_debug_route(int call, int64_t BT, int64_t C, int64_t OC, int64_t r, int a
             tiles(t.kernel, t.pl);
         } else if (t.kernel == NB_ROUTE_LAYER_BWD) {
             LayerBwdParams p;
-            const int rc = plan_layer_bwd(p, BT, C, OC, sms / 2 < kMaxPairs ? sms / 2 : kMaxPairs, gelu, true);
+            const int rc = plan_layer_bwd(p, BT, C, OC, sms / 2 < kMaxPairs ? sms / 2 : kMaxPairs, gelu, true, !accumulate);
             if (rc != NB_OK) return -rc;
             put(t.kernel, p.d_w, 1, 1);
         } else {
@@ -2264,7 +2296,7 @@ int nb_gelu_dbias_noalloc(void *dbias, const void *dout, const void *pre_act, in
         const long long nvec = BT * OC / 8;
         const int rc = launch_chained(gelu_backward_kernel, dim3(elementwise_grid(local, nvec)), 256, stream,
                                       static_cast<uint4 *>(dz), static_cast<const uint4 *>(dout),
-                                      static_cast<const uint4 *>(pre_act), nvec);
+                                      static_cast<const uint4 *>(pre_act), nvec, nullptr, 0, nullptr, 0);
         if (rc != NB_OK) return rc;
         ++g_launches;
     }

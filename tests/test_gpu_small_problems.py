@@ -313,3 +313,32 @@ def test_adapter_forms(BT, C, OC, r, down, up, back):
         got = nb.nb_debug_route(nb.CALL_LORA_BACKWARD, BT, C, OC, r=r, accumulate=accumulate)
         assert [k[0] for k in got] == back, got
     test_small_adapter_layer(BT, C, OC, r)
+
+
+@pytest.mark.parametrize("act,BT,C,OC,whole", [
+    (nb.ACT_NONE, 1500, 1000, 1544, True),      # every unit of dweight is a tile's whole K: stored, nothing cleared
+    (nb.ACT_NONE, 1290, 1032, 4104, True), (nb.ACT_NONE, 2050, 520, 3080, True),  # ragged tiles, one k-block past 32
+    (nb.ACT_NONE, 1300, 2056, 1032, False),     # cut: cleared by a launch of its own
+    (nb.ACT_GELU, 1300, 2056, 1032, False), (nb.ACT_SWIGLU, 1300, 2056, 1040, False),  # cleared with the activation's pass
+    (nb.ACT_GELU, 1290, 1032, 4104, True),
+])
+def test_fresh_gradients_of_the_persistent_backward(act, BT, C, OC, whole):
+    """dweight and dbias start from nothing (over what the buffers held), then a second call adds to them."""
+    route = nb.nb_debug_route(nb.CALL_BACKWARD, BT, C, OC, act=act, accumulate=False)
+    assert route[0][0] == "layer_bwd", route
+    hdr, recs = nb.nb_debug_layer_bwd_plan(BT, C, OC, torch.cuda.get_device_properties(0).multi_processor_count // 2, False,
+                                           launched=True, fresh=True)
+    assert all(k1 - k0 == hdr[5] for _, is_w, _, _, k0, k1 in recs if is_w) == whole
+    inp, w, dout = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (BT, OC // 2 if act == nb.ACT_SWIGLU else OC), 1e-3)
+    pre = gen(4, (BT, OC), 1.0) if act else None
+    r = oracle.linear_backward(f32(dout), f32(inp), f32(w), pre=f32(pre) if act else None, act=act)
+    dinp = Guarded((BT, C), torch.bfloat16)
+    dw, db = Guarded((OC, C), torch.float32, fill=7.0), Guarded((OC,), torch.float32, fill=float("nan"))
+    for acc in range(2):
+        nb.nb_linear_backward_ex(dinp.t, dw.t, db.t, dout, inp, w, pre, None, BT, C, OC, act, acc)
+        check_bf16(dinp.t, r["dinp"], "dinp")
+        check_f32(dw.t, (acc + 1) * r["dweight"], "dweight")
+        check_f32(db.t, (acc + 1) * r["dbias"], "dbias")
+    for g, n in ((dinp, "dinp"), (dw, "dweight"), (db, "dbias")):
+        g.check(n)
+    nb.nb_check_status()
