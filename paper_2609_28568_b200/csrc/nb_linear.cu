@@ -1144,7 +1144,8 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     for (int want = 1; want <= max_chunks; ++want) {
         const int kbc = (p.w_kblocks + want - 1) / want;
         const int chunks = (p.w_kblocks + kbc - 1) / kbc;
-        if (chunks != want || (want < max_chunks && kbc > kMaxChunk)) continue;  // the same length again
+        // the same length again, or one that is too long (the shortest is always tried: it may be both)
+        if (want < max_chunks && (chunks != want || kbc > kMaxChunk)) continue;
         const long long w_units = 1ll * chunks * p.w_tiles;
         if (w_units >= (1ll << 24)) break;
         // the units of the last chunk may be shorter than the others: they all stay in the tail, where lengths are

@@ -184,6 +184,32 @@ def test_layer_backward_plan_on_drawn_shapes(L):
     assert declined < 100   # the drawn set mostly exercises the planner, not its refusal
 
 
+def _check_partition(hdr, recs, pairs, tag):
+    """Every dinp tile once over its whole K, every (dweight tile, k-block) exactly once."""
+    import numpy as np
+    dtm, dtn, dkb, wtm, wtn, wkb, _, rounds = hdr
+    assert rounds <= 64, tag
+    d_seen, w_cov = np.zeros((dtm, dtn), dtype=np.int64), np.zeros((wtm, wtn, wkb), dtype=np.int64)
+    for pr, is_w, m, n, kb0, kb1 in recs:
+        assert 0 <= pr < pairs and 0 <= kb0 < kb1, tag
+        if is_w:
+            assert kb1 <= wkb, tag
+            w_cov[m, n, kb0:kb1] += 1
+        else:
+            assert (kb0, kb1) == (0, dkb), tag
+            d_seen[m, n] += 1
+    assert (d_seen == 1).all() and (w_cov == 1).all(), tag
+
+
+@pytest.mark.parametrize("fresh", [False, True])
+@pytest.mark.parametrize("BT,C,OC", [(303169, 256, 512), (606272, 256, 256), (309000, 256, 512)])
+def test_layer_backward_plan_where_no_chunk_count_gives_short_chunks(L, BT, C, OC, fresh):
+    """Many rows of a narrow layer: the largest number of chunks rounds to fewer, and all smaller ones leave chunks
+    longer than 64 k-blocks. Such a size is planned all the same."""
+    hdr, recs = binding.nb_debug_layer_bwd_plan(BT, C, OC, 74, False, launched=True, fresh=fresh)
+    _check_partition(hdr, recs, 74, (BT, C, OC, fresh))
+
+
 def test_layer_backward_plan_with_halved_dinp_tiles(L):
     """A few dinp tiles over a long K are 128 columns wide in the launch's own plan: they
     partition the work like whole ones. At most a quarter of the pairs as whole tiles, at least 36 and 12 + two a tile of
