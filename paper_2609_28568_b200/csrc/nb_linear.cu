@@ -1089,6 +1089,66 @@ LbCut cut_line(const LbLine &l, int P, int d_tail, double fixed_tail, double lim
     return c;
 }
 
+// A schedule of the W units for the geometry that p holds, found in one pass: about two of them a pair, none shorter than 32
+// k-blocks, and ranges of the line that each level the cost of the pairs still to be served (k-blocks and 3 a unit, 8 for a D unit with
+// gelu'), ending at a multiple of four k-blocks of a unit or at its end. W rounds are taken back until the pairs with a tail D
+// tile have a range as well. It says which sizes have a schedule (more rounds than the order mask holds: none).
+int level_layer_bwd(LayerBwdParams &p, bool gelu_grad)
+{
+    constexpr double eW = 3.0;
+    const int P = p.num_pairs;
+    const double cD = p.d_kblocks * (p.d_w == 128 ? kNarrowD : 1.0) + (gelu_grad ? 8 : 3);
+    int chunks = (2 * P + p.w_tiles - 1) / p.w_tiles;
+    const int max_chunks = p.w_kblocks / 32 > 1 ? p.w_kblocks / 32 : 1;
+    if (chunks > max_chunks) chunks = max_chunks;
+    p.w_kbc = (p.w_kblocks + chunks - 1) / chunks;
+    chunks = (p.w_kblocks + p.w_kbc - 1) / p.w_kbc;
+    const long long w_units = 1ll * chunks * p.w_tiles;
+    if (w_units >= (1ll << 24)) return fail(NB_ERR_UNSUPPORTED, "too many work units");
+    p.w_units = static_cast<int>(w_units);
+    p.w_last_len = p.w_kblocks - (chunks - 1) * p.w_kbc;
+    const int even_units = p.w_last_len == p.w_kbc ? p.w_units : p.w_units - p.w_tiles;
+    const long long ragged = 1ll * (p.w_units - even_units) * p.w_last_len;
+    long long full = 0;
+    for (p.w_rounds = even_units / P;; --p.w_rounds) {
+        full = 1ll * (even_units - p.w_rounds * P) * p.w_kbc;
+        const double mean = static_cast<double>(full + ragged) / P;
+        if (p.w_rounds == 0 || (p.d_tail == 0 ? full + ragged == 0 || mean >= 8.0 : mean + cD * p.d_tail / P - cD >= 8.0)) break;
+    }
+    const long long total = full + ragged;
+    if (total >= (1ll << 30)) return fail(NB_ERR_UNSUPPORTED, "weight-gradient tail too long");
+    if (p.d_rounds + p.w_rounds > kLbMaxRounds) return fail(NB_ERR_UNSUPPORTED, "more than %d rounds", kLbMaxRounds);
+    p.w_tail_full = static_cast<int>(full);
+    long long x = 0, units = p.w_units - 1ll * p.w_rounds * P;  // still on the line, the one that x is in among them
+    long long left = full > 0 ? p.w_kbc : p.w_last_len;         // of that one
+    for (int q = 0; q < P; ++q) {
+        p.w_tail_begin[q] = static_cast<int>(x);
+        const double line_cost = static_cast<double>(total - x) + eW * static_cast<double>(units + P - q - 1);
+        double rem = (line_cost + cD * (p.d_tail > q ? p.d_tail - q : 0)) / (P - q) - (q < p.d_tail ? cD : 0.0);
+        while (x < total && rem >= eW + 4) {
+            const int unit = x < full ? p.w_kbc : p.w_last_len;
+            if (rem - eW < static_cast<double>(left)) {
+                const long long take = static_cast<long long>(rem - eW) / 4 * 4;
+                x += take;
+                left -= take;
+                break;
+            }
+            long long n = 1;  // units that end here: this one's rest, or whole ones as many as fit
+            if (left == unit && unit >= 4) {
+                n = static_cast<long long>(rem / (eW + unit));
+                const long long have = ((x < full ? full : total) - x) / unit;
+                if (n > have) n = have;
+            }
+            x += n * left;
+            units -= n;
+            rem -= static_cast<double>(n) * (eW + static_cast<double>(left));
+            left = x < full ? p.w_kbc : p.w_last_len;
+        }
+    }
+    for (int q = P; q <= kMaxPairs; ++q) p.w_tail_begin[q] = static_cast<int>(total);
+    return NB_OK;
+}
+
 // The schedule of layer_bwd_kernel for P CTA pairs (layer_bwd_sm100.cuh describes the unit list). Costs are counted in
 // k-blocks of tensor-core time (kCostD, kCostW above); every pair should end up with the same cost.
 //  1. K = BT of the weight gradient is cut into chunks. Every number of them from one to the one that gives two W units per
@@ -1108,7 +1168,7 @@ LbCut cut_line(const LbLine &l, int P, int d_tail, double fixed_tail, double lim
 // 768 -> 3072, 18 tiles of 48 k-blocks, 18.9 -> 16.4 us; 1024 rows, 1024 -> 6144, 32.5 -> 24.4 us. With
 // more tiles the operand traffic of halved ones costs more than the shorter chain gives (2021 rows,
 // 768 -> 2304, 24 tiles: 16.0 -> 19.4 us). A 128-wide k-block is counted as 0.6 of a 256-wide one.
-// Returns NB_ERR_UNSUPPORTED when the shape needs more rounds than the order mask holds.
+// Returns NB_ERR_UNSUPPORTED when the shape needs more rounds than the order mask holds (level_layer_bwd).
 int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad, bool narrow, bool fresh)
 {
     memset(&p, 0, sizeof(p));
@@ -1135,6 +1195,9 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     p.d_rounds = p.d_tiles / P;
     p.d_tail = p.d_tiles % P;
     const double cD = p.d_kblocks * (p.d_w == 128 ? kNarrowD : 1.0) + (gelu_grad ? kCostDGelu : kCostD);
+    // stands where the search below has nothing, as for a head whose tail D tiles leave room for more rounds than there are
+    const int rc = level_layer_bwd(p, gelu_grad);
+    if (rc != NB_OK) return rc;
 
     int max_chunks = (2 * P + p.w_tiles - 1) / p.w_tiles;
     if (max_chunks > p.w_kblocks / 16) max_chunks = p.w_kblocks / 16;
@@ -1220,11 +1283,11 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
             (void)cut_line(line, P, p.d_tail, cD, limit, p.w_tail_begin, pieces, slack);
         }
     }
-    if (best < 0.0) return fail(NB_ERR_UNSUPPORTED, "more than %d rounds", kLbMaxRounds);
     const int rounds = p.d_rounds + p.w_rounds;
     for (int r = 0; r < rounds; ++r)
         if (1ll * (r + 1) * p.w_rounds / rounds > 1ll * r * p.w_rounds / rounds) p.round_is_w |= 1ull << r;
-    for (int q = P + 1; q <= kMaxPairs; ++q) p.w_tail_begin[q] = static_cast<int>(best_total);
+    if (best >= 0.0)
+        for (int q = P + 1; q <= kMaxPairs; ++q) p.w_tail_begin[q] = static_cast<int>(best_total);
     p.w_whole = p.w_kbc == p.w_kblocks;
     for (int q = 0; q < P; ++q) p.w_whole &= p.w_tail_begin[q] % p.w_kbc == 0;
     return NB_OK;

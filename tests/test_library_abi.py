@@ -210,6 +210,17 @@ def test_layer_backward_plan_where_no_chunk_count_gives_short_chunks(L, BT, C, O
     _check_partition(hdr, recs, 74, (BT, C, OC, fresh))
 
 
+@pytest.mark.parametrize("fresh", [False, True])
+@pytest.mark.parametrize("BT,C,OC", [(520, 4096, 151936), (712, 4096, 128256), (2312, 4096, 128256), (648, 8192, 65536),
+                                     (136, 12288, 50304), (776, 3072, 256000)])
+def test_layer_backward_plan_of_large_heads(L, BT, C, OC, fresh):
+    """Heads whose weight gradient has far more tiles than 64 rounds of the pairs hold: what the tail dinp tiles leave
+    room for is dealt in rounds, the rest is the line."""
+    hdr, recs = binding.nb_debug_layer_bwd_plan(BT, C, OC, 74, False, launched=True, fresh=fresh)
+    _check_partition(hdr, recs, 74, (BT, C, OC, fresh))
+    assert binding.nb_debug_route(binding.CALL_BACKWARD, BT, C, OC, accumulate=not fresh)[0][0] == "layer_bwd"
+
+
 def test_layer_backward_plan_with_halved_dinp_tiles(L):
     """A few dinp tiles over a long K are 128 columns wide in the launch's own plan: they
     partition the work like whole ones. At most a quarter of the pairs as whole tiles, at least 36 and 12 + two a tile of
