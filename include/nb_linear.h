@@ -352,7 +352,8 @@ int nb_debug_split_plan(int64_t M, int64_t N, int64_t K, int slots, int tile_m, 
  * epilogue (it makes those units dearer in the balance); NB_PLAN_LAUNCHED, the plan of the launch
  * itself, whose dinp tiles are 256 x 128 where a few whole ones over a long K would be the longest
  * chain (without it the plan in whole tiles); NB_PLAN_FRESH, dweight starts from nothing, where a
- * plan whose units are all a tile's whole K saves the clearing. out[0..7] = dinp row tiles, dinp column tiles, k-blocks of
+ * plan whose units are all a tile's whole K saves the clearing; NB_PLAN_SUMS, a record per sum of one
+ * accumulator instead of per unit (a long dweight unit is summed in parts). out[0..7] = dinp row tiles, dinp column tiles, k-blocks of
  * a dinp tile, dweight row tiles, dweight column tiles, k-blocks of K = BT, k-blocks per dweight
  * chunk, whole rounds. Then one record of six ints per unit in execution order of each pair:
  * (pair, is_dweight, row tile, column tile, first k-block, end k-block). Returns the number of
@@ -361,6 +362,7 @@ int nb_debug_split_plan(int64_t M, int64_t N, int64_t K, int slots, int tile_m, 
 #define NB_PLAN_GELU_GRAD 1
 #define NB_PLAN_LAUNCHED 2
 #define NB_PLAN_FRESH 4
+#define NB_PLAN_SUMS 8
 int nb_debug_layer_bwd_plan(int64_t BT, int64_t C, int64_t OC, int pairs, int flags, int *out,
                             int64_t cap);
 

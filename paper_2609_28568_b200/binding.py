@@ -256,15 +256,17 @@ def nb_debug_split_plan(M: int, N: int, K: int, slots: int, tile_m: int):
     return tuple(out)
 
 
-def nb_debug_layer_bwd_plan(BT: int, C: int, OC: int, pairs: int, gelu_grad: bool, launched: bool = False, fresh: bool = False):
+def nb_debug_layer_bwd_plan(BT: int, C: int, OC: int, pairs: int, gelu_grad: bool, launched: bool = False, fresh: bool = False,
+                            sums: bool = False):
     """(header of eight ints, list of (pair, is_dweight, row tile, column tile, kb0, kb1)) of the
     one-launch layer backward; raises NbError for shapes its schedule does not cover. launched: with
-    dinp tiles as wide as the launch has them, else in whole ones; fresh: for gradients that start from nothing."""
+    dinp tiles as wide as the launch has them, else in whole ones; fresh: for gradients that start from nothing; sums: the k-blocks that one accumulator
+    sums are a record, not a unit's."""
     cap = 8 + 6 * (4 * pairs + 64 + 2 * (-(-BT // 256)) * (-(-C // 256))
-                   + 2 * (-(-OC // 256)) * (-(-C // 256)) * max(1, BT // 1024))
+                   + 2 * (-(-OC // 256)) * (-(-C // 256)) * max(1, BT // 1024)) * (8 if sums else 1)
     out = (_int * cap)()
-    n = lib().nb_debug_layer_bwd_plan(BT, C, OC, pairs, int(bool(gelu_grad)) + 2 * int(bool(launched)) + 4 * int(bool(fresh)),
-                                      out, cap)
+    n = lib().nb_debug_layer_bwd_plan(BT, C, OC, pairs, int(bool(gelu_grad)) + 2 * int(bool(launched)) + 4 * int(bool(fresh))
+                                      + 8 * int(bool(sums)), out, cap)
     if n < 0:
         raise NbError(-n, lib().nb_last_error().decode())
     recs = [tuple(out[8 + 6 * i: 14 + 6 * i]) for i in range(n)]

@@ -46,6 +46,7 @@ struct LayerBwdParams {
     // of tile j % w_tiles
     int w_tiles_m, w_tiles_n, w_tiles, w_kblocks, w_kbc, w_units;
     int w_rounds;  // full rounds (num_pairs units each)
+    int w_chain;   // k-blocks of a W unit that one accumulator sums at most (chain_len)
     unsigned long long round_is_w;  // order of the d_rounds + w_rounds full rounds, bit r: W round
     // what is left of the W units after the full rounds, as one line of k-blocks: w_kbc per unit for
     // the first w_tail_full k-blocks, then w_last_len per unit (the units of the last chunk, when K
@@ -67,6 +68,20 @@ struct LbUnit {
     int m_blk, n_blk;
     int kb0, kb1;
 };
+
+// The tensor core's fp32 accumulator drops what a sum's last bit cannot hold instead of rounding it, so the error of a long sum
+// grows with its length, and all of it towards zero: an fp32 dweight over 4096 rows is off by 1.7e-6 (2-norm, standard normal
+// operands) where most of it is summed 32 k-blocks at a time and by 3.4e-6 where 64 at a time. So a W unit that is longer than the
+// plan's w_chain is summed in equal parts, in the two accumulators in turn, and the epilogue adds the parts in registers, rounding
+// to nearest, while the next part is being multiplied. Reading 128 KB of TMEM once more costs the tensor core 0.15 us a part
+// (every unit in four parts: 3.5 % of a launch), so the plan takes no more of them than it needs.
+__host__ __device__ __forceinline__ int chain_len(const LbUnit &u, int w_chain)
+{
+    const int len = u.kb1 - u.kb0;
+    if (!u.is_w || len <= w_chain) return len;
+    const int parts = (len + w_chain - 1) / w_chain;
+    return (len + parts - 1) / parts;
+}
 
 // The sequence of units of one CTA pair; every role of both CTAs walks the same sequence.
 struct LbIter {
@@ -325,44 +340,48 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                 uint32_t acc_phase = 0;
                 bool ok = true;
                 while (ok && it.next(p, u)) {
-                    ok = wait_barrier(wctx, tempty_bar(acc), acc_phase ^ 1u, 200 + acc);
-                    if (!ok) break;
-                    ptx::tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * 256);
+                    const int chain = chain_len(u, p.w_chain);
                     const uint32_t idesc = u.is_w ? idesc_w : idesc_d;
                     // K-major A (D unit): 16 k = 32 B inside the swizzle row; MN-major: 16 k = 2048 B
                     const uint32_t a_step = u.is_w ? (2048u >> 4) : (32u >> 4);
                     const bool mine = DBIAS && u.is_w && u.n_blk == 0;
-                    for (int kb = u.kb0; kb < u.kb1; ++kb) {
-                        ok = wait_barrier(wctx, full_bar(stage), phase, 300 + stage);
+                    for (int c0 = u.kb0; c0 < u.kb1; c0 += chain) {
+                        const int c1 = LbIter::imin(c0 + chain, u.kb1);
+                        ok = wait_barrier(wctx, tempty_bar(acc), acc_phase ^ 1u, 200 + acc);
                         if (!ok) break;
                         ptx::tc_fence_after();
-                        const uint32_t sa = smem + Cfg::OFF_A + stage * Cfg::A_BYTES;
-                        const uint32_t sb = smem + Cfg::OFF_B + stage * Cfg::B_BYTES;
-                        const uint64_t adesc = u.is_w ? make_smem_desc(sa, 8192, 1024)
-                                                      : make_smem_desc(sa, 16, 1024);
-                        const uint64_t bdesc = make_smem_desc(sb, 8192, 1024);
+                        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * 256);
+                        for (int kb = c0; kb < c1; ++kb) {
+                            ok = wait_barrier(wctx, full_bar(stage), phase, 300 + stage);
+                            if (!ok) break;
+                            ptx::tc_fence_after();
+                            const uint32_t sa = smem + Cfg::OFF_A + stage * Cfg::A_BYTES;
+                            const uint32_t sb = smem + Cfg::OFF_B + stage * Cfg::B_BYTES;
+                            const uint64_t adesc = u.is_w ? make_smem_desc(sa, 8192, 1024)
+                                                          : make_smem_desc(sa, 16, 1024);
+                            const uint64_t bdesc = make_smem_desc(sb, 8192, 1024);
 #pragma unroll
-                        for (int k = 0; k < kBlockK / kUmmaK; ++k) {
-                            ptx::umma_bf16<2>(d_tmem, adesc + static_cast<uint64_t>(k * a_step),
-                                              bdesc + static_cast<uint64_t>(k * (2048u >> 4)), idesc,
-                                              (kb > u.kb0 || k > 0) ? 1u : 0u);
+                            for (int k = 0; k < kBlockK / kUmmaK; ++k) {
+                                ptx::umma_bf16<2>(d_tmem, adesc + static_cast<uint64_t>(k * a_step),
+                                                  bdesc + static_cast<uint64_t>(k * (2048u >> 4)), idesc,
+                                                  (kb > c0 || k > 0) ? 1u : 0u);
+                            }
+                            // Without reducers the producer waits on empty[s]. With them it waits on
+                            // free[s], which a stage they do not read gets from here and a stage they
+                            // read gets from them; empty[s] then counts only the uses they read.
+                            if (!DBIAS || mine) ptx::umma_commit<2>(empty_bar(stage));
+                            else ptx::umma_commit<2>(free_bar(stage));
+                            if (++stage == STAGES) {
+                                stage = 0;
+                                phase ^= 1u;
+                            }
                         }
-                        // Without reducers the producer waits on empty[s]. With them it waits on
-                        // free[s], which a stage they do not read gets from here and a stage they
-                        // read gets from them; empty[s] then counts only the uses they read.
-                        if (!DBIAS || mine) ptx::umma_commit<2>(empty_bar(stage));
-                        else ptx::umma_commit<2>(free_bar(stage));
-                        if (++stage == STAGES) {
-                            stage = 0;
-                            phase ^= 1u;
+                        if (!ok) break;
+                        ptx::umma_commit<2>(tfull_bar(acc));
+                        if (++acc == 2) {
+                            acc = 0;
+                            acc_phase ^= 1u;
                         }
-                    }
-                    if (!ok) break;
-                    ptx::umma_commit<2>(tfull_bar(acc));
-                    if (++acc == 2) {
-                        acc = 0;
-                        acc_phase ^= 1u;
                     }
                 }
             }
@@ -493,12 +512,15 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                 const int tw = u.is_w ? 256 : p.d_w;
                 const int nw = u.n_blk * tw + hf * (tw / 2);  // this warp's first column
                 bool ok = true;
-                if (lane == 0) ok = wait_barrier(wctx_epi, tfull_bar(acc), acc_phase, 400 + acc);
-                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                if (!ok) ptx::st_shared_u32_volatile(epi_abort_addr, 1);
-                ptx::tc_fence_after();
-                const uint32_t t_acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
-                                       static_cast<uint32_t>(acc * 256 + hf * (tw / 2));
+                // waits for the accumulator `acc`; where this warp's part of it starts
+                auto accumulated = [&]() {
+                    if (lane == 0 && ok) ok = wait_barrier(wctx_epi, tfull_bar(acc), acc_phase, 400 + acc);
+                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                    if (!ok) ptx::st_shared_u32_volatile(epi_abort_addr, 1);
+                    ptx::tc_fence_after();
+                    return tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(acc * 256 + hf * (tw / 2));
+                };
+                uint32_t t_acc = accumulated();
                 uint32_t rr[4][32];
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
@@ -513,6 +535,26 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                 release_acc(acc);  // the accumulator is in registers
 
                 if (u.is_w) {
+                    // the sums over the rest of the unit's K, added to the first one's
+                    const int chain = chain_len(u, p.w_chain);
+                    for (int c0 = u.kb0 + chain; c0 < u.kb1; c0 += chain) {
+                        if (++acc == 2) {
+                            acc = 0;
+                            acc_phase ^= 1u;
+                        }
+                        t_acc = accumulated();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {  // 16 columns at a time: 32 would spill
+                            uint32_t more[16];
+                            ptx::tmem_ld_32x16_wait(t_acc + static_cast<uint32_t>(i * 16), more);
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                uint32_t &sum = rr[i >> 1][(i & 1) * 16 + j];
+                                sum = __float_as_uint(__uint_as_float(sum) + __uint_as_float(more[j]));
+                            }
+                        }
+                        release_acc(acc);
+                    }
                     // ---------------- fp32 tile of dweight: 32-column boxes, reduce-added (whole ones of a fresh one stored)
 #pragma unroll
                     for (int s4 = 0; s4 < 4; ++s4) {

@@ -1149,6 +1149,65 @@ int level_layer_bwd(LayerBwdParams &p, bool gelu_grad)
     return NB_OK;
 }
 
+// What the error of a schedule's weight gradient goes with: the squares of the lengths of its sums (products of one sign, whose
+// running sum grows with the length) and their cubes (products of either sign, where it grows with the root of it), each as
+// often as the tile has elements of dweight.
+struct LbSums {
+    double squares = 0.0, cubes = 0.0;
+    int longest = 0;
+    void add(int len, double elements)
+    {
+        squares += elements * len * len;
+        cubes += elements * len * len * len;
+        if (len > longest) longest = len;
+    }
+    // (with room for tiles that are cut differently: alike in both sums, errors measured up to 1.2 of each other)
+    bool no_worse_than(const LbSums &o) const
+    {
+        return squares <= 0.85 * o.squares && cubes <= 0.75 * o.cubes && longest <= o.longest;
+    }
+};
+LbSums sums_of(const LayerBwdParams &p, int w_chain)
+{
+    LbSums s;
+    // elements of the tiles of the units before j, in order
+    auto elements_to = [&](long long j) {
+        const long long t = j % p.w_tiles, m = t / p.w_tiles_n, n = t % p.w_tiles_n;
+        const long long rows = p.OC - 256 * m < 256 ? p.OC - 256 * m : 256;
+        return static_cast<double>(j / p.w_tiles) * p.OC * p.C + static_cast<double>(256 * m) * p.C +
+               static_cast<double>(rows * (256 * n < p.C ? 256 * n : p.C));
+    };
+    long long j = 0;  // the unit that the line is in, after the rounds' units
+    auto piece = [&](int len, long long units) {
+        const LbUnit u{1, 0, 0, 0, len};
+        const int part = chain_len(u, w_chain);
+        const double elements = elements_to(j + units) - elements_to(j);
+        s.add(part, elements * (len / part));
+        if (len % part) s.add(len % part, elements);
+    };
+    if (p.w_rounds) piece(p.w_kbc, 1ll * p.w_rounds * p.num_pairs);
+    j += 1ll * p.w_rounds * p.num_pairs;
+    int left = p.w_tail_full > 0 ? p.w_kbc : p.w_last_len;  // of the unit
+    for (int q = 0, x = 0; q < p.num_pairs; ++q) {
+        while (x < p.w_tail_begin[q + 1]) {
+            const int unit = x < p.w_tail_full ? p.w_kbc : p.w_last_len;
+            int end = p.w_tail_begin[q + 1];
+            if (x < p.w_tail_full && end > p.w_tail_full) end = p.w_tail_full;
+            const int len = left < end - x ? left : end - x;
+            const int n = left == unit && end - x > unit ? (end - x) / unit : 1;
+            piece(len, n);
+            x += n * len;
+            if (len < left) {
+                left -= len;
+            } else {
+                j += n;
+                left = x < p.w_tail_full ? p.w_kbc : p.w_last_len;
+            }
+        }
+    }
+    return s;
+}
+
 // The schedule of layer_bwd_kernel for P CTA pairs (layer_bwd_sm100.cuh describes the unit list). Costs are counted in
 // k-blocks of tensor-core time (kCostD, kCostW above); every pair should end up with the same cost.
 //  1. K = BT of the weight gradient is cut into chunks. Every number of them from one to the one that gives two W units per
@@ -1198,6 +1257,7 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     // stands where the search below has nothing, as for a head whose tail D tiles leave room for more rounds than there are
     const int rc = level_layer_bwd(p, gelu_grad);
     if (rc != NB_OK) return rc;
+    const LbSums level = sums_of(p, p.w_kblocks);
 
     int max_chunks = (2 * P + p.w_tiles - 1) / p.w_tiles;
     if (max_chunks > p.w_kblocks / 16) max_chunks = p.w_kblocks / 16;
@@ -1290,6 +1350,13 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
         for (int q = P + 1; q <= kMaxPairs; ++q) p.w_tail_begin[q] = static_cast<int>(best_total);
     p.w_whole = p.w_kbc == p.w_kblocks;
     for (int q = 0; q < P; ++q) p.w_whole &= p.w_tail_begin[q] % p.w_kbc == 0;
+    // as few parts as leave dweight no less exact than the levelled schedule
+    const int longest = sums_of(p, p.w_kblocks).longest;
+    p.w_chain = longest;
+    for (int parts = 1; best >= 0.0; ++parts) {
+        p.w_chain = (longest + parts - 1) / parts;
+        if (p.w_chain <= 1 || sums_of(p, p.w_chain).no_worse_than(level)) break;
+    }
     return NB_OK;
 }
 
@@ -2199,10 +2266,13 @@ int nb_debug_layer_bwd_plan(int64_t BT, int64_t C, int64_t OC, int pairs, int fl
         LbIter it(p, q);
         LbUnit u;
         while (it.next(p, u)) {
-            if (n + 6 > cap) return -fail(NB_ERR_INVALID_ARG, "output buffer too small");
-            out[n++] = q; out[n++] = u.is_w; out[n++] = u.m_blk; out[n++] = u.n_blk;
-            out[n++] = u.kb0; out[n++] = u.kb1;
-            ++records;
+            const int part = flags & NB_PLAN_SUMS ? chain_len(u, p.w_chain) : u.kb1 - u.kb0;
+            for (int kb = u.kb0; kb < u.kb1; kb += part) {
+                if (n + 6 > cap) return -fail(NB_ERR_INVALID_ARG, "output buffer too small");
+                out[n++] = q; out[n++] = u.is_w; out[n++] = u.m_blk; out[n++] = u.n_blk;
+                out[n++] = kb; out[n++] = LbIter::imin(kb + part, u.kb1);
+                ++records;
+            }
         }
     }
     return records;

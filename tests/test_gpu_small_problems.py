@@ -342,3 +342,25 @@ def test_fresh_gradients_of_the_persistent_backward(act, BT, C, OC, whole):
     for g, n in ((dinp, "dinp"), (dw, "dweight"), (db, "dbias")):
         g.check(n)
     nb.nb_check_status()
+
+
+@pytest.mark.parametrize("BT,C,OC", [(4096, 768, 3072), (8192, 768, 3072), (5000, 776, 2056)])
+def test_long_sums_of_the_persistent_backward(BT, C, OC):
+    """The error of a sum in a tensor core's accumulator goes with its length, and the schedule promises sums of at most 32
+    k-blocks at these sizes: dweight is at most twice as far from its value in 64 bits as when the same rows are
+    added up 1024 at a time, in sums of 16 (by a kernel that does not cut K)."""
+    for rows, accumulate, kernel in ((BT, False, "layer_bwd"), (1024, False, "tile_pair"), (1024, True, "tile_pair")):
+        assert nb.nb_debug_route(nb.CALL_BACKWARD, rows, C, OC, dbias=False, accumulate=accumulate)[0][0] == kernel
+    inp, w, dout = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (BT, OC), 1e-3)
+    ref = dout.double().t() @ inp.double()
+    dinp = torch.empty((BT, C), dtype=torch.bfloat16, device="cuda")
+    error = {}
+    for rows in (BT, 1024):
+        dw = torch.empty((OC, C), dtype=torch.float32, device="cuda")
+        for m in range(0, BT, rows):
+            n = min(rows, BT - m)
+            nb.nb_linear_backward_ex(dinp[m:m + n], dw, None, dout[m:m + n], inp[m:m + n], w, None, None, n, C, OC, nb.ACT_NONE,
+                                     int(m > 0))
+        error[rows] = float((dw.double() - ref).norm() / ref.norm())
+    nb.nb_check_status()
+    assert error[BT] <= 2 * error[1024], error

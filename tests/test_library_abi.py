@@ -202,6 +202,21 @@ def _check_partition(hdr, recs, pairs, tag):
 
 
 @pytest.mark.parametrize("fresh", [False, True])
+@pytest.mark.parametrize("gelu", [False, True])
+def test_sums_of_the_layer_backward_plan(L, gelu, fresh):
+    """An accumulator loses accuracy with the length of its sum. No sum of dweight is longer than the chunks of the one-pass
+    schedule are, about two units a pair of at least 32 k-blocks, and the sums are as good a partition as the units."""
+    for BT, C, OC in [(4096, 768, 2304), (4096, 768, 3072), (4096, 3072, 768), (4096, 1024, 6144), (4096, 3072, 1024), (2021, 768, 3072),
+                      (2021, 768, 50304), (8192, 768, 3072), (16384, 768, 768), (16384, 768, 3072), (1500, 1000, 1544), (65536, 768, 768),
+                      (2826, 240, 2040), (9000, 136, 264)]:
+        tiles, wkb = -(-OC // 256) * -(-C // 256), -(-BT // 64)
+        chunks = min(-(-148 // tiles), max(1, wkb // 32))
+        hdr, recs = binding.nb_debug_layer_bwd_plan(BT, C, OC, 74, gelu, launched=True, fresh=fresh, sums=True)
+        _check_partition(hdr, recs, 74, (BT, C, OC, gelu, fresh))
+        assert max(kb1 - kb0 for _, is_w, _, _, kb0, kb1 in recs if is_w) <= -(-wkb // chunks), (BT, C, OC, gelu, fresh)
+
+
+@pytest.mark.parametrize("fresh", [False, True])
 @pytest.mark.parametrize("BT,C,OC", [(303169, 256, 512), (606272, 256, 256), (309000, 256, 512)])
 def test_layer_backward_plan_where_no_chunk_count_gives_short_chunks(L, BT, C, OC, fresh):
     """Many rows of a narrow layer: the largest number of chunks rounds to fewer, and all smaller ones leave chunks
