@@ -537,7 +537,7 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                 if (u.is_w) {
                     // the sums over the rest of the unit's K, added to the first one's
                     const int chain = chain_len(u, p.w_chain);
-                    for (int c0 = u.kb0 + chain; c0 < u.kb1; c0 += chain) {
+                    for (int c0 = u.kb0 + chain; __builtin_expect(c0 < u.kb1, 0); c0 += chain) {
                         if (++acc == 2) {
                             acc = 0;
                             acc_phase ^= 1u;
@@ -548,9 +548,11 @@ layer_bwd_kernel(const __grid_constant__ CUtensorMap tmDz,    // dz   [BT, OC] b
                             uint32_t more[16];
                             ptx::tmem_ld_32x16_wait(t_acc + static_cast<uint32_t>(i * 16), more);
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) {
-                                uint32_t &sum = rr[i >> 1][(i & 1) * 16 + j];
-                                sum = __float_as_uint(__uint_as_float(sum) + __uint_as_float(more[j]));
+                            for (int j = 0; j < 16; j += 2) {
+                                uint32_t &lo = rr[i >> 1][(i & 1) * 16 + j], &hi = rr[i >> 1][(i & 1) * 16 + j + 1];
+                                const ptx::f2 t = ptx::add2(ptx::make_f2_bits(lo, hi), ptx::make_f2_bits(more[j], more[j + 1]));
+                                lo = static_cast<uint32_t>(t.v);
+                                hi = static_cast<uint32_t>(t.v >> 32);
                             }
                         }
                         release_acc(acc);
