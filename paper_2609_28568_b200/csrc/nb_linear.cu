@@ -1028,6 +1028,7 @@ bool layer_bwd_narrow(int d_tiles, int d_kblocks, int w_tiles, int w_kblocks, in
 // several of them 3 to 5 us behind the others.)
 constexpr int kCostD = 1, kCostDGelu = 2, kCostW = 5;
 constexpr int kMaxChunk = 64;  // k-blocks
+constexpr int kLbTries = 4;
 constexpr int kCostClear = 8;  // the launch that clears a fresh dweight, 2.5 to 3 us on the chain
 constexpr int kMinPiece = 2;  // k-blocks of a W unit that are worth a cut
 
@@ -1036,56 +1037,50 @@ constexpr int kMinPiece = 2;  // k-blocks of a W unit that are worth a cut
 struct LbLine {
     long long total, full;
     int kbc, last;
-    long long unit_left(long long x) const  // k-blocks from x to the end of its unit
-    {
-        return x < full ? kbc - x % kbc : last - (x - full) % last;
-    }
 };
-// Cuts the line into a range per pair such that no pair's cost (fixed_tail for the first d_tail of them, a range, kCostW
-// for each unit that it touches) exceeds `limit`; ranges end at their unit's end or at least kMinPiece k-blocks from either
-// end of it, and the last pair takes what is left. begin (or null): P + 1 range borders. pieces: set to their number; where it is given (not 0), as the number that such a cut
-// makes, a pair takes no more than the mean of what is left and `slack`, so that what the limit leaves over is spread and not
-// all the last pair's.
 struct LbCut {
-    double most, least, mean;  // of the pairs' costs
+    double most = 0.0, sum = 0.0, end = 0.0;  // cost of the dearest pair, of all of them, of the last one
 };
-LbCut cut_line(const LbLine &l, int P, int d_tail, double fixed_tail, double limit, int *begin, int &pieces, double slack = 0.0)
+// Cuts the line into a range per pair (begin: P + 1 borders) such that no pair's cost (cD for the first d_tail of them, a range,
+// kCostW for each unit that it touches) exceeds `limit`; a range ends with a unit or at least kMinPiece k-blocks from either end of
+// one (whole: with a unit), and the last pair takes what is left. Units that fit whole are taken at once.
+LbCut cut_line(const LbLine &l, int P, int d_tail, double cD, double limit, bool whole, int *begin)
 {
-    long long x = 0;
-    int n = 0;
-    double carry = 0.0;  // of a k-block that the pair before this one had room for
-    LbCut c{0.0, 1e30, 0.0};
+    LbCut c;
+    long long x = 0, left = l.full > 0 ? l.kbc : l.last;  // of the unit that x is in
     for (int q = 0; q < P; ++q) {
-        if (begin) begin[q] = static_cast<int>(x);
-        double target = limit;
-        if (pieces > 0) {
-            const double mean = (static_cast<double>(l.total - x) + kCostW * (pieces > n ? pieces - n : 0) +
-                                 fixed_tail * (q < d_tail ? d_tail - q : 0)) / (P - q) + slack;
-            if (mean < target) target = mean;
-        }
-        target += carry;
-        carry = 0.0;
-        double cost = q < d_tail ? fixed_tail : 0.0;
+        begin[q] = static_cast<int>(x);
+        double cost = q < d_tail ? cD : 0.0;
+        const long long most = q == P - 1 ? 1ll << 40 : static_cast<long long>(limit - cost);
+        long long spent = 0;
         while (x < l.total) {
-            const long long left = l.unit_left(x);
-            const long long room = q == P - 1 ? left : static_cast<long long>(target - cost - kCostW);
-            long long take = room < left ? room : left;
-            if (take < left && take > left - kMinPiece) take = left - kMinPiece;
-            if (take < left && take < kMinPiece) break;
-            x += take;
-            ++n;
-            cost += kCostW + static_cast<double>(take);
-            if (take < left) {
-                carry = target - cost < 1.0 ? target - cost : 1.0;
+            const long long end = x < l.full ? l.full : l.total;
+            const int unit = x < l.full ? l.kbc : l.last;
+            const long long room = most - spent - kCostW;
+            if (room < left) {
+                const long long take = room < left - kMinPiece ? room : left - kMinPiece;
+                if (!whole && take >= kMinPiece) {
+                    x += take;
+                    left -= take;
+                    spent += kCostW + take;
+                }
                 break;
             }
+            long long n = 1;
+            if (left == unit) {
+                n = (most - spent) / (unit + kCostW);
+                if (n > (end - x) / unit) n = (end - x) / unit;
+            }
+            x += n * left;
+            spent += n * (kCostW + left);
+            left = x < l.full ? l.kbc : l.last;
         }
+        cost += static_cast<double>(spent);
         if (cost > c.most) c.most = cost;
-        if (cost < c.least) c.least = cost;
-        c.mean += cost / P;
+        c.sum += cost;
+        c.end = cost;
     }
-    if (begin) begin[P] = static_cast<int>(l.total);
-    if (pieces == 0) pieces = n;
+    begin[P] = static_cast<int>(l.total);
     return c;
 }
 
@@ -1171,22 +1166,25 @@ LbSums sums_of(const LayerBwdParams &p, int w_chain)
 {
     LbSums s;
     // elements of the tiles of the units before j, in order
-    auto elements_to = [&](long long j) {
-        const long long t = j % p.w_tiles, m = t / p.w_tiles_n, n = t % p.w_tiles_n;
-        const long long rows = p.OC - 256 * m < 256 ? p.OC - 256 * m : 256;
-        return static_cast<double>(j / p.w_tiles) * p.OC * p.C + static_cast<double>(256 * m) * p.C +
-               static_cast<double>(rows * (256 * n < p.C ? 256 * n : p.C));
+    auto elements_to = [&](unsigned j) {
+        const unsigned t = j % p.w_tiles, m = t / p.w_tiles_n, n = t % p.w_tiles_n;
+        const int rows = p.OC - 256 * static_cast<int>(m) < 256 ? p.OC - 256 * static_cast<int>(m) : 256;
+        return static_cast<double>(j / p.w_tiles) * p.OC * p.C + 256.0 * m * p.C + 256.0 * rows * n;  // (n is not the last column's end)
     };
-    long long j = 0;  // the unit that the line is in, after the rounds' units
-    auto piece = [&](int len, long long units) {
+    unsigned j = 0;  // the unit that the line is in, after the rounds' units
+    double before = 0.0;
+    auto piece = [&](int len, unsigned units, bool ends) {
         const LbUnit u{1, 0, 0, 0, len};
         const int part = chain_len(u, w_chain);
-        const double elements = elements_to(j + units) - elements_to(j);
+        const double after = elements_to(j + units), elements = after - before;
+        if (ends) {
+            before = after;
+            j += units;
+        }
         s.add(part, elements * (len / part));
         if (len % part) s.add(len % part, elements);
     };
-    if (p.w_rounds) piece(p.w_kbc, 1ll * p.w_rounds * p.num_pairs);
-    j += 1ll * p.w_rounds * p.num_pairs;
+    if (p.w_rounds) piece(p.w_kbc, static_cast<unsigned>(p.w_rounds) * p.num_pairs, true);
     int left = p.w_tail_full > 0 ? p.w_kbc : p.w_last_len;  // of the unit
     for (int q = 0, x = 0; q < p.num_pairs; ++q) {
         while (x < p.w_tail_begin[q + 1]) {
@@ -1195,14 +1193,9 @@ LbSums sums_of(const LayerBwdParams &p, int w_chain)
             if (x < p.w_tail_full && end > p.w_tail_full) end = p.w_tail_full;
             const int len = left < end - x ? left : end - x;
             const int n = left == unit && end - x > unit ? (end - x) / unit : 1;
-            piece(len, n);
+            piece(len, n, len == left);
             x += n * len;
-            if (len < left) {
-                left -= len;
-            } else {
-                j += n;
-                left = x < p.w_tail_full ? p.w_kbc : p.w_last_len;
-            }
+            left = len < left ? left - len : x < p.w_tail_full ? p.w_kbc : p.w_last_len;
         }
     }
     return s;
@@ -1210,12 +1203,12 @@ LbSums sums_of(const LayerBwdParams &p, int w_chain)
 
 // The schedule of layer_bwd_kernel for P CTA pairs (layer_bwd_sm100.cuh describes the unit list). Costs are counted in
 // k-blocks of tensor-core time (kCostD, kCostW above); every pair should end up with the same cost.
-//  1. K = BT of the weight gradient is cut into chunks. Every number of them from one to the one that gives two W units per
-//     pair is tried, of 16 to kMaxChunk k-blocks where that leaves a choice, and the one whose dearest pair is cheapest is taken.
-//  2. Whole rounds (one unit per pair) are dealt first; W rounds are spread evenly among D rounds.
-//  3. The last D round is partial: pairs [0, d_tail) take one more tile. The W units left over are laid out as one line of
-//     k-blocks and cut into P ranges at the lowest limit at which cut_line finds a place for all of it. If the line is so
-//     short that the tail D tiles alone exceed the level, a W round is taken back into it.
+//  1. Whole rounds (one unit per pair) are dealt first; W rounds are spread evenly among D rounds.
+//  2. The last D round is partial: pairs [0, d_tail) take one more tile. The W units left over are laid out as one line of
+//     k-blocks and cut into P ranges at the lowest limit on a pair's cost at which cut_line finds a place for all of it.
+//  3. K = BT of the weight gradient is cut into chunks, as many as give two W units per pair or fewer, of 16 to kMaxChunk k-blocks
+//     where that leaves a choice. For each number of chunks and each number of W rounds that leaves the pairs with a tail
+//     D tile about level, the cost of a pair is estimated; the kLbTries cheapest are cut and the one with the cheapest dearest pair is taken.
 // Against ranges levelled one after the other with 3 k-blocks a unit, over about two chunks a pair of 32 k-blocks or more
 // (chained launches, accumulating, us): 4096 rows, 768 -> 768 16.3 -> 14.1, 768 -> 2304 27.0 -> 25.5, 1024 -> 6144 77.8 -> 73.6,
 // 3072 -> 1024 42.8 -> 40.0; 8192 rows, 768 -> 768 23.5 -> 20.4; 16384 rows, 768 -> 768 38.5 -> 34.9, 768 -> 2304
@@ -1259,11 +1252,18 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     if (rc != NB_OK) return rc;
     const LbSums level = sums_of(p, p.w_kblocks);
 
+    struct Form {
+        LbLine line;
+        long long units;  // on the line
+        int chunks, rounds;
+        double estimate;  // of what it costs, in the terms of `price`, less the clearing if it may be saved
+    } forms[kLbTries];
+    int n_forms = 0;
     int max_chunks = (2 * P + p.w_tiles - 1) / p.w_tiles;
     if (max_chunks > p.w_kblocks / 16) max_chunks = p.w_kblocks / 16;
     if (max_chunks < 1) max_chunks = 1;
-    double best = -1.0;
-    long long best_total = 0;
+    // The dearest pair counts and, where the chip is at its power limit, what all of them do.
+    auto price = [&](double most, double sum, int rounds, int kbc) { return most + 0.5 * sum / P + 1.5 * rounds * (kbc + kCostW); };
     for (int want = 1; want <= max_chunks; ++want) {
         const int kbc = (p.w_kblocks + want - 1) / want;
         const int chunks = (p.w_kblocks + kbc - 1) / kbc;
@@ -1271,96 +1271,94 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
         if (want < max_chunks && (chunks != want || kbc > kMaxChunk)) continue;
         const long long w_units = 1ll * chunks * p.w_tiles;
         if (w_units >= (1ll << 24)) break;
-        // the units of the last chunk may be shorter than the others: they all stay in the tail, where lengths are
-        // counted exactly
+        // the units of the last chunk may be shorter than the others: they all stay on the line, where lengths are counted exactly
         const int last = p.w_kblocks - (chunks - 1) * kbc;
         const long long even = last == kbc ? w_units : w_units - p.w_tiles;
-        const int aW_max = static_cast<int>(even / P);
-        // as many W rounds as leave the pairs with a tail D tile below the level, give or take one
         const double mean = (1.0 * p.w_kblocks * p.w_tiles + 1.0 * kCostW * (w_units + P) + cD * p.d_tail) / P;
-        int aW_hi = p.d_tail ? static_cast<int>((mean - cD) / (kbc + kCostW)) + 1 : aW_max;
-        aW_hi = aW_hi < 0 ? 0 : aW_hi < aW_max ? aW_hi : aW_max;
-        for (int aW = aW_hi; aW >= 0 && aW >= aW_hi - 2; --aW) {
-            const long long full = (even - 1ll * aW * P) * kbc;
-            const LbLine line{full + (w_units - even) * last, full, kbc, last};
-            if (line.total >= (1ll << 30) || p.d_rounds + aW > kLbMaxRounds) continue;
-            const double rounds = 1.0 * aW * (kbc + kCostW);  // beside the D rounds, which are the same for all plans
-            // no cut costs less than this: every pair with a range pays for a piece at least, and every unit
-            const long long units = w_units - 1ll * aW * P;
-            const double floor_ = (1.0 * line.total + kCostW * static_cast<double>(units > P - p.d_tail ? units : P - p.d_tail) + cD * p.d_tail) / P;
-            if (best >= 0.0 && (rounds + floor_) * 1.5 >= best) continue;
-            double lo = floor_ - 1.0, hi = floor_ + kCostW;
-            auto fits = [&](double limit) {
-                int n = 0;
-                return cut_line(line, P, p.d_tail, cD, limit, nullptr, n).most <= (cD > limit && p.d_tail ? cD : limit) + 1.0;
-            };
-            while (!fits(hi)) hi = 1.25 * hi + kCostW;
-            while (hi - lo > 0.25) {
-                const double mid = 0.5 * (lo + hi);
-                if (fits(mid)) hi = mid;
-                else lo = mid;
-            }
-            // That cut, or one that spreads its room over the pairs. The dearest pair counts and, where the chip is at its
-            // power limit, what all of them do (each piece adds to it); a very cheap one is a share that could be others'.
-            // Where the tail D tiles are the longest chain whatever the others do, higher limits leave more units whole.
-            const bool chain = p.d_tail && cD > hi;
-            auto price = [&](const LbCut &c) { return c.most + 0.5 * c.mean + (chain ? 0.0 : (c.most - c.least) / 8); };
-            int pieces = 0;
-            double slack = 1e9, limit = hi, cost = price(cut_line(line, P, p.d_tail, cD, hi, nullptr, pieces));
-            const bool may_store = fresh && chunks == 1;
-            if (chain || may_store) {
-                const double end = may_store ? (chain ? cD : hi) + 2.0 * kCostClear : 0.9 * cD;
-                for (double at = hi; at < end; at *= 1.05) {
-                    int n = 0;
-                    double c = price(cut_line(line, P, p.d_tail, cD, at, nullptr, n));
-                    if (may_store && n == units) c -= kCostClear;
-                    if (c >= cost) continue;
-                    cost = c;
-                    limit = at;
-                }
-            }
-            if (chain) {
-                pieces = 0;
-            } else {
-                for (int i = 0; i < 24; ++i) {
-                    const double c = price(cut_line(line, P, p.d_tail, cD, 1e9, nullptr, pieces, 0.125 * i));
-                    if (c >= cost) continue;
-                    cost = c;
-                    slack = 0.125 * i;
-                    limit = 1e9;
-                }
-                if (slack == 1e9) pieces = 0;
-            }
-            cost += rounds * 1.5;
-            if (best >= 0.0 && cost >= best) continue;
-            best = cost;
-            best_total = line.total;
-            p.w_kbc = kbc;
-            p.w_units = static_cast<int>(w_units);
-            p.w_rounds = aW;
-            p.w_last_len = last;
-            p.w_tail_full = static_cast<int>(full);
-            (void)cut_line(line, P, p.d_tail, cD, limit, p.w_tail_begin, pieces, slack);
+        long long hi = even / P;
+        if (p.d_tail && static_cast<long long>((mean - cD) / (kbc + kCostW)) + 1 < hi) hi = static_cast<long long>((mean - cD) / (kbc + kCostW)) + 1;
+        if (hi > kLbMaxRounds - p.d_rounds) hi = kLbMaxRounds - p.d_rounds;
+        if (hi < 0) hi = 0;
+        for (long long aW = hi; aW >= 0 && aW >= hi - 2; --aW) {
+            Form f;
+            f.units = w_units - aW * P;
+            f.line = {(even - aW * P) * kbc + (w_units - even) * last, (even - aW * P) * kbc, kbc, last};
+            f.chunks = chunks;
+            f.rounds = static_cast<int>(aW);
+            if (f.line.total >= (1ll << 30)) break;
+            const double pieces = static_cast<double>(f.units > P - p.d_tail ? f.units : P - p.d_tail);
+            const double level = (static_cast<double>(f.line.total) + kCostW * pieces + cD * p.d_tail) / P;
+            f.estimate = price(p.d_tail && cD > level ? cD : level, level * P, f.rounds, kbc) - (fresh && chunks == 1 ? kCostClear : 0);
+            int at = n_forms < kLbTries ? n_forms++ : kLbTries;
+            for (; at > 0 && forms[at - 1].estimate > f.estimate; --at)
+                if (at < kLbTries) forms[at] = forms[at - 1];
+            if (at < kLbTries) forms[at] = f;
         }
+    }
+    double best = -1.0;
+    const Form *best_form = nullptr;
+    // cuts, keeps what is cheaper; the cost of the last pair where that has more than its share, else 0
+    auto take = [&](const Form &f, double limit, bool whole) {
+        int begin[kMaxPairs + 1];
+        const LbCut c = cut_line(f.line, P, p.d_tail, cD, limit, whole, begin);
+        if (c.end >= c.most && c.end > limit + 1.0) return c.end;
+        const double cost = price(c.most, c.sum, f.rounds, f.line.kbc) - (whole ? kCostClear : 0);
+        if (best < 0.0 || cost < best) {
+            best = cost;
+            best_form = &f;
+            for (int q = 0; q <= kMaxPairs; ++q) p.w_tail_begin[q] = begin[q < P ? q : P];
+        }
+        return 0.0;
+    };
+    for (int i = 0; i < n_forms; ++i) {
+        const Form &f = forms[i];
+        if (best >= 0.0 && f.estimate >= best) break;
+        // the lowest limit: what is too much for the last pair is spread over all of them
+        const double pieces = static_cast<double>(f.units > P - p.d_tail ? f.units : P - p.d_tail);
+        double limit = (static_cast<double>(f.line.total) + kCostW * pieces + cD * p.d_tail) / P;
+        for (double end; (end = take(f, limit, false)) > 0.0;) limit += (end - limit) / P > 0.5 ? (end - limit) / P : 0.5;
+        // where the tail D tiles are the longest chain whatever the others do, a higher limit leaves more units whole
+        if (p.d_tail && cD > limit)
+            for (double at = limit + (cD - limit) / 3; at < cD; at += (cD - limit) / 3) (void)take(f, at, false);
+        // a fresh dweight of whole tiles is not cleared: the lowest limit at which every unit has a place
+        if (fresh && f.chunks == 1) {
+            const double unit = f.line.kbc + kCostW;
+            auto held = [&](double at) {
+                return static_cast<double>(p.d_tail) * (at > cD ? floor((at - cD) / unit) : 0.0) +
+                       static_cast<double>(P - p.d_tail) * floor(at / unit);
+            };
+            double with_d = cD + unit, without = unit, at = without < with_d || !p.d_tail ? without : with_d;
+            while (held(at) < static_cast<double>(f.units)) {
+                if (at >= without) without += unit;
+                if (at >= with_d) with_d += unit;
+                at = without < with_d || !p.d_tail ? without : with_d;
+            }
+            (void)take(f, at, true);
+        }
+    }
+    if (best_form) {
+        const Form &f = *best_form;
+        p.w_kbc = f.line.kbc;
+        p.w_units = f.chunks * p.w_tiles;
+        p.w_rounds = f.rounds;
+        p.w_last_len = f.line.last;
+        p.w_tail_full = static_cast<int>(f.line.full);
+    }
+    // as few parts as leave dweight no less exact than the one-pass schedule
+    p.w_chain = sums_of(p, p.w_kblocks).longest;
+    for (int parts = 1, longest = p.w_chain; best_form; ++parts) {
+        p.w_chain = (longest + parts - 1) / parts;
+        if (p.w_chain <= 1 || sums_of(p, p.w_chain).no_worse_than(level)) break;
     }
     const int rounds = p.d_rounds + p.w_rounds;
     for (int r = 0; r < rounds; ++r)
         if (1ll * (r + 1) * p.w_rounds / rounds > 1ll * r * p.w_rounds / rounds) p.round_is_w |= 1ull << r;
-    if (best >= 0.0)
-        for (int q = P + 1; q <= kMaxPairs; ++q) p.w_tail_begin[q] = static_cast<int>(best_total);
     p.w_whole = p.w_kbc == p.w_kblocks;
     for (int q = 0; q < P; ++q) p.w_whole &= p.w_tail_begin[q] % p.w_kbc == 0;
-    // as few parts as leave dweight no less exact than the levelled schedule
-    const int longest = sums_of(p, p.w_kblocks).longest;
-    p.w_chain = longest;
-    for (int parts = 1; best >= 0.0; ++parts) {
-        p.w_chain = (longest + parts - 1) / parts;
-        if (p.w_chain <= 1 || sums_of(p, p.w_chain).no_worse_than(level)) break;
-    }
     return NB_OK;
 }
 
-// The plan of a launch. Finding one takes 60 to 300 us, so the plans of the last sizes are kept (they hold sizes only).
+// The plan of a launch. Finding one takes 5 to 20 us, so the plans of the last sizes are kept (they hold sizes only).
 int cached_layer_bwd_plan(DeviceState &s, LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad, bool fresh)
 {
     const PlanKey key{BT, C, OC, P, gelu_grad, fresh};

@@ -105,7 +105,7 @@ def test_wgrad_split_plan_covers_every_k_block_once(L):
 def test_layer_backward_plan_covers_every_unit_once(L):
     """Host logic of the one-launch layer backward: over all CTA pairs, every dinp tile appears once
     with its whole K range, and every (dweight tile, k-block) is covered exactly once, whatever
-    the interleaving and the balancing cuts; loads are level across the pairs."""
+    the interleaving and the balancing cuts; no pair is much dearer than the mean."""
     cases = [  # BT, C, OC
         (16384, 768, 2304), (16384, 768, 768), (16384, 768, 3072), (16384, 3072, 768),
         (16384, 768, 50304), (4096, 768, 3072), (4096, 3072, 768), (16384, 1024, 2048),
@@ -125,10 +125,10 @@ def test_layer_backward_plan_covers_every_unit_once(L):
                 assert 1 <= kbc <= wkb and rounds <= 64
                 d_seen = {}
                 w_cov = {}
-                load = [0] * pairs   # in the planner's cost units: k-blocks plus an allowance per unit
+                load = [0] * pairs   # in the planner's cost units: k-blocks, 5 for a unit of dweight, 1 (gelu' 2) for one of dinp
                 for pr, is_w, m, n, kb0, kb1 in recs:
                     assert 0 <= pr < pairs and kb0 < kb1
-                    load[pr] += kb1 - kb0 + (3 if is_w else (8 if gelu else 3))
+                    load[pr] += kb1 - kb0 + (5 if is_w else (2 if gelu else 1))
                     if is_w:
                         assert 0 <= m < wtm and 0 <= n < wtn and kb1 <= wkb
                         cov = w_cov.setdefault((m, n), [0] * wkb)
@@ -141,9 +141,9 @@ def test_layer_backward_plan_covers_every_unit_once(L):
                 assert len(w_cov) == wtm * wtn
                 assert all(c == [1] * wkb for c in w_cov.values())
                 if pairs > 1 and BT >= 4096:
-                    # level to within a few k-blocks (cuts are rounded to four, a cut unit pays
-                    # its allowance twice)
-                    assert max(load) - min(load) <= 16, (BT, C, OC, pairs, gelu, max(load), min(load))
+                    # the dearest pair is what counts: it has a few k-blocks more than the mean, as a range is worth its own
+                    # allowance and a piece at least (a pair with less, or nothing, is fewer pieces for all)
+                    assert max(load) <= sum(load) / pairs + 10, (BT, C, OC, pairs, gelu, max(load), sum(load) / pairs)
 
 
 def test_layer_backward_plan_on_drawn_shapes(L):
@@ -199,6 +199,21 @@ def _check_partition(hdr, recs, pairs, tag):
             assert (kb0, kb1) == (0, dkb), tag
             d_seen[m, n] += 1
     assert (d_seen == 1).all() and (w_cov == 1).all(), tag
+
+
+def test_layer_backward_plan_is_found_quickly(L):
+    """A program whose row count changes from step to step pays for a plan on every call: 5 to 20 us, where
+    a layer takes 15 or more on the GPU. (The limit leaves room for a slow or busy host.)"""
+    import time
+    out = (binding._int * (1 << 17))()
+    for BT, C, OC, flags in [(4096, 768, 2304, 2), (4096, 3072, 768, 3), (16384, 768, 768, 2), (16384, 768, 2304, 6), (16384, 3072, 768, 3),
+                             (16384, 1024, 1024, 2), (200000, 768, 768, 2), (171828, 456, 80, 6)]:
+        best = 1.0
+        for _ in range(20):
+            t0 = time.perf_counter()
+            assert L.nb_debug_layer_bwd_plan(BT, C, OC, 74, flags, out, len(out)) > 0
+            best = min(best, time.perf_counter() - t0)
+        assert best < 100e-6, (BT, C, OC, flags, best)
 
 
 @pytest.mark.parametrize("fresh", [False, True])
