@@ -87,14 +87,14 @@ struct PlanKey {
         return BT == o.BT && C == o.C && OC == o.OC && pairs == o.pairs && gelu_grad == o.gelu_grad && fresh == o.fresh;
     }
 };
-struct PlanKeyHash {
-    size_t operator()(const PlanKey &k) const
-    {
-        const uint64_t h = (static_cast<uint64_t>(k.BT) * 0x9E3779B97F4A7C15ull) ^ (static_cast<uint64_t>(k.C) * 0xBF58476D1CE4E5B9ull) ^
-                           (static_cast<uint64_t>(k.OC) * 0x94D049BB133111EBull) ^ (static_cast<uint64_t>(k.pairs) << 2) ^
-                           (static_cast<uint64_t>(k.gelu_grad) << 1) ^ static_cast<uint64_t>(k.fresh);
-        return static_cast<size_t>(h ^ (h >> 31));
-    }
+// The plans of the sizes used last: a model's layers at a few row counts. A program whose row count is new on every call replaces
+// the one that was not used for longest, and finds those of its other layers again.
+struct PlanCache {
+    static constexpr int kSlots = 64;
+    PlanKey keys[kSlots];
+    uint64_t used[kSlots];  // 0: empty
+    LayerBwdParams plans[kSlots];
+    uint64_t clock;
 };
 
 struct DeviceState {
@@ -104,7 +104,7 @@ struct DeviceState {
     void *workspace = nullptr;
     size_t workspace_bytes = 0;
     std::unordered_map<TmapKey, CUtensorMap, TmapKeyHash> tmaps;
-    std::unordered_map<PlanKey, LayerBwdParams, PlanKeyHash> plans;
+    PlanCache plans{};
 };
 
 std::mutex g_mu;
@@ -1358,19 +1358,27 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     return NB_OK;
 }
 
-// The plan of a launch. Finding one takes 5 to 20 us, so the plans of the last sizes are kept (they hold sizes only).
+// The plan of a launch. Finding one takes 5 to 20 us, so those of the sizes used last are kept (they hold sizes only).
 int cached_layer_bwd_plan(DeviceState &s, LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, bool gelu_grad, bool fresh)
 {
-    const PlanKey key{BT, C, OC, P, gelu_grad, fresh};
-    const auto it = s.plans.find(key);
-    if (it != s.plans.end()) {
-        p = it->second;
-        return NB_OK;
+    // fresh and added-to gradients differ in their plans only where a tile's whole K may be one unit
+    const int64_t tiles = ((OC + 255) / 256) * ((C + 255) / 256);
+    const PlanKey key{BT, C, OC, P, gelu_grad, fresh && (BT <= kMaxChunk * kBlockK || tiles >= 2 * P)};
+    PlanCache &c = s.plans;
+    int at = 0;
+    for (int i = 0; i < PlanCache::kSlots; ++i) {
+        if (c.used[i] && c.keys[i] == key) {
+            c.used[i] = ++c.clock;
+            p = c.plans[i];
+            return NB_OK;
+        }
+        if (c.used[i] < c.used[at]) at = i;
     }
-    const int rc = plan_layer_bwd(p, BT, C, OC, P, gelu_grad, true, fresh);
+    const int rc = plan_layer_bwd(p, BT, C, OC, P, gelu_grad, true, key.fresh);
     if (rc != NB_OK) return rc;
-    if (s.plans.size() >= 512) s.plans.clear();
-    s.plans.emplace(key, p);
+    c.keys[at] = key;
+    c.used[at] = ++c.clock;
+    c.plans[at] = p;
     return NB_OK;
 }
 

@@ -364,3 +364,19 @@ def test_long_sums_of_the_persistent_backward(BT, C, OC):
         error[rows] = float((dw.double() - ref).norm() / ref.norm())
     nb.nb_check_status()
     assert error[BT] <= 2 * error[1024], error
+
+
+def test_many_row_counts_of_the_persistent_backward():
+    """More sizes than the schedules that are kept, each twice over, so that the first ones are found again."""
+    C, OC, most = 1032, 2056, 2600
+    inp, w, dout = gen(1, (most, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (most, OC), 1e-3)
+    dinp = torch.empty((most, C), dtype=torch.bfloat16, device="cuda")
+    dw = torch.empty((OC, C), dtype=torch.float32, device="cuda")
+    for BT in list(range(most - 8 * 69, most + 1, 8)) * 2:
+        assert nb.nb_debug_route(nb.CALL_BACKWARD, BT, C, OC, dbias=False, accumulate=False)[0][0] == "layer_bwd"
+        nb.nb_linear_backward_ex(dinp[:BT], dw, None, dout[:BT], inp[:BT], w, None, None, BT, C, OC, nb.ACT_NONE, 0)
+        ref, dref = dout[:BT].double().t() @ inp[:BT].double(), dout[:BT].double() @ w.double()
+        # fp32 sums of at most 41 k-blocks: 1e-7 a k-block; dinp rounded to bf16 besides, 2^-9 at most
+        assert torch.dist(dw.double(), ref) <= 5e-6 * torch.linalg.norm(ref), BT
+        assert torch.dist(dinp[:BT].double(), dref) <= 2e-3 * torch.linalg.norm(dref), BT
+    nb.nb_check_status()
