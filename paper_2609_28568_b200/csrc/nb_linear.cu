@@ -1382,13 +1382,14 @@ int cached_layer_bwd_plan(DeviceState &s, LayerBwdParams &p, int64_t BT, int64_t
     return NB_OK;
 }
 
-// Whether the launch will store a fresh dweight. (It decides for the pairs that it finds room for; where those are not
-// half the SMs this may be wrong, and the gradient is cleared once too often or by a launch of its own.)
-bool layer_bwd_stores(DeviceState &s, int64_t BT, int64_t C, int64_t OC, bool gelu_grad)
+// Whether the launch will add to a fresh dweight, which then has to be cleared before it: not where it stores whole tiles, and not
+// where there is no such launch (the products by themselves start a fresh dweight their own way). (It decides for half the SMs as
+// pairs; where the launch finds room for fewer this may be wrong, and the gradient is cleared once too often or by a launch of its own.)
+bool layer_bwd_adds(DeviceState &s, int64_t BT, int64_t C, int64_t OC, bool gelu_grad)
 {
     LayerBwdParams p;
     const int P = s.num_sms / 2 < kMaxPairs ? s.num_sms / 2 : kMaxPairs;
-    return cached_layer_bwd_plan(s, p, BT, C, OC, P, gelu_grad, true) == NB_OK && p.w_whole;
+    return cached_layer_bwd_plan(s, p, BT, C, OC, P, gelu_grad, true) == NB_OK && !p.w_whole;
 }
 
 using LayerBwdPlain = LbCfg<false, false>;
@@ -1834,7 +1835,7 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
     float *clear_w = nullptr;
     if (act != NB_ACT_NONE) {
         if (dweight && dweight_dtype == NB_DTYPE_F32 && !accumulate && r.kernel == NB_ROUTE_LAYER_BWD &&
-            !layer_bwd_stores(*s, BT, C, OC, inp_pre_act != nullptr))
+            layer_bwd_adds(*s, BT, C, OC, inp_pre_act != nullptr))
             clear_w = static_cast<float *>(dweight);
         float *const clear_b = clear_w ? static_cast<float *>(dbias) : nullptr;
         const long long nw = clear_w ? static_cast<long long>(OC * C) : 0, nb_ = clear_b ? static_cast<long long>(OC) : 0;
