@@ -344,6 +344,33 @@ def test_fresh_gradients_of_the_persistent_backward(act, BT, C, OC, whole):
     nb.nb_check_status()
 
 
+@pytest.mark.parametrize("fused,bias", [(False, False), (True, True), (True, False)])
+@pytest.mark.parametrize("BT,C,OC,whole", [(1500, 1000, 1544, True), (1290, 1032, 4104, True), (2050, 520, 3080, True),
+                                           (1300, 2056, 1032, False)])
+def test_fresh_gradients_of_the_other_forms(fused, bias, BT, C, OC, whole):
+    """The same for the kernels with the producer's GELU derivative, whose fp32 results leave through a single box, and for
+    those without a bias gradient: stored or added to, in one part or several."""
+    assert nb.nb_debug_route(nb.CALL_BACKWARD, BT, C, OC, dbias=bias, gelu_grad=fused, accumulate=False)[0][0] == "layer_bwd"
+    pairs = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    hdr, recs = nb.nb_debug_layer_bwd_plan(BT, C, OC, pairs, fused, launched=True, fresh=True)
+    assert all(k1 - k0 == hdr[5] for _, is_w, _, _, k0, k1 in recs if is_w) == whole
+    inp, w, dout = gen(1, (BT, C), 1.0), gen(2, (OC, C), 0.05), gen(3, (BT, OC), 1e-3)
+    ipre = gen(4, (BT, C), 1.0) if fused else None
+    r = oracle.linear_backward(f32(dout), f32(inp), f32(w), inp_pre=f32(ipre) if fused else None)
+    dinp, dw = Guarded((BT, C), torch.bfloat16), Guarded((OC, C), torch.float32, fill=7.0)
+    db = Guarded((OC,), torch.float32, fill=float("nan")) if bias else None
+    for acc in range(2):
+        nb.nb_linear_backward_ex(dinp.t, dw.t, db.t if bias else None, dout, inp, w, None, ipre, BT, C, OC, nb.ACT_NONE, acc)
+        check_bf16(dinp.t, r["dinp"], "dinp")
+        check_f32(dw.t, (acc + 1) * r["dweight"], "dweight")
+        if bias:
+            check_f32(db.t, (acc + 1) * r["dbias"], "dbias")
+            db.check("dbias")
+    dinp.check("dinp")
+    dw.check("dweight")
+    nb.nb_check_status()
+
+
 @pytest.mark.parametrize("BT,C,OC", [(4096, 768, 3072), (8192, 768, 3072), (5000, 776, 2056)])
 def test_long_sums_of_the_persistent_backward(BT, C, OC):
     """The error of a sum in a tensor core's accumulator goes with its length, and the schedule promises sums of at most 32

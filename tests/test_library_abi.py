@@ -201,6 +201,33 @@ def _check_partition(hdr, recs, pairs, tag):
     assert (d_seen == 1).all() and (w_cov == 1).all(), tag
 
 
+def test_layer_backward_plan_of_fresh_and_launched_forms(L):
+    """The partition in the forms that are launched: dinp tiles halved where they are, gradients from nothing or added to, units and
+    the sums that they are made in. A plan whose dweight units are all a tile's whole K has one for each tile."""
+    import numpy as np
+    rng = np.random.default_rng(5)
+    whole = cut = 0
+    for case in range(160):
+        BT = int(rng.integers(129, 30_000)) if case % 3 else int(rng.integers(129, 2100))
+        C, OC = 8 * int(rng.integers(1, 400)), 8 * int(rng.integers(1, 700))
+        pairs, gelu, fresh = int(rng.choice((74, 66, 33, 7))), bool(rng.integers(0, 2)), bool(rng.integers(0, 4))
+        try:
+            hdr, recs = binding.nb_debug_layer_bwd_plan(BT, C, OC, pairs, gelu, launched=True, fresh=fresh)
+        except binding.NbError as e:
+            assert e.code == binding.NB_ERR_UNSUPPORTED
+            continue
+        tag = (BT, C, OC, pairs, gelu, fresh)
+        _check_partition(hdr, recs, pairs, tag)
+        _check_partition(hdr, binding.nb_debug_layer_bwd_plan(BT, C, OC, pairs, gelu, launched=True, fresh=fresh, sums=True)[1], pairs, tag)
+        units = [k1 - k0 for _, is_w, _, _, k0, k1 in recs if is_w]
+        if all(u == hdr[5] for u in units):
+            assert len(units) == hdr[3] * hdr[4], tag
+            whole += 1
+        else:
+            cut += 1
+    assert whole > 20 and cut > 60, (whole, cut)
+
+
 def test_layer_backward_plan_is_found_quickly(L):
     """A program whose row count changes from step to step pays for a plan on every call: 5 to 20 us, where
     a layer takes 15 or more on the GPU. (The limit leaves room for a slow or busy host.)"""
