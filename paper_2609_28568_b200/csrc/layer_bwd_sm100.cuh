@@ -1,16 +1,17 @@
 // Backward of one linear layer as ONE persistent launch for sm_100a:
 //
 //     dinp[BT, C]     = dz[BT, OC] . W[OC, C]        (x gelu'(inp_pre) in the epilogue, optional)
-//     dweight[OC, C] += dz^T[OC, BT] . inp[BT, C]    fp32, reduce-added
+//     dweight[OC, C] += dz^T[OC, BT] . inp[BT, C]    fp32, reduce-added (stored where it starts from nothing and no
+//                                                    tile is cut)
 //     dbias[OC]      += column sums of dz            fp32, optional
 //
 // Both products read dz, and neither depends on the other, so their work units share one list:
 // 256 x 256 tiles of dinp over the whole K = OC ("D units"), and 256 x 256 tiles of dweight over
 // a range of 64-row k-blocks of K = BT ("W units"; partial sums meet in memory through TMA
-// reduce-adds, so a W tile may be cut anywhere along K). A launch of its own for each product
+// reduce-adds, so a W tile may be cut anywhere along K; a fresh dweight whose tiles are all whole is stored). A launch of its own for each product
 // runs its last wave partly empty (16384 x 768 outputs are 192 tiles for 74 CTA pairs: 2.59
 // waves run as 3) and pays a start and an end; here the weight-gradient k-blocks fill what the
-// input-gradient tiles leave, every CTA pair gets the same amount of tensor-core work, and the
+// input-gradient tiles leave, no CTA pair gets much more tensor-core work than the mean, and the
 // long epilogue of a D unit (gelu') runs under the long main loop of a W unit.
 //
 // Schedule (computed on the host, see plan_layer_bwd): "rounds" of one unit per CTA pair, D rounds
@@ -73,8 +74,8 @@ struct LbUnit {
 // grows with its length, and all of it towards zero: an fp32 dweight over 4096 rows is off by 1.7e-6 (2-norm, standard normal
 // operands) where most of it is summed 32 k-blocks at a time and by 3.4e-6 where 64 at a time. So a W unit that is longer than the
 // plan's w_chain is summed in equal parts, in the two accumulators in turn, and the epilogue adds the parts in registers, rounding
-// to nearest, while the next part is being multiplied. Reading 128 KB of TMEM once more costs the tensor core 0.15 us a part
-// (every unit in four parts: 3.5 % of a launch), so the plan takes no more of them than it needs.
+// to nearest, while the next part is being multiplied: 1.2e-6. Each part reads 128 KB of TMEM once more (every unit in four
+// parts: 3.5 % of a launch; as planned: 0 to 0.3 %), so the plan takes no more of them than it needs.
 __host__ __device__ __forceinline__ int chain_len(const LbUnit &u, int w_chain)
 {
     const int len = u.kb1 - u.kb0;

@@ -1028,7 +1028,7 @@ bool layer_bwd_narrow(int d_tiles, int d_kblocks, int w_tiles, int w_kblocks, in
 // several of them 3 to 5 us behind the others.)
 constexpr int kCostD = 1, kCostDGelu = 2, kCostW = 5;
 constexpr int kMaxChunk = 64;  // k-blocks
-constexpr int kLbTries = 4;
+constexpr int kLbTries = 4;    // forms that are cut; 0.4 us each
 constexpr int kCostClear = 8;  // the launch that clears a fresh dweight, 2.5 to 3 us on the chain
 constexpr int kMinPiece = 2;  // k-blocks of a W unit that are worth a cut
 
@@ -1208,13 +1208,15 @@ LbSums sums_of(const LayerBwdParams &p, int w_chain)
 //     k-blocks and cut into P ranges at the lowest limit on a pair's cost at which cut_line finds a place for all of it.
 //  3. K = BT of the weight gradient is cut into chunks, as many as give two W units per pair or fewer, of 16 to kMaxChunk k-blocks
 //     where that leaves a choice. For each number of chunks and each number of W rounds that leaves the pairs with a tail
-//     D tile about level, the cost of a pair is estimated; the kLbTries cheapest are cut and the one with the cheapest dearest pair is taken.
-// Against ranges levelled one after the other with 3 k-blocks a unit, over about two chunks a pair of 32 k-blocks or more
-// (chained launches, accumulating, us): 4096 rows, 768 -> 768 16.3 -> 14.1, 768 -> 2304 27.0 -> 25.5, 1024 -> 6144 77.8 -> 73.6,
-// 3072 -> 1024 42.8 -> 40.0; 8192 rows, 768 -> 768 23.5 -> 20.4; 16384 rows, 768 -> 768 38.5 -> 34.9, 768 -> 2304
-// 90.9 -> 88.2. Chunks of up to 256 k-blocks cost 16384 rows, 768 -> 3072 4 % (the pairs drift apart).
-// fresh: dweight starts from nothing. Where every W unit is a tile's whole K it is stored and the clearing launch saved
-// (2021 rows, 768 -> 3072 22.7 -> 20.7 us, 768 -> 50304 298 -> 265; 1100 rows, 1024 -> 4096 34.3 -> 29.4), which is worth kCostClear.
+//     D tile about level, the cost of a pair is estimated; the kLbTries cheapest are cut and the one with the cheapest dearest pair
+//     is taken.
+//  4. Units that are longer than the one-pass schedule's sums are summed in parts (w_chain).
+// Against the one-pass schedule (level_layer_bwd; chains of single launches, below the power cap, accumulating, us): 4096 rows,
+// 768 -> 768 16.4 -> 14.4, 768 -> 2304 27.0 -> 26.1, 768 -> 3072 33.3 -> 31.4, 1024 -> 6144 78.9 -> 74.9; 8192 rows, 768 -> 3072
+// 62.8 -> 60.2; 16384 rows, 768 -> 768 36.6 -> 36.1, 768 -> 2304 91.2 -> 89.8 (no difference in a step at the cap). Chunks of up to
+// 256 k-blocks cost 16384 rows, 768 -> 3072 4 % (the pairs drift apart).
+// fresh: dweight starts from nothing. Where every W unit is a tile's whole K it is stored and the clearing launch saved (2021 rows,
+// 768 -> 2304 19.5 -> 17.7 us, 768 -> 3072 22.3 -> 19.9; 1100 rows, 1024 -> 4096 26.0 -> 23.5), which is worth kCostClear.
 // narrow (as it is launched): D tiles are 128 columns wide (layer_bwd_narrow; not with gelu') where the 256-wide ones are
 // at most a quarter of the pairs, K is long, and a single one takes longer than a pair's share of all the work: 1500 rows,
 // 768 -> 3072, 18 tiles of 48 k-blocks, 18.9 -> 16.4 us; 1024 rows, 1024 -> 6144, 32.5 -> 24.4 us. With
@@ -1262,7 +1264,8 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
     int max_chunks = (2 * P + p.w_tiles - 1) / p.w_tiles;
     if (max_chunks > p.w_kblocks / 16) max_chunks = p.w_kblocks / 16;
     if (max_chunks < 1) max_chunks = 1;
-    // The dearest pair counts and, where the chip is at its power limit, what all of them do.
+    // The dearest pair counts and, where the chip is at its power limit, what all of them do. (A judgement, not a fit: with 0.25 or
+    // 1 in the place of 0.5, 3 to 5 % of 3000 drawn sizes get another plan.)
     auto price = [&](double most, double sum, int rounds, int kbc) { return most + 0.5 * sum / P + 1.5 * rounds * (kbc + kCostW); };
     for (int want = 1; want <= max_chunks; ++want) {
         const int kbc = (p.w_kblocks + want - 1) / want;
@@ -1276,7 +1279,8 @@ int plan_layer_bwd(LayerBwdParams &p, int64_t BT, int64_t C, int64_t OC, int P, 
         const long long even = last == kbc ? w_units : w_units - p.w_tiles;
         const double mean = (1.0 * p.w_kblocks * p.w_tiles + 1.0 * kCostW * (w_units + P) + cD * p.d_tail) / P;
         long long hi = even / P;
-        if (p.d_tail && static_cast<long long>((mean - cD) / (kbc + kCostW)) + 1 < hi) hi = static_cast<long long>((mean - cD) / (kbc + kCostW)) + 1;
+        const long long below = static_cast<long long>((mean - cD) / (kbc + kCostW)) + 1;
+        if (p.d_tail && below < hi) hi = below;
         if (hi > kLbMaxRounds - p.d_rounds) hi = kLbMaxRounds - p.d_rounds;
         if (hi < 0) hi = 0;
         for (long long aW = hi; aW >= 0 && aW >= hi - 2; --aW) {
@@ -1538,7 +1542,9 @@ int run_forward(DeviceState &s, const GemmArgs &a, int act, cudaStream_t stream)
 
 // A layer's backward without the small-problem kernel: layer_bwd_kernel for both products, else a
 // launch per product. An fp32 result that starts from zero costs the clearing besides. (sms / 2: the CTA pairs that
-// the launch's occupancy query finds on B200.)
+// the launch's occupancy query finds on B200.) The launch has become cheaper than this says where it stores a fresh dweight and
+// where its ranges are level: from zero, 256 rows, 2048 -> 3072 takes 13.3 us with it and 17.8 in tiles, 768 rows, 3072 -> 768
+// 11.1 and 12.7 (with gelu' 12.4 and 15.6), and these still go to the tiles; 1003 rows, 776 -> 1416 13.6 and 12.6.
 double backward_us(int sms, int M, int BT, int N, int Mw, int kd, int kw, bool accumulate, bool apart, bool gelu)
 {
     const int slots = sms / 2;
@@ -1826,8 +1832,8 @@ int nb_linear_backward_ex(void *dinp, void *dweight, void *dbias, const void *do
 
     // dz: either dout itself, or dout times this layer's activation derivative (workspace)
     const void *dz = dout;
-    // The pass that forms dz also clears a dweight that layer_bwd_kernel adds to, which saves that launch (4096 rows,
-    // 1024 -> 6144 SwiGLU: 106 -> 96 us with the new schedule).
+    // The pass that forms dz also clears a dweight that layer_bwd_kernel adds to, which saves that launch (4096 rows, from zero,
+    // with the schedule: 1024 -> 6144 SwiGLU 104 -> 98 us, 768 -> 3072 GELU 49.4 -> 45.7).
     Route r;
     if (dweight && dweight_dtype == NB_DTYPE_F32)
         r = route_backward(s->num_sms, dinp != nullptr, dbias != nullptr, inp_pre_act != nullptr, accumulate != 0,
